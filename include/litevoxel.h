@@ -110,9 +110,9 @@ typedef struct {
 
 typedef struct {
   int32_t tile;           /* tile edge in pixels: 8, 16 or 32 */
-  int32_t batch;          /* list entries a warp stages per round (32, 64 or 128; 128 not with tile 32):
-                             their records are loaded together into the warp's shared-memory slice
-                             (64 B each) before its pixels march through them; changes no result */
+  int32_t batch;          /* 32, 64 or 128 (128 not with tile 32): once the list entries a warp staged per
+                             round; the composites now size their rounds themselves, so every value
+                             gives the same launch; changes no result */
   float t_stop;           /* a ray stops after the sample that takes T below t_stop (1e-4) */
   uint32_t flags;         /* LV_FLAG_* */
   int32_t persistent_sms; /* with LV_FLAG_PERSISTENT: run the composite on this many SMs (0 = all): the

@@ -14,16 +14,18 @@
 //               depth key.
 //   radix sort  the pairs by tile id (stable: each tile's list stays in
 //               voxel-id order); its last pass also notes every tile's range.
-//   k_tile_sort_warp, k_tile_sort, k_tile_merge  per tile: its slots sorted by depth key in
-//               shared memory (stable), so every tile's list ends front to back
-//               with ties by voxel id.  The depth keys are sorted per tile,
-//               where they fit in shared memory, instead of by global passes
-//               over all slots.
+//   k_tile_sort_warp, k_tile_sort  per tile: its slots sorted by depth key in
+//               shared memory (stable), front to back with ties by voxel id, and
+//               written with the pixel strips they meet; of very long lists only
+//               the front.  The depth keys are sorted per tile, where they fit
+//               in shared memory, instead of by global passes over all slots.
 //   k_fwd       per tile, one thread per pixel: each warp stages the records
 //               that meet its pixel strip through shared memory and marches
 //               front to back (Eq. 2-4); w_max (Eq. 5) is reduced over the
 //               warp before one global atomicMax; a warp stops when all its
 //               pixels have T < t_stop.
+//   k_tile_rest, k_fwd  the rest of the very long lists whose pixels are still
+//               open, and their march from there on.
 // lv_rasterize_backward walks the same lists back to front (k_bwd) and
 // reduces the SH colour gradient per voxel (k_sh_bwd).
 #include <math.h>
@@ -93,6 +95,14 @@ static void make_views(const lv_camera* cams, int nv, int ts, ViewSet* vs, int64
 }
 
 // ------------------------------------------------------------------ workspace
+// progress of a long tile's depth order
+struct TileProg {
+  uint32_t done;  // entries sorted
+  uint32_t next;  // smallest order key not sorted yet
+  uint32_t kmax;  // largest order key of the list
+  uint32_t open;  // 1: listed in open_tiles
+  uint32_t front; // where the resumed composite starts (list entry)
+};
 // items are (view, voxel) pairs in view-major order: item = view * n + voxel
 struct FwdWs {
   unsigned long long* counters;  // [0] pairs, [1] slots
@@ -106,14 +116,19 @@ struct FwdWs {
   uint2* rec_bb;                 // [slots] pixel box of the render record
   uint32_t* slot_vox;            // [slots] voxel id of the render record
   uint32_t* s_dkey;              // [slots] order key
-  unsigned int* work;            // [16] work-item counters: [0..1] the persistent composites, [2] count
-                                 // of the long tiles' chunks, [3] the merge's work counter, [4..5] count
-                                 // of the medium tiles and k_tile_sort's work counter, [6] count of the
-                                 // long tiles; [8..9] block arrivals of the persistent forward and
-                                 // backward composites (sm_leave)
-  uint2* chunks;                 // [pair capacity / TS_CHUNK + tiles] (tile, chunk) of the long tiles
+  unsigned int* work;            // [16] work-item counters: [0..1] the persistent composites, [2] the
+                                 // resumed composite, [3] k_tile_rest, [4..5] count of the medium tiles
+                                 // and k_tile_sort's work counter, [6] count of the long tiles, [7] count
+                                 // of the open tiles, [11] count of the short tiles; [8..10] block arrivals of the persistent forward,
+                                 // backward and resumed composites (sm_leave)
   uint32_t* mid_tiles;           // [tiles] tiles of medium-length lists
   uint32_t* long_tiles;          // [tiles] tiles of long lists
+  uint32_t* short_tiles;         // [tiles] the other tiles
+  uint32_t* open_tiles;          // [tiles] long tiles with pixels open at the end of the sorted part
+  uint32_t* ready;               // [tiles] end of the list's depth-sorted part
+  TileProg* prog;                // [tiles] progress of the long tiles' depth order
+  float* dep;                    // [pixels] depth and sample count of the pixels of open tiles
+  uint32_t* nsamp;
   void* scan_tmp;
   float4* rec;                   // [slots][4]
   float4* d_rgb;                 // [slots] colour gradient (xyz) scratch of the backward; w = clamp mask
@@ -122,6 +137,7 @@ struct FwdWs {
   void* sort_tmp;                // scratch of the sort by tile
   int32_t* status;               // fallback status word
   uint32_t *k0, *v0, *k1, *v1;   // [pair capacity] (tile, slot) pairs, sorted by tile
+  uint2* plist;                  // [pair capacity] (slot, strip mask) of every tile's list in depth order
   size_t bytes;
 };
 
@@ -146,32 +162,34 @@ static FwdWs carve_fwd(void* base, int64_t n, int nv, int64_t tiles, int64_t pix
   w.rec = c.take<float4>(items * 4);
   w.d_rgb = c.take<float4>(items);
   w.ranges = c.take<uint32_t>(tiles * 2);
-  w.chunks = c.take<uint2>(pair_cap / 4096 + tiles);
   w.mid_tiles = c.take<uint32_t>(tiles);
   w.long_tiles = c.take<uint32_t>(tiles);
+  w.short_tiles = c.take<uint32_t>(tiles);
+  w.open_tiles = c.take<uint32_t>(tiles);
+  w.ready = c.take<uint32_t>(tiles);
+  w.prog = c.take<TileProg>(tiles);
+  w.dep = c.take<float>(pixels);
+  w.nsamp = c.take<uint32_t>(pixels);
   w.tau = c.take<float>(pixels);
   w.sort_tmp = c.take<char>(sort_tmp_bytes(pair_cap));
   w.k0 = c.take<uint32_t>(pair_cap);
   w.v0 = c.take<uint32_t>(pair_cap);
   w.k1 = c.take<uint32_t>(pair_cap);
   w.v1 = c.take<uint32_t>(pair_cap);
+  w.plist = c.take<uint2>(pair_cap);
   w.bytes = c.off + 256;
   return w;
 }
 
-// the sorted (tile, slot) pairs: in (k0, v0) after an even number of tile-digit passes
+// the slots of the pairs sorted by tile (item order within a tile): in v0 after an even number of tile-digit passes
 static int tile_bits(int64_t tiles) {
   int b = 0;
   while (b < 32 && ((int64_t)1 << b) < tiles) ++b;
   return b;
 }
-static const uint32_t* sorted_pair_slots(const FwdWs& w, int64_t tiles) {
+static const uint32_t* tile_pair_slots(const FwdWs& w, int64_t tiles) {
   return (sort_passes(tile_bits(tiles)) & 1) ? w.v1 : w.v0;
 }
-static const uint32_t* sorted_pair_tiles(const FwdWs& w, int64_t tiles) {
-  return (sort_passes(tile_bits(tiles)) & 1) ? w.k1 : w.k0;
-}
-static void launch_tile_sort(const FwdWs& w, int64_t tiles, int64_t pair_cap, cudaStream_t s);
 
 
 // ------------------------------------------------------------------ binning (FP32, fixed op order)
@@ -523,25 +541,37 @@ __device__ __forceinline__ int64_t usable_pairs(const unsigned long long* d_coun
 // ------------------------------------------------------------------ per-tile depth order
 // After the stable sort by tile id, each tile's pairs are in item order (voxel
 // id within a view), and the sort's last pass has left every tile's range in
-// ranges (empty tiles: (0xffffffff, 0)).  Each tile's slots are then sorted by
-// order key: an LSD radix sort of 9-bit digits of the key minus the tile's
-// smallest key (a tile whose keys span less than 2^27 takes 3 passes).  Each
-// pass ranks stably (warp-private digit counts; the lanes holding a digit
-// found by bit ballots or by __match_any_sync), so equal keys keep item order,
-// and each tile's list ends front to back with ties by voxel id: the order one
-// stable sort of (tile, order key) pairs in voxel-id order gives.  The tiles
-// are shared out by list length:
+// ranges (empty tiles: (0xffffffff, 0)).  Each tile's slots are then put in
+// order of their keys, ties in item order, and written with their strip masks
+// to plist: the order one stable sort of (tile, order key) pairs in voxel-id
+// order gives.  A list is sorted in shared memory, by an LSD radix sort of
+// 9-bit digits of the key minus the smallest key (3 passes for spans below
+// 2^27).  Each pass ranks stably (warp-private digit counts; the lanes holding
+// a digit found by bit ballots or by __match_any_sync).  The tiles are shared
+// out by list length:
 //   k_tile_sort_warp  one warp per tile: lists of up to TW_MAX pairs; it also
 //                     writes every tile's range in final form (empty: (0, 0))
 //                     and lists the longer tiles;
-//   k_tile_sort       persistent blocks of 512 threads: lists of up to
-//                     TS_CHUNK pairs in place, and longer lists cut into
-//                     chunks of TS_CHUNK pairs, each sorted into a scratch
-//                     copy of the pair arrays;
-//   k_tile_merge      persistent blocks over the long tiles: the sorted chunks
-//                     merged stably (equal keys of earlier chunks first).
+//   k_tile_sort       persistent blocks of 512 threads: lists of up to TS_CHUNK
+//                     pairs in one go, longer ones range of keys by range of
+//                     keys, and of those above TS_LAZY only the front, the
+//                     TS_FRONT to TS_CHUNK nearest pairs;
+//   k_tile_rest       the rest of those whose pixels are still open after the
+//                     composite of the sorted parts.
+// Opaque scenes seldom read a long list past its front: of eight 980 x 545
+// views of 6M voxels with tile 32 (lists of up to 68,000 pairs, 38M in all) 2-5 %
+// of the tiles do.  Sorting every list whole, in chunks merged afterwards, took
+// 4.7 ms of those views' 8.2 ms.  Lists of a few chunks are sorted whole: where
+// their pixels stay open, the composite in two launches costs more than the sort
+// saves (one 1237 x 822 view of 2M voxels, lists of up to 7,800 pairs: 217 + 151 us
+// against 297 us).  Scenes of up to TS_LAZY_VOXELS seldom have longer lists, and go
+// without the two launches that the rest takes (6 us when there is none).
 constexpr int TS_BITS = 9, TS_BINS = 1 << TS_BITS;
 constexpr int TS_THREADS = 512, TS_WARPS = TS_THREADS / 32, TS_ITEMS = 8, TS_CHUNK = TS_THREADS * TS_ITEMS;
+constexpr int TS_FRONT = 2048;                      // pairs of a long list sorted at first (at least, if its keys allow)
+constexpr uint32_t TS_LAZY = 4 * TS_CHUNK;          // lists up to here are sorted whole at once
+constexpr int64_t TS_LAZY_VOXELS = 1 << 19;         // and all lists of scenes up to here
+constexpr int TL_BITS = 11, TL_BINS = 1 << TL_BITS;  // key histogram of a long list
 constexpr int TW_MAX = 256, TW_ITEMS = TW_MAX / 32, TW_WARPS = 16;
 static_assert(TS_THREADS == TS_BINS, "a thread for each digit");
 
@@ -562,10 +592,10 @@ struct WarpSortSmem {
 struct TileSortWarpSmem {
   WarpSortSmem w[TW_WARPS];
 };
-struct TileMergeSmem {
-  uint32_t k[2][2 * TS_CHUNK];  // two runs side by side, then the first merge's output
-  uint32_t v[2][2 * TS_CHUNK];
-  uint32_t item;
+struct TileLongSmem {
+  TileSortSmem s;
+  uint32_t inc[TL_BINS];  // keys of a bin or an earlier one
+  uint32_t b0, b1;
 };
 
 // exclusive scan of one value per thread over a block of WARPS warps
@@ -649,41 +679,86 @@ __device__ __forceinline__ int ts_passes(uint32_t span) {
   return span ? (32 - __clz(span) + TS_BITS - 1) / TS_BITS : 0;
 }
 
+// The strips (4 x 8 pixel blocks, one warp of a composite each) of a tile that a
+// pixel box meets, as a bit mask: bit s for strip s, ts / 8 strips across.  The
+// sorted list carries it beside the slot, so a composite's warp finds its
+// records from one coalesced 8-byte word per entry.  Before, every one of a
+// tile's 2, 8 or 32 warps gathered the pixel box of every entry by slot; the
+// gather is now done once per pair, where the sorted list is written.
+struct TileBox {
+  int x0, y0;   // the tile's first pixel
+  int cshift;   // log2 of the strips across: ts = 8 << cshift
+  __device__ __forceinline__ TileBox(const ViewSet& vs, uint32_t gtile) {
+    int v = 0;
+    while (v + 1 < vs.n && (int)gtile >= vs.v[v + 1].tile_off) ++v;
+    const int lt = (int)gtile - vs.v[v].tile_off, tx = vs.v[v].tiles_x;
+    x0 = (lt % tx) * vs.ts;
+    y0 = (lt / tx) * vs.ts;
+    cshift = vs.ts == 8 ? 0 : (vs.ts == 16 ? 1 : 2);
+  }
+  // box: (bx0 | bx1 << 16, by0 | by1 << 16), [bx0, bx1) x [by0, by1)
+  __device__ __forceinline__ uint32_t mask(uint2 box) const {
+    const int ts = 8 << cshift;
+    const int bx0 = max((int)(box.x & 0xffffu) - x0, 0), bx1 = min((int)(box.x >> 16) - x0, ts);
+    const int by0 = max((int)(box.y & 0xffffu) - y0, 0), by1 = min((int)(box.y >> 16) - y0, ts);
+    if (bx1 <= bx0 || by1 <= by0) return 0u;
+    const uint32_t cols = (1u << ((bx1 + 7) >> 3)) - (1u << (bx0 >> 3));
+    const int r0 = (by0 >> 2) << cshift, r1 = ((by1 + 3) >> 2) << cshift;  // bit range [r0, r1) of the rows
+    const uint32_t rows = ((r1 < 32 ? 1u << r1 : 0u) - (1u << r0)) &
+                          (cshift == 0 ? 0xffffffffu : (cshift == 1 ? 0x55555555u : 0x11111111u));
+    return rows * cols;  // the column bits at every row: no carries, cols < 2^(strips across)
+  }
+};
+
 // ---- short lists: one warp each, TW_WARPS tiles per block
-__global__ void __launch_bounds__(TW_WARPS * 32, 2) k_tile_sort_warp(uint32_t* __restrict__ tvals,
+__global__ void __launch_bounds__(TW_WARPS * 32, 2) k_tile_sort_warp(const uint32_t* __restrict__ tvals,
                                                                     const uint32_t* __restrict__ s_dkey,
                                                                     const unsigned long long* __restrict__ d_count,
                                                                     int64_t cap, bool ranges_ready, int64_t tiles,
                                                                     uint32_t* __restrict__ ranges,
                                                                     uint32_t* __restrict__ mid_tiles,
                                                                     unsigned int* __restrict__ n_mid,
-                                                                    uint2* __restrict__ chunks,
-                                                                    unsigned int* __restrict__ n_chunks,
                                                                     uint32_t* __restrict__ long_tiles,
-                                                                    unsigned int* __restrict__ n_long) {
+                                                                    unsigned int* __restrict__ n_long,
+                                                                    uint32_t* __restrict__ short_tiles,
+                                                                    unsigned int* __restrict__ n_short,
+                                                                    uint32_t* __restrict__ ready,
+                                                                    TileProg* __restrict__ prog,
+                                                                    const __grid_constant__ ViewSet vs,
+                                                                    const uint2* __restrict__ rec_bb,
+                                                                    uint2* __restrict__ plist) {
   extern __shared__ __align__(16) unsigned char tw_raw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   WarpSortSmem& W = reinterpret_cast<TileSortWarpSmem*>(tw_raw)->w[warp];
+  __shared__ uint32_t s_cnt[3], s_at[3];
   const int64_t tile64 = (int64_t)blockIdx.x * TW_WARPS + warp;
-  if (tile64 >= tiles) return;  // warp-uniform; no block-wide barrier below
   const uint32_t tile = (uint32_t)tile64;
-  uint32_t lo = 0, hi = 0;
-  if (lane == 0) {
+  uint32_t lo = 0, hi = 0, at = 0;
+  int cls = 0;  // 0 short, 1 medium, 2 long
+  if (threadIdx.x < 3) s_cnt[threadIdx.x] = 0u;
+  __syncthreads();
+  if (lane == 0 && tile64 < tiles) {
     ts_range(ranges, tile, usable_pairs(d_count, cap), ranges_ready, &lo, &hi);
     reinterpret_cast<uint2*>(ranges)[tile] = make_uint2(lo, hi);
     const uint32_t L = hi - lo;
-    if (L > (uint32_t)TS_CHUNK) {
-      const uint32_t nc = (L + TS_CHUNK - 1) / TS_CHUNK;
-      const uint32_t at = atomicAdd(n_chunks, nc);
-      for (uint32_t c = 0; c < nc; ++c) chunks[at + c] = make_uint2(tile, c);
-      long_tiles[atomicAdd(n_long, 1u)] = tile;
-    } else if (L > (uint32_t)TW_MAX) {
-      mid_tiles[atomicAdd(n_mid, 1u)] = tile;
-    }
+    ready[tile] = hi;
+    cls = L > (uint32_t)TS_CHUNK ? 2 : (L > (uint32_t)TW_MAX ? 1 : 0);
+    if (cls == 2) prog[tile].open = 0u;
+    at = atomicAdd(&s_cnt[cls], 1u);
   }
+  __syncthreads();
+  // the tiles by length class, for the longer lists' sorts and the composites' order of work
+  if (threadIdx.x < 3) {
+    unsigned int* n_cls = threadIdx.x == 0 ? n_short : (threadIdx.x == 1 ? n_mid : n_long);
+    s_at[threadIdx.x] = s_cnt[threadIdx.x] ? atomicAdd(n_cls, s_cnt[threadIdx.x]) : 0u;
+  }
+  __syncthreads();
+  if (tile64 >= tiles) return;  // warp-uniform; no block-wide barrier below
+  if (lane == 0) (cls == 0 ? short_tiles : (cls == 1 ? mid_tiles : long_tiles))[s_at[cls] + at] = tile;
   lo = __shfl_sync(FULL, lo, 0);
   const int L = (int)(__shfl_sync(FULL, hi, 0) - lo);
-  if (L < 2 || L > TW_MAX) return;  // warp-uniform
+  if (L < 1 || L > TW_MAX) return;  // warp-uniform
+  const TileBox tb(vs, tile);
   const int R = (L + 31) / 32;
   uint32_t mn = ~0u, mx = 0u;
   {
@@ -712,8 +787,7 @@ __global__ void __launch_bounds__(TW_WARPS * 32, 2) k_tile_sort_warp(uint32_t* _
   }
   const uint32_t kmin = __reduce_min_sync(FULL, mn);
   const int npass = ts_passes(__reduce_max_sync(FULL, mx) - kmin);
-  if (npass == 0) return;  // warp-uniform: all keys equal, item order is the order
-  __syncwarp();
+  __syncwarp();  // no pass (one pair, or all keys equal): item order is the order
   int cur = 0;
   for (int pass = 0; pass < npass; ++pass) {
     const int shift = TS_BITS * pass;
@@ -772,53 +846,28 @@ __global__ void __launch_bounds__(TW_WARPS * 32, 2) k_tile_sort_warp(uint32_t* _
   for (int j = 0; j < TW_ITEMS; ++j) {
     if (j >= R) break;
     const int q = j * 32 + lane;
-    if (q < L) tvals[lo + q] = W.v[cur][q];
+    if (q < L) {
+      const uint32_t v = W.v[cur][q];
+      plist[lo + q] = make_uint2(v, tb.mask(rec_bb[v]));
+    }
   }
 }
 
-// Sorts m <= TS_CHUNK slots src[0, m) by order key with the whole block; the
-// sorted slots go to out_v[0, m) (which may be src) and, when out_k is not
-// null, their keys to out_k[0, m).  Returns with the block in step.
-__device__ __forceinline__ void ts_sort_chunk(TileSortSmem& S, const uint32_t* src,
-                                              const uint32_t* __restrict__ s_dkey, int m, uint32_t* out_k,
-                                              uint32_t* out_v) {
+// the blocks' shared memory, named in each function (not handed down as a
+// pointer) so that calls keep its address space
+__device__ __forceinline__ TileLongSmem& ts_smem() {
+  extern __shared__ __align__(16) unsigned char ts_raw[];
+  return *reinterpret_cast<TileLongSmem*>(ts_raw);
+}
+
+// Sorts the m <= TS_CHUNK (key, slot) pairs of S by key, stably, with the whole
+// block (all of it past a barrier since they were written, and S.kmin and S.kmax
+// their extremes), and writes (slot, strip mask) to plist[0, m).
+__device__ __noinline__ void ts_sort_smem(int m, const TileBox& tb, const uint2* __restrict__ rec_bb,
+                                          uint2* __restrict__ plist) {
+  TileSortSmem& S = ts_smem().s;
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  if (t == 0) {
-    S.kmin = ~0u;
-    S.kmax = 0u;
-  }
-  __syncthreads();
   const int R = (m + TS_THREADS - 1) / TS_THREADS;  // items per thread, and rounds per warp
-  {
-    // every slot load, then every key load, in flight at once
-    uint32_t kk[TS_ITEMS], vv[TS_ITEMS];
-#pragma unroll
-    for (int j = 0; j < TS_ITEMS; ++j) {
-      if (j >= R) break;
-      const int q = t + j * TS_THREADS;
-      vv[j] = q < m ? src[q] : 0u;
-    }
-#pragma unroll
-    for (int j = 0; j < TS_ITEMS; ++j) {
-      if (j >= R) break;
-      const int q = t + j * TS_THREADS;
-      kk[j] = q < m ? s_dkey[vv[j]] : 0u;
-    }
-    uint32_t mn = ~0u, mx = 0u;
-#pragma unroll
-    for (int j = 0; j < TS_ITEMS; ++j) {
-      if (j >= R) break;
-      const int q = t + j * TS_THREADS;
-      if (q < m) {
-        S.k[q] = kk[j];
-        S.v[q] = vv[j];
-        mn = min(mn, kk[j]);
-        mx = max(mx, kk[j]);
-      }
-    }
-    ts_min_max(mn, mx, &S.kmin, &S.kmax);
-  }
-  __syncthreads();
   const uint32_t kmin = S.kmin;
   const int npass = ts_passes(S.kmax - kmin);
   for (int pass = 0; pass < npass; ++pass) {
@@ -862,169 +911,320 @@ __device__ __forceinline__ void ts_sort_chunk(TileSortSmem& S, const uint32_t* s
     __syncthreads();
   }
   for (int q = t; q < m; q += TS_THREADS) {
-    out_v[q] = S.v[q];
-    if (out_k) out_k[q] = S.k[q];
+    const uint32_t v = S.v[q];
+    plist[q] = make_uint2(v, tb.mask(rec_bb[v]));
   }
 }
 
-// Persistent blocks over the medium tiles (sorted in place), then over the
-// chunks of the long tiles (sorted into the scratch arrays xk, xv at the
-// chunk's own positions).
-__global__ void __launch_bounds__(TS_THREADS, 2) k_tile_sort(uint32_t* __restrict__ tvals,
-                                                            uint32_t* __restrict__ xk, uint32_t* __restrict__ xv,
+// a whole list of m <= TS_CHUNK slots
+__device__ __noinline__ void ts_sort_list(const uint32_t* __restrict__ src, const uint32_t* __restrict__ s_dkey,
+                                          int m, const TileBox& tb, const uint2* __restrict__ rec_bb,
+                                          uint2* __restrict__ plist) {
+  TileSortSmem& S = ts_smem().s;
+  const int t = threadIdx.x;
+  if (t == 0) {
+    S.kmin = ~0u;
+    S.kmax = 0u;
+  }
+  __syncthreads();
+  const int R = (m + TS_THREADS - 1) / TS_THREADS;
+  // every slot load, then every key load, in flight at once
+  uint32_t kk[TS_ITEMS], vv[TS_ITEMS];
+#pragma unroll
+  for (int j = 0; j < TS_ITEMS; ++j) {
+    if (j >= R) break;
+    const int q = t + j * TS_THREADS;
+    vv[j] = q < m ? src[q] : 0u;
+  }
+#pragma unroll
+  for (int j = 0; j < TS_ITEMS; ++j) {
+    if (j >= R) break;
+    const int q = t + j * TS_THREADS;
+    kk[j] = q < m ? s_dkey[vv[j]] : 0u;
+  }
+  uint32_t mn = ~0u, mx = 0u;
+#pragma unroll
+  for (int j = 0; j < TS_ITEMS; ++j) {
+    if (j >= R) break;
+    const int q = t + j * TS_THREADS;
+    if (q < m) {
+      S.k[q] = kk[j];
+      S.v[q] = vv[j];
+      mn = min(mn, kk[j]);
+      mx = max(mx, kk[j]);
+    }
+  }
+  ts_min_max(mn, mx, &S.kmin, &S.kmax);
+  __syncthreads();
+  ts_sort_smem(m, tb, rec_bb, plist);
+}
+
+// The entries of a long list with keys in [k0, k1], in item order: to S as
+// (key, slot) with their extremes (there are at most TS_CHUNK of them), or, with
+// ALL_EQUAL, straight to plist (any number: one key, so item order is the order).
+template <bool ALL_EQUAL>
+__device__ __forceinline__ void tl_collect(TileSortSmem& S, const uint32_t* __restrict__ sv,
+                                           const uint32_t* xk, uint32_t L, uint32_t k0, uint32_t k1,
+                                           const TileBox& tb, const uint2* __restrict__ rec_bb,
+                                           uint2* __restrict__ plist) {
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  if (t == 0) {
+    S.kmin = ~0u;
+    S.kmax = 0u;
+  }
+  uint32_t at = 0, mn = ~0u, mx = 0u;
+  for (uint32_t base = 0; base < L; base += TS_CHUNK) {  // block-uniform
+    // warp w takes entries [base + 256 w, + 256), 32 at a time
+    uint32_t k[TS_ITEMS], in[TS_ITEMS], c = 0;
+    const uint32_t e0 = base + warp * 32 * TS_ITEMS + lane;
+#pragma unroll
+    for (int j = 0; j < TS_ITEMS; ++j) k[j] = e0 + 32 * j < L ? xk[e0 + 32 * j] : 0u;
+#pragma unroll
+    for (int j = 0; j < TS_ITEMS; ++j) {
+      in[j] = __ballot_sync(FULL, e0 + 32 * j < L && k[j] >= k0 && k[j] <= k1);
+      c += __popc(in[j]);
+    }
+    __syncthreads();  // the last round's counts are read
+    if (lane == 0) S.w[warp] = c;
+    __syncthreads();
+    uint32_t pos = at;
+#pragma unroll
+    for (int w = 0; w < TS_WARPS; ++w) {
+      const uint32_t x = S.w[w];
+      pos += w < warp ? x : 0u;
+      at += x;
+    }
+#pragma unroll
+    for (int j = 0; j < TS_ITEMS; ++j) {
+      if ((in[j] >> lane) & 1u) {
+        const uint32_t q = pos + __popc(in[j] & ((1u << lane) - 1u)), v = sv[e0 + 32 * j];
+        if (ALL_EQUAL) {
+          plist[q] = make_uint2(v, tb.mask(rec_bb[v]));
+        } else {
+          S.k[q] = k[j];
+          S.v[q] = v;
+          mn = min(mn, k[j]);
+          mx = max(mx, k[j]);
+        }
+      }
+      pos += __popc(in[j]);
+    }
+  }
+  if (!ALL_EQUAL) ts_min_max(mn, mx, &S.kmin, &S.kmax);
+  __syncthreads();
+}
+
+// Depth order of a long list, nearest entries first: a histogram of the keys not
+// sorted yet cuts them into ranges of at most TS_CHUNK entries, and each range is
+// collected in item order and sorted in shared memory.  A bin of more than
+// TS_CHUNK entries is cut by a finer histogram of its own keys; once a bin is one
+// key, item order is the order.  START: the keys are gathered first (to xk), and above
+// `lazy` entries the work stops after one range, of TS_FRONT entries or more where the
+// bins allow it; else it goes on from the progress of such a start.
+template <bool START>
+__device__ __noinline__ void tl_order(uint32_t lo, uint32_t L, uint32_t lazy, const uint32_t* __restrict__ sv_all,
+                         uint32_t* xk_all, const uint32_t* __restrict__ s_dkey, TileProg* prog,
+                         uint32_t* ready, const TileBox& tb, const uint2* __restrict__ rec_bb,
+                         uint2* __restrict__ plist_all) {
+  TileLongSmem& M = ts_smem();
+  TileSortSmem& S = M.s;
+  const int t = threadIdx.x;
+  const uint32_t* sv = sv_all + lo;
+  uint32_t* xk = xk_all + lo;
+  uint2* plist = plist_all + lo;
+  uint32_t done, cur, kmax;
+  const bool front = START && L > lazy;
+  if (START) {
+    if (t == 0) {
+      S.kmin = ~0u;
+      S.kmax = 0u;
+    }
+    __syncthreads();
+    uint32_t mn = ~0u, mx = 0u;
+    for (uint32_t base = t; base < L; base += TS_CHUNK) {
+      uint32_t v[TS_ITEMS], k[TS_ITEMS];
+#pragma unroll
+      for (int j = 0; j < TS_ITEMS; ++j) v[j] = base + j * TS_THREADS < L ? sv[base + j * TS_THREADS] : 0u;
+#pragma unroll
+      for (int j = 0; j < TS_ITEMS; ++j) k[j] = base + j * TS_THREADS < L ? s_dkey[v[j]] : 0u;
+#pragma unroll
+      for (int j = 0; j < TS_ITEMS; ++j)
+        if (base + j * TS_THREADS < L) {
+          xk[base + j * TS_THREADS] = k[j];
+          mn = min(mn, k[j]);
+          mx = max(mx, k[j]);
+        }
+    }
+    ts_min_max(mn, mx, &S.kmin, &S.kmax);
+    __syncthreads();  // also orders the block's writes of xk before its reads below
+    done = 0u;
+    cur = S.kmin;
+    kmax = S.kmax;
+  } else {
+    done = prog->done;
+    cur = prog->next;
+    kmax = prog->kmax;
+  }
+  uint32_t top = kmax;  // keys [cur, top] are cut by one histogram
+  while (done < L) {    // block-uniform
+    const uint32_t span = top - cur;
+    const int shift = span < (uint32_t)TL_BINS ? 0 : 32 - __clz(span) - TL_BITS;
+    for (int x = t; x < TL_BINS; x += TS_THREADS) M.inc[x] = 0u;
+    __syncthreads();
+    for (uint32_t base = t; base < L; base += TS_CHUNK) {
+      uint32_t k[TS_ITEMS];
+#pragma unroll
+      for (int j = 0; j < TS_ITEMS; ++j) k[j] = base + j * TS_THREADS < L ? xk[base + j * TS_THREADS] : 0u;
+#pragma unroll
+      for (int j = 0; j < TS_ITEMS; ++j)
+        if (base + j * TS_THREADS < L && k[j] >= cur && k[j] <= top) atomicAdd(&M.inc[(k[j] - cur) >> shift], 1u);
+    }
+    __syncthreads();
+    {
+      constexpr int PER = TL_BINS / TS_THREADS;
+      uint32_t c[PER], sum = 0;
+#pragma unroll
+      for (int i = 0; i < PER; ++i) sum += c[i] = M.inc[PER * t + i];
+      uint32_t run = ts_block_excl<TS_WARPS>(sum, S.w);
+#pragma unroll
+      for (int i = 0; i < PER; ++i) M.inc[PER * t + i] = run += c[i];
+    }
+    __syncthreads();
+    const uint32_t total = M.inc[TL_BINS - 1];
+    uint32_t b0 = 0, cum = 0;
+    bool finer = false;
+    while (cum < total) {  // block-uniform
+      if (t == 0) {
+        // bins [b0, b1): as many as fit (b1 == b0: bin b0 alone does not), and for the front no more
+        // than reach TS_FRONT
+        auto count_upto = [&](uint32_t limit) {  // bins with inc <= limit
+          uint32_t n = 0;
+          for (uint32_t step = TL_BINS; step; step >>= 1)
+            if (n + step <= (uint32_t)TL_BINS && M.inc[n + step - 1] <= limit) n += step;
+          return n;
+        };
+        uint32_t b1 = count_upto(cum + TS_CHUNK);
+        if (front) b1 = min(b1, count_upto(cum + TS_FRONT - 1) + 1u);
+        M.b0 = count_upto(cum);  // past empty bins, so that an oversized bin is met as b0
+        M.b1 = b1;
+      }
+      __syncthreads();
+      b0 = M.b0;
+      const uint32_t b1 = M.b1;
+      __syncthreads();
+      if (b1 > b0) {
+        const uint32_t k0 = cur + (b0 << shift);
+        const uint32_t k1 = b1 < (uint32_t)TL_BINS && top - cur >= b1 << shift ? cur + ((b1 << shift) - 1u) : top;
+        const uint32_t m = M.inc[b1 - 1] - cum;
+        tl_collect<false>(S, sv, xk, L, k0, k1, tb, rec_bb, plist);
+        ts_sort_smem((int)m, tb, rec_bb, plist + done);
+        __syncthreads();  // S is reused
+        done += m;
+        cum += m;
+        b0 = b1;
+        if (front) {
+          if (t == 0) {
+            prog->done = done;
+            prog->next = k1 + 1u;
+            prog->kmax = kmax;
+            *ready = lo + done;
+          }
+          return;
+        }
+      } else if (shift == 0) {  // one key with more entries than TS_CHUNK
+        const uint32_t m = M.inc[b0] - cum;
+        tl_collect<true>(S, sv, xk, L, cur + b0, cur + b0, tb, rec_bb, plist + done);
+        done += m;
+        cum += m;
+        const uint32_t k1 = cur + b0;
+        ++b0;
+        if (front) {
+          if (t == 0) {
+            prog->done = done;
+            prog->next = k1 + 1u;
+            prog->kmax = kmax;
+            *ready = lo + done;
+          }
+          return;
+        }
+      } else {  // the bin's own keys, finer
+        cur += b0 << shift;
+        if (top - cur >= 1u << shift) top = cur + ((1u << shift) - 1u);
+        finer = true;
+        break;
+      }
+    }
+    if (!finer) {  // everything up to top is sorted
+      cur = top + 1u;
+      top = kmax;
+    }
+  }
+  if (t == 0) {
+    prog->done = done;
+    prog->next = prog->kmax = kmax;
+    *ready = lo + done;
+  }
+}
+
+// Persistent blocks over the long tiles (their fronts; first, as they take
+// longest), then over the medium tiles.
+__global__ void __launch_bounds__(TS_THREADS, 2) k_tile_sort(const uint32_t* __restrict__ tvals,
+                                                            uint32_t* xk,
                                                             const uint32_t* __restrict__ s_dkey,
                                                             const uint32_t* __restrict__ ranges,
                                                             const uint32_t* __restrict__ mid_tiles,
                                                             const unsigned int* __restrict__ n_mid,
-                                                            const uint2* __restrict__ chunks,
-                                                            const unsigned int* __restrict__ n_chunks,
-                                                            unsigned int* __restrict__ work) {
-  extern __shared__ __align__(16) unsigned char ts_raw[];
-  TileSortSmem& S = *reinterpret_cast<TileSortSmem*>(ts_raw);
-  const unsigned int nm = *n_mid, total = nm + *n_chunks;
+                                                            const uint32_t* __restrict__ long_tiles,
+                                                            const unsigned int* __restrict__ n_long,
+                                                            unsigned int* __restrict__ work,
+                                                            uint32_t* ready, TileProg* prog, uint32_t lazy,
+                                                            const __grid_constant__ ViewSet vs,
+                                                            const uint2* __restrict__ rec_bb,
+                                                            uint2* __restrict__ plist) {
+  TileLongSmem& M = ts_smem();
+  const unsigned int nl = *n_long, total = nl + *n_mid;
   while (true) {
-    if (threadIdx.x == 0) S.item = atomicAdd(work, 1u);
+    if (threadIdx.x == 0) M.s.item = atomicAdd(work, 1u);
     __syncthreads();
-    const unsigned int item = S.item;
+    const unsigned int item = M.s.item;
     __syncthreads();  // everyone has read the item before it is overwritten
     if (item >= total) return;  // block-uniform
-    uint32_t off, m;
-    const bool mid = item < nm;
-    if (mid) {
-      const uint2 r = reinterpret_cast<const uint2*>(ranges)[mid_tiles[item]];
-      off = r.x;
-      m = r.y - r.x;
-    } else {
-      const uint2 ch = chunks[item - nm];
-      const uint2 r = reinterpret_cast<const uint2*>(ranges)[ch.x];
-      off = r.x + ch.y * (uint32_t)TS_CHUNK;
-      m = min((uint32_t)TS_CHUNK, r.y - off);
-    }
-    ts_sort_chunk(S, tvals + off, s_dkey, (int)m, mid ? nullptr : xk + off, (mid ? tvals : xv) + off);
+    const uint32_t tile = item < nl ? long_tiles[item] : mid_tiles[item - nl];
+    const uint2 r = reinterpret_cast<const uint2*>(ranges)[tile];
+    const TileBox tb(vs, tile);
+    if (item < nl)
+      tl_order<true>(r.x, r.y - r.x, lazy, tvals, xk, s_dkey, prog + tile, ready + tile, tb, rec_bb, plist);
+    else
+      ts_sort_list(tvals + r.x, s_dkey, (int)(r.y - r.x), tb, rec_bb, plist + r.x);
     __syncthreads();
   }
 }
 
-// number of entries of the ascending run[0, n) below k (or, with or_equal, not above k); n <= TS_CHUNK
-__device__ __forceinline__ uint32_t ts_count_below(const uint32_t* run, uint32_t n, uint32_t k, bool or_equal) {
-  uint32_t base = 0;
-#pragma unroll
-  for (uint32_t step = TS_CHUNK; step; step >>= 1) {
-    if (base + step <= n) {
-      const uint32_t x = run[base + step - 1];
-      if (or_equal ? x <= k : x < k) base += step;
-    }
-  }
-  return base;
-}
-
-// (dk, dv)[0, n) = (sk, sv)[0, n), n <= 2 * TS_CHUNK, with every load of a thread in flight at once
-__device__ __forceinline__ void ts_stage(uint32_t* dk, uint32_t* dv, const uint32_t* __restrict__ sk,
-                                         const uint32_t* __restrict__ sv, int n) {
-  constexpr int U = 2 * TS_CHUNK / TS_THREADS;
-  uint32_t k[U], v[U];
-#pragma unroll
-  for (int j = 0; j < U; ++j) {
-    const int q = threadIdx.x + j * TS_THREADS;
-    k[j] = q < n ? sk[q] : 0u;
-    v[j] = q < n ? sv[q] : 0u;
-  }
-  asm volatile("" ::: "memory");  // all loads before the first store
-#pragma unroll
-  for (int j = 0; j < U; ++j) {
-    const int q = threadIdx.x + j * TS_THREADS;
-    if (q < n) {
-      dk[q] = k[j];
-      dv[q] = v[j];
-    }
-  }
-}
-
-// Block-wide stable merge of the ascending runs (ak, av)[0, na) and (bk, bv)[0, nb)
-// into (ok, ov)[0, na + nb) (ok may be null): equal keys take the first run's
-// entries first.  Each thread finds where its share of the output starts in
-// both runs by one binary search along the output's diagonal, then merges its
-// share sequentially.
-__device__ __forceinline__ void ts_merge2(const uint32_t* ak, const uint32_t* av, int na, const uint32_t* bk,
-                                          const uint32_t* bv, int nb, uint32_t* ok, uint32_t* ov) {
-  const int n = na + nb, per = (n + TS_THREADS - 1) / TS_THREADS;
-  const int i0 = min(n, (int)threadIdx.x * per), i1 = min(n, i0 + per);
-  int lo = max(0, i0 - nb), hi = min(i0, na);  // entries of the first run among the first i0 outputs
-  while (lo < hi) {
-    const int mid = (lo + hi) >> 1;
-    if (ak[mid] <= bk[i0 - mid - 1]) lo = mid + 1;
-    else hi = mid;
-  }
-  int ia = lo, ib = i0 - lo;
-  for (int i = i0; i < i1; ++i) {
-    const bool take_a = ia < na && (ib >= nb || ak[ia] <= bk[ib]);
-    const uint32_t k = take_a ? ak[ia] : bk[ib], v = take_a ? av[ia] : bv[ib];
-    if (ok) ok[i] = k;
-    ov[i] = v;
-    ia += take_a ? 1 : 0;
-    ib += take_a ? 0 : 1;
-  }
-}
-
-// Persistent blocks over the long tiles, whose chunks k_tile_sort has sorted
-// into the scratch arrays (xk, xv).  Two or three chunks are merged through
-// shared memory (the first two, then that with the third); a tile of more
-// chunks places each pair behind the pairs of earlier chunks with keys not
-// above its own and of later chunks with keys below it, found by binary
-// searches of those chunks.
-__global__ void __launch_bounds__(TS_THREADS) k_tile_merge(uint32_t* __restrict__ tvals,
-                                                          const uint32_t* __restrict__ xk,
-                                                          const uint32_t* __restrict__ xv,
-                                                          const uint32_t* __restrict__ ranges,
-                                                          const uint32_t* __restrict__ long_tiles,
-                                                          const unsigned int* __restrict__ n_long,
-                                                          unsigned int* __restrict__ work) {
-  extern __shared__ __align__(16) unsigned char tm_raw[];
-  TileMergeSmem& S = *reinterpret_cast<TileMergeSmem*>(tm_raw);
-  const int t = threadIdx.x;
-  const unsigned int total = *n_long;
+// Persistent blocks over the listed long tiles: what k_tile_sort left unsorted.
+__global__ void __launch_bounds__(TS_THREADS, 2) k_tile_rest(const uint32_t* __restrict__ tvals,
+                                                            uint32_t* xk,
+                                                            const uint32_t* __restrict__ ranges,
+                                                            const uint32_t* __restrict__ list,
+                                                            const unsigned int* __restrict__ n_list,
+                                                            unsigned int* __restrict__ work,
+                                                            uint32_t* ready, TileProg* prog,
+                                                            const __grid_constant__ ViewSet vs,
+                                                            const uint2* __restrict__ rec_bb,
+                                                            uint2* __restrict__ plist) {
+  TileLongSmem& M = ts_smem();
+  const unsigned int total = *n_list;
+  if (total == 0u) return;
   while (true) {
-    if (t == 0) S.item = atomicAdd(work, 1u);
+    if (threadIdx.x == 0) M.s.item = atomicAdd(work, 1u);
     __syncthreads();
-    const unsigned int item = S.item;
+    const unsigned int item = M.s.item;
     __syncthreads();
     if (item >= total) return;  // block-uniform
-    const uint2 r = reinterpret_cast<const uint2*>(ranges)[long_tiles[item]];
-    const int L = (int)(r.y - r.x), nc = (L + TS_CHUNK - 1) / TS_CHUNK;
-    const uint32_t* ck = xk + r.x;
-    const uint32_t* cv = xv + r.x;
-    if (nc <= 3) {
-      // chunks 0 and 1 side by side in area 0
-      const int n01 = min(L, 2 * TS_CHUNK);
-      ts_stage(S.k[0], S.v[0], ck, cv, n01);
-      __syncthreads();
-      const int n1 = n01 - TS_CHUNK;
-      if (nc == 2) {
-        ts_merge2(S.k[0], S.v[0], TS_CHUNK, S.k[0] + TS_CHUNK, S.v[0] + TS_CHUNK, n1, nullptr, tvals + r.x);
-      } else {
-        ts_merge2(S.k[0], S.v[0], TS_CHUNK, S.k[0] + TS_CHUNK, S.v[0] + TS_CHUNK, n1, S.k[1], S.v[1]);
-        __syncthreads();  // area 0 is read: chunk 2 goes there
-        const int n2 = L - n01;
-        ts_stage(S.k[0], S.v[0], ck + n01, cv + n01, n2);
-        __syncthreads();
-        ts_merge2(S.k[1], S.v[1], n01, S.k[0], S.v[0], n2, nullptr, tvals + r.x);
-      }
-    } else {
-      for (int c = 0; c < nc; ++c) {
-        const int own = c * TS_CHUNK, m = min(TS_CHUNK, L - own);
-        for (int q = t; q < m; q += TS_THREADS) {
-          const uint32_t k = ck[own + q], v = cv[own + q];
-          uint32_t pos = (uint32_t)q;
-          for (int o = 0; o < nc; ++o) {
-            if (o == c) continue;
-            const int off = o * TS_CHUNK;
-            pos += ts_count_below(ck + off, (uint32_t)min(TS_CHUNK, L - off), k, o < c);
-          }
-          tvals[r.x + pos] = v;
-        }
-      }
-    }
-    __syncthreads();  // shared memory is read before the next tile's loads
+    const uint32_t tile = list[item];
+    const uint2 r = reinterpret_cast<const uint2*>(ranges)[tile];
+    tl_order<false>(r.x, r.y - r.x, 0u, tvals, xk, nullptr, prog + tile, ready + tile, TileBox(vs, tile), rec_bb,
+                    plist);
+    __syncthreads();
   }
 }
 
@@ -1130,6 +1330,18 @@ __device__ __forceinline__ float one_minus_exp(float x, float e) {
   return x < 0.125f ? p : 1.f - e;
 }
 
+// The composites take the tiles by length class, long lists first: a long list
+// begun last would keep its warps marching after all others have ended.
+struct TileOrder {
+  const uint32_t *long_tiles, *mid_tiles, *short_tiles;
+  const unsigned int *n_long, *n_mid;
+  __device__ __forceinline__ int tile(uint32_t i) const {
+    const uint32_t nl = *n_long, nm = *n_mid;
+    if (nl + nm == 0u) return (int)i;  // short lists only: any order does, without one more load
+    return (int)(i < nl ? long_tiles[i] : (i < nl + nm ? mid_tiles[i - nl] : short_tiles[i - nl - nm]));
+  }
+};
+
 __device__ __forceinline__ int find_view(const ViewSet& vs, int gtile) {
   int v = 0;
   while (v + 1 < vs.n && gtile >= vs.v[v + 1].tile_off) ++v;
@@ -1154,13 +1366,9 @@ struct Strip {
   }
   __device__ __forceinline__ int px(int lane) const { return (int)x0 + (lane & 7); }
   __device__ __forceinline__ int py(int lane) const { return (int)y0 + (lane >> 3); }
-  // box: (bx0 | bx1 << 16, by0 | by1 << 16)
-  __device__ __forceinline__ bool misses(uint2 box) const {
-    return (box.x >> 16) <= x0 || (box.x & 0xffffu) >= x1 || (box.y >> 16) <= y0 || (box.y & 0xffffu) >= y1;
-  }
 };
 
-// Work items are (tile, warp strip) pairs, item = tile * (TS*TS/32) + strip.
+// Work items are (tile, warp strip) pairs, item = position in the tile order * (TS*TS/32) + strip.
 // Without PERSIST every warp takes the item of its own block and warp index;
 // with PERSIST a grid sized to the resident warps loops, each warp taking the
 // next item from a global counter (one atomicAdd per item, no waiting), so a
@@ -1205,54 +1413,127 @@ __device__ __forceinline__ bool sm_leave(int sm_cut, int n_sms, unsigned int* ar
 }
 
 // ------------------------------------------------------------------ forward composite
-// Each warp walks its strip's tile list on its own: CH list entries at a time
-// (the batch: 32, 64 or 128, CH / 32 per lane, all loads of a batch issued
-// before any is used), the entries whose pixel box meets the strip are
-// compacted with ballots and their 64-byte records staged in the warp's slice
-// of shared memory, then every lane marches its pixel through them front to
-// back.  No block-wide barrier: a warp stops as soon as all its pixels have
-// stopped.
-// per-warp staging slice: CH records (64 B) + voxel id + list entry (+ slot id in the backward)
-__host__ __device__ constexpr size_t fwd_slice(int ch) { return (size_t)ch * 64 + (size_t)ch * 4 * 2; }
-__host__ __device__ constexpr size_t bwd_slice(int ch) { return (size_t)ch * 64 + (size_t)ch * 4 * 3; }
+// Each warp walks its strip's list on its own, with no block-wide barrier, and
+// stops as soon as all its pixels have.  The list entries carry the strips they
+// meet, so a warp reads WALK_ENTRIES of them at a time (coalesced 8-byte words,
+// four per lane) and queues the few that meet its strip; the records of 32
+// queued entries are then copied to shared memory and every lane marches its
+// pixel through them.  A pixel that stays open walks thousands of entries, and
+// the walk is then one serial chain per warp, so its memory latency is taken out
+// of the chain: the entries of the next round are loaded before they are needed,
+// and the records of the next 32 are copied (cp.async) while the current 32 are
+// marched.  The rounds and batches are the same for every lv_raster_opts.batch,
+// which chose the entries per round when a round gathered pixel boxes and records.
+//
+// per-warp slice of shared memory: two buffers of 32 records (64 B) and voxel
+// ids, and the queue of (slot, list entry): at most 32 marched, 32 in flight, 31
+// left over and one round of new ones
+constexpr int WALK_ENTRIES = 128;
+constexpr int QUEUE_LEN = 256;
+static_assert(32 + 32 + 31 + WALK_ENTRIES <= QUEUE_LEN, "the queue holds every entry in use");
+constexpr size_t WARP_SLICE = 2 * 32 * (64 + 4) + (size_t)QUEUE_LEN * 8;
 
-// Stage the entries [base, base + CH) below `end` whose pixel box meets the
-// strip: records in list order at positions 0 .. m - 1 of the warp's slice
-// (voxel id, list entry and, with slot_out, the slot id beside them); returns m.
-template <int TS, int CH>
-__device__ __forceinline__ int stage_batch(uint32_t base, uint32_t end, int lane, const Strip<TS>& strip,
-                                           const uint32_t* __restrict__ svals, const float4* __restrict__ rec,
-                                           const uint2* __restrict__ rec_bb, const uint32_t* __restrict__ slot_vox,
-                                           float4* wr, uint32_t* w_vox, uint32_t* w_ent, uint32_t* w_slot) {
-  constexpr int K = CH / 32;
-  uint32_t sl[K];
-  bool ov[K];
-#pragma unroll
-  for (int k = 0; k < K; ++k) {
-    const uint32_t e = base + 32 * k + lane;
-    sl[k] = e < end ? svals[e] : 0u;
-  }
-#pragma unroll
-  for (int k = 0; k < K; ++k) ov[k] = base + 32 * k + lane < end && !strip.misses(rec_bb[sl[k]]);
-  int m = 0;
-#pragma unroll
-  for (int k = 0; k < K; ++k) {
-    const uint32_t mask = __ballot_sync(FULL, ov[k]);
-    if (ov[k]) {
-      const int pos = m + __popc(mask & ((1u << lane) - 1u));
-      const float4* src = rec + 4 * (size_t)sl[k];
-      wr[4 * pos + 0] = src[0];
-      wr[4 * pos + 1] = src[1];
-      wr[4 * pos + 2] = src[2];
-      wr[4 * pos + 3] = src[3];
-      w_vox[pos] = slot_vox[sl[k]];
-      w_ent[pos] = base + 32 * k + lane;
-      if (w_slot) w_slot[pos] = sl[k];
-    }
-    m += __popc(mask);
-  }
-  return m;
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
 }
+__device__ __forceinline__ void cp_async4(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+// The records of one strip in list order (REV: from the last entry to the
+// first), 32 at a time.  All members are called by the whole warp.
+template <bool REV>
+struct StripWalk {
+  static constexpr int K = WALK_ENTRIES / 32;
+  static constexpr uint32_t QM = QUEUE_LEN - 1;
+  const uint2* __restrict__ plist;
+  const float4* __restrict__ rec;
+  const uint32_t* __restrict__ slot_vox;
+  float4* s_rec;     // [2][32][4]
+  uint32_t* s_vox;   // [2][32]
+  uint2* s_q;        // (slot, entry)
+  uint32_t lo, hi;   // entries [lo, hi) not scanned yet, those in `ahead` not counted
+  uint32_t base;     // first entry of `ahead`
+  uint2 ahead[K];
+  uint32_t head, tail;  // queue positions: next to copy, next to fill
+  uint32_t bit;
+  bool live;            // `ahead` holds entries not queued yet
+  int lane;
+
+  __device__ __forceinline__ void load_ahead() {
+    if (REV) {
+      base = hi - lo > (uint32_t)WALK_ENTRIES ? hi - WALK_ENTRIES : lo;
+#pragma unroll
+      for (int k = 0; k < K; ++k) {
+        const uint32_t e = base + 32 * k + lane;
+        ahead[k] = e < hi ? plist[e] : make_uint2(0u, 0u);
+      }
+      hi = base;
+    } else {
+      base = lo;
+#pragma unroll
+      for (int k = 0; k < K; ++k) {
+        const uint32_t e = base + 32 * k + lane;
+        ahead[k] = e < hi ? plist[e] : make_uint2(0u, 0u);
+      }
+      lo = hi - lo > (uint32_t)WALK_ENTRIES ? lo + WALK_ENTRIES : hi;
+    }
+  }
+  __device__ __forceinline__ void begin(uint32_t start, uint32_t end, int strip) {
+    lo = start;
+    hi = end;
+    head = tail = 0u;
+    bit = 1u << strip;
+    live = start < end;
+    load_ahead();
+  }
+  // queue entries until 32 wait or the list ends
+  __device__ __forceinline__ void fill() {
+    while (tail - head < 32u && live) {
+      const uint32_t b = base;
+      uint2 cur[K];
+#pragma unroll
+      for (int k = 0; k < K; ++k) cur[k] = ahead[k];
+      live = lo < hi;
+      load_ahead();
+#pragma unroll
+      for (int kk = 0; kk < K; ++kk) {
+        const int k = REV ? K - 1 - kk : kk;
+        const bool in = (cur[k].y & bit) != 0u;
+        const uint32_t m = __ballot_sync(FULL, in);
+        if (in) {
+          const uint32_t before = REV ? m & (0xfffffffeu << lane) : m & ((1u << lane) - 1u);
+          s_q[(tail + __popc(before)) & QM] = make_uint2(cur[k].x, b + 32 * k + lane);
+        }
+        tail += __popc(m);
+      }
+    }
+    __syncwarp();
+  }
+  // start copying the next (up to) 32 records into buffer b; returns their number
+  __device__ __forceinline__ int copy(int b) {
+    const int m = (int)min(32u, tail - head);
+    // four lanes per record: a record's 64 bytes in one request
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int r = 8 * k + (lane >> 2);
+      if (r < m) {
+        const uint32_t sl = s_q[(head + r) & QM].x;
+        cp_async16(s_rec + 128 * b + 4 * r + (lane & 3), rec + 4 * (size_t)sl + (lane & 3));
+      }
+    }
+    if (lane < m) cp_async4(s_vox + 32 * b + lane, slot_vox + s_q[(head + lane) & QM].x);
+    cp_async_commit();
+    head += m;
+    return m;
+  }
+};
+
 // The LF-weighted loss fused into the backward composite (Sec. IV-B, Eq. 8 and
 // 18): per pixel dL/drgb = 2 / (3 |P_v|) * (w / <w>) * (rgb - gt), in the
 // operation order lv_lf_loss_from_weights uses, and the view's summed
@@ -1268,60 +1549,114 @@ struct LfFuse {
   float* dL;           // [P][3] dL/drgb, also written out (nullable)
 };
 
-template <int TS>
-constexpr int min_blocks() { return TS == 16 ? 5 : (TS == 8 ? 16 : 1); }
+// The composite of a list's sorted part and, for the tiles whose pixels were
+// still open at its end, of the rest in a second launch (resume): the pixels'
+// sums are read back from the outputs (the depth and the sample count, which a
+// caller may not want, from dep and nsamp) and the march goes on where it
+// stopped, so the results are those of one march.
+struct Front {
+  uint32_t* ready;
+  TileProg* prog;
+  uint32_t* open_tiles;
+  unsigned int* n_open;
+  float* dep;
+  uint32_t* nsamp;
+  bool resume;
+};
 
-template <int TS, bool SEG, bool PERSIST, int CH>
+template <int TS>
+constexpr int min_blocks() { return TS == 16 ? 4 : (TS == 8 ? 16 : 1); }
+
+template <int TS, bool SEG, bool PERSIST>
 __global__ void __launch_bounds__(TS* TS, min_blocks<TS>()) k_fwd(const __grid_constant__ ViewSet vs, const uint32_t* __restrict__ ranges,
-                                                const uint32_t* __restrict__ svals, const float4* __restrict__ rec,
-                                                const uint2* __restrict__ rec_bb,
+                                                const uint2* __restrict__ plist, const float4* __restrict__ rec,
                                                 const uint32_t* __restrict__ slot_vox, float t_stop,
                                                 float* __restrict__ rgb, float* __restrict__ depth,
                                                 float* __restrict__ T_out, uint32_t* __restrict__ n_contrib,
                                                 uint32_t* __restrict__ n_samples, float* __restrict__ tau_out,
                                                 unsigned long long* __restrict__ wmax, unsigned int* work,
-                                                uint32_t n_items, int sm_cut, int n_sms, unsigned int* arrivals) {
+                                                uint32_t n_items, int sm_cut, int n_sms, unsigned int* arrivals,
+                                                const TileOrder order, const Front fr) {
   constexpr int NW = TS * TS / 32;
   extern __shared__ float4 smem_f4[];
   if (PERSIST && sm_leave(sm_cut, n_sms, arrivals)) return;  // block-uniform
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  float4* wr = (float4*)((char*)smem_f4 + fwd_slice(CH) * warp);
-  uint32_t* w_vox = (uint32_t*)(wr + 4 * CH);
-  uint32_t* w_ent = w_vox + CH;
+  if (PERSIST && fr.resume) {  // grid-uniform
+    n_items = *fr.n_open * NW;
+    if (n_items == 0u) return;
+  }
+  StripWalk<false> walk;
+  walk.plist = plist;
+  walk.rec = rec;
+  walk.slot_vox = slot_vox;
+  walk.lane = lane;
+  walk.s_rec = (float4*)((char*)smem_f4 + WARP_SLICE * warp);
+  walk.s_vox = (uint32_t*)(walk.s_rec + 2 * 32 * 4);
+  walk.s_q = (uint2*)(walk.s_vox + 2 * 32);
   for (uint32_t item = PERSIST ? next_item(work, lane) : blockIdx.x * NW + warp; item < n_items;
        item = PERSIST ? next_item(work, lane) : n_items) {  // warp-uniform
-    const int gtile = (int)(item / NW);
+    const int gtile = PERSIST && fr.resume ? (int)fr.open_tiles[item / NW] : order.tile(item / NW);
     const int view = find_view(vs, gtile);
     const DevView& c = vs.v[view];
+    const uint32_t start = ranges[2 * gtile], end = fr.ready[gtile];
+    walk.begin(PERSIST && fr.resume ? fr.prog[gtile].front : start, end, (int)(item % NW));
     const int lt = gtile - c.tile_off;
     const int tile_x = lt % c.tiles_x, tile_y = lt / c.tiles_x;
     const Strip<TS> strip(tile_x, tile_y, (int)(item % NW));
     const int px = strip.px(lane), py = strip.py(lane);
     const bool inside = px < c.W && py < c.H;
     const Ray r = make_ray(c, px, py);
-    const uint32_t start = ranges[2 * gtile], end = ranges[2 * gtile + 1];
     const unsigned long long gid = (unsigned long long)(c.pix_off + (long long)py * c.W + px);
     const unsigned long long gid_key = 0xffffffffull - ((gid + (unsigned long long)vs.id_base) & 0xffffffffull);
     float T = 1.f, tau = 0.f, cr = 0.f, cg = 0.f, cb = 0.f, dep = 0.f;
     uint32_t last = 0, nsamp = 0;
     bool done = !inside;
-    for (uint32_t base = start; base < end && !__all_sync(FULL, done); base += CH) {
-      const int m = stage_batch<TS, CH>(base, end, lane, strip, svals, rec, rec_bb, slot_vox, wr, w_vox, w_ent,
-                                        nullptr);
-      if (!m) continue;
+    if (PERSIST && fr.resume) {
+      if (inside) {
+        const size_t p = (size_t)gid;
+        T = T_out[p];
+        done = T < t_stop;
+      }
+      if (__all_sync(FULL, done)) continue;  // the strip stopped within the front
+      if (inside) {
+        const size_t p = (size_t)gid;
+        cr = rgb[3 * p + 0];
+        cg = rgb[3 * p + 1];
+        cb = rgb[3 * p + 2];
+        dep = fr.dep[p];
+        tau = tau_out[p];
+        last = n_contrib[p];
+        nsamp = fr.nsamp[p];
+      }
+    }
+    walk.fill();
+    int m = walk.copy(0);
+    for (int b = 0; m; b ^= 1) {  // warp-uniform
+      const uint32_t q0 = walk.head - (uint32_t)m;  // this batch's queue entries
+      walk.fill();
+      const int m_next = walk.copy(b ^ 1);
+      cp_async_wait<1>();
       __syncwarp();
+      const float4* wr = walk.s_rec + 128 * b;
+      const uint32_t* w_vox = walk.s_vox + 32 * b;
       int last_j = -1;  // the lane's last sample of this batch (its list entry is read once, below)
+      float4 g = wr[0];
+      float t_in, t_out;
+      bool h = chord(r, g, t_in, t_out);
       for (int j = 0; j < m; ++j) {
-        if (CH > 32 && (j & 31) == 31 && __all_sync(FULL, done)) break;  // warp-uniform
-        const float4 g = wr[4 * j];
-        float t_in, t_out;
-        const bool hit = !done && chord(r, g, t_in, t_out);
+        const bool hit = h && !done;
+        const float4 gj = g;
+        const float ti = t_in, to = t_out;
+        // the next record's chord does not wait for this sample (past the last one: the last again)
+        g = wr[4 * min(j + 1, m - 1)];
+        h = chord(r, g, t_in, t_out);
+        if (!__any_sync(FULL, hit)) continue;
         float w = 0.f;
         if (hit) {
           const float4 d0 = wr[4 * j + 1], d1 = wr[4 * j + 2], col = wr[4 * j + 3];
-          const float l = t_out - t_in, tm = 0.5f * (t_in + t_out);
+          const float l = to - ti, tm = 0.5f * (ti + to);
           float u[SEG ? 9 : 3];
-          const float sigma = fmaxf(sample_density<SEG>(r, g, d0, d1, col.w, t_in, tm, t_out, u), 0.f);
+          const float sigma = fmaxf(sample_density<SEG>(r, gj, d0, d1, col.w, ti, tm, to, u), 0.f);
           const float x = sigma * l;
           const float ex = __expf(-x);
           const float alpha = one_minus_exp(x, ex);
@@ -1334,21 +1669,34 @@ __global__ void __launch_bounds__(TS* TS, min_blocks<TS>()) k_fwd(const __grid_c
           T *= ex;
           last_j = j;
           ++nsamp;
+          done = T < t_stop;
         }
-        if (__any_sync(FULL, hit)) {
+        if (wmax) {  // grid-uniform
           // the warp's largest w (ties to the lowest lane = smallest pixel id), one global atomic
           const uint32_t v = hit ? __float_as_uint(w) + 1u : 0u;
           const uint32_t mx = __reduce_max_sync(FULL, v);
           const uint32_t who = __ballot_sync(FULL, v == mx);
-          if (wmax && lane == __ffs(who) - 1)
+          if (lane == __ffs(who) - 1)
             atomicMax(&wmax[w_vox[j]], ((unsigned long long)(mx - 1u) << 32) | gid_key);
-          if (hit && T < t_stop) done = true;
         }
       }
-      if (last_j >= 0) last = w_ent[last_j] - start + 1;
-      __syncwarp();
+      if (last_j >= 0) last = walk.s_q[(q0 + last_j) & walk.QM].y - start + 1;
+      m = m_next;
+      if (__all_sync(FULL, done)) break;
+      __syncwarp();  // the buffer is copied into next
+    }
+    cp_async_wait<0>();  // a batch copied ahead of the stop
+    // a long list sorted only so far, and pixels that go on: listed for k_tile_rest and the second launch
+    const bool open = end < ranges[2 * gtile + 1] && !__all_sync(FULL, done);
+    if (open && lane == 0 && atomicExch(&fr.prog[gtile].open, 1u) == 0u) {
+      fr.prog[gtile].front = end;
+      fr.open_tiles[atomicAdd(fr.n_open, 1u)] = (uint32_t)gtile;
     }
     if (inside) {
+      if (open) {
+        fr.dep[gid] = dep;
+        fr.nsamp[gid] = nsamp;
+      }
       const size_t p = (size_t)gid;
       rgb[3 * p + 0] = cr;
       rgb[3 * p + 1] = cg;
@@ -1398,20 +1746,20 @@ __device__ __forceinline__ float warp_reduce16(float* v, int lane) {
 }
 
 // Backward: each warp walks its strip's list back to front from the last entry
-// any of its pixels used, in the same 32-entry chunks and with the same
-// compaction as the forward; the per-record gradients (8 corners + colour) are
+// any of its pixels used, through the same queue and copies as the forward; the
+// per-record gradients (8 corners + colour) are
 // reduced over the warp and sent with three 16-byte global reductions.
-template <int TS, bool SEG, bool PERSIST, int CH>
+template <int TS, bool SEG, bool PERSIST>
 __global__ void __launch_bounds__(TS* TS, min_blocks<TS>()) k_bwd(const __grid_constant__ ViewSet vs, const uint32_t* __restrict__ ranges,
-                                                const uint32_t* __restrict__ svals, const float4* __restrict__ rec,
-                                                const uint2* __restrict__ rec_bb,
+                                                const uint2* __restrict__ plist, const float4* __restrict__ rec,
                                                 const uint32_t* __restrict__ slot_vox, const float* __restrict__ T_fwd,
                                                 const float* __restrict__ tau_in,
                                                 const uint32_t* __restrict__ n_contrib,
                                                 const float* __restrict__ dL_drgb, const float* __restrict__ dL_ddepth,
                                                 const float* __restrict__ dL_dT, float* __restrict__ d_density,
                                                 float4* __restrict__ d_rgb, unsigned int* work, uint32_t n_items,
-                                                int sm_cut, int n_sms, unsigned int* arrivals, const LfFuse lf) {
+                                                int sm_cut, int n_sms, unsigned int* arrivals, const TileOrder order,
+                                                const LfFuse lf) {
   constexpr int NW = TS * TS / 32;
   extern __shared__ float4 smem_f4[];
   __shared__ double s_lf[NW][LV_MAX_VIEWS];  // each warp's loss sums (fused LF loss; no atomics)
@@ -1429,13 +1777,17 @@ __global__ void __launch_bounds__(TS* TS, min_blocks<TS>()) k_bwd(const __grid_c
     }
     __syncthreads();
   }
-  float4* wr = (float4*)((char*)smem_f4 + bwd_slice(CH) * warp);
-  uint32_t* w_vox = (uint32_t*)(wr + 4 * CH);
-  uint32_t* w_slot = w_vox + CH;
-  uint32_t* w_ent = w_slot + CH;
+  StripWalk<true> walk;
+  walk.plist = plist;
+  walk.rec = rec;
+  walk.slot_vox = slot_vox;
+  walk.lane = lane;
+  walk.s_rec = (float4*)((char*)smem_f4 + WARP_SLICE * warp);
+  walk.s_vox = (uint32_t*)(walk.s_rec + 2 * 32 * 4);
+  walk.s_q = (uint2*)(walk.s_vox + 2 * 32);
   for (uint32_t item = PERSIST ? next_item(work, lane) : blockIdx.x * NW + warp; item < n_items;
        item = PERSIST ? next_item(work, lane) : n_items) {  // warp-uniform
-    const int gtile = (int)(item / NW);
+    const int gtile = order.tile(item / NW);
     const int view = find_view(vs, gtile);
     const DevView& c = vs.v[view];
     const int lt = gtile - c.tile_off;
@@ -1487,17 +1839,31 @@ __global__ void __launch_bounds__(TS* TS, min_blocks<TS>()) k_bwd(const __grid_c
     const float tgT = Tf * gT;
     float S = 0.f;
     float Tcur = __expf(-tau);  // T after the last sample, from the stored optical depth
-    // batches aligned as in the forward: [start + CH k, start + CH k + CH), walked back to front
-    for (uint32_t cb = start + (warp_hi - start + CH - 1) / CH * CH; cb > start; cb -= CH) {
-      const uint32_t base = cb - CH;
-      const int m = stage_batch<TS, CH>(base, warp_hi, lane, strip, svals, rec, rec_bb, slot_vox, wr, w_vox,
-                                        w_ent, w_slot);
-      if (!m) continue;
+    walk.begin(start, warp_hi, (int)(item % NW));
+    walk.fill();
+    int m = walk.copy(0);
+    for (int b = 0; m; b ^= 1) {  // warp-uniform
+      const uint32_t q0 = walk.head - (uint32_t)m;  // this batch's queue entries
+      walk.fill();
+      const int m_next = walk.copy(b ^ 1);
+      cp_async_wait<1>();
       __syncwarp();
-      for (int j = m - 1; j >= 0; --j) {
-        const float4 g = wr[4 * j];
-        float t_in, t_out;
-        const bool hit = w_ent[j] < my_hi && chord(r, g, t_in, t_out);
+      const float4* wr = walk.s_rec + 128 * b;
+      const uint32_t* w_vox = walk.s_vox + 32 * b;
+      uint2 qe = walk.s_q[q0 & walk.QM];
+      float4 gn = wr[0];
+      float tn_in, tn_out;
+      bool h = chord(r, gn, tn_in, tn_out) && qe.y < my_hi;
+      for (int j = 0; j < m; ++j) {
+        const bool hit = h;
+        const float4 g = gn;
+        const float t_in = tn_in, t_out = tn_out;
+        const uint32_t slot = qe.x;
+        // the next record's chord does not wait for this sample (past the last one: the last again)
+        const int jn = min(j + 1, m - 1);
+        qe = walk.s_q[(q0 + jn) & walk.QM];
+        gn = wr[4 * jn];
+        h = chord(r, gn, tn_in, tn_out) && qe.y < my_hi;
         const unsigned hb = __ballot_sync(FULL, hit);
         if (!hb) continue;
         float v[16];
@@ -1531,7 +1897,7 @@ __global__ void __launch_bounds__(TS* TS, min_blocks<TS>()) k_bwd(const __grid_c
           v[10] = w * gb;
         }
         float* dd = d_density + 8 * (size_t)w_vox[j];
-        float* dc = (float*)(d_rgb + w_slot[j]);
+        float* dc = (float*)(d_rgb + slot);
         if (__popc(hb) <= 8) {
           // up to eight lanes: each sends its own values, cheaper than the butterfly (measured: 8 lanes
           // 2 % faster than 2; every lane, 12x slower, the reductions to one address serialise)
@@ -1553,8 +1919,11 @@ __global__ void __launch_bounds__(TS* TS, min_blocks<TS>()) k_bwd(const __grid_c
           else if (lane == 2) red_add_v4(dc, q0, q1, q2, 0.f);
         }
       }
-      __syncwarp();
+      m = m_next;
+      __syncwarp();  // the buffer is copied into next
     }
+    cp_async_wait<0>();
+    __syncwarp();  // the slice is reused by the next item
   }
   if (lf.w) {
     __syncthreads();
@@ -1660,13 +2029,17 @@ __global__ void k_gather_edge(const int64_t* __restrict__ argmax, int64_t n, con
   edge[i] = (a >= 0 && a < n_pix) ? edge_map[a] : 0.f;
 }
 
-__global__ void k_debug_pairs(const uint32_t* __restrict__ k, const uint32_t* __restrict__ v,
+// a block per tile, in turn
+__global__ void k_debug_pairs(const uint2* __restrict__ ranges, int64_t tiles, const uint2* __restrict__ plist,
                               const uint32_t* __restrict__ slot_vox, const uint32_t* __restrict__ s_dkey,
-                              const unsigned long long* d_count, int64_t cap, uint64_t* ko, uint32_t* vo) {
-  const int64_t n = usable_pairs(d_count, cap);
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    if (ko) ko[i] = ((uint64_t)k[i] << 32) | s_dkey[v[i]];
-    if (vo) vo[i] = slot_vox[v[i]];
+                              uint64_t* ko, uint32_t* vo) {
+  for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+    const uint2 r = ranges[tile];
+    for (uint32_t i = r.x + threadIdx.x; i < r.y; i += blockDim.x) {
+      const uint32_t s = plist[i].x;
+      if (ko) ko[i] = ((uint64_t)tile << 32) | s_dkey[s];
+      if (vo) vo[i] = slot_vox[s];
+    }
   }
 }
 
@@ -1692,7 +2065,7 @@ __device__ __forceinline__ void sh_basis64(double x, double y, double z, double*
 
 template <typename DT, typename ST>
 __global__ void k_render_f64(const __grid_constant__ ViewSet vs, const uint32_t* __restrict__ ranges,
-                             const uint32_t* __restrict__ svals, const uint32_t* __restrict__ slot_vox,
+                             const uint2* __restrict__ plist, const uint32_t* __restrict__ slot_vox,
                              const float4* __restrict__ geom, const DT* __restrict__ dens, const ST* __restrict__ sh,
                              int sh_nb, const int64_t* __restrict__ pixels, int64_t n_px, double t_stop,
                              int segment, const uint32_t* __restrict__ vidx, double* __restrict__ rgb_out,
@@ -1723,7 +2096,7 @@ __global__ void k_render_f64(const __grid_constant__ ViewSet vs, const uint32_t*
   double T = 1.0, cr = 0.0, cg = 0.0, cb = 0.0;
   const uint32_t start = ranges[2 * gtile], end = ranges[2 * gtile + 1];
   for (uint32_t e = start; e < end; ++e) {
-    const uint32_t vox = slot_vox[svals[e]];
+    const uint32_t vox = slot_vox[plist[e].x];
     const float4 g = geom[vox];
     const double h = (double)g.w, cc[3] = {(double)g.x, (double)g.y, (double)g.z};
     double lo_t = t_near, hi_t = 1e300;
@@ -1844,42 +2217,50 @@ static void sm_limits(int sm_limit, int dev, int* sms, int* sm_cut) {
   *sm_cut = (sm_limit > 0 && *sms > 0 && sm_limit < *sms) ? sm_limit : 0;
 }
 
-template <int TS, bool SEG, bool PERSIST, int CH>
-static void launch_fwd_t(int64_t tiles, cudaStream_t s, const ViewSet& vs, const FwdWs& w, const uint32_t* sv,
-                         float t_stop, const lv_fwd_out* out, int sm_limit) {
-  const size_t smem = fwd_slice(CH) * (TS * TS / 32);
+static TileOrder tile_order(const FwdWs& w) {
+  return {w.long_tiles, w.mid_tiles, w.short_tiles, w.work + 6, w.work + 4};
+}
+
+// resume: the second launch, over the open tiles (its grid is persistent whatever the schedule: only the
+// device knows their number)
+template <int TS, bool SEG, bool PERSIST>
+static void launch_fwd_t(int64_t tiles, cudaStream_t s, const ViewSet& vs, const FwdWs& w, float t_stop,
+                         const lv_fwd_out* out, int sm_limit, bool resume) {
+  const size_t smem = WARP_SLICE * (TS * TS / 32);
   static int pblocks[64];  // per device
   static std::atomic<unsigned long long> done{0};
   const int dev = current_device();
   once_per_device(done, [&] {
-    cudaFuncSetAttribute(k_fwd<TS, SEG, PERSIST, CH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (PERSIST && dev < 64) pblocks[dev] = persistent_blocks(k_fwd<TS, SEG, PERSIST, CH>, TS * TS, smem);
+    cudaFuncSetAttribute(k_fwd<TS, SEG, PERSIST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (PERSIST && dev < 64) pblocks[dev] = persistent_blocks(k_fwd<TS, SEG, PERSIST>, TS * TS, smem);
   });
-  const int pb = dev < 64 ? pblocks[dev] : persistent_blocks(k_fwd<TS, SEG, PERSIST, CH>, TS * TS, smem);
+  const int pb = dev < 64 ? pblocks[dev] : persistent_blocks(k_fwd<TS, SEG, PERSIST>, TS * TS, smem);
   int sms = 0, sm_cut = 0;
   sm_limits(sm_limit, dev, &sms, &sm_cut);
   const uint32_t n_items = (uint32_t)tiles * (TS * TS / 32);
   unsigned grid = (unsigned)tiles;
-  if (PERSIST) grid = (unsigned)(tiles < pb ? tiles : pb);  // work[0] was cleared at the start of the forward
-  k_fwd<TS, SEG, PERSIST, CH><<<grid, TS * TS, smem, s>>>(vs, w.ranges, sv, w.rec, w.rec_bb, w.slot_vox, t_stop,
+  if (PERSIST) grid = (unsigned)(tiles < pb ? tiles : pb);  // the work counters were cleared at the start of the forward
+  const Front fr = {w.ready, w.prog, w.open_tiles, w.work + 7, w.dep, w.nsamp, resume};
+  k_fwd<TS, SEG, PERSIST><<<grid, TS * TS, smem, s>>>(vs, w.ranges, w.plist, w.rec, w.slot_vox, t_stop,
                                                        out->rgb, out->depth, out->T, out->n_contrib,
-                                                       out->n_samples, w.tau, out->wmax_packed, w.work, n_items,
-                                                       sm_cut, sms, w.work + 8);
+                                                       out->n_samples, w.tau, out->wmax_packed,
+                                                       w.work + (resume ? 2 : 0), n_items, sm_cut, sms,
+                                                       w.work + (resume ? 10 : 8), tile_order(w), fr);
 }
 
-template <int TS, bool SEG, bool PERSIST, int CH>
-static void launch_bwd_t(int64_t tiles, cudaStream_t s, const ViewSet& vs, const FwdWs& w, const uint32_t* sv,
-                         const lv_fwd_out* fwd, const float* gC, const float* gD, const float* gT, float* dd,
+template <int TS, bool SEG, bool PERSIST>
+static void launch_bwd_t(int64_t tiles, cudaStream_t s, const ViewSet& vs, const FwdWs& w, const lv_fwd_out* fwd,
+                         const float* gC, const float* gD, const float* gT, float* dd,
                          int sm_limit, const LfFuse& lf) {
-  const size_t smem = bwd_slice(CH) * (TS * TS / 32);
+  const size_t smem = WARP_SLICE * (TS * TS / 32);
   static int pblocks[64];  // per device
   static std::atomic<unsigned long long> done{0};
   const int dev = current_device();
   once_per_device(done, [&] {
-    cudaFuncSetAttribute(k_bwd<TS, SEG, PERSIST, CH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (PERSIST && dev < 64) pblocks[dev] = persistent_blocks(k_bwd<TS, SEG, PERSIST, CH>, TS * TS, smem);
+    cudaFuncSetAttribute(k_bwd<TS, SEG, PERSIST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (PERSIST && dev < 64) pblocks[dev] = persistent_blocks(k_bwd<TS, SEG, PERSIST>, TS * TS, smem);
   });
-  const int pb = dev < 64 ? pblocks[dev] : persistent_blocks(k_bwd<TS, SEG, PERSIST, CH>, TS * TS, smem);
+  const int pb = dev < 64 ? pblocks[dev] : persistent_blocks(k_bwd<TS, SEG, PERSIST>, TS * TS, smem);
   int sms = 0, sm_cut = 0;
   sm_limits(sm_limit, dev, &sms, &sm_cut);
   const uint32_t n_items = (uint32_t)tiles * (TS * TS / 32);
@@ -1888,93 +2269,87 @@ static void launch_bwd_t(int64_t tiles, cudaStream_t s, const ViewSet& vs, const
     zero_async(s, w.work + 1, sizeof(unsigned int), w.work + 9, sizeof(unsigned int));
     grid = (unsigned)(tiles < pb ? tiles : pb);
   }
-  k_bwd<TS, SEG, PERSIST, CH><<<grid, TS * TS, smem, s>>>(vs, w.ranges, sv, w.rec, w.rec_bb, w.slot_vox, fwd->T,
+  k_bwd<TS, SEG, PERSIST><<<grid, TS * TS, smem, s>>>(vs, w.ranges, w.plist, w.rec, w.slot_vox, fwd->T,
                                                        w.tau, fwd->n_contrib, gC, gD, gT, dd, w.d_rgb, w.work + 1,
-                                                       n_items, sm_cut, sms, w.work + 9, lf);
+                                                       n_items, sm_cut, sms, w.work + 9, tile_order(w), lf);
 }
 
-// tile size, batch, density model (midpoint, or the exact-segment variant) and scheduling
-// (one block per tile, or persistent warps on a work counter) from the options; a batch of
-// 128 needs more than the 227 KB of shared memory of a block for 32 x 32 tiles (refused by
-// check_common)
-// The tile-sorted pairs are in (k0, v0) after an even number of digit passes,
-// else in (k1, v1); the other pair of arrays is scratch.  One warp per tile
-// first (short lists, ranges, the lists of longer tiles), then persistent
-// blocks over the medium tiles and the long tiles' chunks, then the merge.
-static void launch_tile_sort(const FwdWs& w, int64_t tiles, int64_t pair_cap, cudaStream_t s) {
+// tile size, density model (midpoint, or the exact-segment variant) and scheduling (one block per
+// tile, or persistent warps on a work counter) from the options
+// The pairs sorted by tile are in (k0, v0) after an even number of digit passes, else in (k1, v1); the
+// other keys are scratch for the long lists' order keys.  One warp per tile first (short lists, ranges,
+// the lists of longer tiles), then persistent blocks over the long tiles' fronts and the medium tiles.
+static int tile_sort_blocks() {
   static std::atomic<unsigned long long> attr_done{0};
-  static int sort_blocks[64], merge_blocks[64];
-  int dev = 0;
-  cudaGetDevice(&dev);
+  static int blocks[64];
+  const int dev = current_device();
   once_per_device(attr_done, [dev] {
     cudaFuncSetAttribute(k_tile_sort_warp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TileSortWarpSmem));
-    cudaFuncSetAttribute(k_tile_sort, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TileSortSmem));
-    cudaFuncSetAttribute(k_tile_merge, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TileMergeSmem));
-    if (dev < 64) {
-      sort_blocks[dev] = persistent_blocks(k_tile_sort, TS_THREADS, sizeof(TileSortSmem));
-      merge_blocks[dev] = persistent_blocks(k_tile_merge, TS_THREADS, sizeof(TileMergeSmem));
-    }
+    cudaFuncSetAttribute(k_tile_sort, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TileLongSmem));
+    cudaFuncSetAttribute(k_tile_rest, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TileLongSmem));
+    if (dev < 64) blocks[dev] = persistent_blocks(k_tile_sort, TS_THREADS, sizeof(TileLongSmem));
   });
-  const int ns = dev < 64 ? sort_blocks[dev] : persistent_blocks(k_tile_sort, TS_THREADS, sizeof(TileSortSmem));
-  const int nmg = dev < 64 ? merge_blocks[dev] : persistent_blocks(k_tile_merge, TS_THREADS, sizeof(TileMergeSmem));
-  const int passes = sort_passes(tile_bits(tiles));
-  const bool odd = passes & 1, ready = passes > 0;
-  uint32_t* sv = odd ? w.v1 : w.v0;
-  uint32_t* xk = odd ? w.k0 : w.k1;
-  uint32_t* xv = odd ? w.v0 : w.v1;
+  return dev < 64 ? blocks[dev] : persistent_blocks(k_tile_sort, TS_THREADS, sizeof(TileLongSmem));
+}
+static uint32_t* long_keys(const FwdWs& w, int64_t tiles) {
+  return (sort_passes(tile_bits(tiles)) & 1) ? w.k0 : w.k1;
+}
+static void launch_tile_sort(const FwdWs& w, const ViewSet& vs, int64_t n, int64_t tiles, int64_t pair_cap,
+                             cudaStream_t s) {
+  const int64_t nb = std::min<int64_t>(tile_sort_blocks(), tiles);
+  const bool ready = sort_passes(tile_bits(tiles)) > 0;
+  const uint32_t* sv = tile_pair_slots(w, tiles);
   const unsigned wblocks = (unsigned)((tiles + TW_WARPS - 1) / TW_WARPS);
-  k_tile_sort_warp<<<wblocks, TW_WARPS * 32, sizeof(TileSortWarpSmem), s>>>(sv, w.s_dkey, w.counters, pair_cap, ready,
-                                                                          tiles, w.ranges, w.mid_tiles, w.work + 4,
-                                                                          w.chunks, w.work + 2, w.long_tiles,
-                                                                          w.work + 6);
-  k_tile_sort<<<(unsigned)ns, TS_THREADS, sizeof(TileSortSmem), s>>>(sv, xk, xv, w.s_dkey, w.ranges, w.mid_tiles,
-                                                                     w.work + 4, w.chunks, w.work + 2, w.work + 5);
-  k_tile_merge<<<(unsigned)nmg, TS_THREADS, sizeof(TileMergeSmem), s>>>(sv, xk, xv, w.ranges, w.long_tiles,
-                                                                        w.work + 6, w.work + 3);
-  count_launch(3);
+  k_tile_sort_warp<<<wblocks, TW_WARPS * 32, sizeof(TileSortWarpSmem), s>>>(
+      sv, w.s_dkey, w.counters, pair_cap, ready, tiles, w.ranges, w.mid_tiles, w.work + 4, w.long_tiles, w.work + 6,
+      w.short_tiles, w.work + 11, w.ready, w.prog, vs, w.rec_bb, w.plist);
+  count_launch(1);
+  if (n <= TW_MAX) return;  // a tile lists a voxel once: every list is short
+  k_tile_sort<<<(unsigned)nb, TS_THREADS, sizeof(TileLongSmem), s>>>(
+      sv, long_keys(w, tiles), w.s_dkey, w.ranges, w.mid_tiles, w.work + 4, w.long_tiles, w.work + 6, w.work + 5,
+      w.ready, w.prog, n > TS_LAZY_VOXELS ? TS_LAZY : ~0u, vs, w.rec_bb, w.plist);
+  count_launch(1);
+}
+// the rest of the open tiles' lists, or (all) of every long list, for the calls that read whole lists
+static void launch_tile_rest(const FwdWs& w, const ViewSet& vs, int64_t tiles, bool all, cudaStream_t s) {
+  const int64_t nb = std::min<int64_t>(tile_sort_blocks(), tiles);
+  if (all) zero_async(s, w.work + 3, sizeof(unsigned int));
+  k_tile_rest<<<(unsigned)nb, TS_THREADS, sizeof(TileLongSmem), s>>>(
+      tile_pair_slots(w, tiles), long_keys(w, tiles), w.ranges, all ? w.long_tiles : w.open_tiles,
+      w.work + (all ? 6 : 7), w.work + 3, w.ready, w.prog, vs, w.rec_bb, w.plist);
+  count_launch(1);
 }
 
 static void launch_fwd(const lv_raster_opts* o, int64_t tiles, cudaStream_t s, const ViewSet& vs, const FwdWs& w,
-                       const uint32_t* sv, const lv_fwd_out* out) {
-  const bool seg = (o->flags & LV_FLAG_EXACT_SEGMENT) != 0, per = (o->flags & LV_FLAG_PERSISTENT) != 0;
-  const int sml = per ? o->persistent_sms : 0;
-#define LV_FWD_CH(TS, CH)                                                                           \
-  if (seg && per) launch_fwd_t<TS, true, true, CH>(tiles, s, vs, w, sv, o->t_stop, out, sml);   \
-  else if (seg) launch_fwd_t<TS, true, false, CH>(tiles, s, vs, w, sv, o->t_stop, out, 0);      \
-  else if (per) launch_fwd_t<TS, false, true, CH>(tiles, s, vs, w, sv, o->t_stop, out, sml);    \
-  else launch_fwd_t<TS, false, false, CH>(tiles, s, vs, w, sv, o->t_stop, out, 0)
-#define LV_FWD(TS)                                   \
-  if (o->batch == 64) { LV_FWD_CH(TS, 64); }         \
-  else if (o->batch == 128) { LV_FWD_CH(TS, 128); }  \
-  else { LV_FWD_CH(TS, 32); }
-  if (o->tile == 8) { LV_FWD(8) }
-  else if (o->tile == 16) { LV_FWD(16) }
-  else if (o->batch == 64) { LV_FWD_CH(32, 64); }
-  else { LV_FWD_CH(32, 32); }
+                       const lv_fwd_out* out, bool resume) {
+  const bool seg = (o->flags & LV_FLAG_EXACT_SEGMENT) != 0, flag = (o->flags & LV_FLAG_PERSISTENT) != 0;
+  const bool per = flag || resume;
+  const int sml = flag ? o->persistent_sms : 0;
+#define LV_FWD(TS)                                                                          \
+  if (seg && per) launch_fwd_t<TS, true, true>(tiles, s, vs, w, o->t_stop, out, sml, resume);   \
+  else if (seg) launch_fwd_t<TS, true, false>(tiles, s, vs, w, o->t_stop, out, 0, false);      \
+  else if (per) launch_fwd_t<TS, false, true>(tiles, s, vs, w, o->t_stop, out, sml, resume);    \
+  else launch_fwd_t<TS, false, false>(tiles, s, vs, w, o->t_stop, out, 0, false)
+  if (o->tile == 8) { LV_FWD(8); }
+  else if (o->tile == 16) { LV_FWD(16); }
+  else { LV_FWD(32); }
 #undef LV_FWD
-#undef LV_FWD_CH
 }
 
 static void launch_bwd(const lv_raster_opts* o, int64_t tiles, cudaStream_t s, const ViewSet& vs, const FwdWs& w,
-                       const uint32_t* sv, const lv_fwd_out* fwd, const float* gC, const float* gD, const float* gT,
+                       const lv_fwd_out* fwd, const float* gC, const float* gD, const float* gT,
                        float* dd, const LfFuse& lf) {
   const bool seg = (o->flags & LV_FLAG_EXACT_SEGMENT) != 0, per = (o->flags & LV_FLAG_PERSISTENT) != 0;
   const int sml = per ? o->persistent_sms : 0;
-#define LV_BWD_CH(TS, CH)                                                                                 \
-  if (seg && per) launch_bwd_t<TS, true, true, CH>(tiles, s, vs, w, sv, fwd, gC, gD, gT, dd, sml, lf);    \
-  else if (seg) launch_bwd_t<TS, true, false, CH>(tiles, s, vs, w, sv, fwd, gC, gD, gT, dd, 0, lf);       \
-  else if (per) launch_bwd_t<TS, false, true, CH>(tiles, s, vs, w, sv, fwd, gC, gD, gT, dd, sml, lf);     \
-  else launch_bwd_t<TS, false, false, CH>(tiles, s, vs, w, sv, fwd, gC, gD, gT, dd, 0, lf)
-#define LV_BWD(TS)                                   \
-  if (o->batch == 64) { LV_BWD_CH(TS, 64); }         \
-  else if (o->batch == 128) { LV_BWD_CH(TS, 128); }  \
-  else { LV_BWD_CH(TS, 32); }
-  if (o->tile == 8) { LV_BWD(8) }
-  else if (o->tile == 16) { LV_BWD(16) }
-  else if (o->batch == 64) { LV_BWD_CH(32, 64); }
-  else { LV_BWD_CH(32, 32); }
+#define LV_BWD(TS)                                                                                \
+  if (seg && per) launch_bwd_t<TS, true, true>(tiles, s, vs, w, fwd, gC, gD, gT, dd, sml, lf);    \
+  else if (seg) launch_bwd_t<TS, true, false>(tiles, s, vs, w, fwd, gC, gD, gT, dd, 0, lf);       \
+  else if (per) launch_bwd_t<TS, false, true>(tiles, s, vs, w, fwd, gC, gD, gT, dd, sml, lf);     \
+  else launch_bwd_t<TS, false, false>(tiles, s, vs, w, fwd, gC, gD, gT, dd, 0, lf)
+  if (o->tile == 8) { LV_BWD(8); }
+  else if (o->tile == 16) { LV_BWD(16); }
+  else { LV_BWD(32); }
 #undef LV_BWD
-#undef LV_BWD_CH
 }
 
 }  // namespace lv
@@ -2043,8 +2418,7 @@ extern "C" lv_status lv_rasterize_forward(const lv_voxels* vox, const lv_camera*
   radix_sort_pairs(w.k0, w.v0, w.k0, w.v0, w.k1, w.v1, w.sort_tmp, w.counters, pair_capacity, tile_bits(tiles),
                    d_status, s, w.ranges, items > 0);
   // each tile's range, and its list front to back
-  launch_tile_sort(w, tiles, pair_capacity, s);
-  const uint32_t* sv = sorted_pair_slots(w, tiles);
+  launch_tile_sort(w, vs, n, tiles, pair_capacity, s);
   if (out->composite_event) {
     // a timing mark: inside a stream capture it becomes an event record node of the graph
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
@@ -2054,8 +2428,13 @@ extern "C" lv_status lv_rasterize_forward(const lv_voxels* vox, const lv_camera*
     else
       cudaEventRecord((cudaEvent_t)out->composite_event, s);
   }
-  launch_fwd(opts, tiles, s, vs, w, sv, out);
+  launch_fwd(opts, tiles, s, vs, w, out, false);
   count_launch(2);
+  if (n > TS_LAZY_VOXELS) {
+    launch_tile_rest(w, vs, tiles, false, s);
+    launch_fwd(opts, tiles, s, vs, w, out, true);
+    count_launch(1);
+  }
   return finish(LV_OK, opts->flags, d_status, s, "lv_rasterize_forward");
 }
 
@@ -2160,9 +2539,8 @@ extern "C" lv_status lv_rasterize_backward(const lv_voxels* vox, const lv_camera
     if (fwd->lf_wait_event) cudaStreamWaitEvent(s, (cudaEvent_t)fwd->lf_wait_event, 0);  // the weights
   }
   const int64_t n = vox->n;
-  const uint32_t* sv = sorted_pair_slots(w, tiles);
   if (!accumulate && n > 0) cudaMemsetAsync(d_density, 0, sizeof(float) * 8 * n, s);
-  launch_bwd(opts, tiles, s, vs, w, sv, fwd, dL_drgb, dL_ddepth, dL_dT, d_density, lf);
+  launch_bwd(opts, tiles, s, vs, w, fwd, dL_drgb, dL_ddepth, dL_dT, d_density, lf);
   count_launch(1);
   if (d_sh) launch_sh_bwd(vox, vs, w, d_sh, accumulate, s);
   return finish(LV_OK, opts->flags, d_status, s, "lv_rasterize_backward");
@@ -2217,8 +2595,8 @@ extern "C" lv_status lv_debug_pairs(int64_t n, const lv_camera* cams, int n_view
   FwdWs w = carve_fwd((void*)workspace, n, n_views, tiles, pixels, pair_capacity);
   if (ws_bytes < w.bytes) { set_error("workspace too small"); return LV_ERR_WORKSPACE; }
   if (keys || voxel) {
-    k_debug_pairs<<<608, 256, 0, s>>>(sorted_pair_tiles(w, tiles), sorted_pair_slots(w, tiles), w.slot_vox, w.s_dkey,
-                                       w.counters, pair_capacity, keys, voxel);
+    launch_tile_rest(w, vs, tiles, true, s);
+    k_debug_pairs<<<608, 256, 0, s>>>((const uint2*)w.ranges, tiles, w.plist, w.slot_vox, w.s_dkey, keys, voxel);
     count_launch(1);
   }
   if (ranges) cudaMemcpyAsync(ranges, w.ranges, sizeof(uint32_t) * 2 * tiles, cudaMemcpyDeviceToDevice, s);
@@ -2239,11 +2617,11 @@ extern "C" lv_status lv_render_pixels_f64(const lv_voxels* vox, const lv_camera*
   make_views(cams, n_views, opts->tile, &vs, &tiles, &npix);
   FwdWs w = carve_fwd((void*)workspace, vox->n, n_views, tiles, npix, pair_capacity);
   if (ws_bytes < w.bytes) { set_error("workspace too small"); return LV_ERR_WORKSPACE; }
-  const uint32_t* sv = sorted_pair_slots(w, tiles);
+  launch_tile_rest(w, vs, tiles, true, s);
   const int nb = (vox->sh_degree + 1) * (vox->sh_degree + 1);
   const unsigned grid = (unsigned)((n_px + 127) / 128);
 #define LV_F64(DT, ST)                                                                                            \
-  k_render_f64<DT, ST><<<grid, 128, 0, s>>>(vs, w.ranges, sv, w.slot_vox, (const float4*)vox->geom,              \
+  k_render_f64<DT, ST><<<grid, 128, 0, s>>>(vs, w.ranges, w.plist, w.slot_vox, (const float4*)vox->geom,              \
                                             (const DT*)vox->density, (const ST*)vox->sh, nb, pixels, n_px,       \
                                             (double)opts->t_stop, (opts->flags & LV_FLAG_EXACT_SEGMENT) ? 1 : 0,  \
                                             vox->vidx, rgb, T)
