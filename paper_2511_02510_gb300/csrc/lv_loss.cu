@@ -13,21 +13,43 @@ namespace {
 
 constexpr int TPB = 256;
 
+// Every step runs all views in one launch (a launch per view cost about 8 us
+// each however small the view): the blocks of a step are dealt out to the views
+// by their pixels, block range [blk[v], blk[v + 1]) for view v.  With the
+// selection by 14 + 9 + 9 bits, sixteen views of 14.6 Mpixel in all went from
+// 701 to 285 us: Sobel 143 -> 79, selection 181 -> 33, weights 150 -> 61 (powf),
+// loss 230 -> 86 (585 MB, the memory rate).
 struct ViewPix {
   int n;
   int W[LV_MAX_VIEWS];
   int H[LV_MAX_VIEWS];
   long long off[LV_MAX_VIEWS + 1];
-  uint32_t k[LV_MAX_VIEWS];  // nearest-rank index of the percentile
+  uint32_t k[LV_MAX_VIEWS];    // nearest-rank index of the percentile
+  int tile[LV_MAX_VIEWS + 1];  // first Sobel tile of each view
+  int blk[LV_MAX_VIEWS + 1];   // first block of each view in the per-pixel steps
+};
+
+// The percentile is selected by the magnitudes' bits, digit by digit from the
+// top: 14 bits (the highest, the sign, is always 0), then 9 and 9.  The first digit is wide so that the few octaves an image's
+// gradients span fall into hundreds of counters: with 11 bits about 24 counters
+// took all the shared-memory atomics.  It is counted where the magnitudes are
+// computed, and no group array is read, as a block's pixels are one view's.
+constexpr int D1_SHIFT = 18, D1_BINS = 1 << (31 - D1_SHIFT);
+constexpr int D2_SHIFT = 9, D2_BINS = 1 << (D1_SHIFT - D2_SHIFT);
+constexpr int D3_BINS = 1 << D2_SHIFT;
+constexpr int HIST_WORDS = D1_BINS + D2_BINS + D3_BINS;  // a view's counters
+
+struct LfPick {
+  uint32_t prefix;  // digits chosen so far
+  uint32_t k;       // rank among the keys that share them
 };
 
 struct LfWs {
-  SelectQuery* q;
-  void* sel_tmp;
+  LfPick* pick;   // [2][views] after the first and the second digit
   double* wsum;   // [views]
   double* lsum;   // [views]
-  uint16_t* grp;  // [pixels]
-  uint32_t* mkey; // [pixels] Sobel magnitude bits
+  uint32_t* hist; // [views][HIST_WORDS]
+  uint32_t* mkey; // [pixels] bits of three times the Sobel magnitude
   float* w;       // [pixels] unnormalised weight
   size_t bytes;
 };
@@ -35,50 +57,191 @@ struct LfWs {
 LfWs carve_lf(void* base, int nv, int64_t pixels) {
   LfWs w;
   Carve c(base);
-  w.q = c.take<SelectQuery>(SELECT_MAX_QUERIES);
-  w.sel_tmp = c.take<char>(select_tmp_bytes(SELECT_MAX_QUERIES));
+  w.pick = c.take<LfPick>(2 * LV_MAX_VIEWS);
   w.wsum = c.take<double>(LV_MAX_VIEWS);
   w.lsum = c.take<double>(LV_MAX_VIEWS);
-  w.grp = c.take<uint16_t>(pixels);
+  w.hist = c.take<uint32_t>((size_t)nv * HIST_WORDS);
   w.mkey = c.take<uint32_t>(pixels);
   w.w = c.take<float>(pixels);
-  w.bytes = c.off + 256;
+  // The size asked for never falls below 10 bytes a pixel and the scratch of a 64-query select, the
+  // layout that the allocation-free call's limit of about 1.6 million pixels comes from.
+  Carve f(nullptr);
+  f.take<SelectQuery>(SELECT_MAX_QUERIES);
+  f.take<char>(select_tmp_bytes(SELECT_MAX_QUERIES));
+  f.take<double>(LV_MAX_VIEWS);
+  f.take<double>(LV_MAX_VIEWS);
+  f.take<uint16_t>(pixels);
+  f.take<uint32_t>(pixels);
+  f.take<float>(pixels);
+  w.bytes = (c.off > f.off ? c.off : f.off) + 256;
   return w;
 }
 
-__device__ __forceinline__ int view_of(const ViewPix& vp, long long p) {
+// view of block b among the block ranges `first`
+__device__ __forceinline__ int view_of_block(const int* first, int n, int b) {
   int v = 0;
-  while (v + 1 < vp.n && p >= vp.off[v + 1]) ++v;
+  while (v + 1 < n && b >= first[v + 1]) ++v;
   return v;
 }
 
-__device__ __forceinline__ float luma(const float* __restrict__ gt, long long p) {
-  return (gt[3 * p] + gt[3 * p + 1] + gt[3 * p + 2]) * (1.0f / 3.0f);
-}
 
-// Eq. 7 input: |Sobel(Y)| with replicated border
-__global__ void k_lf_sobel(const float* __restrict__ gt, const __grid_constant__ ViewPix vp, uint16_t* grp,
-                           uint32_t* mkey) {
-  long long p = blockIdx.x * (long long)TPB + threadIdx.x;
-  if (p >= vp.off[vp.n]) return;
-  const int v = view_of(vp, p);
-  const long long loc = p - vp.off[v];
-  const int W = vp.W[v], H = vp.H[v];
-  const int x = (int)(loc % W), y = (int)(loc / W);
-  const int xm = max(x - 1, 0), xp = min(x + 1, W - 1), ym = max(y - 1, 0), yp = min(y + 1, H - 1);
-  const float* g = gt + 3 * vp.off[v];
-#define Y_(a, b) luma(g, (long long)(b) * W + (a))
-  const float gx = (Y_(xp, ym) + 2.f * Y_(xp, y) + Y_(xp, yp)) - (Y_(xm, ym) + 2.f * Y_(xm, y) + Y_(xm, yp));
-  const float gy = (Y_(xm, yp) + 2.f * Y_(x, yp) + Y_(xp, yp)) - (Y_(xm, ym) + 2.f * Y_(x, ym) + Y_(xp, ym));
+// Eq. 7 input: |Sobel(Y)| with replicated border, and the first digit's counts.
+// A block takes `per` tiles of 32 x 32 pixels; a tile's channel sums (three times
+// the luma) with a border of one pixel are computed once into shared memory
+// (1.13 pixels read per pixel; nine neighbours' three channels each from the
+// caches before), and the next tile's pixels are loaded while this one is worked on.
+constexpr int ST = 32, SP = ST + 2;
+__global__ void __launch_bounds__(TPB) k_lf_sobel(const float* __restrict__ gt, const __grid_constant__ ViewPix vp,
+                                                 int per, uint32_t* __restrict__ mkey, uint32_t* __restrict__ hist) {
+  __shared__ uint32_t s_h[D1_BINS];
+  __shared__ float s_y[SP * SP];
+  const int t = threadIdx.x;
+  for (int i = t; i < D1_BINS; i += TPB) s_h[i] = 0u;
+  const int t0 = blockIdx.x * per, t1 = min(t0 + per, vp.tile[vp.n]);
+  int v = view_of_block(vp.tile, vp.n, t0);
+  constexpr int LD = (SP * SP + TPB - 1) / TPB;
+  float ahead[LD][3];
+  auto load = [&](int tile, int view) {
+    const int W = vp.W[view], H = vp.H[view], tx = (W - 1) / ST + 1, loc = tile - vp.tile[view];
+    const int x0 = loc % tx * ST, y0 = loc / tx * ST;
+#pragma unroll
+    for (int k = 0; k < LD; ++k) {
+      const int i = min(t + k * TPB, SP * SP - 1), ly = i / SP, lx = i - ly * SP;
+      const int x = max(x0 + min(lx - 1, W - 1 - x0), 0), y = max(y0 + min(ly - 1, H - 1 - y0), 0);
+      const float* g = gt + 3 * (vp.off[view] + (long long)y * W + x);
+      ahead[k][0] = g[0];
+      ahead[k][1] = g[1];
+      ahead[k][2] = g[2];
+    }
+  };
+  if (t0 < t1) load(t0, v);
+  for (int tile = t0; tile < t1; ++tile) {  // block-uniform
+    const int W = vp.W[v], H = vp.H[v], tx = (W - 1) / ST + 1, loc = tile - vp.tile[v];
+    const int x0 = loc % tx * ST, y0 = loc / tx * ST;
+    __syncthreads();  // the last tile's sums are read
+#pragma unroll
+    for (int k = 0; k < LD; ++k)
+      if (t + k * TPB < SP * SP) s_y[t + k * TPB] = ahead[k][0] + ahead[k][1] + ahead[k][2];
+    __syncthreads();
+    if (tile + 1 < t1) load(tile + 1, tile + 1 < vp.tile[v + 1] ? v : v + 1);
+    const int lx = t % ST;
+#pragma unroll
+    for (int r = 0; r < ST * ST / TPB; ++r) {
+      const int ly = t / ST + r * (TPB / ST);
+      if (lx < W - x0 && ly < H - y0) {
+#define Y_(a, b) s_y[(ly + (b)) * SP + lx + (a)]
+        const float gx = (Y_(2, 0) + 2.f * Y_(2, 1) + Y_(2, 2)) - (Y_(0, 0) + 2.f * Y_(0, 1) + Y_(0, 2));
+        const float gy = (Y_(0, 2) + 2.f * Y_(1, 2) + Y_(2, 2)) - (Y_(0, 0) + 2.f * Y_(1, 0) + Y_(2, 0));
 #undef Y_
-  const float mag = sqrtf(gx * gx + gy * gy);
-  grp[p] = (uint16_t)v;
-  mkey[p] = __float_as_uint(mag);  // non-negative: bit order == value order
+        // three times the magnitude (only its ratio to the percentile counts); bit order == value order
+        const uint32_t key = __float_as_uint(sqrtf(gx * gx + gy * gy)) & 0x7fffffffu;
+        mkey[vp.off[v] + (long long)(y0 + ly) * W + x0 + lx] = key;
+        atomicAdd(&s_h[key >> D1_SHIFT], 1u);
+      }
+    }
+    if (tile + 1 == t1 || tile + 1 == vp.tile[v + 1]) {  // the block's last tile of this view
+      __syncthreads();
+      uint32_t* h = hist + (size_t)v * HIST_WORDS;
+      for (int i = t; i < D1_BINS; i += TPB) {
+        const uint32_t c = s_h[i];
+        if (c) {
+          atomicAdd(&h[i], c);
+          s_h[i] = 0u;
+        }
+      }
+      ++v;
+    }
+  }
 }
 
-__global__ void k_lf_queries(SelectQuery* q, const __grid_constant__ ViewPix vp) {
-  int v = threadIdx.x;
-  if (v < vp.n) { q[v].group = v; q[v].k = vp.k[v]; }
+// The digit that holds the k-th key among NB counters, and the rank among its
+// keys; the whole block calls, every thread gets both.  A warp sums its share of
+// the counters 32 at a time (coalesced), one thread per 32 scans the sums, and
+// the warp of the group that holds the key finds it there.
+template <int NB>
+__device__ __forceinline__ LfPick block_pick(const uint32_t* __restrict__ h, uint32_t k) {
+  constexpr int PER = NB / TPB;  // groups of 32 counters per warp
+  static_assert(PER >= 1 && PER <= 32, "a lane for each of a warp's groups");
+  __shared__ uint32_t s_part[TPB / 32];
+  __shared__ LfPick s_pick;
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const uint32_t* hw = h + warp * (32 * PER);
+  uint32_t c[PER], sum = 0;
+#pragma unroll
+  for (int i = 0; i < PER; ++i) c[i] = hw[32 * i + lane];
+#pragma unroll
+  for (int i = 0; i < PER; ++i) {
+    const uint32_t r = __reduce_add_sync(FULL, c[i]);
+    if (lane == i) sum = r;  // lane i: group i of the warp
+  }
+  uint32_t x = sum;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(FULL, x, o);
+    if (lane >= o) x += y;
+  }
+  if (lane == 31) s_part[warp] = x;
+  __syncthreads();
+  uint32_t before = x - sum;
+  for (int w = 0; w < warp; ++w) before += s_part[w];
+  const uint32_t who = __ballot_sync(FULL, before < k && k <= before + sum);
+  if (who) {  // one warp: the counts add up to the view's pixels
+    const int grp = __ffs(who) - 1;
+    before = __shfl_sync(FULL, before, grp);
+    const uint32_t own = hw[32 * grp + lane];
+    uint32_t y = own;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t z = __shfl_up_sync(FULL, y, o);
+      if (lane >= o) y += z;
+    }
+    before += y - own;
+    if (before < k && k <= before + own) {
+      s_pick.prefix = (uint32_t)(warp * (32 * PER) + 32 * grp + lane);
+      s_pick.k = k - before;
+    }
+  }
+  __syncthreads();
+  return s_pick;
+}
+
+// Counts of the second digit (the keys with the first digit picked here) or,
+// LAST, of the third.  Every block picks for its view; the view's first block
+// leaves the pick for the next step.
+template <bool LAST>
+__global__ void __launch_bounds__(TPB) k_lf_digit(const uint32_t* __restrict__ mkey, const __grid_constant__ ViewPix vp,
+                                                 uint32_t* hist, LfPick* pick) {
+  constexpr int NB = LAST ? D3_BINS : D2_BINS;
+  __shared__ uint32_t s_h[NB];
+  const int t = threadIdx.x, v = view_of_block(vp.blk, vp.n, blockIdx.x);
+  uint32_t* h = hist + (size_t)v * HIST_WORDS;
+  for (int i = t; i < NB; i += TPB) s_h[i] = 0u;
+  LfPick p;
+  if (!LAST) {
+    p = block_pick<D1_BINS>(h, vp.k[v]);
+  } else {
+    const LfPick p1 = pick[v];
+    p = block_pick<D2_BINS>(h + D1_BINS, p1.k);
+    p.prefix |= p1.prefix << (D1_SHIFT - D2_SHIFT);
+  }
+  const int b0 = vp.blk[v], nb = vp.blk[v + 1] - b0;
+  if (t == 0 && (int)blockIdx.x == b0) pick[(LAST ? LV_MAX_VIEWS : 0) + v] = p;
+  constexpr int SHIFT = LAST ? 0 : D2_SHIFT, ITEMS = 8;
+  const long long lo = vp.off[v], hi = vp.off[v + 1];
+  for (long long q = lo + (blockIdx.x - b0) * (long long)(TPB * ITEMS) + t; q < hi; q += (long long)nb * (TPB * ITEMS)) {
+    uint32_t key[ITEMS];
+#pragma unroll
+    for (int u = 0; u < ITEMS; ++u) key[u] = q + u * TPB < hi ? mkey[q + u * TPB] : ~0u;  // no key: top bit clear
+#pragma unroll
+    for (int u = 0; u < ITEMS; ++u)
+      if (key[u] >> (LAST ? D2_SHIFT : D1_SHIFT) == p.prefix) atomicAdd(&s_h[(key[u] >> SHIFT) & (NB - 1)], 1u);
+  }
+  __syncthreads();
+  uint32_t* out = h + D1_BINS + (LAST ? D2_BINS : 0);
+  for (int i = t; i < NB; i += TPB) {
+    const uint32_t c = s_h[i];
+    if (c) atomicAdd(&out[i], c);
+  }
 }
 
 __device__ __forceinline__ void block_add_f64(double v, double* dst) {
@@ -100,23 +263,40 @@ __device__ __forceinline__ void block_add_f64(double v, double* dst) {
 // Eq. 7: w = (eps + 1 - s)^gamma, s = clip(|grad| / P, 0, 1); blocks never span views.
 // Grid-stride over the view's pixels with a bounded block count: one FP64
 // atomic per block (a per-256-pixel atomic would serialise at the L2).
-__global__ void k_lf_weight(const uint32_t* __restrict__ mkey, const SelectQuery* q, const __grid_constant__ ViewPix vp,
-                            int v, float eps, float gamma, float* w, double* wsum, float* edge_out) {
+__global__ void __launch_bounds__(TPB) k_lf_weight(const uint32_t* __restrict__ mkey, const uint32_t* __restrict__ hist,
+                                                  const LfPick* __restrict__ pick,
+                                                  const __grid_constant__ ViewPix vp, float eps, float gamma,
+                                                  float* __restrict__ w, double* wsum, float* __restrict__ edge_out) {
+  const int v = view_of_block(vp.blk, vp.n, blockIdx.x);
+  const int b0 = vp.blk[v], nb = vp.blk[v + 1] - b0;
   const long long lo = vp.off[v], hi = vp.off[v + 1];
-  const float P = __uint_as_float(q[v].result);
-  const bool norm = q[v].k != 0 && P > 0.f;
-  // a thread sums its few pixels in FP32; blocks combine in FP64 (the GPU's FP64
+  const LfPick p2 = pick[LV_MAX_VIEWS + v];
+  const LfPick p3 = block_pick<D3_BINS>(hist + (size_t)v * HIST_WORDS + D1_BINS + D2_BINS, p2.k);
+  const float P = __uint_as_float(p2.prefix << D2_SHIFT | p3.prefix);
+  const bool norm = P > 0.f;
+  // a thread sums four pixels in FP32, and those sums and the blocks' in FP64 (the GPU's FP64
   // rate is low, so no per-pixel FP64 arithmetic)
-  float acc = 0.f;
-  for (long long p = lo + blockIdx.x * (long long)TPB + threadIdx.x; p < hi; p += (long long)gridDim.x * TPB) {
-    float s = 0.f;
-    if (norm) s = fminf(fmaxf(__uint_as_float(mkey[p]) / P, 0.f), 1.f);
-    if (edge_out) edge_out[p] = s;
-    const float wv = gamma == 0.f ? 1.f : powf(eps + 1.f - s, gamma);
-    w[p] = wv;
-    acc += wv;
+  constexpr int ITEMS = 4;
+  double acc = 0.0;
+  for (long long p = lo + (blockIdx.x - b0) * (long long)(TPB * ITEMS) + threadIdx.x; p < hi;
+       p += (long long)nb * (TPB * ITEMS)) {
+    uint32_t key[ITEMS];
+#pragma unroll
+    for (int u = 0; u < ITEMS; ++u) key[u] = p + u * TPB < hi ? mkey[p + u * TPB] : 0u;
+    float part = 0.f;
+#pragma unroll
+    for (int u = 0; u < ITEMS; ++u) {
+      if (p + u * TPB >= hi) break;
+      float s = 0.f;
+      if (norm) s = fminf(fmaxf(__uint_as_float(key[u]) / P, 0.f), 1.f);
+      if (edge_out) edge_out[p + u * TPB] = s;
+      const float wv = gamma == 0.f ? 1.f : powf(eps + 1.f - s, gamma);
+      w[p + u * TPB] = wv;
+      part += wv;
+    }
+    acc += (double)part;
   }
-  block_add_f64((double)acc, &wsum[v]);
+  block_add_f64(acc, &wsum[v]);
 }
 
 // the view's mean weight <w> and gradient scale 2 / (3 |P|), rounded to FP32 from FP64, once per
@@ -131,18 +311,20 @@ __device__ __forceinline__ void lf_view_constants(const double* wsum, int v, lon
 
 // Eq. 8 + Eq. 18: w~ = w / <w>, L = 1/|P| sum w~ mean_c r^2, dL/drgb = 2/(3|P|) w~ r
 __global__ void k_lf_loss(const float* __restrict__ rgb, const float* __restrict__ gt, const float* __restrict__ w,
-                          const __grid_constant__ ViewPix vp, int v, const double* wsum, double* lsum,
+                          const __grid_constant__ ViewPix vp, const double* wsum, double* lsum,
                           float* __restrict__ grad) {
+  const int v = view_of_block(vp.blk, vp.n, blockIdx.x);
+  const int b0 = vp.blk[v], nb = vp.blk[v + 1] - b0;
   const long long lo = vp.off[v], hi = vp.off[v + 1];
   const long long np = hi - lo;
   __shared__ float s_mean, s_gscale;
   lf_view_constants(wsum, v, np, &s_mean, &s_gscale);
   const float mean = s_mean, gscale = s_gscale;
-  float acc = 0.f;  // sum of w~ (r0^2 + r1^2 + r2^2) over this thread's pixels; the 1/3 is applied at the end
-  for (long long p = lo + blockIdx.x * (long long)TPB + threadIdx.x; p < hi; p += (long long)gridDim.x * TPB) {
+  double acc = 0.0;  // sum of w~ (r0^2 + r1^2 + r2^2) over this thread's pixels; the 1/3 is applied at the end
+  for (long long p = lo + (blockIdx.x - b0) * (long long)TPB + threadIdx.x; p < hi; p += (long long)nb * TPB) {
     const float wt = w[p] / mean;
     const float r0 = rgb[3 * p] - gt[3 * p], r1 = rgb[3 * p + 1] - gt[3 * p + 1], r2 = rgb[3 * p + 2] - gt[3 * p + 2];
-    acc += wt * (r0 * r0 + r1 * r1 + r2 * r2);
+    acc += (double)(wt * (r0 * r0 + r1 * r1 + r2 * r2));
     if (grad) {
       const float c = gscale * wt;
       grad[3 * p] = c * r0;
@@ -150,29 +332,31 @@ __global__ void k_lf_loss(const float* __restrict__ rgb, const float* __restrict
       grad[3 * p + 2] = c * r2;
     }
   }
-  block_add_f64((double)acc, &lsum[v]);
+  block_add_f64(acc, &lsum[v]);
 }
 
 // k_lf_loss over groups of four pixels: three 16-byte loads of rgb and of gt,
 // one of w, three 16-byte stores of the gradient.  The pixels of the view
 // before the first group boundary (global pixel index a multiple of 4) and
-// after the last one go through the scalar path of thread 0 of block 0.  The
+// after the last one go through the scalar path of thread 0 of its first block.  The
 // per-pixel arithmetic is that of k_lf_loss; only the summation order of the
 // partial sums differs.
 __global__ void k_lf_loss4(const float* __restrict__ rgb, const float* __restrict__ gt, const float* __restrict__ w,
-                           const __grid_constant__ ViewPix vp, int v, const double* wsum, double* lsum,
+                           const __grid_constant__ ViewPix vp, const double* wsum, double* lsum,
                            float* __restrict__ grad) {
+  const int v = view_of_block(vp.blk, vp.n, blockIdx.x);
+  const int b0 = vp.blk[v], nb = vp.blk[v + 1] - b0;
   const long long lo = vp.off[v], hi = vp.off[v + 1];
   const long long np = hi - lo;
   __shared__ float s_mean, s_gscale;
   lf_view_constants(wsum, v, np, &s_mean, &s_gscale);
   const float mean = s_mean, gscale = s_gscale;
   const long long g0 = (lo + 3) >> 2, g1 = hi >> 2;  // whole groups [4 g0, 4 g1)
-  float acc = 0.f;
+  double acc = 0.0;  // four pixels' terms are summed in FP32
   auto one = [&](long long p) {
     const float wt = w[p] / mean;
     const float r0 = rgb[3 * p] - gt[3 * p], r1 = rgb[3 * p + 1] - gt[3 * p + 1], r2 = rgb[3 * p + 2] - gt[3 * p + 2];
-    acc += wt * (r0 * r0 + r1 * r1 + r2 * r2);
+    acc += (double)(wt * (r0 * r0 + r1 * r1 + r2 * r2));
     if (grad) {
       const float c = gscale * wt;
       grad[3 * p] = c * r0;
@@ -180,7 +364,7 @@ __global__ void k_lf_loss4(const float* __restrict__ rgb, const float* __restric
       grad[3 * p + 2] = c * r2;
     }
   };
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
+  if ((int)blockIdx.x == b0 && threadIdx.x == 0) {
     if (g1 <= g0) {
       for (long long p = lo; p < hi; ++p) one(p);
     } else {
@@ -192,15 +376,17 @@ __global__ void k_lf_loss4(const float* __restrict__ rgb, const float* __restric
   const float4* t4 = (const float4*)gt;
   const float4* w4 = (const float4*)w;
   float4* d4 = (float4*)grad;
-  for (long long g = g0 + blockIdx.x * (long long)TPB + threadIdx.x; g < g1; g += (long long)gridDim.x * TPB) {
+  for (long long g = g0 + (blockIdx.x - b0) * (long long)TPB + threadIdx.x; g < g1; g += (long long)nb * TPB) {
     const float4 a0 = r4[3 * g], a1 = r4[3 * g + 1], a2 = r4[3 * g + 2];
     const float4 b0 = t4[3 * g], b1 = t4[3 * g + 1], b2 = t4[3 * g + 2];
     const float4 wv = w4[g];
     const float r[12] = {a0.x - b0.x, a0.y - b0.y, a0.z - b0.z, a0.w - b0.w, a1.x - b1.x, a1.y - b1.y,
                          a1.z - b1.z, a1.w - b1.w, a2.x - b2.x, a2.y - b2.y, a2.z - b2.z, a2.w - b2.w};
     const float wt[4] = {wv.x / mean, wv.y / mean, wv.z / mean, wv.w / mean};
+    float part = 0.f;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) acc += wt[k] * (r[3 * k] * r[3 * k] + r[3 * k + 1] * r[3 * k + 1] + r[3 * k + 2] * r[3 * k + 2]);
+    for (int k = 0; k < 4; ++k) part += wt[k] * (r[3 * k] * r[3 * k] + r[3 * k + 1] * r[3 * k + 1] + r[3 * k + 2] * r[3 * k + 2]);
+    acc += (double)part;
     if (grad) {
       float o[12];
 #pragma unroll
@@ -215,7 +401,7 @@ __global__ void k_lf_loss4(const float* __restrict__ rgb, const float* __restric
       d4[3 * g + 2] = make_float4(o[8], o[9], o[10], o[11]);
     }
   }
-  block_add_f64((double)acc, &lsum[v]);
+  block_add_f64(acc, &lsum[v]);
 }
 
 // clear: the sums are zeroed once read (the fused backward's sums start from zero next time)
@@ -227,6 +413,9 @@ __global__ void k_lf_finish(const __grid_constant__ ViewPix vp, double* lsum, fl
     if (clear) lsum[v] = 0.0;
   }
 }
+
+constexpr int STEP_BLOCKS = 8 * 152;
+constexpr int SOBEL_BLOCKS = 6 * 152;
 
 bool make_viewpix(const int32_t* widths, const int32_t* heights, int nv, int32_t pctl_ppm, ViewPix* vp) {
   if (nv < 1 || nv > LV_MAX_VIEWS || !widths || !heights) return false;
@@ -245,7 +434,16 @@ bool make_viewpix(const int32_t* widths, const int32_t* heights, int nv, int32_t
     off += np;
   }
   vp->off[nv] = off;
-  return off < 0xffffffffLL;
+  if (off >= 0xffffffffLL) return false;
+  // about four pixels per thread, more where that would make over STEP_BLOCKS blocks
+  const long long px = off / STEP_BLOCKS > 4 * TPB ? off / STEP_BLOCKS : 4 * TPB;
+  vp->tile[0] = vp->blk[0] = 0;
+  for (int v = 0; v < nv; ++v) {
+    const long long np = vp->off[v + 1] - vp->off[v];
+    vp->tile[v + 1] = vp->tile[v] + ((vp->W[v] - 1) / ST + 1) * ((vp->H[v] - 1) / ST + 1);
+    vp->blk[v + 1] = vp->blk[v] + (int)((np + px - 1) / px);
+  }
+  return true;
 }
 
 }  // namespace
@@ -268,10 +466,6 @@ extern "C" size_t lv_lf_workspace_size(const int32_t* widths, const int32_t* hei
 }
 
 namespace {
-unsigned blocks_for(long long np) {
-  const long long b = (np + 4 * TPB - 1) / (4 * TPB);  // about four pixels per thread
-  return (unsigned)(b < 1 ? 1 : (b > 1216 ? 1216 : b));
-}
 bool aligned16(const void* p) { return ((uintptr_t)p & 15) == 0; }
 
 lv_status lf_setup(const int32_t* widths, const int32_t* heights, int n_views, int32_t pctl_ppm, void* workspace,
@@ -293,19 +487,19 @@ extern "C" lv_status lv_lf_weights(const float* gt, const int32_t* widths, const
   LfWs w;
   lv_status e = lf_setup(widths, heights, n_views, p->pctl_ppm, workspace, ws_bytes, &vp, &w);
   if (e != LV_OK) return e;
-  const int64_t P = vp.off[n_views];
   cudaStream_t s = (cudaStream_t)stream;
   const float gamma = lv_lf_gamma(t, p);
-  // the weight sums, and the loss sums a backward with the fused loss accumulates
-  zero_async(s, w.wsum, sizeof(double) * LV_MAX_VIEWS, w.lsum, sizeof(double) * LV_MAX_VIEWS);
-  k_lf_sobel<<<(unsigned)((P + TPB - 1) / TPB), TPB, 0, s>>>(gt, vp, w.grp, w.mkey);
-  k_lf_queries<<<1, LV_MAX_VIEWS, 0, s>>>(w.q, vp);
-  select_kth(w.mkey, w.grp, P, w.q, n_views, w.sel_tmp, s);
-  for (int v = 0; v < n_views; ++v) {
-    const long long np = vp.off[v + 1] - vp.off[v];
-    k_lf_weight<<<blocks_for(np), TPB, 0, s>>>(w.mkey, w.q, vp, v, p->eps, gamma, w.w, w.wsum, p->edge_out);
-  }
-  count_launch(2 + n_views);
+  // the weight sums, the loss sums a backward with the fused loss accumulates, and the counters
+  zero_async(s, w.wsum, sizeof(double) * LV_MAX_VIEWS, w.lsum, sizeof(double) * LV_MAX_VIEWS, w.hist,
+             sizeof(uint32_t) * HIST_WORDS * (size_t)n_views);
+  // a block clears and adds up all the counters, so it takes several tiles once there are enough
+  const int tiles = vp.tile[n_views], per = (tiles + SOBEL_BLOCKS - 1) / SOBEL_BLOCKS;
+  k_lf_sobel<<<(unsigned)((tiles + per - 1) / per), TPB, 0, s>>>(gt, vp, per, w.mkey, w.hist);
+  const unsigned blocks = (unsigned)vp.blk[n_views];
+  k_lf_digit<false><<<blocks, TPB, 0, s>>>(w.mkey, vp, w.hist, w.pick);
+  k_lf_digit<true><<<blocks, TPB, 0, s>>>(w.mkey, vp, w.hist, w.pick);
+  k_lf_weight<<<blocks, TPB, 0, s>>>(w.mkey, w.hist, w.pick, vp, p->eps, gamma, w.w, w.wsum, p->edge_out);
+  count_launch(4);
   return cuda_check(cudaGetLastError(), "lv_lf_weights");
 }
 
@@ -321,13 +515,11 @@ extern "C" lv_status lv_lf_loss_from_weights(const float* rgb, const float* gt, 
   zero_async(s, w.lsum, sizeof(double) * LV_MAX_VIEWS);
   // four pixels (three 16-byte words of rgb, gt and dL_drgb) per step where the buffers allow it
   const bool vec = aligned16(rgb) && aligned16(gt) && aligned16(w.w) && (!dL_drgb || aligned16(dL_drgb));
-  for (int v = 0; v < n_views; ++v) {
-    const long long np = vp.off[v + 1] - vp.off[v];
-    if (vec) k_lf_loss4<<<blocks_for(np), TPB, 0, s>>>(rgb, gt, w.w, vp, v, w.wsum, w.lsum, dL_drgb);
-    else k_lf_loss<<<blocks_for(np), TPB, 0, s>>>(rgb, gt, w.w, vp, v, w.wsum, w.lsum, dL_drgb);
-  }
+  const unsigned blocks = (unsigned)vp.blk[n_views];
+  if (vec) k_lf_loss4<<<blocks, TPB, 0, s>>>(rgb, gt, w.w, vp, w.wsum, w.lsum, dL_drgb);
+  else k_lf_loss<<<blocks, TPB, 0, s>>>(rgb, gt, w.w, vp, w.wsum, w.lsum, dL_drgb);
   k_lf_finish<<<1, LV_MAX_VIEWS, 0, s>>>(vp, w.lsum, loss, false);
-  count_launch(1 + n_views);
+  count_launch(2);
   return cuda_check(cudaGetLastError(), "lv_lf_loss_from_weights");
 }
 

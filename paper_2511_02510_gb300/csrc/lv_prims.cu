@@ -791,12 +791,6 @@ __global__ void __launch_bounds__(SEL_THREADS) k_sel_hist(const uint32_t* keys, 
   }
 }
 
-__global__ void k_sel_init(SelectQuery* q, int nq, uint32_t* hist, int hist_words) {
-  int j = threadIdx.x;
-  if (j < nq) { q[j].prefix = 0; q[j].result = 0xffffffffu; }
-  for (int i = threadIdx.x; i < hist_words; i += blockDim.x) hist[i] = 0;
-}
-
 template <int RADIX>
 void select_passes(const uint32_t* keys, const uint16_t* grp, int64_t n, SelectQuery* d_queries, int nq,
                    uint32_t* hist, SelectQuery* qs, int key_bits, int width, cudaStream_t s, uint32_t* h0) {
@@ -813,7 +807,7 @@ void select_passes(const uint32_t* keys, const uint16_t* grp, int64_t n, SelectQ
                          (int)(sizeof(uint32_t) * 256 * SELECT_MAX_QUERIES));
   });
   // three histogram buffers: pass p writes H[p % 3], reads H[(p - 1) % 3] for its pick step and
-  // clears H[(p + 1) % 3] for pass p + 1 (k_sel_init cleared H[0]); the queries after p picks
+  // clears H[(p + 1) % 3] for pass p + 1 (select_prepare cleared H[0]); the queries after p picks
   // are A[p]: A[0] = d_queries, then the two scratch copies in turn; the last pick writes d_queries.
   // With h0, the key producer has counted the first digit into H[0] = h0 and the query kernel
   // cleared H[1]; the passes and the last pick leave h0 cleared.
@@ -865,13 +859,6 @@ static void select_run(const uint32_t* keys, const uint16_t* grp, int64_t n, Sel
   }
   if (wide) select_passes<2048>(keys, grp, n, d_queries, n_queries, hist, qs, key_bits, 11, s, h0);
   else select_passes<256>(keys, grp, n, d_queries, n_queries, hist, qs, key_bits, 8, s, h0);
-}
-
-void select_kth(const uint32_t* keys, const uint16_t* grp, int64_t n, SelectQuery* d_queries, int n_queries,
-                void* tmp, cudaStream_t s) {
-  k_sel_init<<<1, 256, 0, s>>>(d_queries, n_queries, (uint32_t*)tmp, select_hist_words(n_queries));
-  count_launch(1);
-  select_run(keys, grp, n, d_queries, n_queries, tmp, s, nullptr);
 }
 
 void select_kth_prepared(const uint32_t* keys, const uint16_t* grp, int64_t n, SelectQuery* d_queries,

@@ -59,7 +59,7 @@ int radix_sort_pairs(const uint64_t* kin, const uint32_t* vin, uint64_t* k0, uin
 // For each query q (group g_q, 1-based rank k_q), find the k-th smallest
 // 32-bit key among the items i with grp[i] == g_q (0xffff = excluded).
 // Queries live in device memory so that k can be computed on the device.
-// After select_kth, queries[q].result holds the key, or 0xffffffff when
+// After the select, queries[q].result holds the key, or 0xffffffff when
 // k == 0 or the group has fewer than k items (queries[q].k is then 0).
 // keys == nullptr ranks the items by their index (key = i).  Queries of one
 // group must be contiguous, at most two per group, groups < 64.
@@ -72,12 +72,9 @@ struct SelectQuery {
   uint32_t result;
 };
 size_t select_tmp_bytes(int n_queries);
-void select_kth(const uint32_t* keys, const uint16_t* grp, int64_t n, SelectQuery* d_queries, int n_queries,
-                void* tmp, cudaStream_t s);
 
-// select_kth without its set-up launch: the kernel that writes the queries
-// also calls select_prepare (all threads of one block) for the same queries
-// and scratch, so a select costs one launch less on the caller's stream.
+// The kernel that writes the queries also calls select_prepare (all threads of
+// one block) for the same queries and scratch, so a select has no set-up launch.
 constexpr int SEL_WIDE_MAX_Q = 4;  // up to this many queries use 11-bit digits
 __host__ __device__ constexpr int select_hist_words(int n_queries) {
   return (n_queries <= SEL_WIDE_MAX_Q ? 2048 : 256) * n_queries;
