@@ -310,6 +310,17 @@ __global__ void __launch_bounds__(Os<K>::THREADS, Os<K>::MIN_BLOCKS) k_os_pass(c
   if (t < RADIX) look_next[tile * RADIX + t] = 0ull;      // and its look-back words
 
   const uint32_t gcount = t < RADIX ? ghist[pass * RADIX + t] : 0u;  // read early: its latency overlaps the loads
+  if constexpr (sizeof(K) == 8) {
+    // every key has the same digit (the high bytes of keys packed from the bottom): the pass is a copy.
+    // (32-bit keys are tile ids, whose digits differ whenever there is a second tile.)
+    if (__syncthreads_or(gcount == (uint32_t)n)) {
+      for (int64_t i = tile * OS_TILE + t; i < min(n, (tile + 1) * OS_TILE); i += OS_THREADS) {
+        kout[i] = kin[i];
+        vout[i] = vin ? vin[i] : (uint32_t)i;
+      }
+      return;
+    }
+  }
   // ---- load (warp-striped: lane l of warp w holds items w*256 + j*32 + l)
   const int64_t base = tile * OS_TILE;
   const int m = (int)min((int64_t)OS_TILE, n - base);

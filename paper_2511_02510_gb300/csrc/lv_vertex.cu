@@ -5,15 +5,18 @@
 // corners trilinearly, Eq. 2-4 are unchanged).
 //
 //   lv_build_vertex_index: corner -> vertex id.  Every corner's integer
-//     coordinates on the finest grid (half-size units) form a 63-bit key; the
-//     8n keys are radix-sorted (stable, 64-bit) and numbered in key order, so
-//     vertex ids are the ranks of the distinct corner points (deterministic).
+//     coordinates on the finest grid (half-size units) form a 63-bit key.  The
+//     distinct keys are found with a hash table, radix-sorted and numbered in
+//     key order, so vertex ids are the ranks of the distinct corner points
+//     (deterministic).
 //   lv_vertex_gather: vertex values -> per-voxel corners [n][8] (FP32).
 //   lv_vertex_scatter_add: per-voxel corner values [n][8] -> vertex sums
 //     (atomics across the voxels sharing a vertex): turns the rasterizer's
 //     per-corner density gradient into the vertex gradient, or averages
 //     per-voxel corners into vertices with a count array.
 #include <math.h>
+
+#include <algorithm>
 
 #include "lv_prims.cuh"
 
@@ -24,14 +27,18 @@ constexpr int TPB = 256;
 constexpr int COORD_BITS = 21;
 constexpr long long COORD_OFF = 1ll << (COORD_BITS - 1);  // coordinates in [-2^20, 2^20)
 
+constexpr uint32_t COORD_MASK = (1u << COORD_BITS) - 1;
+constexpr uint64_t TAKEN = 1ull << 63;  // set in an occupied table word: the table starts as zeros
+
 struct VxWs {
-  unsigned long long* counters;  // [0] 8n (sort count), [1..2] scan totals
-  uint64_t *k0, *k1;
-  uint32_t *v0, *v1;
-  uint32_t* flag;
-  uint32_t* rank;
+  unsigned long long* counters;  // [0] distinct keys
+  uint32_t* bounds;              // [3] largest coordinate, [3] COORD_MASK - smallest coordinate
+  int32_t* status;
+  uint64_t* table;               // [1 << bits] TAKEN | key, then the vertex id
+  uint64_t *k0, *k1;             // [8n] distinct keys
+  uint32_t *v0, *v1;             // [8n] their table slots
   void* sort_tmp;
-  void* scan_tmp;
+  int bits;
   size_t bytes;
 };
 
@@ -39,62 +46,158 @@ VxWs carve_vx(void* base, int64_t n) {
   VxWs w;
   Carve c(base);
   const int64_t m = 8 * n;
+  w.bits = 10;
+  while (w.bits < 32 && (1ll << w.bits) < m + m / 4) ++w.bits;  // at most 0.8 full, 0.1 to 0.2 in real scenes
   w.counters = c.take<unsigned long long>(4);
+  w.bounds = c.take<uint32_t>(6);
+  w.status = c.take<int32_t>(1);
+  w.table = c.take<uint64_t>((size_t)1 << w.bits);
   w.k0 = c.take<uint64_t>(m);
   w.k1 = c.take<uint64_t>(m);
   w.v0 = c.take<uint32_t>(m);
   w.v1 = c.take<uint32_t>(m);
-  w.flag = c.take<uint32_t>(m);
-  w.rank = c.take<uint32_t>(m);
   w.sort_tmp = c.take<char>(sort_tmp_bytes(m));
-  w.scan_tmp = c.take<char>(scan2_tmp_bytes());
   w.bytes = c.off + 256;
   return w;
 }
 
-// corner c of voxel v at (centre +- h) on the finest grid; misaligned corners report
-__global__ void k_vx_keys(const float4* __restrict__ geom, int64_t n, double inv_unit, uint64_t* __restrict__ keys,
-                          int32_t* status) {
+// Grid coordinate of x + h (h signed) in units of 1 / inv_unit, COORD_OFF added;
+// false if it is more than 1e-3 off the grid or out of range.  The definition
+// is the FP64 one at the end; FP64 is slow on this part (24 coordinates a voxel
+// in FP64 took 131 us for 300,000 voxels), so pairs of FP32 values, good to
+// 2^-44 relative, decide wherever the distance is clear of the limit.
+__device__ __forceinline__ bool grid_coord(float x, float h, double inv_unit, float ih, float il, uint32_t* q) {
+  const float s = __fadd_rn(x, h), bb = __fsub_rn(s, x);
+  const float e = __fadd_rn(__fsub_rn(x, __fsub_rn(s, bb)), __fsub_rn(h, bb));  // s + e == x + h exactly
+  const float p = __fmul_rn(s, ih);
+  const float lo = __fmaf_rn(e, ih, __fmaf_rn(s, il, __fmaf_rn(s, ih, -p)));
+  const float rf = rintf(p);
+  if (fabsf(__fadd_rn(__fsub_rn(p, rf), lo)) <= 9.9e-4f && fabsf(rf) < (float)COORD_OFF) {
+    *q = (uint32_t)((int)rf + (int)COORD_OFF);
+    return true;
+  }
+  const double xd = ((double)x + (double)h) * inv_unit;
+  const double r = rint(xd);
+  *q = (uint32_t)((uint64_t)((long long)r + COORD_OFF) & COORD_MASK);
+  return fabs(xd - r) <= 1e-3 && r >= -(double)COORD_OFF && r < (double)COORD_OFF;
+}
+
+// The corners' keys entered in the table, a corner per thread (a voxel per
+// thread, its eight probes one after another, took 81 us for 300,000 voxels):
+// vidx gets each corner's table slot, a key's first finder appends it to the
+// distinct keys, and the coordinates' bounds are reduced.  Octree neighbours
+// share corners, so the distinct keys are a fraction of the corners: sorting only
+// those, and reading each corner's id from the table, replaced eight 64-bit sort
+// passes over all corners (the whole index of 300,000 voxels: 404 -> 176 us, of
+// which this kernel is 40 and the sort 95, bound by its passes' latencies).
+__global__ void __launch_bounds__(TPB) k_vx_hash(const float4* __restrict__ geom, int64_t n, double inv_unit,
+                                                unsigned long long* table, int bits, uint32_t* __restrict__ vidx,
+                                                uint64_t* __restrict__ keys, uint32_t* __restrict__ slots,
+                                                unsigned long long* count, uint32_t* bounds, int32_t* status) {
+  __shared__ uint32_t s_b[6], s_n;
+  __shared__ unsigned long long s_at;
+  if (threadIdx.x < 6) s_b[threadIdx.x] = 0u;
+  if (threadIdx.x == 0) s_n = 0u;
+  __syncthreads();
   const int64_t i = blockIdx.x * (int64_t)TPB + threadIdx.x;
-  if (i >= 8 * n) return;
-  const int64_t v = i >> 3;
-  const int c = (int)(i & 7);
-  const float4 g = geom[v];
-  const double h = (double)g.w;
-  const double p[3] = {(double)g.x + ((c & 1) ? h : -h), (double)g.y + ((c & 2) ? h : -h),
-                       (double)g.z + ((c & 4) ? h : -h)};
+  const int lane = threadIdx.x & 31, c = (int)(i & 7);
+  const float ih = (float)inv_unit, il = (float)(inv_unit - (double)ih);
+  uint32_t q[3] = {0u, 0u, 0u}, mn[3] = {0u, 0u, 0u}, slot = 0;
   uint64_t key = 0;
-  bool ok = true;
+  bool fresh = false;
+  if (i < 8 * n) {
+    const float4 g = geom[i >> 3];
+    bool ok = grid_coord(g.x, c & 1 ? g.w : -g.w, inv_unit, ih, il, &q[0]);
+    ok &= grid_coord(g.y, c & 2 ? g.w : -g.w, inv_unit, ih, il, &q[1]);
+    ok &= grid_coord(g.z, c & 4 ? g.w : -g.w, inv_unit, ih, il, &q[2]);
+    if (!ok) report(status, LV_ERR_INVALID_ARG);
+    key = TAKEN | (uint64_t)q[0] | (uint64_t)q[1] << COORD_BITS | (uint64_t)q[2] << (2 * COORD_BITS);
+    slot = (uint32_t)((key * 0x9e3779b97f4a7c15ull) >> (64 - bits));
+    // the table is never full, so a probe meets its key or an empty word
+    uint64_t cur = __ldcg(table + slot);
+    while (cur != key) {
+      if (cur == 0ull) {
+        cur = atomicCAS(table + slot, 0ull, (unsigned long long)key);
+        fresh = cur == 0ull;
+        if (fresh) break;
+      } else {
+        slot = (slot + 1u) & (uint32_t)((1ull << bits) - 1ull);
+        cur = __ldcg(table + slot);
+      }
+    }
+    vidx[i] = slot;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) mn[a] = COORD_MASK - q[a];
+  }
+  // one atomic per block on the count (same-address atomics serialise: one per warp cost 25 us)
+  const uint32_t who = __ballot_sync(FULL, fresh);
+  uint32_t rank = 0;
+  if (lane == 0 && who) rank = atomicAdd(&s_n, __popc(who));
+  rank = __shfl_sync(FULL, rank, 0) + __popc(who & ((1u << lane) - 1u));
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    const double x = p[a] * inv_unit;
-    const double r = rint(x);
-    ok = ok && fabs(x - r) <= 1e-3 && r >= -(double)COORD_OFF && r < (double)COORD_OFF;
-    const uint64_t q = (uint64_t)((long long)r + COORD_OFF) & ((1ull << COORD_BITS) - 1);
-    key |= q << (COORD_BITS * a);
+    const uint32_t x = __reduce_max_sync(FULL, q[a]), y = __reduce_max_sync(FULL, mn[a]);
+    if (lane == 0) {
+      atomicMax(&s_b[a], x);
+      atomicMax(&s_b[3 + a], y);
+    }
   }
-  keys[i] = key;
-  if (!ok) report(status, LV_ERR_INVALID_ARG);
+  __syncthreads();
+  if (threadIdx.x == 0 && s_n) s_at = atomicAdd(count, (unsigned long long)s_n);
+  // the bounds settle after a few blocks: most need no atomic
+  if (threadIdx.x < 6 && s_b[threadIdx.x] > __ldcg(&bounds[threadIdx.x])) atomicMax(&bounds[threadIdx.x], s_b[threadIdx.x]);
+  __syncthreads();
+  if (fresh) {
+    keys[s_at + rank] = key & ~TAKEN;
+    slots[s_at + rank] = slot;
+  }
 }
 
-__global__ void k_vx_set_count(unsigned long long* c, unsigned long long v) {
-  if (threadIdx.x == 0) *c = v;
+// The distinct keys packed: each coordinate less its smallest value, in just the
+// bits its range needs.  The order stays, and the sort's passes over the high
+// bytes, all zero, are plain copies.
+__global__ void __launch_bounds__(TPB) k_vx_pack(uint64_t* __restrict__ keys, const unsigned long long* count,
+                                                const uint32_t* __restrict__ bounds) {
+  const int64_t m = (int64_t)*count;
+  uint32_t lo[3];
+  int sh[3], at = 0;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    lo[a] = COORD_MASK - bounds[3 + a];
+    sh[a] = at;
+    at += 32 - __clz(bounds[a] - lo[a]);
+  }
+  for (int64_t i = blockIdx.x * (int64_t)TPB + threadIdx.x; i < m; i += (int64_t)gridDim.x * TPB) {
+    const uint64_t k = keys[i];
+    uint64_t r = 0;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) r |= (uint64_t)(((uint32_t)(k >> (COORD_BITS * a)) & COORD_MASK) - lo[a]) << sh[a];
+    keys[i] = r;
+  }
 }
 
-__global__ void k_vx_flags(const uint64_t* __restrict__ keys, int64_t m, uint32_t* __restrict__ flag) {
-  const int64_t r = blockIdx.x * (int64_t)TPB + threadIdx.x;
-  if (r < m) flag[r] = (r == 0 || keys[r] != keys[r - 1]) ? 1u : 0u;
+// a vertex's id is its key's rank
+__global__ void __launch_bounds__(TPB) k_vx_rank(const uint32_t* __restrict__ slots, const unsigned long long* count,
+                                                uint64_t* __restrict__ table, int64_t* __restrict__ n_vert) {
+  const int64_t m = (int64_t)*count;
+  for (int64_t i = blockIdx.x * (int64_t)TPB + threadIdx.x; i < m; i += (int64_t)gridDim.x * TPB)
+    table[slots[i]] = (uint64_t)i;
+  if (blockIdx.x == 0 && threadIdx.x == 0) *n_vert = m;
 }
 
-// the vertex id of sorted position r is the number of distinct keys before it
-__global__ void k_vx_assign(const uint32_t* __restrict__ slot, const uint32_t* __restrict__ flag,
-                            const uint32_t* __restrict__ excl, int64_t m, uint32_t* __restrict__ vidx) {
-  const int64_t r = blockIdx.x * (int64_t)TPB + threadIdx.x;
-  if (r < m) vidx[slot[r]] = excl[r] + flag[r] - 1u;
-}
-
-__global__ void k_vx_count(const unsigned long long* totals, int64_t* n_vert) {
-  if (threadIdx.x == 0) *n_vert = (int64_t)totals[1];
+// four corners per thread
+__global__ void __launch_bounds__(TPB) k_vx_assign(const uint64_t* __restrict__ table, int64_t n4,
+                                                  uint32_t* __restrict__ vidx) {
+  const int64_t i = blockIdx.x * (int64_t)TPB + threadIdx.x;
+  if (i >= n4) return;
+  uint32_t* p = vidx + 4 * i;
+  if (((uintptr_t)vidx & 15) == 0) {  // grid-uniform
+    const uint4 s = *(const uint4*)p;
+    *(uint4*)p = make_uint4((uint32_t)table[s.x], (uint32_t)table[s.y], (uint32_t)table[s.z], (uint32_t)table[s.w]);
+  } else {
+#pragma unroll
+    for (int c = 0; c < 4; ++c) p[c] = (uint32_t)table[p[c]];
+  }
 }
 
 template <typename DT>
@@ -144,22 +247,23 @@ extern "C" lv_status lv_build_vertex_index(const float* geom, int64_t n, double 
   if (ws_bytes < w.bytes) { set_error("workspace %zu < %zu bytes", ws_bytes, w.bytes); return LV_ERR_WORKSPACE; }
   cudaStream_t s = (cudaStream_t)stream;
   const int64_t m = 8 * n;
-  cudaMemsetAsync(d_n_vert, 0, sizeof(int64_t), s);
-  if (n == 0) return cuda_check(cudaGetLastError(), "lv_build_vertex_index");
-  k_vx_set_count<<<1, 32, 0, s>>>(w.counters, (unsigned long long)m);  // the sort's item count
-  int32_t* st = d_status ? d_status : (int32_t*)(w.counters + 3);
-  if (!d_status) cudaMemsetAsync(st, 0, sizeof(int32_t), s);
-  const unsigned blocks = (unsigned)((m + TPB - 1) / TPB);
-  k_vx_keys<<<blocks, TPB, 0, s>>>((const float4*)geom, n, 1.0 / unit, w.k0, st);
-  const int which = radix_sort_pairs(w.k0, nullptr, w.k0, w.v0, w.k1, w.v1, w.sort_tmp, w.counters, m,
+  if (n == 0) {
+    cudaMemsetAsync(d_n_vert, 0, sizeof(int64_t), s);
+    return cuda_check(cudaGetLastError(), "lv_build_vertex_index");
+  }
+  int32_t* st = d_status ? d_status : w.status;
+  zero_async(s, w.table, sizeof(uint64_t) << w.bits, w.counters, sizeof(unsigned long long), w.bounds,
+             6 * sizeof(uint32_t), d_status ? nullptr : w.status, sizeof(int32_t));
+  k_vx_hash<<<(unsigned)((m + TPB - 1) / TPB), TPB, 0, s>>>((const float4*)geom, n, 1.0 / unit,
+                                                            (unsigned long long*)w.table, w.bits, vidx, w.k0, w.v0,
+                                                            w.counters, w.bounds, st);
+  const unsigned grid = (unsigned)std::min<int64_t>((m + TPB - 1) / TPB, 8 * 152);  // the count is on the device
+  k_vx_pack<<<grid, TPB, 0, s>>>(w.k0, w.counters, w.bounds);
+  const int which = radix_sort_pairs(w.k0, w.v0, w.k0, w.v0, w.k1, w.v1, w.sort_tmp, w.counters, m,
                                      3 * COORD_BITS, st, s);
-  const uint64_t* sk = which ? w.k1 : w.k0;
-  const uint32_t* sv = which ? w.v1 : w.v0;
-  k_vx_flags<<<blocks, TPB, 0, s>>>(sk, m, w.flag);
-  scan2(w.flag, w.flag, m, nullptr, w.rank, w.counters + 1, w.scan_tmp, s);
-  k_vx_assign<<<blocks, TPB, 0, s>>>(sv, w.flag, w.rank, m, vidx);
-  k_vx_count<<<1, 32, 0, s>>>(w.counters + 1, d_n_vert);
-  count_launch(5);
+  k_vx_rank<<<grid, TPB, 0, s>>>(which ? w.v1 : w.v0, w.counters, w.table, d_n_vert);
+  k_vx_assign<<<(unsigned)((m / 4 + TPB - 1) / TPB), TPB, 0, s>>>(w.table, m / 4, vidx);
+  count_launch(4);
   return cuda_check(cudaGetLastError(), "lv_build_vertex_index");
 }
 
