@@ -4,9 +4,9 @@
 // Pipeline of lv_rasterize_forward (one stream, no host synchronisation):
 //   k_bin       per (voxel, view): FP32 cull / near-plane clipping / corner
 //               projection / tile rect / depth key with a fixed operation
-//               order; depth statistics.
-//   scan2       visible-slot ids and each item's first pair (item order),
-//               with the slot and pair totals.
+//               order; depth statistics; each block's pair and slot totals.
+//   k_block_offsets  the blocks' first pairs and slots (item order), with the
+//               slot and pair totals.
 //   k_emit      per (voxel, view): the item's (tile, slot) pairs, written in
 //               item order by whole warps; per visible item the 64-byte render
 //               record (centre relative to the camera, half-size, 8 corner
@@ -106,13 +106,15 @@ struct TileProg {
 // items are (view, voxel) pairs in view-major order: item = view * n + voxel
 struct FwdWs {
   unsigned long long* counters;  // [0] pairs, [1] slots
-  uint32_t* cnt;                 // [items] tiles covered
-  uint32_t* vis;                 // [items] 1 if cnt > 0
-  uint2* rect;                   // [items] (tx0 | tx1 << 16, ty0 | ty1 << 16)
-  uint2* pbox;                   // [items] conservative pixel box (x0 | x1 << 16, y0 | y1 << 16), [x0, x1)
-  uint32_t* dkey;                // [items] order key of z_centre
-  uint32_t* slot;                // [items] render slot of a visible item
-  unsigned long long* poff;      // [items] first pair of the item (pairs in item order)
+  uint32_t* cnt;                 // [items] tiles covered (visible: not 0)
+  uint2* rect;                   // [items] of visible items: (tx0 | tx1 << 16, ty0 | ty1 << 16)
+  uint2* pbox;                   // [items] of visible items: conservative pixel box (x0 | x1 << 16, y0 | y1 << 16), [x0, x1)
+  uint32_t* dkey;                // [items] of visible items: order key of z_centre
+  uint32_t* slot;                // [items] of visible items: render slot
+  unsigned long long* blk_pairs; // [blocks of 256 voxels x views, view-major] pairs, then the block's first within its group
+  uint32_t* blk_slots;           // the same for slots
+  unsigned long long* grp_pairs; // totals of groups of BO_GROUP blocks
+  uint32_t* grp_slots;
   uint2* rec_bb;                 // [slots] pixel box of the render record
   uint32_t* slot_vox;            // [slots] voxel id of the render record
   uint32_t* s_dkey;              // [slots] order key
@@ -129,7 +131,6 @@ struct FwdWs {
   TileProg* prog;                // [tiles] progress of the long tiles' depth order
   float* dep;                    // [pixels] depth and sample count of the pixels of open tiles
   uint32_t* nsamp;
-  void* scan_tmp;
   float4* rec;                   // [slots][4]
   float4* d_rgb;                 // [slots] colour gradient (xyz) scratch of the backward; w = clamp mask
   uint32_t* ranges;              // [tiles][2]
@@ -141,6 +142,9 @@ struct FwdWs {
   size_t bytes;
 };
 
+constexpr int BIN_THREADS = 256;  // voxels per block of k_bin and k_emit
+static int64_t bin_blocks(int64_t n) { return (n + BIN_THREADS - 1) / BIN_THREADS; }
+
 static FwdWs carve_fwd(void* base, int64_t n, int nv, int64_t tiles, int64_t pixels, int64_t pair_cap) {
   FwdWs w;
   Carve c(base);
@@ -149,16 +153,17 @@ static FwdWs carve_fwd(void* base, int64_t n, int nv, int64_t tiles, int64_t pix
   w.status = c.take<int32_t>(4);
   w.work = c.take<unsigned int>(16);
   w.cnt = c.take<uint32_t>(items);
-  w.vis = c.take<uint32_t>(items);
   w.rect = c.take<uint2>(items);
   w.pbox = c.take<uint2>(items);
   w.dkey = c.take<uint32_t>(items);
   w.slot = c.take<uint32_t>(items);
-  w.poff = c.take<unsigned long long>(items);
+  w.blk_pairs = c.take<unsigned long long>(bin_blocks(n) * nv);
+  w.blk_slots = c.take<uint32_t>(bin_blocks(n) * nv);
+  w.grp_pairs = c.take<unsigned long long>(bin_blocks(n) * nv / 4096 + 1);
+  w.grp_slots = c.take<uint32_t>(bin_blocks(n) * nv / 4096 + 1);
   w.rec_bb = c.take<uint2>(items);
   w.slot_vox = c.take<uint32_t>(items);
   w.s_dkey = c.take<uint32_t>(items);
-  w.scan_tmp = c.take<char>(scan2_tmp_bytes());
   w.rec = c.take<float4>(items * 4);
   w.d_rgb = c.take<float4>(items);
   w.ranges = c.take<uint32_t>(tiles * 2);
@@ -192,6 +197,17 @@ static const uint32_t* tile_pair_slots(const FwdWs& w, int64_t tiles) {
 }
 
 
+__device__ __forceinline__ float max3(float a, float b, float c) {
+  float d;
+  asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
+}
+__device__ __forceinline__ float min3(float a, float b, float c) {
+  float d;
+  asm("min.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
+}
+
 // ------------------------------------------------------------------ binning (FP32, fixed op order)
 __device__ __forceinline__ void cam_point32(const DevView& c, float X, float Y, float Z, float* q) {
 #pragma unroll
@@ -205,22 +221,14 @@ __device__ __forceinline__ void cam_point32(const DevView& c, float X, float Y, 
   }
 }
 
-__global__ void __launch_bounds__(256) k_bin(const float4* __restrict__ geom, int64_t n,
-                                             const __grid_constant__ ViewSet vs, uint32_t* cnt, uint32_t* vis,
-                                             uint2* rect, uint2* pbox, uint32_t* dkey, float* z_min,
-                                             float* delta_min, uint8_t* seen) {
-  int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= n * vs.n) return;
-  // items are view-major (i = view * n + voxel): a warp's lanes share one view, so the camera
-  // fields are warp-uniform loads, and the statistics' atomics hit distinct voxels
-  const int view = (int)(i / n);
-  const int64_t vox = i - (int64_t)view * n;
-  const DevView& c = vs.v[view];
-  const int ts = vs.ts;
+// one (voxel, view) item: its number of tiles, and the outputs of a visible one
+__device__ __forceinline__ uint32_t bin_item(const DevView& c, int ts, const float4* __restrict__ geom, int64_t vox,
+                                             int64_t i, uint2* __restrict__ rect, uint2* __restrict__ pbox,
+                                             uint32_t* __restrict__ dkey, float* z_min, float* delta_min,
+                                             uint8_t* seen) {
   float4 g = geom[vox];
   float qc[3];
   cam_point32(c, g.x, g.y, g.z, qc);
-  dkey[i] = order_key(qc[2]);
   {
     // Early out for voxels far outside the view: the circumscribed sphere lies behind the near
     // plane or beyond a side plane of the frustum of the tile grid (which may reach past the image
@@ -235,18 +243,11 @@ __global__ void __launch_bounds__(256) k_bin(const float4* __restrict__ geom, in
                      c.fx * qc[0] + c.cull_m[1] * qc[2] > rs * c.cull_n[1] ||
                      c.fy * qc[1] + c.cull_m[2] * qc[2] < -rs * c.cull_n[2] ||
                      c.fy * qc[1] + c.cull_m[3] * qc[2] > rs * c.cull_n[3];
-    if (out) {
-      cnt[i] = 0u;
-      vis[i] = 0u;
-      rect[i] = make_uint2(0u, 0u);
-      pbox[i] = make_uint2(0u, 0u);
-      return;
-    }
+    if (out) return 0u;
   }
-  int n_front = 0;
   float umin = 0.f, umax = 0.f, vmin = 0.f, vmax = 0.f;
-  bool first = true;
   float px[8], py[8], pz[8];
+  int n_front = 0;
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
     float X = (k & 1) ? __fadd_rn(g.x, g.w) : __fsub_rn(g.x, g.w);
@@ -255,13 +256,33 @@ __global__ void __launch_bounds__(256) k_bin(const float4* __restrict__ geom, in
     float p[3];
     cam_point32(c, X, Y, Z, p);
     px[k] = p[0]; py[k] = p[1]; pz[k] = p[2];
-    if (p[2] >= c.z_near) {
-      ++n_front;
-      const float iz = __frcp_rn(p[2]);  // one correctly rounded reciprocal per corner
-      float u = __fadd_rn(__fmul_rn(c.fx, __fmul_rn(p[0], iz)), c.cx);
-      float v = __fadd_rn(__fmul_rn(c.fy, __fmul_rn(p[1], iz)), c.cy);
-      if (first) { umin = umax = u; vmin = vmax = v; first = false; }
-      else { umin = fminf(umin, u); umax = fmaxf(umax, u); vmin = fminf(vmin, v); vmax = fmaxf(vmax, v); }
+    n_front += p[2] >= c.z_near ? 1 : 0;
+  }
+  auto project = [&](int k, float* u, float* v) {
+    const float iz = __frcp_rn(pz[k]);  // one correctly rounded reciprocal per corner
+    *u = __fadd_rn(__fmul_rn(c.fx, __fmul_rn(px[k], iz)), c.cx);
+    *v = __fadd_rn(__fmul_rn(c.fy, __fmul_rn(py[k], iz)), c.cy);
+  };
+  if (n_front == 8) {
+    // the usual case, with no test per corner: 3-input minima and maxima of all eight (the order of
+    // minima and maxima changes nothing)
+    float u[8], v[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) project(k, &u[k], &v[k]);
+    umin = fminf(min3(u[0], u[1], u[2]), fminf(min3(u[3], u[4], u[5]), fminf(u[6], u[7])));
+    umax = fmaxf(max3(u[0], u[1], u[2]), fmaxf(max3(u[3], u[4], u[5]), fmaxf(u[6], u[7])));
+    vmin = fminf(min3(v[0], v[1], v[2]), fminf(min3(v[3], v[4], v[5]), fminf(v[6], v[7])));
+    vmax = fmaxf(max3(v[0], v[1], v[2]), fmaxf(max3(v[3], v[4], v[5]), fmaxf(v[6], v[7])));
+  } else {
+    bool first = true;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      if (pz[k] >= c.z_near) {
+        float u, v;
+        project(k, &u, &v);
+        if (first) { umin = umax = u; vmin = vmax = v; first = false; }
+        else { umin = fminf(umin, u); umax = fmaxf(umax, u); vmin = fminf(vmin, v); vmax = fmaxf(vmax, v); }
+      }
     }
   }
   int tx0 = 0, tx1 = 0, ty0 = 0, ty1 = 0;
@@ -309,16 +330,137 @@ __global__ void __launch_bounds__(256) k_bin(const float4* __restrict__ geom, in
     py1 = (int)fminf(fmaxf(floorf(vmax + ev - 0.5f) + 1.0f, (float)py0), (float)c.H);
   }
   uint32_t count = (tx1 > tx0 && ty1 > ty0) ? (uint32_t)(tx1 - tx0) * (uint32_t)(ty1 - ty0) : 0u;
-  cnt[i] = count;
-  vis[i] = count ? 1u : 0u;
+  if (!count) return 0u;
+  dkey[i] = order_key(qc[2]);
   rect[i] = make_uint2((uint32_t)tx0 | ((uint32_t)tx1 << 16), (uint32_t)ty0 | ((uint32_t)ty1 << 16));
   pbox[i] = make_uint2((uint32_t)px0 | ((uint32_t)px1 << 16), (uint32_t)py0 | ((uint32_t)py1 << 16));
-  if (count) {
-    float zs = fmaxf(qc[2], c.z_near);
-    float dl = __fdiv_rn(zs, c.fx);
-    if (z_min) atomicMin((unsigned int*)&z_min[vox], __float_as_uint(zs));
-    if (delta_min) atomicMin((unsigned int*)&delta_min[vox], __float_as_uint(dl));
-    if (seen) seen[vox] = 1;
+  float zs = fmaxf(qc[2], c.z_near);
+  float dl = __fdiv_rn(zs, c.fx);
+  if (z_min) atomicMin((unsigned int*)&z_min[vox], __float_as_uint(zs));
+  if (delta_min) atomicMin((unsigned int*)&delta_min[vox], __float_as_uint(dl));
+  if (seen) seen[vox] = 1;
+  return count;
+}
+
+// Block b covers 256 consecutive voxels of view b % views, as in k_emit: the
+// views' blocks of one voxel range run side by side, so its geometry comes from
+// HBM once; a warp's lanes share one view (warp-uniform camera loads; the
+// statistics' atomics hit distinct voxels).  The block leaves its pair and slot
+// totals, from which k_block_offsets and k_emit place the items: per-item
+// offsets, scanned by three more launches, cost 28 bytes of traffic an item
+// (48M items: 290 us), and only visible items write anything but their count
+// (48M items: 854 -> 634 us with that, the geometry read once and the usual case's
+// projections without a test per corner; 2M items: 39 -> 32 us).
+__global__ void __launch_bounds__(BIN_THREADS) k_bin(const float4* __restrict__ geom, int64_t n, int64_t blocks,
+                                                     const __grid_constant__ ViewSet vs, uint32_t* __restrict__ cnt,
+                                                     uint2* __restrict__ rect, uint2* __restrict__ pbox,
+                                                     uint32_t* __restrict__ dkey,
+                                                     unsigned long long* __restrict__ blk_pairs,
+                                                     uint32_t* __restrict__ blk_slots, float* z_min,
+                                                     float* delta_min, uint8_t* seen) {
+  __shared__ unsigned long long s_pairs[BIN_THREADS / 32];
+  __shared__ uint32_t s_slots[BIN_THREADS / 32];
+  const int view = (int)(blockIdx.x % (unsigned)vs.n);
+  const int64_t vb = blockIdx.x / (unsigned)vs.n, vox = vb * BIN_THREADS + threadIdx.x;
+  const int64_t i = (int64_t)view * n + vox;  // items are view-major
+  uint32_t count = 0;
+  if (vox < n) {
+    count = bin_item(vs.v[view], vs.ts, geom, vox, i, rect, pbox, dkey, z_min, delta_min, seen);
+    cnt[i] = count;
+  }
+  // (32 counts can exceed 32 bits: halves are summed)
+  const uint32_t lo = __reduce_add_sync(FULL, count & 0xffffu), hi = __reduce_add_sync(FULL, count >> 16);
+  const uint32_t vis = __popc(__ballot_sync(FULL, count != 0u));
+  if ((threadIdx.x & 31) == 0) {
+    s_pairs[threadIdx.x >> 5] = ((unsigned long long)hi << 16) + lo;
+    s_slots[threadIdx.x >> 5] = vis;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    unsigned long long p = 0;
+    uint32_t q = 0;
+#pragma unroll
+    for (int w = 0; w < BIN_THREADS / 32; ++w) {
+      p += s_pairs[w];
+      q += s_slots[w];
+    }
+    blk_pairs[view * blocks + vb] = p;
+    blk_slots[view * blocks + vb] = q;
+  }
+}
+
+// Offsets of the binning blocks' pairs and slots within groups of BO_GROUP
+// blocks, in place, the groups' totals, and the grand totals added to
+// counters[0] and [1] (zero before).  k_emit sums the groups before its own: up
+// to 1M items there is one group, at 48M items 46.  (One block over all entries
+// took 196 us for 48M items, 4 us a round of 4096.)
+constexpr int BO_THREADS = 1024, BO_ITEMS = 4, BO_GROUP = BO_THREADS * BO_ITEMS;
+__global__ void __launch_bounds__(BO_THREADS) k_block_offsets(unsigned long long* __restrict__ pairs,
+                                                              uint32_t* __restrict__ slots, int64_t m,
+                                                              unsigned long long* __restrict__ grp_pairs,
+                                                              uint32_t* __restrict__ grp_slots,
+                                                              unsigned long long* __restrict__ counters) {
+  __shared__ unsigned long long s_a[BO_THREADS / 32];
+  __shared__ uint32_t s_b[BO_THREADS / 32];
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const int64_t i0 = blockIdx.x * (int64_t)BO_GROUP + BO_ITEMS * t;
+  unsigned long long a[BO_ITEMS], xa = 0;
+  uint32_t b[BO_ITEMS], xb = 0;
+#pragma unroll
+  for (int k = 0; k < BO_ITEMS; ++k) {
+    a[k] = i0 + k < m ? pairs[i0 + k] : 0ull;
+    b[k] = i0 + k < m ? slots[i0 + k] : 0u;
+  }
+#pragma unroll
+  for (int k = 0; k < BO_ITEMS; ++k) {
+    xa += a[k];
+    xb += b[k];
+  }
+  const unsigned long long own_a = xa;
+  const uint32_t own_b = xb;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned long long ya = __shfl_up_sync(FULL, xa, o);
+    const uint32_t yb = __shfl_up_sync(FULL, xb, o);
+    if (lane >= o) {
+      xa += ya;
+      xb += yb;
+    }
+  }
+  if (lane == 31) {
+    s_a[warp] = xa;
+    s_b[warp] = xb;
+  }
+  __syncthreads();
+  unsigned long long wa = s_a[lane];
+  uint32_t wb = s_b[lane];
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned long long ya = __shfl_up_sync(FULL, wa, o);
+    const uint32_t yb = __shfl_up_sync(FULL, wb, o);
+    if (lane >= o) {
+      wa += ya;
+      wb += yb;
+    }
+  }
+  const unsigned long long pa = __shfl_sync(FULL, wa, (warp + 31) & 31);
+  const uint32_t pb = __shfl_sync(FULL, wb, (warp + 31) & 31);
+  unsigned long long ra = (warp ? pa : 0ull) + xa - own_a;
+  uint32_t rb = (warp ? pb : 0u) + xb - own_b;
+#pragma unroll
+  for (int k = 0; k < BO_ITEMS; ++k) {
+    if (i0 + k < m) {
+      pairs[i0 + k] = ra;
+      slots[i0 + k] = rb;
+    }
+    ra += a[k];
+    rb += b[k];
+  }
+  if (t == BO_THREADS - 1) {
+    grp_pairs[blockIdx.x] = wa;  // lane 31: the whole group
+    grp_slots[blockIdx.x] = wb;
+    atomicAdd(&counters[0], wa);
+    atomicAdd(&counters[1], (unsigned long long)wb);
   }
 }
 
@@ -354,8 +496,32 @@ __device__ __forceinline__ void sh_basis(float x, float y, float z, float* Y) {
   Y[15] = C3a * x * (xx - 3.f * yy);
 }
 
-// one voxel's 48 SH coefficients into registers with 16-byte loads
+// A lane's own row in 32-byte loads, whole sectors, where the row is aligned for
+// them: with 16-byte loads every sector of a row is asked for twice, and by the
+// second time the other lanes' rows may have pushed it out of L1.
+__device__ __forceinline__ void ld_row32(const void* p, uint32_t* w) {
+  asm("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+      : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7])
+      : "l"(p));
+}
+__device__ __forceinline__ bool aligned32(const void* p) { return ((uintptr_t)p & 31) == 0; }
+__device__ __forceinline__ void bf16_pair(uint32_t w, float* c) {
+  c[0] = __uint_as_float(w << 16);
+  c[1] = __uint_as_float(w & 0xffff0000u);
+}
+
+// one voxel's 48 SH coefficients into registers (rows are 16-byte aligned)
 __device__ __forceinline__ void load_sh_row(const float* __restrict__ row, float* c) {
+  if (aligned32(row)) {
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+      uint32_t w[8];
+      ld_row32(row + 8 * k, w);
+#pragma unroll
+      for (int h = 0; h < 8; ++h) c[8 * k + h] = __uint_as_float(w[h]);
+    }
+    return;
+  }
   const float4* v = (const float4*)row;
 #pragma unroll
   for (int k = 0; k < 12; ++k) {
@@ -364,16 +530,51 @@ __device__ __forceinline__ void load_sh_row(const float* __restrict__ row, float
   }
 }
 __device__ __forceinline__ void load_sh_row(const __nv_bfloat16* __restrict__ row, float* c) {
+  if (aligned32(row)) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      uint32_t w[8];
+      ld_row32(row + 16 * k, w);
+#pragma unroll
+      for (int h = 0; h < 8; ++h) bf16_pair(w[h], c + 16 * k + 2 * h);
+    }
+    return;
+  }
   const uint4* v = (const uint4*)row;
 #pragma unroll
   for (int k = 0; k < 6; ++k) {
     const uint4 q = __ldg(v + k);
     const uint32_t w[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
-    for (int h = 0; h < 4; ++h) {
-      c[8 * k + 2 * h] = __uint_as_float(w[h] << 16);
-      c[8 * k + 2 * h + 1] = __uint_as_float(w[h] & 0xffff0000u);
+    for (int h = 0; h < 4; ++h) bf16_pair(w[h], c + 8 * k + 2 * h);
+  }
+}
+
+// one voxel's 8 corner densities (any alignment)
+__device__ __forceinline__ void load_corners(const float* __restrict__ row, float* d) {
+  if (aligned32(row)) {
+    uint32_t w[8];
+    ld_row32(row, w);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) d[k] = __uint_as_float(w[k]);
+  } else {
+#pragma unroll
+    for (int k = 0; k < 8; ++k) d[k] = row[k];
+  }
+}
+__device__ __forceinline__ void load_corners(const __half* __restrict__ row, float* d) {
+  if (((uintptr_t)row & 15) == 0) {
+    const uint4 q = __ldg((const uint4*)row);
+    const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const float2 f = __half22float2(*(const __half2*)&w[k]);
+      d[2 * k] = f.x;
+      d[2 * k + 1] = f.y;
     }
+  } else {
+#pragma unroll
+    for (int k = 0; k < 8; ++k) d[k] = to_f32(row[k]);
   }
 }
 
@@ -404,7 +605,8 @@ __device__ __forceinline__ void unit_dir(float rx, float ry, float rz, float* d)
 }
 
 // ------------------------------------------------------------------ emit
-// One thread per (voxel, view) item.  First the warp writes the (tile, slot)
+// One thread per (voxel, view) item, blocks as in k_bin: an item's slot and first
+// pair are its block's plus a scan inside the block.  First the warp writes the (tile, slot)
 // pairs of its 32 items: items are consecutive, so their pairs form one
 // contiguous range in item order (view-major, voxel id within a view), which
 // the warp fills 32 pairs per step, each lane finding the item of its pair by
@@ -421,8 +623,11 @@ __global__ void __launch_bounds__(256) k_emit(const float4* __restrict__ geom, c
                                               const uint2* __restrict__ pbox, uint2* __restrict__ rec_bb,
                                               uint32_t* __restrict__ slot_vox,
                                               const uint32_t* __restrict__ dkey,
-                                              const uint32_t* __restrict__ slot,
-                                              const unsigned long long* __restrict__ poff,
+                                              uint32_t* __restrict__ slot, int64_t blocks,
+                                              const unsigned long long* __restrict__ blk_pairs,
+                                              const uint32_t* __restrict__ blk_slots,
+                                              const unsigned long long* __restrict__ grp_pairs,
+                                              const uint32_t* __restrict__ grp_slots,
                                               const unsigned long long* __restrict__ counters, int64_t pair_cap,
                                               uint32_t* __restrict__ pair_tile, uint32_t* __restrict__ pair_slot,
                                               int32_t* status, uint2* __restrict__ ranges, int64_t tiles,
@@ -450,44 +655,77 @@ __global__ void __launch_bounds__(256) k_emit(const float4* __restrict__ geom, c
     const int64_t words = (int64_t)((total + sc.tile - 1) / sc.tile) * 256;
     for (int64_t x = blockIdx.x * 256ll + threadIdx.x; x < words; x += (int64_t)gridDim.x * 256) sc.look0[x] = 0ull;
   }
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t blk = view * blocks + blockIdx.x / (unsigned)vs.n;
+  // items of the warp before this one: visible, and their pairs (32 bits do: nothing is written when
+  // the pairs exceed the capacity, and that is below 2^32)
+  const uint32_t vism = __ballot_sync(FULL, cn != 0u);
+  uint32_t pre = cn;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(FULL, pre, o);
+    if (lane >= o) pre += y;
+  }
+  __shared__ uint32_t s_wp[8], s_wv[8];
+  if (lane == 31) {
+    s_wp[warp] = pre;
+    s_wv[warp] = __popc(vism);
+  }
+  uint32_t sl = blk_slots[blk];
+  unsigned long long p_block = blk_pairs[blk];
+  const int64_t grp = blk / BO_GROUP;
+  if (grp) {  // grid-uniform within a group: every warp sums the groups before
+    unsigned long long a = 0;
+    uint32_t b = 0;
+    for (int64_t g = lane; g < grp; g += 32) {
+      a += grp_pairs[g];
+      b += grp_slots[g];
+    }
+#pragma unroll
+    for (int o = 16; o; o >>= 1) a += __shfl_xor_sync(FULL, a, o);
+    p_block += a;
+    sl += __reduce_add_sync(FULL, b);
+  }
   __syncthreads();
+  uint32_t wp = 0;
+#pragma unroll
+  for (int w = 0; w < 8; ++w) {
+    wp += w < warp ? s_wp[w] : 0u;
+    sl += w < warp ? s_wv[w] : 0u;
+  }
+  sl += __popc(vism & ((1u << lane) - 1u));
   if (total > (unsigned long long)pair_cap) {
     if (blockIdx.x == 0 && threadIdx.x == 0) report(status, LV_ERR_CAPACITY);
   } else {
-    const int lane = threadIdx.x & 31;
-    const uint32_t inm = __ballot_sync(FULL, in);  // a prefix of the lanes
-    if (inm) {                                     // warp-uniform
-      const int last = 31 - __clz(inm);
-      // lanes past the last voxel start after every pair, so the search never picks them
-      const unsigned long long po = in ? poff[i] : ~0ull;
-      uint32_t rx = 0u, ry = 0u, sl = 0u;
+    const uint32_t wn = __shfl_sync(FULL, pre, 31);  // the warp's pairs
+    if (wn) {                                        // warp-uniform
+      const uint32_t po = pre - cn;  // first pair of the item within the warp's
+      uint32_t rx = 0u, ry = 0u;
       if (cn) {
         const uint2 rc = rect[i];
         rx = rc.x;
         ry = rc.y;
-        sl = slot[i];
       }
-      const unsigned long long p_begin = __shfl_sync(FULL, po, 0);
-      const unsigned long long p_end = __shfl_sync(FULL, po + cn, last);
+      const unsigned long long p_begin = p_block + wp;
       const DevView& c = vs.v[view];
       const uint32_t toff = (uint32_t)c.tile_off, tiles_x = (uint32_t)c.tiles_x;
-      for (unsigned long long p0 = p_begin; p0 < p_end; p0 += 32) {  // warp-uniform
-        const unsigned long long e = p0 + lane;
-        int j = 0;  // the largest lane whose first pair is <= e (lane 0's is <= p0)
+      for (uint32_t e0 = 0; e0 < wn; e0 += 32) {  // warp-uniform
+        const uint32_t e = e0 + lane;
+        int j = 0;  // the largest lane whose first pair is <= e (lane 0's is 0)
 #pragma unroll
         for (int step = 16; step; step >>= 1) {
-          const unsigned long long x = __shfl_sync(FULL, po, (j + step) & 31);
+          const uint32_t x = __shfl_sync(FULL, po, (j + step) & 31);
           if (j + step < 32 && x <= e) j += step;
         }
-        const unsigned long long pj = __shfl_sync(FULL, po, j);
+        const uint32_t pj = __shfl_sync(FULL, po, j);
         const uint32_t jx = __shfl_sync(FULL, rx, j), jy = __shfl_sync(FULL, ry, j);
         const uint32_t js = __shfl_sync(FULL, sl, j);
-        if (e < p_end) {
-          const uint32_t q = (uint32_t)(e - pj);
+        if (e < wn) {
+          const uint32_t q = e - pj;
           const uint32_t tx0 = jx & 0xffffu, wx = (jx >> 16) - tx0, ty0 = jy & 0xffffu;
           const uint32_t key = toff + (ty0 + q / wx) * tiles_x + tx0 + q % wx;
-          pair_tile[e] = key;
-          pair_slot[e] = js;
+          pair_tile[p_begin + e] = key;
+          pair_slot[p_begin + e] = js;
           for (int p = 0; p < passes; ++p) atomicAdd(&s_cnt[p * 256 + ((key >> (8 * p)) & 255u)], 1u);
         }
       }
@@ -498,7 +736,8 @@ __global__ void __launch_bounds__(256) k_emit(const float4* __restrict__ geom, c
     if (s_cnt[x]) atomicAdd(&sc.counts[x], s_cnt[x]);
   if (!cn) return;
   const DevView& c = vs.v[view];
-  const uint32_t s = slot[i];
+  const uint32_t s = sl;
+  slot[i] = s;
   const float4 g = geom[vox];
   const float rx = g.x - c.o[0], ry = g.y - c.o[1], rz = g.z - c.o[2];
   float dir[3];
@@ -515,8 +754,7 @@ __global__ void __launch_bounds__(256) k_emit(const float4* __restrict__ geom, c
     d[0] = to_f32(dens[i0.x]); d[1] = to_f32(dens[i0.y]); d[2] = to_f32(dens[i0.z]); d[3] = to_f32(dens[i0.w]);
     d[4] = to_f32(dens[i1.x]); d[5] = to_f32(dens[i1.y]); d[6] = to_f32(dens[i1.z]); d[7] = to_f32(dens[i1.w]);
   } else {
-#pragma unroll
-    for (int k = 0; k < 8; ++k) d[k] = to_f32(dens[8 * vox + k]);
+    load_corners(dens + 8 * vox, d);
   }
   float4* r = rec + 4 * (int64_t)s;
   r[0] = make_float4(rx, ry, rz, g.w);
@@ -1253,17 +1491,6 @@ __device__ __forceinline__ Ray make_ray(const DevView& c, int px, int py) {
   return r;
 }
 
-__device__ __forceinline__ float max3(float a, float b, float c) {
-  float d;
-  asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
-  return d;
-}
-__device__ __forceinline__ float min3(float a, float b, float c) {
-  float d;
-  asm("min.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
-  return d;
-}
-
 // Chord of the ray (origin at the camera) through the box centred at rc
 // (relative to the camera) with half-size h, clipped to start at the near
 // plane: slab a enters at (rc_a - h sign) / d_a and leaves at (rc_a + h sign) / d_a.
@@ -1945,7 +2172,7 @@ __global__ void __launch_bounds__(TS* TS, min_blocks<TS>()) k_bwd(const __grid_c
 // without any visible voxel touch nothing.
 __global__ void __launch_bounds__(128) k_sh_bwd(const float4* __restrict__ rec, int sh_nb, int64_t n,
                                                 const __grid_constant__ ViewSet vs,
-                                                const uint32_t* __restrict__ vis, const uint32_t* __restrict__ slot,
+                                                const uint32_t* __restrict__ cnt, const uint32_t* __restrict__ slot,
                                                 float4* __restrict__ d_rgb, float* __restrict__ d_sh,
                                                 int accumulate) {
   constexpr int RS = 49;
@@ -1963,7 +2190,7 @@ __global__ void __launch_bounds__(128) k_sh_bwd(const float4* __restrict__ rec, 
     const int64_t vox = v0 + lane;
     for (int view = 0; view < vs.n; ++view) {
       const int64_t i = (int64_t)view * n + vox;  // view-major items
-      if (!vis[i]) continue;
+      if (!cnt[i]) continue;
       any_vis = true;
       const uint32_t s = slot[i];
       // the record holds the centre relative to this view's camera, as k_emit computed it, so the
@@ -2392,17 +2619,19 @@ extern "C" lv_status lv_rasterize_forward(const lv_voxels* vox, const lv_camera*
   zero_async(s, w.counters, 8 * sizeof(unsigned long long), d_status == w.status ? w.status : nullptr,
              sizeof(int32_t), w.work, 16 * sizeof(unsigned int), sc.counts, sc.zero_bytes);
   if (items > 0) {
-    int blocks = (int)((items + 255) / 256);
-    const unsigned emit_blocks = (unsigned)(((n + 255) / 256) * n_views);  // (voxel range, view) blocks
-    k_bin<<<blocks, 256, 0, s>>>((const float4*)vox->geom, n, vs, w.cnt, w.vis, w.rect, w.pbox, w.dkey, out->z_min,
-                                 out->delta_min, out->seen);
+    const int64_t blocks = bin_blocks(n);
+    const unsigned item_blocks = (unsigned)(blocks * n_views);  // (voxel range, view) blocks
+    k_bin<<<item_blocks, BIN_THREADS, 0, s>>>((const float4*)vox->geom, n, blocks, vs, w.cnt, w.rect, w.pbox, w.dkey,
+                                              w.blk_pairs, w.blk_slots, out->z_min, out->delta_min, out->seen);
     if (out->stats_event) cudaEventRecord((cudaEvent_t)out->stats_event, s);  // statistics final
-    scan2(w.cnt, w.vis, items, w.poff, w.slot, w.counters, w.scan_tmp, s);
+    k_block_offsets<<<(unsigned)((blocks * n_views + BO_GROUP - 1) / BO_GROUP), BO_THREADS, 0, s>>>(
+        w.blk_pairs, w.blk_slots, blocks * n_views, w.grp_pairs, w.grp_slots, w.counters);
     const int nb = (vox->sh_degree + 1) * (vox->sh_degree + 1);
 #define LV_EMIT(DT, ST)                                                                                             \
-  k_emit<DT, ST><<<emit_blocks, 256, 0, s>>>((const float4*)vox->geom, (const DT*)vox->density, (const ST*)vox->sh, \
+  k_emit<DT, ST><<<item_blocks, BIN_THREADS, 0, s>>>((const float4*)vox->geom, (const DT*)vox->density, (const ST*)vox->sh, \
                                              nb, n, vs, w.cnt, w.rect, w.pbox, w.rec_bb, w.slot_vox, w.dkey,          \
-                                             w.slot, w.poff, w.counters, pair_capacity, w.k0, w.v0, d_status,         \
+                                             w.slot, blocks, w.blk_pairs, w.blk_slots, w.grp_pairs, w.grp_slots,     \
+                                             w.counters, pair_capacity, w.k0, w.v0, d_status,         \
                                              (uint2*)w.ranges, tiles, sc, passes, w.rec, w.d_rgb, w.s_dkey,   \
                                              vox->vidx)
     if (vox->density_dtype == LV_F32 && vox->sh_dtype == LV_F32) LV_EMIT(float, float);
@@ -2410,7 +2639,7 @@ extern "C" lv_status lv_rasterize_forward(const lv_voxels* vox, const lv_camera*
     else if (vox->density_dtype == LV_F32 && vox->sh_dtype == LV_BF16) LV_EMIT(float, __nv_bfloat16);
     else LV_EMIT(__half, __nv_bfloat16);
 #undef LV_EMIT
-    count_launch(2);
+    count_launch(3);
   } else if (out->stats_event) {
     cudaEventRecord((cudaEvent_t)out->stats_event, s);  // no voxel: nothing to bin
   }
@@ -2500,7 +2729,7 @@ static lv_status launch_sh_bwd(const lv_voxels* vox, const ViewSet& vs, const Fw
   if (n == 0) return LV_OK;
   const int nb = (vox->sh_degree + 1) * (vox->sh_degree + 1);
   const int blocks = (int)((n + 127) / 128);  // 4 warps x 32 voxels
-  k_sh_bwd<<<blocks, 128, 0, s>>>(w.rec, nb, n, vs, w.vis, w.slot, w.d_rgb, d_sh, accumulate);
+  k_sh_bwd<<<blocks, 128, 0, s>>>(w.rec, nb, n, vs, w.cnt, w.slot, w.d_rgb, d_sh, accumulate);
   count_launch(1);
   return LV_OK;
 }
