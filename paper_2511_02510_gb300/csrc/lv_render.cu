@@ -137,13 +137,23 @@ struct FwdWs {
   float* tau;                    // [pixels] final optical depth
   void* sort_tmp;                // scratch of the sort by tile
   int32_t* status;               // fallback status word
-  uint32_t *k0, *v0, *k1, *v1;   // [pair capacity] (tile, slot) pairs, sorted by tile
+  uint32_t *k0, *v0, *k1, *v1;   // [pair capacity] (tile, slot) pairs and the sort's other buffer
+  // once the pairs are sorted by tile, their slots in one of v0 and v1 (item order within a tile), the
+  // sort's other buffer and the sorted tile ids, which the ranges replace, serve the depth order:
+  uint32_t* tile_slots;          // the sorted slots
   uint2* plist;                  // [pair capacity] (slot, strip mask) of every tile's list in depth order
+  uint32_t* long_keys;           // [pair capacity] the long lists' order keys
   size_t bytes;
 };
 
 constexpr int BIN_THREADS = 256;  // voxels per block of k_bin and k_emit
 static int64_t bin_blocks(int64_t n) { return (n + BIN_THREADS - 1) / BIN_THREADS; }
+
+static int tile_bits(int64_t tiles) {
+  int b = 0;
+  while (b < 32 && ((int64_t)1 << b) < tiles) ++b;
+  return b;
+}
 
 static FwdWs carve_fwd(void* base, int64_t n, int nv, int64_t tiles, int64_t pixels, int64_t pair_cap) {
   FwdWs w;
@@ -177,24 +187,20 @@ static FwdWs carve_fwd(void* base, int64_t n, int nv, int64_t tiles, int64_t pix
   w.nsamp = c.take<uint32_t>(pixels);
   w.tau = c.take<float>(pixels);
   w.sort_tmp = c.take<char>(sort_tmp_bytes(pair_cap));
-  w.k0 = c.take<uint32_t>(pair_cap);
-  w.v0 = c.take<uint32_t>(pair_cap);
-  w.k1 = c.take<uint32_t>(pair_cap);
-  w.v1 = c.take<uint32_t>(pair_cap);
-  w.plist = c.take<uint2>(pair_cap);
+  // keys and values of a buffer side by side, so that the unused buffer holds 8-byte words
+  const size_t half = align_up((size_t)pair_cap, 64);
+  w.k0 = c.take<uint32_t>(2 * half);
+  w.k1 = c.take<uint32_t>(2 * half);
+  w.v0 = w.k0 ? w.k0 + half : nullptr;
+  w.v1 = w.k1 ? w.k1 + half : nullptr;
+  const bool odd = sort_passes(tile_bits(tiles)) & 1;  // the sorted pairs are in (k1, v1)
+  w.tile_slots = odd ? w.v1 : w.v0;
+  w.long_keys = odd ? w.k1 : w.k0;
+  w.plist = (uint2*)(odd ? w.k0 : w.k1);
   w.bytes = c.off + 256;
   return w;
 }
 
-// the slots of the pairs sorted by tile (item order within a tile): in v0 after an even number of tile-digit passes
-static int tile_bits(int64_t tiles) {
-  int b = 0;
-  while (b < 32 && ((int64_t)1 << b) < tiles) ++b;
-  return b;
-}
-static const uint32_t* tile_pair_slots(const FwdWs& w, int64_t tiles) {
-  return (sort_passes(tile_bits(tiles)) & 1) ? w.v1 : w.v0;
-}
 
 
 __device__ __forceinline__ float max3(float a, float b, float c) {
@@ -357,9 +363,14 @@ __global__ void __launch_bounds__(BIN_THREADS) k_bin(const float4* __restrict__ 
                                                      uint32_t* __restrict__ dkey,
                                                      unsigned long long* __restrict__ blk_pairs,
                                                      uint32_t* __restrict__ blk_slots, float* z_min,
-                                                     float* delta_min, uint8_t* seen) {
+                                                     float* delta_min, uint8_t* seen, const ZeroRanges zr) {
   __shared__ unsigned long long s_pairs[BIN_THREADS / 32];
   __shared__ uint32_t s_slots[BIN_THREADS / 32];
+  // the later kernels' counters are cleared here, not by a launch of their own (whole 32-bit words)
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+    for (size_t x = blockIdx.x * (size_t)BIN_THREADS + threadIdx.x; x < zr.bytes[k] / 4; x += (size_t)gridDim.x * BIN_THREADS)
+      ((uint32_t*)zr.p[k])[x] = 0u;
   const int view = (int)(blockIdx.x % (unsigned)vs.n);
   const int64_t vb = blockIdx.x / (unsigned)vs.n, vox = vb * BIN_THREADS + threadIdx.x;
   const int64_t i = (int64_t)view * n + vox;  // items are view-major
@@ -2503,9 +2514,8 @@ static void launch_bwd_t(int64_t tiles, cudaStream_t s, const ViewSet& vs, const
 
 // tile size, density model (midpoint, or the exact-segment variant) and scheduling (one block per
 // tile, or persistent warps on a work counter) from the options
-// The pairs sorted by tile are in (k0, v0) after an even number of digit passes, else in (k1, v1); the
-// other keys are scratch for the long lists' order keys.  One warp per tile first (short lists, ranges,
-// the lists of longer tiles), then persistent blocks over the long tiles' fronts and the medium tiles.
+// One warp per tile first (short lists, ranges, the lists of longer tiles), then persistent blocks over
+// the long tiles' fronts and the medium tiles.
 static int tile_sort_blocks() {
   static std::atomic<unsigned long long> attr_done{0};
   static int blocks[64];
@@ -2518,14 +2528,11 @@ static int tile_sort_blocks() {
   });
   return dev < 64 ? blocks[dev] : persistent_blocks(k_tile_sort, TS_THREADS, sizeof(TileLongSmem));
 }
-static uint32_t* long_keys(const FwdWs& w, int64_t tiles) {
-  return (sort_passes(tile_bits(tiles)) & 1) ? w.k0 : w.k1;
-}
 static void launch_tile_sort(const FwdWs& w, const ViewSet& vs, int64_t n, int64_t tiles, int64_t pair_cap,
                              cudaStream_t s) {
   const int64_t nb = std::min<int64_t>(tile_sort_blocks(), tiles);
   const bool ready = sort_passes(tile_bits(tiles)) > 0;
-  const uint32_t* sv = tile_pair_slots(w, tiles);
+  const uint32_t* sv = w.tile_slots;
   const unsigned wblocks = (unsigned)((tiles + TW_WARPS - 1) / TW_WARPS);
   k_tile_sort_warp<<<wblocks, TW_WARPS * 32, sizeof(TileSortWarpSmem), s>>>(
       sv, w.s_dkey, w.counters, pair_cap, ready, tiles, w.ranges, w.mid_tiles, w.work + 4, w.long_tiles, w.work + 6,
@@ -2533,7 +2540,7 @@ static void launch_tile_sort(const FwdWs& w, const ViewSet& vs, int64_t n, int64
   count_launch(1);
   if (n <= TW_MAX) return;  // a tile lists a voxel once: every list is short
   k_tile_sort<<<(unsigned)nb, TS_THREADS, sizeof(TileLongSmem), s>>>(
-      sv, long_keys(w, tiles), w.s_dkey, w.ranges, w.mid_tiles, w.work + 4, w.long_tiles, w.work + 6, w.work + 5,
+      sv, w.long_keys, w.s_dkey, w.ranges, w.mid_tiles, w.work + 4, w.long_tiles, w.work + 6, w.work + 5,
       w.ready, w.prog, n > TS_LAZY_VOXELS ? TS_LAZY : ~0u, vs, w.rec_bb, w.plist);
   count_launch(1);
 }
@@ -2542,7 +2549,7 @@ static void launch_tile_rest(const FwdWs& w, const ViewSet& vs, int64_t tiles, b
   const int64_t nb = std::min<int64_t>(tile_sort_blocks(), tiles);
   if (all) zero_async(s, w.work + 3, sizeof(unsigned int));
   k_tile_rest<<<(unsigned)nb, TS_THREADS, sizeof(TileLongSmem), s>>>(
-      tile_pair_slots(w, tiles), long_keys(w, tiles), w.ranges, all ? w.long_tiles : w.open_tiles,
+      w.tile_slots, w.long_keys, w.ranges, all ? w.long_tiles : w.open_tiles,
       w.work + (all ? 6 : 7), w.work + 3, w.ready, w.prog, vs, w.rec_bb, w.plist);
   count_launch(1);
 }
@@ -2616,13 +2623,17 @@ extern "C" lv_status lv_rasterize_forward(const lv_voxels* vox, const lv_camera*
   // sort by tile's digit counts, which k_emit accumulates (k_tile_sort_warp writes every tile's range)
   const SortCountTargets sc = sort_count_targets(w.sort_tmp, pair_capacity);
   const int passes = std::min(sort_passes(tile_bits(tiles)), 4);
-  zero_async(s, w.counters, 8 * sizeof(unsigned long long), d_status == w.status ? w.status : nullptr,
-             sizeof(int32_t), w.work, 16 * sizeof(unsigned int), sc.counts, sc.zero_bytes);
+  const bool own_status = d_status == w.status;
+  const ZeroRanges zr = {{w.counters, w.status, w.work, sc.counts},
+                         {8 * sizeof(unsigned long long), own_status ? sizeof(int32_t) : 0, 16 * sizeof(unsigned int),
+                          sc.zero_bytes}};
+  if (items == 0)
+    zero_async(s, zr.p[0], zr.bytes[0], zr.p[1], zr.bytes[1], zr.p[2], zr.bytes[2], zr.p[3], zr.bytes[3]);
   if (items > 0) {
     const int64_t blocks = bin_blocks(n);
     const unsigned item_blocks = (unsigned)(blocks * n_views);  // (voxel range, view) blocks
     k_bin<<<item_blocks, BIN_THREADS, 0, s>>>((const float4*)vox->geom, n, blocks, vs, w.cnt, w.rect, w.pbox, w.dkey,
-                                              w.blk_pairs, w.blk_slots, out->z_min, out->delta_min, out->seen);
+                                              w.blk_pairs, w.blk_slots, out->z_min, out->delta_min, out->seen, zr);
     if (out->stats_event) cudaEventRecord((cudaEvent_t)out->stats_event, s);  // statistics final
     k_block_offsets<<<(unsigned)((blocks * n_views + BO_GROUP - 1) / BO_GROUP), BO_THREADS, 0, s>>>(
         w.blk_pairs, w.blk_slots, blocks * n_views, w.grp_pairs, w.grp_slots, w.counters);
