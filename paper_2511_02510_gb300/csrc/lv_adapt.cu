@@ -205,6 +205,7 @@ PruneWs carve_prune(void* base, int64_t n) {
 
 __global__ void k_pr_seen(int64_t n, const uint8_t* __restrict__ seen, const float* __restrict__ z, uint16_t* grp,
                           uint32_t* zkey, PruneState* st) {
+  grid_begin();
   const int64_t i0 = first_item();
   uint8_t sv[IPT];
   float zv[IPT];
@@ -230,6 +231,7 @@ __global__ void k_pr_seen(int64_t n, const uint8_t* __restrict__ seen, const flo
 // order keys of w_max; the per-bin selection's first digit is counted here (row = depth bin)
 __global__ void k_pr_wkey(int64_t n, const float* __restrict__ w_max, const uint16_t* __restrict__ grp,
                           uint32_t* __restrict__ wkey, const FirstHist fh) {
+  grid_begin();
   __shared__ uint32_t sh[FH_WORDS];
   fh_clear(fh, sh);
   const int64_t i0 = first_item();
@@ -249,6 +251,7 @@ __global__ void k_pr_wkey(int64_t n, const float* __restrict__ w_max, const uint
 
 __global__ void k_pr_pct_queries(SelectQuery* q, const PruneState* st, uint32_t lo_ppm, uint32_t hi_ppm,
                                  void* sel_tmp) {
+  grid_begin();
   select_prepare(q, 2, sel_tmp);
   if (threadIdx.x == 0) {
     q[0].group = 0; q[0].k = rank_ppm(lo_ppm, st->ns);
@@ -277,12 +280,14 @@ __device__ __forceinline__ void running_pct(const SelectQuery* pct, float* state
 }
 
 __global__ void k_pr_pct_apply(const SelectQuery* pct, PruneState* st, float* state, float r, float omr) {
+  grid_begin();
   if (threadIdx.x == 0 && st->ns > 0) running_pct(pct, state, r, omr, &st->p_lo);
 }
 
 // bin counts go through a block-local histogram (one global add per bin and block)
 __global__ void k_pr_bin(int64_t n, const uint8_t* __restrict__ seen, const float* __restrict__ z, int nb,
                          uint16_t* grp, PruneState* st) {
+  grid_begin();
   __shared__ uint32_t sh[SELECT_MAX_QUERIES];
   if (threadIdx.x < SELECT_MAX_QUERIES) sh[threadIdx.x] = 0;
   __syncthreads();
@@ -318,6 +323,7 @@ __device__ __forceinline__ long long q_bin(long long q_ppm, long long anneal_ppm
 // a bin with q_b = 0 gets k = 0: no threshold (result stays 0xffffffff)
 __global__ void k_pr_tau_queries(SelectQuery* q, const PruneState* st, int nb, uint32_t q_ppm, int anneal,
                                  uint32_t anneal_ppm, uint32_t relax_ppm, void* sel_tmp) {
+  grid_begin();
   select_prepare(q, nb, sel_tmp);
   int b = threadIdx.x;
   if (b < nb) {
@@ -342,6 +348,7 @@ __global__ void k_pr_update(int64_t n, const uint16_t* __restrict__ grp, const u
                             const SelectQuery* tau, float alpha, float oma, float m_low, float m_high, float* ema_m,
                             uint8_t* state, const Halo halo, uint8_t* mask, uint16_t* cand_grp, PruneState* st,
                             const FirstHist fh) {
+  grid_begin();
   __shared__ uint32_t sh[FH_WORDS];
   fh_clear(fh, sh);
   const int64_t i0 = first_item();
@@ -392,6 +399,7 @@ __global__ void k_pr_update(int64_t n, const uint16_t* __restrict__ grp, const u
 }
 
 __global__ void k_pr_cap_query(SelectQuery* q, PruneState* st, uint32_t cap, void* sel_tmp) {
+  grid_begin();
   select_prepare(q, 1, sel_tmp);
   if (threadIdx.x == 0) {
     st->all = st->n_cand <= cap ? 1u : 0u;
@@ -404,6 +412,7 @@ __global__ void k_pr_cap_query(SelectQuery* q, PruneState* st, uint32_t cap, voi
 // (the ties compete by id: the need = cap - c_lt smallest ids among them go)
 __global__ void k_pr_ties(int64_t n, const uint32_t* __restrict__ wkey, const SelectQuery* thr,
                           const uint8_t* __restrict__ cand, uint32_t* blk, PruneState* st) {
+  grid_begin();
   const int64_t i0 = first_item();
   uint32_t clt = 0, ceq = 0;
   if (thr[0].k != 0) {
@@ -435,6 +444,7 @@ __global__ void k_pr_ties(int64_t n, const uint32_t* __restrict__ wkey, const Se
 __global__ void k_pr_mask(int64_t n, const uint32_t* __restrict__ wkey, const SelectQuery* thr,
                           const uint32_t* __restrict__ blk, const PruneState* st, uint8_t* mask,
                           int64_t* n_pruned, uint32_t cap) {
+  grid_begin();
   const int64_t i0 = first_item();
   const bool all = st->all != 0;
   const bool thr_ok = thr[0].k != 0;
@@ -525,6 +535,7 @@ SubWs carve_sub(void* base, int64_t n) {
 __global__ void k_sd_flags(int64_t n, const uint8_t* __restrict__ seen, const uint8_t* __restrict__ pm,
                            const float* __restrict__ z, uint16_t* grp, uint32_t* zkey, SubState* st,
                            const FirstHist fh) {
+  grid_begin();
   __shared__ uint32_t sh[FH_WORDS];
   fh_clear(fh, sh);
   const int64_t i0 = first_item();
@@ -559,6 +570,7 @@ __global__ void k_sd_flags(int64_t n, const uint8_t* __restrict__ seen, const ui
 // (when h0 is not null), and row 1 gets a copy
 __global__ void k_sd_pct_queries(SelectQuery* q, uint32_t lo_ppm, uint32_t hi_ppm, const uint32_t* counter,
                                  void* sel_tmp, uint32_t* h0) {
+  grid_begin();
   select_prepare(q, 2, sel_tmp);
   if (h0)
     for (int i = threadIdx.x; i < select_radix(2); i += blockDim.x) h0[select_radix(2) + i] = h0[i];
@@ -571,6 +583,7 @@ __global__ void k_sd_pct_queries(SelectQuery* q, uint32_t lo_ppm, uint32_t hi_pp
 
 // also clears n_el (the alive and seen count until now) for the eligible count
 __global__ void k_sd_pct_apply(const SelectQuery* pct, SubState* st, float* state, float r, float omr) {
+  grid_begin();
   if (threadIdx.x == 0) {
     if (st->n_el > 0) running_pct(pct, state, r, omr, &st->p_lo);
     st->n_el = 0u;
@@ -582,6 +595,7 @@ __global__ void k_sd_priority(int64_t n, const float4* __restrict__ geom, const 
                               const float* __restrict__ delta, const float* __restrict__ z,
                               const float* __restrict__ u, float kappa, float beta, int l_max, uint16_t* grp,
                               uint32_t* pkey, SubState* st, const FirstHist fh) {
+  grid_begin();
   __shared__ uint32_t sh[FH_WORDS];
   fh_clear(fh, sh);
   const int64_t i0 = first_item();
@@ -624,6 +638,7 @@ __global__ void k_sd_priority(int64_t n, const float4* __restrict__ geom, const 
 }
 
 __global__ void k_sd_k(SelectQuery* q, SubState* st, uint32_t top_ppm, long long budget, void* sel_tmp) {
+  grid_begin();
   select_prepare(q + 2, 1, sel_tmp);
   if (threadIdx.x == 0) {
     const unsigned long long na = st->n_alive;
@@ -641,6 +656,7 @@ __global__ void k_sd_k(SelectQuery* q, SubState* st, uint32_t top_ppm, long long
 // (the ties compete by id: the need = k - c_gt smallest ids among them split)
 __global__ void k_sd_ties(int64_t n, const uint32_t* __restrict__ pkey, const SelectQuery* thr,
                           const uint16_t* __restrict__ grp, uint32_t* blk, SubState* st) {
+  grid_begin();
   const int64_t i0 = first_item();
   uint32_t cgt = 0, ceq = 0;
   if (thr->k != 0) {
@@ -672,6 +688,7 @@ __global__ void k_sd_select(int64_t n, const uint8_t* __restrict__ pm, const uin
                             const uint32_t* __restrict__ pkey, const SelectQuery* q,
                             const uint32_t* __restrict__ blk, const SubState* st, uint8_t* selected,
                             uint32_t* surv, uint32_t* sel, uint32_t* blk_surv, uint32_t* blk_sel) {
+  grid_begin();
   const int64_t i0 = first_item();
   const bool any_k = q[2].k != 0;
   const uint32_t v = q[2].result;
@@ -719,6 +736,7 @@ __global__ void k_sd_select(int64_t n, const uint8_t* __restrict__ pm, const uin
 
 __global__ void k_sd_check(const unsigned long long* totals, SubState* st, int64_t capacity, int64_t* n_new,
                            int32_t* status) {
+  grid_begin();
   if (threadIdx.x == 0) {
     const long long nn = (long long)totals[0] + 8ll * (long long)totals[1];
     st->fits = nn <= capacity ? 1u : 0u;
@@ -813,6 +831,7 @@ __device__ __forceinline__ float lerp_rn(float a, float b, float t) {
 }
 
 __global__ void k_cp_flags(int64_t n, const uint8_t* __restrict__ keep, uint32_t* __restrict__ surv) {
+  grid_begin();
   const int64_t i = blockIdx.x * (int64_t)TPB + threadIdx.x;
   if (i < n) surv[i] = keep[i] ? 1u : 0u;
 }
@@ -831,6 +850,7 @@ __global__ void k_sd_list(int64_t n, const uint32_t* __restrict__ sel, const uin
                           unsigned long long* __restrict__ surv_pos, uint32_t* __restrict__ list,
                           uint32_t* __restrict__ holes, unsigned long long* totals, SubState* st, int64_t capacity,
                           int64_t* n_new, int32_t* status) {
+  grid_begin();
   const int64_t i0 = first_item();
   uint32_t sl[IPT], sv[IPT], cs = 0, cl = 0;
   load4(sel, i0, n, sl, 0u);
@@ -935,6 +955,7 @@ __global__ void k_sd_write(int64_t n, int64_t max_children, const uint32_t* __re
                            const unsigned long long* totals, const SubState* st, const float4* __restrict__ geom,
                            const uint8_t* __restrict__ level, const DT* __restrict__ dens, const ST* __restrict__ sh,
                            float4* ogeom, uint8_t* olevel, DT* odens, ST* osh, const __grid_constant__ AuxSet aux) {
+  grid_wait();
   if (!st->fits) return;
   const int64_t gw = (blockIdx.x * (int64_t)TPB + threadIdx.x) >> 5;  // global warp
   const int64_t sw = (n + 31) / 32;
@@ -1005,6 +1026,7 @@ __global__ void __launch_bounds__(TPB) k_ip_children(int64_t n, const uint32_t* 
                                                      const unsigned long long* totals, const SubState* st,
                                                      float4* geom, uint8_t* level, DT* dens, ST* sh,
                                                      const __grid_constant__ AuxSet aux) {
+  grid_wait();
   constexpr int WPR = (int)(48 * sizeof(ST) / 16);  // 16-byte words per SH row
   __shared__ uint4 s_sh[TPB / 32][4 * WPR];
   __shared__ int64_t s_dst[TPB / 32][32];
@@ -1114,6 +1136,7 @@ template <typename DT, typename ST>
 __global__ void __launch_bounds__(TPB) k_ip_tail(int64_t n, const uint32_t* __restrict__ holes,
                                                  const unsigned long long* totals, const SubState* st, float4* geom,
                                                  uint8_t* level, DT* dens, ST* sh, const __grid_constant__ AuxSet aux) {
+  grid_wait();
   if (!st->fits) return;
   const int64_t k = (int64_t)totals[1];
   const int64_t h = n - (int64_t)totals[0] - k;
@@ -1184,12 +1207,12 @@ extern "C" lv_status lv_prune_bins(int64_t n, const uint8_t* seen, const float* 
   cudaStream_t s = (cudaStream_t)stream;
   const int blocks = eblocks(n);  // IPT voxels per thread
   zero_async(s, w.st, sizeof(PruneState));
-  k_pr_seen<<<blocks, TPB, 0, s>>>(n, seen, z, w.grp, w.zkey, w.st);
-  k_pr_pct_queries<<<1, 256, 0, s>>>(w.q, w.st, (uint32_t)p->lo_ppm, (uint32_t)p->hi_ppm, w.sel_tmp);
+  chain(k_pr_seen, blocks, TPB, 0, s)(n, seen, z, w.grp, w.zkey, w.st);
+  chain(k_pr_pct_queries, 1, 256, 0, s)(w.q, w.st, (uint32_t)p->lo_ppm, (uint32_t)p->hi_ppm, w.sel_tmp);
   select_kth_prepared(w.zkey, w.grp, n, w.q, 2, w.sel_tmp, s);
   const float r = p->pct_ema, omr = 1.0f - r;  // rounded to FP32 once, as the oracle does
-  k_pr_pct_apply<<<1, 32, 0, s>>>(w.q, w.st, p->pct_state, r, omr);
-  k_pr_bin<<<blocks, TPB, 0, s>>>(n, seen, z, p->n_bins, w.grp, w.st);
+  chain(k_pr_pct_apply, 1, 32, 0, s)(w.q, w.st, p->pct_state, r, omr);
+  chain(k_pr_bin, blocks, TPB, 0, s)(n, seen, z, p->n_bins, w.grp, w.st);
   count_launch(4);
   return cuda_check(cudaGetLastError(), "lv_prune_bins");
 }
@@ -1218,9 +1241,9 @@ extern "C" lv_status lv_prune_finish(int64_t n, const float* w_max, const uint8_
   // the two selections' first digits are counted by the kernels that write their keys
   const FirstHist fh_tau = first_hist(w.h0_tau, nb, nb), fh_cap = first_hist(w.h0_cap, 1, 1);
   zero_async(s, w.h0_tau, sizeof(uint32_t) * 2 * FH_WORDS, w.h0_cap, sizeof(uint32_t) * select_radix(1));
-  k_pr_wkey<<<blocks, TPB, 0, s>>>(n, w_max, w.grp, w.wkey, fh_tau);
+  chain(k_pr_wkey, blocks, TPB, 0, s)(n, w_max, w.grp, w.wkey, fh_tau);
   // the percentiles in q[0..1] are consumed: q is reused per bin
-  k_pr_tau_queries<<<1, 256, 0, s>>>(w.q, w.st, nb, (uint32_t)p->q_ppm, p->anneal, (uint32_t)p->anneal_ppm,
+  chain(k_pr_tau_queries, 1, 256, 0, s)(w.q, w.st, nb, (uint32_t)p->q_ppm, p->anneal, (uint32_t)p->anneal_ppm,
                                      (uint32_t)p->relax_ppm, w.sel_tmp);
   if (fh_tau.h0) select_kth_first(w.wkey, w.grp, n, w.q, nb, w.h0_tau, w.sel_tmp, s);
   else select_kth_prepared(w.wkey, w.grp, n, w.q, nb, w.sel_tmp, s);
@@ -1234,13 +1257,13 @@ extern "C" lv_status lv_prune_finish(int64_t n, const float* w_max, const uint8_
   halo.delta = p->delta;
   halo.edge_score = p->edge;
   halo.w_max = w_max;
-  k_pr_update<<<blocks, TPB, 0, s>>>(n, w.grp, w.wkey, w.q, alpha, oma, p->m_low, p->m_high, ema_m, state, halo,
+  chain(k_pr_update, blocks, TPB, 0, s)(n, w.grp, w.wkey, w.q, alpha, oma, p->m_low, p->m_high, ema_m, state, halo,
                                       prune_mask, cand, w.st, fh_cap);
   SelectQuery* qc = w.q + SELECT_MAX_QUERIES - 2;  // cap threshold
-  k_pr_cap_query<<<1, 256, 0, s>>>(qc, w.st, cap, w.sel_tmp);
+  chain(k_pr_cap_query, 1, 256, 0, s)(qc, w.st, cap, w.sel_tmp);
   select_kth_first(w.wkey, cand, n, qc, 1, w.h0_cap, w.sel_tmp, s);
-  k_pr_ties<<<blocks, TPB, 0, s>>>(n, w.wkey, qc, prune_mask, w.blk, w.st);
-  k_pr_mask<<<blocks, TPB, 0, s>>>(n, w.wkey, qc, w.blk, w.st, prune_mask, d_n_pruned, cap);
+  chain(k_pr_ties, blocks, TPB, 0, s)(n, w.wkey, qc, prune_mask, w.blk, w.st);
+  chain(k_pr_mask, blocks, TPB, 0, s)(n, w.wkey, qc, w.blk, w.st, prune_mask, d_n_pruned, cap);
   count_launch(7);
   return cuda_check(cudaGetLastError(), "lv_prune_finish");
 }
@@ -1319,19 +1342,19 @@ extern "C" lv_status lv_subdivide_select(const lv_voxels* in, const float* delta
     return cuda_check(cudaGetLastError(), "lv_subdivide_select");
   }
   const int blocks = eblocks(n);  // IPT voxels per thread
-  k_sd_flags<<<blocks, TPB, 0, s>>>(n, seen, prune_mask, z, w.grp, w.zkey, w.st, first_hist(w.h0_pct, 2, 1));
-  k_sd_pct_queries<<<1, 256, 0, s>>>(w.q, (uint32_t)p->lo_ppm, (uint32_t)p->hi_ppm, &w.st->n_el, w.sel_tmp,
+  chain(k_sd_flags, blocks, TPB, 0, s)(n, seen, prune_mask, z, w.grp, w.zkey, w.st, first_hist(w.h0_pct, 2, 1));
+  chain(k_sd_pct_queries, 1, 256, 0, s)(w.q, (uint32_t)p->lo_ppm, (uint32_t)p->hi_ppm, &w.st->n_el, w.sel_tmp,
                                      w.h0_pct);
   select_kth_first(w.zkey, w.grp, n, w.q, 2, w.h0_pct, w.sel_tmp, s);
-  k_sd_pct_apply<<<1, 32, 0, s>>>(w.q, w.st, p->pct_state, p->pct_ema, 1.0f - p->pct_ema);
-  k_sd_priority<<<blocks, TPB, 0, s>>>(n, (const float4*)in->geom, in->level, delta, z, u, p->kappa, p->beta,
+  chain(k_sd_pct_apply, 1, 32, 0, s)(w.q, w.st, p->pct_state, p->pct_ema, 1.0f - p->pct_ema);
+  chain(k_sd_priority, blocks, TPB, 0, s)(n, (const float4*)in->geom, in->level, delta, z, u, p->kappa, p->beta,
                                         p->l_max, w.grp, w.pkey, w.st, first_hist(w.h0_top, 1, 1));
-  k_sd_k<<<1, 256, 0, s>>>(w.q, w.st, (uint32_t)p->top_ppm, (long long)p->budget, w.sel_tmp);
+  chain(k_sd_k, 1, 256, 0, s)(w.q, w.st, (uint32_t)p->top_ppm, (long long)p->budget, w.sel_tmp);
   select_kth_first(w.pkey, w.grp, n, w.q + 2, 1, w.h0_top, w.sel_tmp, s);
-  k_sd_ties<<<blocks, TPB, 0, s>>>(n, w.pkey, w.q + 2, w.grp, w.blk, w.st);
-  k_sd_select<<<blocks, TPB, 0, s>>>(n, prune_mask, w.grp, w.pkey, w.q, w.blk, w.st, selected, w.surv, w.sel,
+  chain(k_sd_ties, blocks, TPB, 0, s)(n, w.pkey, w.q + 2, w.grp, w.blk, w.st);
+  chain(k_sd_select, blocks, TPB, 0, s)(n, prune_mask, w.grp, w.pkey, w.q, w.blk, w.st, selected, w.surv, w.sel,
                                       w.blk_surv, w.blk_sel);
-  k_sd_list<<<blocks, TPB, 0, s>>>(n, w.sel, w.surv, w.blk_surv, w.blk_sel, w.surv_pos, w.sel_list, w.zkey,
+  chain(k_sd_list, blocks, TPB, 0, s)(n, w.sel, w.surv, w.blk_surv, w.blk_sel, w.surv_pos, w.sel_list, w.zkey,
                                    w.totals, w.st, out_capacity, d_n_new, d_status);
   count_launch(9);
   return cuda_check(cudaGetLastError(), "lv_subdivide_select");
@@ -1357,7 +1380,7 @@ extern "C" lv_status lv_subdivide_apply(const lv_voxels* in, const lv_subdiv_par
   const int64_t warps = (n + 31) / 32 + (max_children + 31) / 32;
   const unsigned grid = (unsigned)((warps * 32 + TPB - 1) / TPB);
 #define LV_SUB(DT, ST)                                                                                                 \
-  k_sd_write<DT, ST><<<grid, TPB, 0, s>>>(n, max_children, w.surv, w.surv_pos, w.sel_list, w.totals, w.st,           \
+  launch(k_sd_write<DT, ST>, grid, TPB, 0, s)(n, max_children, w.surv, w.surv_pos, w.sel_list, w.totals, w.st,           \
                                           (const float4*)in->geom, in->level, (const DT*)in->density,                \
                                           (const ST*)in->sh, (float4*)out->geom, (uint8_t*)out->level,               \
                                           (DT*)out->density, (ST*)out->sh, as)
@@ -1408,9 +1431,9 @@ extern "C" lv_status lv_subdivide_apply_inplace(const lv_voxels* vox, int64_t ca
 #define LV_IP(DT, ST)                                                                                                  \
   do {                                                                                                                \
     if (grid > 0)                                                                                                     \
-      k_ip_children<DT, ST><<<grid, TPB, 0, s>>>(n, w.sel_list, holes, w.totals, w.st, (float4*)vox->geom,            \
+      launch(k_ip_children<DT, ST>, grid, TPB, 0, s)(n, w.sel_list, holes, w.totals, w.st, (float4*)vox->geom,            \
                                                  (uint8_t*)vox->level, (DT*)vox->density, (ST*)vox->sh, as);          \
-    k_ip_tail<DT, ST><<<tail_grid, TPB, 0, s>>>(n, holes, w.totals, w.st, (float4*)vox->geom, (uint8_t*)vox->level,   \
+    chain(k_ip_tail<DT, ST>, tail_grid, TPB, 0, s)(n, holes, w.totals, w.st, (float4*)vox->geom, (uint8_t*)vox->level,   \
                                                 (DT*)vox->density, (ST*)vox->sh, as);                                 \
   } while (0)
   if (vox->density_dtype == LV_F32 && vox->sh_dtype == LV_F32) LV_IP(float, float);
@@ -1448,12 +1471,12 @@ extern "C" lv_status lv_compact(const lv_voxels* in, const uint8_t* keep, const 
   for (int a = 0; a < n_aux; ++a) as.a[a] = aux[a];
   cudaMemsetAsync(w.st, 0, sizeof(SubState), s);
   const int blocks = blocks_for(n);
-  k_cp_flags<<<blocks, TPB, 0, s>>>(n, keep, w.surv);
+  launch(k_cp_flags, blocks, TPB, 0, s)(n, keep, w.surv);
   scan2(w.surv, nullptr, n, w.surv_pos, nullptr, w.totals, w.scan_tmp, s);  // totals[1] = 0: no children
-  k_sd_check<<<1, 32, 0, s>>>(w.totals, w.st, out->n, d_n_new, d_status);
+  chain(k_sd_check, 1, 32, 0, s)(w.totals, w.st, out->n, d_n_new, d_status);
   const unsigned grid = (unsigned)((((n + 31) / 32) * 32 + TPB - 1) / TPB);  // one warp per 32 voxels
 #define LV_CP(DT, ST)                                                                                         \
-  k_sd_write<DT, ST><<<grid, TPB, 0, s>>>(n, 0, w.surv, w.surv_pos, w.sel_list, w.totals, w.st,            \
+  chain(k_sd_write<DT, ST>, grid, TPB, 0, s)(n, 0, w.surv, w.surv_pos, w.sel_list, w.totals, w.st,            \
                                           (const float4*)in->geom, in->level, (const DT*)in->density,       \
                                           (const ST*)in->sh, (float4*)out->geom, (uint8_t*)out->level,      \
                                           (DT*)out->density, (ST*)out->sh, as)

@@ -29,6 +29,7 @@ void count_launch(int k) { g_launches.fetch_add(k, std::memory_order_relaxed); }
 namespace {
 // 16-byte words where the range allows, bytes at the ragged ends
 __global__ void k_zero(const ZeroRanges r) {
+  grid_begin();
   const size_t stride = (size_t)gridDim.x * blockDim.x;
   const size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
 #pragma unroll
@@ -60,6 +61,7 @@ struct RowsArg {
 };
 
 __global__ void k_rows_scatter(const __grid_constant__ RowsArg r) {
+  grid_wait();
   const int64_t total = r.start[r.n];
   for (int64_t u = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; u < total; u += (int64_t)gridDim.x * blockDim.x) {
     int a = 0;
@@ -88,7 +90,7 @@ void zero_async(cudaStream_t s, void* p0, size_t b0, void* p1, size_t b1, void* 
   size_t blocks = (most / 16 + 255) / 256;
   if (blocks < 1) blocks = 1;
   if (blocks > 1216) blocks = 1216;
-  k_zero<<<(unsigned)blocks, 256, 0, s>>>(r);
+  launch(k_zero, (unsigned)blocks, 256, 0, s)(r);
   count_launch(1);
 }
 
@@ -158,7 +160,7 @@ extern "C" lv_status lv_rows_scatter(const lv_rows* arrays, int n_arrays, void* 
   const int64_t total = r.start[r.n];
   const int64_t want = (total + 255) / 256;
   const unsigned blocks = (unsigned)(want < 4 * 1216 ? (want < 1 ? 1 : want) : 4 * 1216);
-  k_rows_scatter<<<blocks, 256, 0, (cudaStream_t)stream>>>(r);
+  launch(k_rows_scatter, blocks, 256, 0, (cudaStream_t)stream)(r);
   count_launch(1);
   return cuda_check(cudaGetLastError(), "lv_rows_scatter");
 }

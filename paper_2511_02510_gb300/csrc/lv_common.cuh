@@ -47,6 +47,50 @@ void once_per_device(std::atomic<unsigned long long>& done, F&& f) {
   if (bit) done.fetch_or(bit, std::memory_order_release);
 }
 
+// Kernel launches.  chain(k, grid, block, smem, stream)(args...) launches k so
+// that it may become resident while the kernel before it in the stream still runs
+// (programmatic stream serialization): every kernel of the library starts with
+// grid_begin() or grid_wait(), which waits until the grids before it have
+// completed and their writes are visible, so only the launch latency overlaps.
+// A call of many short kernels (25 in a small training iteration, 23 in a
+// pruning) spent 1 to 2 us of each on that latency.  launch(...) does not
+// overlap: for the first kernel of a call and after an event record, where what
+// comes before in the stream is the caller's.
+template <typename T>
+struct SameType {
+  using type = T;
+};
+template <typename... K>
+struct Launcher {
+  void (*kernel)(K...);
+  dim3 grid, block;
+  size_t smem;
+  cudaStream_t stream;
+  bool chained;
+  void operator()(const typename SameType<K>::type&... args) const {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = chained ? 1 : 0;
+    void* ptrs[] = {(void*)&args...};
+    cudaLaunchKernelExC(&cfg, (const void*)kernel, ptrs);
+  }
+};
+template <typename... K>
+Launcher<K...> chain(void (*k)(K...), dim3 grid, dim3 block, size_t smem, cudaStream_t s) {
+  return {k, grid, block, smem, s, true};
+}
+template <typename... K>
+Launcher<K...> launch(void (*k)(K...), dim3 grid, dim3 block, size_t smem, cudaStream_t s) {
+  return {k, grid, block, smem, s, false};
+}
+
 // Bump allocator over a caller-owned workspace (also used to size it).
 struct Carve {
   char* base;
@@ -74,6 +118,16 @@ void zero_async(cudaStream_t s, void* p0, size_t b0, void* p1 = nullptr, size_t 
                 size_t b2 = 0, void* p3 = nullptr, size_t b3 = 0);
 
 // ---------------------------------------------------------------- device-side
+// The first statement of every kernel (see chain): waits for the grids before
+// it.  grid_begin also lets the next grid become resident from now on, as far as
+// this one leaves room; long kernels, beside which it would only hold resources, use
+// grid_wait, and the next grid follows their last blocks.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_begin() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  grid_wait();
+}
+
 __device__ __forceinline__ void report(int32_t* st, int code) {
   if (st) atomicCAS(st, 0, code);
 }

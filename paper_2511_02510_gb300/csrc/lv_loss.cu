@@ -93,6 +93,7 @@ __device__ __forceinline__ int view_of_block(const int* first, int n, int b) {
 constexpr int ST = 32, SP = ST + 2;
 __global__ void __launch_bounds__(TPB) k_lf_sobel(const float* __restrict__ gt, const __grid_constant__ ViewPix vp,
                                                  int per, uint32_t* __restrict__ mkey, uint32_t* __restrict__ hist) {
+  grid_begin();
   __shared__ uint32_t s_h[D1_BINS];
   __shared__ float s_y[SP * SP];
   const int t = threadIdx.x;
@@ -211,6 +212,7 @@ __device__ __forceinline__ LfPick block_pick(const uint32_t* __restrict__ h, uin
 template <bool LAST>
 __global__ void __launch_bounds__(TPB) k_lf_digit(const uint32_t* __restrict__ mkey, const __grid_constant__ ViewPix vp,
                                                  uint32_t* hist, LfPick* pick) {
+  grid_begin();
   constexpr int NB = LAST ? D3_BINS : D2_BINS;
   __shared__ uint32_t s_h[NB];
   const int t = threadIdx.x, v = view_of_block(vp.blk, vp.n, blockIdx.x);
@@ -267,6 +269,7 @@ __global__ void __launch_bounds__(TPB) k_lf_weight(const uint32_t* __restrict__ 
                                                   const LfPick* __restrict__ pick,
                                                   const __grid_constant__ ViewPix vp, float eps, float gamma,
                                                   float* __restrict__ w, double* wsum, float* __restrict__ edge_out) {
+  grid_begin();
   const int v = view_of_block(vp.blk, vp.n, blockIdx.x);
   const int b0 = vp.blk[v], nb = vp.blk[v + 1] - b0;
   const long long lo = vp.off[v], hi = vp.off[v + 1];
@@ -313,6 +316,7 @@ __device__ __forceinline__ void lf_view_constants(const double* wsum, int v, lon
 __global__ void k_lf_loss(const float* __restrict__ rgb, const float* __restrict__ gt, const float* __restrict__ w,
                           const __grid_constant__ ViewPix vp, const double* wsum, double* lsum,
                           float* __restrict__ grad) {
+  grid_begin();
   const int v = view_of_block(vp.blk, vp.n, blockIdx.x);
   const int b0 = vp.blk[v], nb = vp.blk[v + 1] - b0;
   const long long lo = vp.off[v], hi = vp.off[v + 1];
@@ -344,6 +348,7 @@ __global__ void k_lf_loss(const float* __restrict__ rgb, const float* __restrict
 __global__ void k_lf_loss4(const float* __restrict__ rgb, const float* __restrict__ gt, const float* __restrict__ w,
                            const __grid_constant__ ViewPix vp, const double* wsum, double* lsum,
                            float* __restrict__ grad) {
+  grid_begin();
   const int v = view_of_block(vp.blk, vp.n, blockIdx.x);
   const int b0 = vp.blk[v], nb = vp.blk[v + 1] - b0;
   const long long lo = vp.off[v], hi = vp.off[v + 1];
@@ -406,6 +411,7 @@ __global__ void k_lf_loss4(const float* __restrict__ rgb, const float* __restric
 
 // clear: the sums are zeroed once read (the fused backward's sums start from zero next time)
 __global__ void k_lf_finish(const __grid_constant__ ViewPix vp, double* lsum, float* loss, bool clear) {
+  grid_begin();
   int v = threadIdx.x;
   if (v < vp.n) {
     const long long np = vp.off[v + 1] - vp.off[v];
@@ -494,11 +500,11 @@ extern "C" lv_status lv_lf_weights(const float* gt, const int32_t* widths, const
              sizeof(uint32_t) * HIST_WORDS * (size_t)n_views);
   // a block clears and adds up all the counters, so it takes several tiles once there are enough
   const int tiles = vp.tile[n_views], per = (tiles + SOBEL_BLOCKS - 1) / SOBEL_BLOCKS;
-  k_lf_sobel<<<(unsigned)((tiles + per - 1) / per), TPB, 0, s>>>(gt, vp, per, w.mkey, w.hist);
+  chain(k_lf_sobel, (unsigned)((tiles + per - 1) / per), TPB, 0, s)(gt, vp, per, w.mkey, w.hist);
   const unsigned blocks = (unsigned)vp.blk[n_views];
-  k_lf_digit<false><<<blocks, TPB, 0, s>>>(w.mkey, vp, w.hist, w.pick);
-  k_lf_digit<true><<<blocks, TPB, 0, s>>>(w.mkey, vp, w.hist, w.pick);
-  k_lf_weight<<<blocks, TPB, 0, s>>>(w.mkey, w.hist, w.pick, vp, p->eps, gamma, w.w, w.wsum, p->edge_out);
+  chain(k_lf_digit<false>, blocks, TPB, 0, s)(w.mkey, vp, w.hist, w.pick);
+  chain(k_lf_digit<true>, blocks, TPB, 0, s)(w.mkey, vp, w.hist, w.pick);
+  chain(k_lf_weight, blocks, TPB, 0, s)(w.mkey, w.hist, w.pick, vp, p->eps, gamma, w.w, w.wsum, p->edge_out);
   count_launch(4);
   return cuda_check(cudaGetLastError(), "lv_lf_weights");
 }
@@ -516,9 +522,9 @@ extern "C" lv_status lv_lf_loss_from_weights(const float* rgb, const float* gt, 
   // four pixels (three 16-byte words of rgb, gt and dL_drgb) per step where the buffers allow it
   const bool vec = aligned16(rgb) && aligned16(gt) && aligned16(w.w) && (!dL_drgb || aligned16(dL_drgb));
   const unsigned blocks = (unsigned)vp.blk[n_views];
-  if (vec) k_lf_loss4<<<blocks, TPB, 0, s>>>(rgb, gt, w.w, vp, w.wsum, w.lsum, dL_drgb);
-  else k_lf_loss<<<blocks, TPB, 0, s>>>(rgb, gt, w.w, vp, w.wsum, w.lsum, dL_drgb);
-  k_lf_finish<<<1, LV_MAX_VIEWS, 0, s>>>(vp, w.lsum, loss, false);
+  if (vec) chain(k_lf_loss4, blocks, TPB, 0, s)(rgb, gt, w.w, vp, w.wsum, w.lsum, dL_drgb);
+  else chain(k_lf_loss, blocks, TPB, 0, s)(rgb, gt, w.w, vp, w.wsum, w.lsum, dL_drgb);
+  chain(k_lf_finish, 1, LV_MAX_VIEWS, 0, s)(vp, w.lsum, loss, false);
   count_launch(2);
   return cuda_check(cudaGetLastError(), "lv_lf_loss_from_weights");
 }
@@ -530,7 +536,7 @@ extern "C" lv_status lv_lf_loss_finish(const int32_t* widths, const int32_t* hei
   LfWs w;
   lv_status e = lf_setup(widths, heights, n_views, 990000, workspace, ws_bytes, &vp, &w);
   if (e != LV_OK) return e;
-  k_lf_finish<<<1, LV_MAX_VIEWS, 0, (cudaStream_t)stream>>>(vp, w.lsum, loss, true);
+  launch(k_lf_finish, 1, LV_MAX_VIEWS, 0, (cudaStream_t)stream)(vp, w.lsum, loss, true);
   count_launch(1);
   return cuda_check(cudaGetLastError(), "lv_lf_loss_finish");
 }

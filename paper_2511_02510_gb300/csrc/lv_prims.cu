@@ -44,6 +44,7 @@ __device__ __forceinline__ void block_exclusive_scan2(unsigned long long& a, uin
 
 __global__ void k_scan2_reduce(const uint32_t* a, const uint32_t* b, int64_t n, int64_t chunk,
                                unsigned long long* bsa, uint32_t* bsb) {
+  grid_begin();
   __shared__ unsigned long long sa[32];
   __shared__ uint32_t sb[32];
   int64_t lo = blockIdx.x * chunk, hi = min(n, lo + chunk);
@@ -60,6 +61,7 @@ __global__ void k_scan2_reduce(const uint32_t* a, const uint32_t* b, int64_t n, 
 }
 
 __global__ void k_scan2_blocks(unsigned long long* bsa, uint32_t* bsb, int nb, unsigned long long* totals) {
+  grid_begin();
   __shared__ unsigned long long sa[32];
   __shared__ uint32_t sb[32];
   // nb <= SCAN_BLOCKS = 2 * SCAN_THREADS: two items per thread
@@ -85,6 +87,7 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan2_apply(const uint32_t* a,
                                                              int64_t chunk, const unsigned long long* bsa,
                                                              const uint32_t* bsb, unsigned long long* out_a,
                                                              uint32_t* out_b) {
+  grid_begin();
   __shared__ unsigned long long sa[32];
   __shared__ uint32_t sb[32];
   // one pad word per 8 items: a thread's 8 consecutive items then sit in
@@ -146,9 +149,9 @@ void scan2(const uint32_t* a, const uint32_t* b, int64_t n, unsigned long long* 
   uint32_t* bsb = (uint32_t*)(bsa + SCAN_BLOCKS);
   int64_t chunk = (n + SCAN_BLOCKS - 1) / SCAN_BLOCKS;
   if (chunk < 1) chunk = 1;
-  k_scan2_reduce<<<SCAN_BLOCKS, SCAN_THREADS, 0, s>>>(a, b, n, chunk, bsa, bsb);
-  k_scan2_blocks<<<1, SCAN_THREADS, 0, s>>>(bsa, bsb, SCAN_BLOCKS, totals);
-  k_scan2_apply<<<SCAN_BLOCKS, SCAN_THREADS, 0, s>>>(a, b, n, chunk, bsa, bsb, out_a, out_b);
+  chain(k_scan2_reduce, SCAN_BLOCKS, SCAN_THREADS, 0, s)(a, b, n, chunk, bsa, bsb);
+  chain(k_scan2_blocks, 1, SCAN_THREADS, 0, s)(bsa, bsb, SCAN_BLOCKS, totals);
+  chain(k_scan2_apply, SCAN_BLOCKS, SCAN_THREADS, 0, s)(a, b, n, chunk, bsa, bsb, out_a, out_b);
   count_launch(3);
 }
 
@@ -238,6 +241,7 @@ template <typename K>
 __global__ void __launch_bounds__(OS_HIST_THREADS) k_os_hist(const K* __restrict__ keys, const unsigned long long* d_count,
                                                        int64_t cap, int passes, uint32_t* __restrict__ ghist,
                                                        unsigned long long* __restrict__ look0) {
+  grid_begin();
   __shared__ uint32_t sh[OS_MAX_PASSES * RADIX];
   for (int i = threadIdx.x; i < passes * RADIX; i += OS_HIST_THREADS) sh[i] = 0;
   __syncthreads();
@@ -289,6 +293,7 @@ __global__ void __launch_bounds__(Os<K>::THREADS, Os<K>::MIN_BLOCKS) k_os_pass(c
                                                          unsigned long long* look, unsigned long long* look_next,
                                                          int32_t* status, unsigned spin_limit,
                                                          uint32_t* __restrict__ key_ranges) {
+  grid_begin();
   constexpr int OS_THREADS = Os<K>::THREADS, OS_WARPS = Os<K>::WARPS, OS_TILE = Os<K>::TILE;
   __shared__ uint32_t s_wh[OS_WARPS][RADIX + 1];  // warp digit counts -> warp prefixes (bin RADIX: padding items)
   __shared__ uint32_t s_start[RADIX];             // tile-local start of each digit
@@ -503,14 +508,14 @@ static int radix_sort_t(const K* kin, const uint32_t* vin, K* k0, uint32_t* v0, 
   if (!counted) {
     zero_async(s, st.ghist, sizeof(uint32_t) * (OS_MAX_PASSES * RADIX + 2));  // counts and tickets
     const int hb = (int)min((int64_t)OS_HIST_BLOCKS, tiles);
-    k_os_hist<K><<<hb, OS_HIST_THREADS, 0, s>>>(kin, d_count, cap, passes, st.ghist, st.look[0]);
+    chain(k_os_hist<K>, hb, OS_HIST_THREADS, 0, s)(kin, d_count, cap, passes, st.ghist, st.look[0]);
   }
   for (int p = 0; p < passes; ++p) {
     // pass 0 reads the input (kept intact unless it is k0 / v0), pass p writes buffer (p + 1) & 1
     const K* ks = p == 0 ? kin : kb[p & 1];
     const uint32_t* vs = p == 0 ? vin : vb[p & 1];
     const int dst = (p + 1) & 1;
-    k_os_pass<K><<<(unsigned)tiles, Os<K>::THREADS, 0, s>>>(ks, vs, kb[dst], vb[dst], d_count, cap, p, st.ghist,
+    chain(k_os_pass<K>, (unsigned)tiles, Os<K>::THREADS, 0, s)(ks, vs, kb[dst], vb[dst], d_count, cap, p, st.ghist,
                                                        st.ticket, st.look[p & 1], st.look[(p + 1) & 1], status,
                                                        OS_SPIN_LIMIT, p == passes - 1 ? key_ranges : nullptr);
   }
@@ -565,6 +570,7 @@ DbgWs carve_dbg(void* base) {
   return w;
 }
 __global__ void k_dbg_setup(unsigned long long* count, uint32_t* ticket) {
+  grid_begin();
   if (threadIdx.x == 0) {
     *count = (unsigned long long)DBG_ITEMS;
     ticket[0] = 1u;  // the one block launched takes tile 1
@@ -587,8 +593,8 @@ extern "C" lv_status lv_debug_sort_timeout(int32_t spin_limit, void* workspace, 
   SortTmp st = carve_sort(w.tmp, DBG_ITEMS);
   cudaMemsetAsync(workspace, 0, w.bytes, s);  // keys, counts, tickets and look-back words
   cudaMemsetAsync(d_status, 0, sizeof(int32_t), s);
-  k_dbg_setup<<<1, 32, 0, s>>>(w.count, st.ticket);
-  k_os_pass<uint32_t><<<1, Os<uint32_t>::THREADS, 0, s>>>(w.k0, nullptr, w.k1, w.v1, w.count, DBG_ITEMS, 0, st.ghist,
+  launch(k_dbg_setup, 1, 32, 0, s)(w.count, st.ticket);
+  chain(k_os_pass<uint32_t>, 1, Os<uint32_t>::THREADS, 0, s)(w.k0, nullptr, w.k1, w.v1, w.count, DBG_ITEMS, 0, st.ghist,
                                                           st.ticket, st.look[0], st.look[1], d_status,
                                                           (unsigned)spin_limit, nullptr);
   count_launch(2);
@@ -677,6 +683,7 @@ __device__ __forceinline__ SelectQuery warp_pick(const uint32_t* __restrict__ ro
 // histogram row cleared.
 template <int RADIX>
 __global__ void k_sel_pick(const SelectQuery* q_in, SelectQuery* q, int nq, int shift, uint32_t* hist) {
+  grid_begin();
   const int lane = threadIdx.x & 31;
   const int j = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (j >= nq) return;  // warp-uniform
@@ -702,6 +709,7 @@ __global__ void __launch_bounds__(SEL_THREADS) k_sel_hist(const uint32_t* keys, 
                                                          const SelectQuery* q, int nq, int shift, int width,
                                                          uint32_t* hist, const uint32_t* hist_prev, int prev_shift,
                                                          SelectQuery* q_out, uint32_t* clear, int clear_words) {
+  grid_begin();
   extern __shared__ uint4 sh4[];  // nq * RADIX counters
   uint32_t* sh = (uint32_t*)sh4;
   __shared__ SelectQuery sq[SELECT_MAX_QUERIES];
@@ -837,12 +845,12 @@ void select_passes(const uint32_t* keys, const uint16_t* grp, int64_t n, SelectQ
     const int wbits = p == 0 ? key_bits - width * (npass - 1) : width;
     shift -= wbits;
     if (p > 0 || !h0)
-      k_sel_hist<RADIX><<<blocks, SEL_THREADS, smem, s>>>(keys, grp, n, A(p > 0 ? p - 1 : 0), nq, shift, wbits,
+      chain(k_sel_hist<RADIX>, blocks, SEL_THREADS, smem, s)(keys, grp, n, A(p > 0 ? p - 1 : 0), nq, shift, wbits,
                                                           H[p % 3], p > 0 ? H[(p - 1) % 3] : nullptr, prev_shift,
                                                           p > 0 ? A(p) : nullptr, H[(p + 1) % 3], words);
     prev_shift = shift;
   }
-  k_sel_pick<RADIX><<<(nq + 7) / 8, 256, 0, s>>>(A(npass - 1), d_queries, nq, 0, H[(npass - 1) % 3]);
+  chain(k_sel_pick<RADIX>, (nq + 7) / 8, 256, 0, s)(A(npass - 1), d_queries, nq, 0, H[(npass - 1) % 3]);
   count_launch(npass + (h0 ? 0 : 1));
 }
 

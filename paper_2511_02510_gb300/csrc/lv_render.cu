@@ -364,6 +364,7 @@ __global__ void __launch_bounds__(BIN_THREADS) k_bin(const float4* __restrict__ 
                                                      unsigned long long* __restrict__ blk_pairs,
                                                      uint32_t* __restrict__ blk_slots, float* z_min,
                                                      float* delta_min, uint8_t* seen, const ZeroRanges zr) {
+  grid_begin();
   __shared__ unsigned long long s_pairs[BIN_THREADS / 32];
   __shared__ uint32_t s_slots[BIN_THREADS / 32];
   // the later kernels' counters are cleared here, not by a launch of their own (whole 32-bit words)
@@ -411,6 +412,7 @@ __global__ void __launch_bounds__(BO_THREADS) k_block_offsets(unsigned long long
                                                               unsigned long long* __restrict__ grp_pairs,
                                                               uint32_t* __restrict__ grp_slots,
                                                               unsigned long long* __restrict__ counters) {
+  grid_begin();
   __shared__ unsigned long long s_a[BO_THREADS / 32];
   __shared__ uint32_t s_b[BO_THREADS / 32];
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
@@ -646,6 +648,7 @@ __global__ void __launch_bounds__(256) k_emit(const float4* __restrict__ geom, c
                                               float4* __restrict__ rec,
                                               float4* __restrict__ d_rgb, uint32_t* __restrict__ s_dkey,
                                               const uint32_t* __restrict__ vidx) {
+  grid_begin();
   // Block b covers 256 consecutive voxels of view b % views, so the blocks of
   // all views of one voxel range run side by side: a voxel's SH row comes
   // from HBM once and from L2 for its other views.  Items are view-major
@@ -976,6 +979,7 @@ __global__ void __launch_bounds__(TW_WARPS * 32, 2) k_tile_sort_warp(const uint3
                                                                     const __grid_constant__ ViewSet vs,
                                                                     const uint2* __restrict__ rec_bb,
                                                                     uint2* __restrict__ plist) {
+  grid_begin();
   extern __shared__ __align__(16) unsigned char tw_raw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   WarpSortSmem& W = reinterpret_cast<TileSortWarpSmem*>(tw_raw)->w[warp];
@@ -1430,6 +1434,7 @@ __global__ void __launch_bounds__(TS_THREADS, 2) k_tile_sort(const uint32_t* __r
                                                             const __grid_constant__ ViewSet vs,
                                                             const uint2* __restrict__ rec_bb,
                                                             uint2* __restrict__ plist) {
+  grid_begin();
   TileLongSmem& M = ts_smem();
   const unsigned int nl = *n_long, total = nl + *n_mid;
   while (true) {
@@ -1460,6 +1465,7 @@ __global__ void __launch_bounds__(TS_THREADS, 2) k_tile_rest(const uint32_t* __r
                                                             const __grid_constant__ ViewSet vs,
                                                             const uint2* __restrict__ rec_bb,
                                                             uint2* __restrict__ plist) {
+  grid_begin();
   TileLongSmem& M = ts_smem();
   const unsigned int total = *n_list;
   if (total == 0u) return;
@@ -1815,6 +1821,7 @@ __global__ void __launch_bounds__(TS* TS, min_blocks<TS>()) k_fwd(const __grid_c
                                                 unsigned long long* __restrict__ wmax, unsigned int* work,
                                                 uint32_t n_items, int sm_cut, int n_sms, unsigned int* arrivals,
                                                 const TileOrder order, const Front fr) {
+  grid_wait();
   constexpr int NW = TS * TS / 32;
   extern __shared__ float4 smem_f4[];
   if (PERSIST && sm_leave(sm_cut, n_sms, arrivals)) return;  // block-uniform
@@ -1998,6 +2005,7 @@ __global__ void __launch_bounds__(TS* TS, min_blocks<TS>()) k_bwd(const __grid_c
                                                 float4* __restrict__ d_rgb, unsigned int* work, uint32_t n_items,
                                                 int sm_cut, int n_sms, unsigned int* arrivals, const TileOrder order,
                                                 const LfFuse lf) {
+  grid_wait();
   constexpr int NW = TS * TS / 32;
   extern __shared__ float4 smem_f4[];
   __shared__ double s_lf[NW][LV_MAX_VIEWS];  // each warp's loss sums (fused LF loss; no atomics)
@@ -2186,6 +2194,7 @@ __global__ void __launch_bounds__(128) k_sh_bwd(const float4* __restrict__ rec, 
                                                 const uint32_t* __restrict__ cnt, const uint32_t* __restrict__ slot,
                                                 float4* __restrict__ d_rgb, float* __restrict__ d_sh,
                                                 int accumulate) {
+  grid_wait();
   constexpr int RS = 49;
   __shared__ float s_rows[4][32 * RS];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -2247,6 +2256,7 @@ __global__ void __launch_bounds__(128) k_sh_bwd(const float4* __restrict__ rec, 
 
 __global__ void k_unpack_wmax(const unsigned long long* __restrict__ packed, int64_t n, float* __restrict__ w,
                               int64_t* __restrict__ arg) {
+  grid_begin();
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= n) return;
   unsigned long long v = packed[i];
@@ -2261,6 +2271,7 @@ __global__ void k_unpack_wmax(const unsigned long long* __restrict__ packed, int
 
 __global__ void k_gather_edge(const int64_t* __restrict__ argmax, int64_t n, const float* __restrict__ edge_map,
                               int64_t n_pix, float* __restrict__ edge) {
+  grid_begin();
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= n) return;
   const int64_t a = argmax[i];
@@ -2271,6 +2282,7 @@ __global__ void k_gather_edge(const int64_t* __restrict__ argmax, int64_t n, con
 __global__ void k_debug_pairs(const uint2* __restrict__ ranges, int64_t tiles, const uint2* __restrict__ plist,
                               const uint32_t* __restrict__ slot_vox, const uint32_t* __restrict__ s_dkey,
                               uint64_t* ko, uint32_t* vo) {
+  grid_begin();
   for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
     const uint2 r = ranges[tile];
     for (uint32_t i = r.x + threadIdx.x; i < r.y; i += blockDim.x) {
@@ -2308,6 +2320,7 @@ __global__ void k_render_f64(const __grid_constant__ ViewSet vs, const uint32_t*
                              int sh_nb, const int64_t* __restrict__ pixels, int64_t n_px, double t_stop,
                              int segment, const uint32_t* __restrict__ vidx, double* __restrict__ rgb_out,
                              double* __restrict__ T_out) {
+  grid_begin();
   const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (q >= n_px) return;
   const long long gp = pixels[q];
@@ -2479,7 +2492,9 @@ static void launch_fwd_t(int64_t tiles, cudaStream_t s, const ViewSet& vs, const
   unsigned grid = (unsigned)tiles;
   if (PERSIST) grid = (unsigned)(tiles < pb ? tiles : pb);  // the work counters were cleared at the start of the forward
   const Front fr = {w.ready, w.prog, w.open_tiles, w.work + 7, w.dep, w.nsamp, resume};
-  k_fwd<TS, SEG, PERSIST><<<grid, TS * TS, smem, s>>>(vs, w.ranges, w.plist, w.rec, w.slot_vox, t_stop,
+  auto k = out->composite_event && !resume ? launch(k_fwd<TS, SEG, PERSIST>, grid, TS * TS, smem, s)
+                                           : chain(k_fwd<TS, SEG, PERSIST>, grid, TS * TS, smem, s);
+  k(vs, w.ranges, w.plist, w.rec, w.slot_vox, t_stop,
                                                        out->rgb, out->depth, out->T, out->n_contrib,
                                                        out->n_samples, w.tau, out->wmax_packed,
                                                        w.work + (resume ? 2 : 0), n_items, sm_cut, sms,
@@ -2507,7 +2522,7 @@ static void launch_bwd_t(int64_t tiles, cudaStream_t s, const ViewSet& vs, const
     zero_async(s, w.work + 1, sizeof(unsigned int), w.work + 9, sizeof(unsigned int));
     grid = (unsigned)(tiles < pb ? tiles : pb);
   }
-  k_bwd<TS, SEG, PERSIST><<<grid, TS * TS, smem, s>>>(vs, w.ranges, w.plist, w.rec, w.slot_vox, fwd->T,
+  launch(k_bwd<TS, SEG, PERSIST>, grid, TS * TS, smem, s)(vs, w.ranges, w.plist, w.rec, w.slot_vox, fwd->T,
                                                        w.tau, fwd->n_contrib, gC, gD, gT, dd, w.d_rgb, w.work + 1,
                                                        n_items, sm_cut, sms, w.work + 9, tile_order(w), lf);
 }
@@ -2534,12 +2549,12 @@ static void launch_tile_sort(const FwdWs& w, const ViewSet& vs, int64_t n, int64
   const bool ready = sort_passes(tile_bits(tiles)) > 0;
   const uint32_t* sv = w.tile_slots;
   const unsigned wblocks = (unsigned)((tiles + TW_WARPS - 1) / TW_WARPS);
-  k_tile_sort_warp<<<wblocks, TW_WARPS * 32, sizeof(TileSortWarpSmem), s>>>(
+  chain(k_tile_sort_warp, wblocks, TW_WARPS * 32, sizeof(TileSortWarpSmem), s)(
       sv, w.s_dkey, w.counters, pair_cap, ready, tiles, w.ranges, w.mid_tiles, w.work + 4, w.long_tiles, w.work + 6,
       w.short_tiles, w.work + 11, w.ready, w.prog, vs, w.rec_bb, w.plist);
   count_launch(1);
   if (n <= TW_MAX) return;  // a tile lists a voxel once: every list is short
-  k_tile_sort<<<(unsigned)nb, TS_THREADS, sizeof(TileLongSmem), s>>>(
+  chain(k_tile_sort, (unsigned)nb, TS_THREADS, sizeof(TileLongSmem), s)(
       sv, w.long_keys, w.s_dkey, w.ranges, w.mid_tiles, w.work + 4, w.long_tiles, w.work + 6, w.work + 5,
       w.ready, w.prog, n > TS_LAZY_VOXELS ? TS_LAZY : ~0u, vs, w.rec_bb, w.plist);
   count_launch(1);
@@ -2548,7 +2563,7 @@ static void launch_tile_sort(const FwdWs& w, const ViewSet& vs, int64_t n, int64
 static void launch_tile_rest(const FwdWs& w, const ViewSet& vs, int64_t tiles, bool all, cudaStream_t s) {
   const int64_t nb = std::min<int64_t>(tile_sort_blocks(), tiles);
   if (all) zero_async(s, w.work + 3, sizeof(unsigned int));
-  k_tile_rest<<<(unsigned)nb, TS_THREADS, sizeof(TileLongSmem), s>>>(
+  chain(k_tile_rest, (unsigned)nb, TS_THREADS, sizeof(TileLongSmem), s)(
       w.tile_slots, w.long_keys, w.ranges, all ? w.long_tiles : w.open_tiles,
       w.work + (all ? 6 : 7), w.work + 3, w.ready, w.prog, vs, w.rec_bb, w.plist);
   count_launch(1);
@@ -2632,14 +2647,16 @@ extern "C" lv_status lv_rasterize_forward(const lv_voxels* vox, const lv_camera*
   if (items > 0) {
     const int64_t blocks = bin_blocks(n);
     const unsigned item_blocks = (unsigned)(blocks * n_views);  // (voxel range, view) blocks
-    k_bin<<<item_blocks, BIN_THREADS, 0, s>>>((const float4*)vox->geom, n, blocks, vs, w.cnt, w.rect, w.pbox, w.dkey,
+    const unsigned bo_blocks = (unsigned)((blocks * n_views + BO_GROUP - 1) / BO_GROUP);
+    launch(k_bin, item_blocks, BIN_THREADS, 0, s)((const float4*)vox->geom, n, blocks, vs, w.cnt, w.rect, w.pbox, w.dkey,
                                               w.blk_pairs, w.blk_slots, out->z_min, out->delta_min, out->seen, zr);
     if (out->stats_event) cudaEventRecord((cudaEvent_t)out->stats_event, s);  // statistics final
-    k_block_offsets<<<(unsigned)((blocks * n_views + BO_GROUP - 1) / BO_GROUP), BO_THREADS, 0, s>>>(
-        w.blk_pairs, w.blk_slots, blocks * n_views, w.grp_pairs, w.grp_slots, w.counters);
+    auto offsets = out->stats_event ? launch(k_block_offsets, bo_blocks, BO_THREADS, 0, s)
+                                    : chain(k_block_offsets, bo_blocks, BO_THREADS, 0, s);
+    offsets(w.blk_pairs, w.blk_slots, blocks * n_views, w.grp_pairs, w.grp_slots, w.counters);
     const int nb = (vox->sh_degree + 1) * (vox->sh_degree + 1);
 #define LV_EMIT(DT, ST)                                                                                             \
-  k_emit<DT, ST><<<item_blocks, BIN_THREADS, 0, s>>>((const float4*)vox->geom, (const DT*)vox->density, (const ST*)vox->sh, \
+  chain(k_emit<DT, ST>, item_blocks, BIN_THREADS, 0, s)((const float4*)vox->geom, (const DT*)vox->density, (const ST*)vox->sh, \
                                              nb, n, vs, w.cnt, w.rect, w.pbox, w.rec_bb, w.slot_vox, w.dkey,          \
                                              w.slot, blocks, w.blk_pairs, w.blk_slots, w.grp_pairs, w.grp_slots,     \
                                              w.counters, pair_capacity, w.k0, w.v0, d_status,         \
@@ -2683,6 +2700,7 @@ namespace {
 // four voxels per thread: one 32-byte store of w_max, 16-byte stores of the
 // depths, one 4-byte store of seen (scalar at a ragged end or misaligned arrays)
 __global__ void k_reset_stats(int64_t n, unsigned long long* wmax, float* z_min, float* delta_min, uint8_t* seen) {
+  grid_begin();
   const float inf = __int_as_float(0x7f800000);
   const int64_t stride = (int64_t)gridDim.x * blockDim.x * 4;
   const bool vec = (((uintptr_t)wmax | (uintptr_t)z_min | (uintptr_t)delta_min) & 15) == 0 &&
@@ -2716,7 +2734,7 @@ extern "C" lv_status lv_reset_stats(int64_t n, unsigned long long* wmax_packed, 
   int64_t blocks = (n / 4 + 255) / 256;
   if (blocks < 1) blocks = 1;
   if (blocks > 4 * 1216) blocks = 4 * 1216;
-  k_reset_stats<<<(unsigned)blocks, 256, 0, (cudaStream_t)stream>>>(n, wmax_packed, z_min, delta_min, seen);
+  launch(k_reset_stats, (unsigned)blocks, 256, 0, (cudaStream_t)stream)(n, wmax_packed, z_min, delta_min, seen);
   count_launch(1);
   return cuda_check(cudaGetLastError(), "lv_reset_stats");
 }
@@ -2735,12 +2753,13 @@ extern "C" lv_status lv_workspace_counters(const void* workspace, size_t ws_byte
 }
 
 static lv_status launch_sh_bwd(const lv_voxels* vox, const ViewSet& vs, const FwdWs& w, float* d_sh, int accumulate,
-                               cudaStream_t s) {
+                               cudaStream_t s, bool chained) {
   const int64_t n = vox->n;
   if (n == 0) return LV_OK;
   const int nb = (vox->sh_degree + 1) * (vox->sh_degree + 1);
   const int blocks = (int)((n + 127) / 128);  // 4 warps x 32 voxels
-  k_sh_bwd<<<blocks, 128, 0, s>>>(w.rec, nb, n, vs, w.cnt, w.slot, w.d_rgb, d_sh, accumulate);
+  auto k = chained ? chain(k_sh_bwd, blocks, 128, 0, s) : launch(k_sh_bwd, blocks, 128, 0, s);
+  k(w.rec, nb, n, vs, w.cnt, w.slot, w.d_rgb, d_sh, accumulate);
   count_launch(1);
   return LV_OK;
 }
@@ -2782,7 +2801,7 @@ extern "C" lv_status lv_rasterize_backward(const lv_voxels* vox, const lv_camera
   if (!accumulate && n > 0) cudaMemsetAsync(d_density, 0, sizeof(float) * 8 * n, s);
   launch_bwd(opts, tiles, s, vs, w, fwd, dL_drgb, dL_ddepth, dL_dT, d_density, lf);
   count_launch(1);
-  if (d_sh) launch_sh_bwd(vox, vs, w, d_sh, accumulate, s);
+  if (d_sh) launch_sh_bwd(vox, vs, w, d_sh, accumulate, s, true);
   return finish(LV_OK, opts->flags, d_status, s, "lv_rasterize_backward");
 }
 
@@ -2798,7 +2817,7 @@ extern "C" lv_status lv_sh_backward(const lv_voxels* vox, const lv_camera* cams,
   make_views(cams, n_views, opts->tile, &vs, &tiles, &pixels);
   FwdWs w = carve_fwd(workspace, vox->n, n_views, tiles, pixels, pair_capacity);
   if (ws_bytes < w.bytes) { set_error("workspace %zu bytes < required %zu", ws_bytes, w.bytes); return LV_ERR_WORKSPACE; }
-  launch_sh_bwd(vox, vs, w, d_sh, accumulate, s);
+  launch_sh_bwd(vox, vs, w, d_sh, accumulate, s, false);
   return cuda_check(cudaGetLastError(), "lv_sh_backward");
 }
 
@@ -2806,7 +2825,7 @@ extern "C" lv_status lv_unpack_wmax(const unsigned long long* packed, int64_t n,
                                     void* stream) {
   if (n < 0 || (n > 0 && (!packed || !w_max))) { set_error("bad arguments"); return LV_ERR_INVALID_ARG; }
   if (n == 0) return LV_OK;
-  k_unpack_wmax<<<(unsigned)((n + 255) / 256), 256, 0, (cudaStream_t)stream>>>(packed, n, w_max, argmax);
+  launch(k_unpack_wmax, (unsigned)((n + 255) / 256), 256, 0, (cudaStream_t)stream)(packed, n, w_max, argmax);
   count_launch(1);
   return cuda_check(cudaGetLastError(), "lv_unpack_wmax");
 }
@@ -2818,7 +2837,7 @@ extern "C" lv_status lv_gather_edge(const int64_t* argmax, int64_t n, const floa
     return LV_ERR_INVALID_ARG;
   }
   if (n == 0) return LV_OK;
-  k_gather_edge<<<(unsigned)((n + 255) / 256), 256, 0, (cudaStream_t)stream>>>(argmax, n, edge_map, n_pix, edge);
+  launch(k_gather_edge, (unsigned)((n + 255) / 256), 256, 0, (cudaStream_t)stream)(argmax, n, edge_map, n_pix, edge);
   count_launch(1);
   return cuda_check(cudaGetLastError(), "lv_gather_edge");
 }
@@ -2836,7 +2855,7 @@ extern "C" lv_status lv_debug_pairs(int64_t n, const lv_camera* cams, int n_view
   if (ws_bytes < w.bytes) { set_error("workspace too small"); return LV_ERR_WORKSPACE; }
   if (keys || voxel) {
     launch_tile_rest(w, vs, tiles, true, s);
-    k_debug_pairs<<<608, 256, 0, s>>>((const uint2*)w.ranges, tiles, w.plist, w.slot_vox, w.s_dkey, keys, voxel);
+    chain(k_debug_pairs, 608, 256, 0, s)((const uint2*)w.ranges, tiles, w.plist, w.slot_vox, w.s_dkey, keys, voxel);
     count_launch(1);
   }
   if (ranges) cudaMemcpyAsync(ranges, w.ranges, sizeof(uint32_t) * 2 * tiles, cudaMemcpyDeviceToDevice, s);
@@ -2861,7 +2880,7 @@ extern "C" lv_status lv_render_pixels_f64(const lv_voxels* vox, const lv_camera*
   const int nb = (vox->sh_degree + 1) * (vox->sh_degree + 1);
   const unsigned grid = (unsigned)((n_px + 127) / 128);
 #define LV_F64(DT, ST)                                                                                            \
-  k_render_f64<DT, ST><<<grid, 128, 0, s>>>(vs, w.ranges, w.plist, w.slot_vox, (const float4*)vox->geom,              \
+  chain(k_render_f64<DT, ST>, grid, 128, 0, s)(vs, w.ranges, w.plist, w.slot_vox, (const float4*)vox->geom,              \
                                             (const DT*)vox->density, (const ST*)vox->sh, nb, pixels, n_px,       \
                                             (double)opts->t_stop, (opts->flags & LV_FLAG_EXACT_SEGMENT) ? 1 : 0,  \
                                             vox->vidx, rgb, T)

@@ -56,6 +56,7 @@ __device__ __forceinline__ void block_add(float v, double* dst) {
 // L_Tc: sum of T (1 - T) and dL/dT = weight (1 - 2T) / |P|
 __global__ void __launch_bounds__(TPB) k_tc(const float* __restrict__ T, int64_t n, float weight, float inv_p,
                                            float* __restrict__ dT, int accumulate, double* acc) {
+  grid_begin();
   float part = 0.f;
   const float gs = weight * inv_p;
   for (int64_t i = blockIdx.x * (int64_t)TPB + threadIdx.x; i < n; i += (int64_t)gridDim.x * TPB) {
@@ -70,6 +71,7 @@ __global__ void __launch_bounds__(TPB) k_tc(const float* __restrict__ T, int64_t
 }
 
 __global__ void k_train_finish(const double* acc, double scale, float* out) {
+  grid_begin();
   if (threadIdx.x == 0) *out = (float)(*acc * scale);
 }
 
@@ -117,6 +119,7 @@ __global__ void __launch_bounds__(TPB) k_adam_density(int64_t n, DT* __restrict_
                                                      const float4* __restrict__ grad, float4* __restrict__ m4,
                                                      float4* __restrict__ v4, const AdamK k, float tv2,
                                                      double* tv_acc) {
+  grid_wait();
   const int lane = threadIdx.x & 31;
   const int64_t total = 2 * n;  // float4 words, two per voxel
   const int64_t stride = (int64_t)gridDim.x * TPB;
@@ -162,6 +165,7 @@ __global__ void __launch_bounds__(TPB) k_adam_density(int64_t n, DT* __restrict_
 template <typename ST>
 __global__ void __launch_bounds__(TPB) k_adam_flat(int64_t n4, ST* __restrict__ p, const float4* __restrict__ grad,
                                                   float4* __restrict__ m4, float4* __restrict__ v4, const AdamK k) {
+  grid_wait();
   for (int64_t i = blockIdx.x * (int64_t)TPB + threadIdx.x; i < n4; i += (int64_t)gridDim.x * TPB) {
     const float4 g = grad[i];
     float4 m = m4[i], v = v4[i];
@@ -183,6 +187,7 @@ template <>
 __global__ void __launch_bounds__(TPB) k_adam_flat<float>(int64_t n4, float* __restrict__ p,
                                                          const float4* __restrict__ grad, float4* __restrict__ m4,
                                                          float4* __restrict__ v4, const AdamK k) {
+  grid_wait();
   float4* p4 = (float4*)p;
   const int64_t stride = (int64_t)gridDim.x * TPB;
   // two independent words per step: more loads in flight
@@ -215,6 +220,7 @@ __global__ void __launch_bounds__(TPB) k_adam_flat<float>(int64_t n4, float* __r
 template <typename ST>
 __global__ void k_adam_tail(int64_t first, int64_t count, ST* __restrict__ p, const float* __restrict__ grad,
                             float* __restrict__ m, float* __restrict__ v, const AdamK k) {
+  grid_wait();
   const int64_t i = first + threadIdx.x;
   if (i < count) {
     float mm = m[i], vv = v[i];
@@ -255,8 +261,8 @@ extern "C" lv_status lv_transmittance_loss(const float* T, int64_t n_pix, float 
   cudaStream_t s = (cudaStream_t)stream;
   cudaMemsetAsync(w.acc, 0, sizeof(double), s);
   if (n_pix > 0)
-    k_tc<<<grid_for(n_pix), TPB, 0, s>>>(T, n_pix, weight, 1.0f / (float)n_pix, dL_dT, accumulate, w.acc);
-  k_train_finish<<<1, 32, 0, s>>>(w.acc, n_pix > 0 ? (double)weight / (double)n_pix : 0.0, loss);
+    launch(k_tc, grid_for(n_pix), TPB, 0, s)(T, n_pix, weight, 1.0f / (float)n_pix, dL_dT, accumulate, w.acc);
+  chain(k_train_finish, 1, 32, 0, s)(w.acc, n_pix > 0 ? (double)weight / (double)n_pix : 0.0, loss);
   count_launch(n_pix > 0 ? 2 : 1);
   return cuda_check(cudaGetLastError(), "lv_transmittance_loss");
 }
@@ -286,26 +292,26 @@ extern "C" lv_status lv_adam_voxels(int64_t n, void* density, lv_dtype density_d
   if (n > 0) {
     const AdamK kd = make_adam(p->lr_density, p);
     if (density_dtype == LV_F32)
-      k_adam_density<float><<<grid_for(2 * n), TPB, 0, s>>>(n, (float*)density, (const float4*)d_density,
+      launch(k_adam_density<float>, grid_for(2 * n), TPB, 0, s)(n, (float*)density, (const float4*)d_density,
                                                         (float4*)m_density, (float4*)v_density, kd, tv2, tv_acc);
     else
-      k_adam_density<__half><<<grid_for(2 * n), TPB, 0, s>>>(n, (__half*)density, (const float4*)d_density,
+      launch(k_adam_density<__half>, grid_for(2 * n), TPB, 0, s)(n, (__half*)density, (const float4*)d_density,
                                                          (float4*)m_density, (float4*)v_density, kd, tv2, tv_acc);
     count_launch(1);
     if (d_sh) {
       const AdamK ks = make_adam(p->lr_sh, p);
       const int64_t n4 = n * 12;
       if (sh_dtype == LV_F32)
-        k_adam_flat<float><<<grid_for(n4), TPB, 0, s>>>(n4, (float*)sh, (const float4*)d_sh, (float4*)m_sh,
+        chain(k_adam_flat<float>, grid_for(n4), TPB, 0, s)(n4, (float*)sh, (const float4*)d_sh, (float4*)m_sh,
                                                         (float4*)v_sh, ks);
       else
-        k_adam_flat<__nv_bfloat16><<<grid_for(n4), TPB, 0, s>>>(n4, (__nv_bfloat16*)sh, (const float4*)d_sh,
+        chain(k_adam_flat<__nv_bfloat16>, grid_for(n4), TPB, 0, s)(n4, (__nv_bfloat16*)sh, (const float4*)d_sh,
                                                                 (float4*)m_sh, (float4*)v_sh, ks);
       count_launch(1);
     }
   }
   if (tv_loss) {
-    k_train_finish<<<1, 32, 0, s>>>(tv_acc, n > 0 ? (double)p->tv_weight / (double)n : 0.0, tv_loss);
+    chain(k_train_finish, 1, 32, 0, s)(tv_acc, n > 0 ? (double)p->tv_weight / (double)n : 0.0, tv_loss);
     count_launch(1);
   }
   return cuda_check(cudaGetLastError(), "lv_adam_voxels");
@@ -325,17 +331,17 @@ extern "C" lv_status lv_adam_array(int64_t count, void* param, lv_dtype dtype, c
   const AdamK k = make_adam(lr, p);
   const int64_t n4 = count / 4, first = 4 * n4;
   if (dtype == LV_F32) {
-    if (n4) k_adam_flat<float><<<grid_for(n4), TPB, 0, s>>>(n4, (float*)param, (const float4*)grad, (float4*)m,
+    if (n4) launch(k_adam_flat<float>, grid_for(n4), TPB, 0, s)(n4, (float*)param, (const float4*)grad, (float4*)m,
                                                            (float4*)v, k);
-    if (first < count) k_adam_tail<float><<<1, 32, 0, s>>>(first, count, (float*)param, grad, m, v, k);
+    if (first < count) chain(k_adam_tail<float>, 1, 32, 0, s)(first, count, (float*)param, grad, m, v, k);
   } else if (dtype == LV_F16) {
-    if (n4) k_adam_flat<__half><<<grid_for(n4), TPB, 0, s>>>(n4, (__half*)param, (const float4*)grad, (float4*)m,
+    if (n4) launch(k_adam_flat<__half>, grid_for(n4), TPB, 0, s)(n4, (__half*)param, (const float4*)grad, (float4*)m,
                                                             (float4*)v, k);
-    if (first < count) k_adam_tail<__half><<<1, 32, 0, s>>>(first, count, (__half*)param, grad, m, v, k);
+    if (first < count) chain(k_adam_tail<__half>, 1, 32, 0, s)(first, count, (__half*)param, grad, m, v, k);
   } else {
-    if (n4) k_adam_flat<__nv_bfloat16><<<grid_for(n4), TPB, 0, s>>>(n4, (__nv_bfloat16*)param, (const float4*)grad,
+    if (n4) launch(k_adam_flat<__nv_bfloat16>, grid_for(n4), TPB, 0, s)(n4, (__nv_bfloat16*)param, (const float4*)grad,
                                                                     (float4*)m, (float4*)v, k);
-    if (first < count) k_adam_tail<__nv_bfloat16><<<1, 32, 0, s>>>(first, count, (__nv_bfloat16*)param, grad, m, v, k);
+    if (first < count) chain(k_adam_tail<__nv_bfloat16>, 1, 32, 0, s)(first, count, (__nv_bfloat16*)param, grad, m, v, k);
   }
   count_launch(2);
   return cuda_check(cudaGetLastError(), "lv_adam_array");

@@ -94,6 +94,7 @@ __global__ void __launch_bounds__(TPB) k_vx_hash(const float4* __restrict__ geom
                                                 unsigned long long* table, int bits, uint32_t* __restrict__ vidx,
                                                 uint64_t* __restrict__ keys, uint32_t* __restrict__ slots,
                                                 unsigned long long* count, uint32_t* bounds, int32_t* status) {
+  grid_begin();
   __shared__ uint32_t s_b[6], s_n;
   __shared__ unsigned long long s_at;
   if (threadIdx.x < 6) s_b[threadIdx.x] = 0u;
@@ -158,6 +159,7 @@ __global__ void __launch_bounds__(TPB) k_vx_hash(const float4* __restrict__ geom
 // bytes, all zero, are plain copies.
 __global__ void __launch_bounds__(TPB) k_vx_pack(uint64_t* __restrict__ keys, const unsigned long long* count,
                                                 const uint32_t* __restrict__ bounds) {
+  grid_begin();
   const int64_t m = (int64_t)*count;
   uint32_t lo[3];
   int sh[3], at = 0;
@@ -179,6 +181,7 @@ __global__ void __launch_bounds__(TPB) k_vx_pack(uint64_t* __restrict__ keys, co
 // a vertex's id is its key's rank
 __global__ void __launch_bounds__(TPB) k_vx_rank(const uint32_t* __restrict__ slots, const unsigned long long* count,
                                                 uint64_t* __restrict__ table, int64_t* __restrict__ n_vert) {
+  grid_begin();
   const int64_t m = (int64_t)*count;
   for (int64_t i = blockIdx.x * (int64_t)TPB + threadIdx.x; i < m; i += (int64_t)gridDim.x * TPB)
     table[slots[i]] = (uint64_t)i;
@@ -188,6 +191,7 @@ __global__ void __launch_bounds__(TPB) k_vx_rank(const uint32_t* __restrict__ sl
 // four corners per thread
 __global__ void __launch_bounds__(TPB) k_vx_assign(const uint64_t* __restrict__ table, int64_t n4,
                                                   uint32_t* __restrict__ vidx) {
+  grid_begin();
   const int64_t i = blockIdx.x * (int64_t)TPB + threadIdx.x;
   if (i >= n4) return;
   uint32_t* p = vidx + 4 * i;
@@ -203,6 +207,7 @@ __global__ void __launch_bounds__(TPB) k_vx_assign(const uint64_t* __restrict__ 
 template <typename DT>
 __global__ void k_vx_gather(const uint32_t* __restrict__ vidx, int64_t m, const DT* __restrict__ vals,
                             float* __restrict__ out) {
+  grid_begin();
   const int64_t i = blockIdx.x * (int64_t)TPB + threadIdx.x;
   if (i < m) out[i] = to_f32(vals[vidx[i]]);
 }
@@ -210,6 +215,7 @@ __global__ void k_vx_gather(const uint32_t* __restrict__ vidx, int64_t m, const 
 // zero rows (voxels the views never reached) cost one 32-byte read and no atomics
 __global__ void k_vx_scatter(const uint32_t* __restrict__ vidx, int64_t n, const float4* __restrict__ corner,
                              float* __restrict__ out, float* __restrict__ count) {
+  grid_begin();
   const int64_t v = blockIdx.x * (int64_t)TPB + threadIdx.x;
   if (v >= n) return;
   const float4 a = corner[2 * v], b = corner[2 * v + 1];
@@ -254,15 +260,15 @@ extern "C" lv_status lv_build_vertex_index(const float* geom, int64_t n, double 
   int32_t* st = d_status ? d_status : w.status;
   zero_async(s, w.table, sizeof(uint64_t) << w.bits, w.counters, sizeof(unsigned long long), w.bounds,
              6 * sizeof(uint32_t), d_status ? nullptr : w.status, sizeof(int32_t));
-  k_vx_hash<<<(unsigned)((m + TPB - 1) / TPB), TPB, 0, s>>>((const float4*)geom, n, 1.0 / unit,
+  chain(k_vx_hash, (unsigned)((m + TPB - 1) / TPB), TPB, 0, s)((const float4*)geom, n, 1.0 / unit,
                                                             (unsigned long long*)w.table, w.bits, vidx, w.k0, w.v0,
                                                             w.counters, w.bounds, st);
   const unsigned grid = (unsigned)std::min<int64_t>((m + TPB - 1) / TPB, 8 * 152);  // the count is on the device
-  k_vx_pack<<<grid, TPB, 0, s>>>(w.k0, w.counters, w.bounds);
+  chain(k_vx_pack, grid, TPB, 0, s)(w.k0, w.counters, w.bounds);
   const int which = radix_sort_pairs(w.k0, w.v0, w.k0, w.v0, w.k1, w.v1, w.sort_tmp, w.counters, m,
                                      3 * COORD_BITS, st, s);
-  k_vx_rank<<<grid, TPB, 0, s>>>(which ? w.v1 : w.v0, w.counters, w.table, d_n_vert);
-  k_vx_assign<<<(unsigned)((m / 4 + TPB - 1) / TPB), TPB, 0, s>>>(w.table, m / 4, vidx);
+  chain(k_vx_rank, grid, TPB, 0, s)(which ? w.v1 : w.v0, w.counters, w.table, d_n_vert);
+  chain(k_vx_assign, (unsigned)((m / 4 + TPB - 1) / TPB), TPB, 0, s)(w.table, m / 4, vidx);
   count_launch(4);
   return cuda_check(cudaGetLastError(), "lv_build_vertex_index");
 }
@@ -275,8 +281,8 @@ extern "C" lv_status lv_vertex_gather(const uint32_t* vidx, int64_t n, const voi
   const int64_t m = 8 * n;
   const unsigned blocks = (unsigned)((m + TPB - 1) / TPB);
   cudaStream_t s = (cudaStream_t)stream;
-  if (dtype == LV_F32) k_vx_gather<float><<<blocks, TPB, 0, s>>>(vidx, m, (const float*)vertex_values, corners);
-  else k_vx_gather<__half><<<blocks, TPB, 0, s>>>(vidx, m, (const __half*)vertex_values, corners);
+  if (dtype == LV_F32) launch(k_vx_gather<float>, blocks, TPB, 0, s)(vidx, m, (const float*)vertex_values, corners);
+  else launch(k_vx_gather<__half>, blocks, TPB, 0, s)(vidx, m, (const __half*)vertex_values, corners);
   count_launch(1);
   return cuda_check(cudaGetLastError(), "lv_vertex_gather");
 }
@@ -286,7 +292,7 @@ extern "C" lv_status lv_vertex_scatter_add(const uint32_t* vidx, int64_t n, cons
   if (n < 0 || (n > 0 && (!vidx || !corners || !vertex_sum))) { set_error("bad arguments"); return LV_ERR_INVALID_ARG; }
   if (!aligned16(vidx) || !aligned16(corners)) { set_error("vidx and corners must be 16-byte aligned"); return LV_ERR_INVALID_ARG; }
   if (n == 0) return LV_OK;
-  k_vx_scatter<<<(unsigned)((n + TPB - 1) / TPB), TPB, 0, (cudaStream_t)stream>>>(
+  launch(k_vx_scatter, (unsigned)((n + TPB - 1) / TPB), TPB, 0, (cudaStream_t)stream)(
       vidx, n, (const float4*)corners, vertex_sum, vertex_count);
   count_launch(1);
   return cuda_check(cudaGetLastError(), "lv_vertex_scatter_add");
