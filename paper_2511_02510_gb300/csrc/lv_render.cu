@@ -355,9 +355,9 @@ __device__ __forceinline__ uint32_t bin_item(const DevView& c, int ts, const flo
 // totals, from which k_block_offsets and k_emit place the items: per-item
 // offsets, scanned by three more launches, cost 28 bytes of traffic an item
 // (48M items: 290 us), and only visible items write anything but their count
-// (48M items: 854 -> 634 us with that, the geometry read once and the usual case's
-// projections without a test per corner; 2M items: 39 -> 32 us).
-__global__ void __launch_bounds__(BIN_THREADS) k_bin(const float4* __restrict__ geom, int64_t n, int64_t blocks,
+// (48M items: 854 -> 607 us with that, the geometry read once, the usual case's
+// projections without a test per corner and six blocks an SM; 2M items: 39 -> 31 us).
+__global__ void __launch_bounds__(BIN_THREADS, 6) k_bin(const float4* __restrict__ geom, int64_t n, int64_t blocks,
                                                      const __grid_constant__ ViewSet vs, uint32_t* __restrict__ cnt,
                                                      uint2* __restrict__ rect, uint2* __restrict__ pbox,
                                                      uint32_t* __restrict__ dkey,
@@ -367,11 +367,15 @@ __global__ void __launch_bounds__(BIN_THREADS) k_bin(const float4* __restrict__ 
   grid_begin();
   __shared__ unsigned long long s_pairs[BIN_THREADS / 32];
   __shared__ uint32_t s_slots[BIN_THREADS / 32];
-  // the later kernels' counters are cleared here, not by a launch of their own (whole 32-bit words)
-#pragma unroll
-  for (int k = 0; k < 4; ++k)
-    for (size_t x = blockIdx.x * (size_t)BIN_THREADS + threadIdx.x; x < zr.bytes[k] / 4; x += (size_t)gridDim.x * BIN_THREADS)
-      ((uint32_t*)zr.p[k])[x] = 0u;
+  // the later kernels' counters are cleared by the first blocks, not by a launch of their own (about
+  // 2100 32-bit words)
+  constexpr unsigned ZERO_BLOCKS = 8;
+  if (blockIdx.x < ZERO_BLOCKS) {
+    const size_t stride = (size_t)min(gridDim.x, ZERO_BLOCKS) * BIN_THREADS;
+    for (int k = 0; k < 4; ++k)
+      for (size_t x = blockIdx.x * (size_t)BIN_THREADS + threadIdx.x; x < zr.bytes[k] / 4; x += stride)
+        ((uint32_t*)zr.p[k])[x] = 0u;
+  }
   const int view = (int)(blockIdx.x % (unsigned)vs.n);
   const int64_t vb = blockIdx.x / (unsigned)vs.n, vox = vb * BIN_THREADS + threadIdx.x;
   const int64_t i = (int64_t)view * n + vox;  // items are view-major
@@ -517,50 +521,75 @@ __device__ __forceinline__ void ld_row32(const void* p, uint32_t* w) {
       : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7])
       : "l"(p));
 }
+__device__ __forceinline__ void st_row32(void* p, float4 a, float4 b) {  // p: 32-byte aligned
+  asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(a.x), "f"(a.y), "f"(a.z),
+               "f"(a.w), "f"(b.x), "f"(b.y), "f"(b.z), "f"(b.w)
+               : "memory");
+}
 __device__ __forceinline__ bool aligned32(const void* p) { return ((uintptr_t)p & 31) == 0; }
 __device__ __forceinline__ void bf16_pair(uint32_t w, float* c) {
   c[0] = __uint_as_float(w << 16);
   c[1] = __uint_as_float(w & 0xffff0000u);
 }
 
-// one voxel's 48 SH coefficients into registers (rows are 16-byte aligned)
-__device__ __forceinline__ void load_sh_row(const float* __restrict__ row, float* c) {
-  if (aligned32(row)) {
+// c = max(0, raw) with raw = sum_j coef[j] Y_j + 0.5 per channel, from a voxel's row of 48 coefficients
+// ([j][rgb], 16-byte aligned).  The row is read 32 bytes at a time, each word used before the next is
+// asked for, and only as far as the degree needs, to keep k_emit's registers few: it is bound by the
+// latency of its scattered reads and writes, so warps in flight count for more than loads in flight per
+// warp.  Eight views of 6M voxels, FP16 and BF16: 1474 us at 5 blocks an SM, 1362 at 6, 1271 at 8 (32
+// registers), 1100 with the records stored in whole sectors; one view of 2M, FP32: 97, 91, 97 us, and 86.
+template <int PER, typename F>
+__device__ __forceinline__ void sh_add(int k, const F (&c)[PER], int nb, const float* Y, float* raw) {
 #pragma unroll
-    for (int k = 0; k < 6; ++k) {
-      uint32_t w[8];
-      ld_row32(row + 8 * k, w);
-#pragma unroll
-      for (int h = 0; h < 8; ++h) c[8 * k + h] = __uint_as_float(w[h]);
-    }
-    return;
-  }
-  const float4* v = (const float4*)row;
-#pragma unroll
-  for (int k = 0; k < 12; ++k) {
-    const float4 q = __ldg(v + k);
-    c[4 * k] = q.x; c[4 * k + 1] = q.y; c[4 * k + 2] = q.z; c[4 * k + 3] = q.w;
+  for (int h = 0; h < PER; ++h) {
+    const int i = PER * k + h, j = i / 3;
+    if (j < nb) raw[i % 3] = fmaf(c[h], Y[j], raw[i % 3]);
   }
 }
-__device__ __forceinline__ void load_sh_row(const __nv_bfloat16* __restrict__ row, float* c) {
-  if (aligned32(row)) {
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      uint32_t w[8];
-      ld_row32(row + 16 * k, w);
-#pragma unroll
-      for (int h = 0; h < 8; ++h) bf16_pair(w[h], c + 16 * k + 2 * h);
-    }
-    return;
-  }
-  const uint4* v = (const uint4*)row;
+__device__ __forceinline__ void sh_raw_row(const float* __restrict__ row, int nb, const float* dir, float* raw) {
+  float Y[16];
+  sh_basis(dir[0], dir[1], dir[2], Y);
+  raw[0] = raw[1] = raw[2] = 0.f;
+  const bool wide = aligned32(row);
 #pragma unroll
   for (int k = 0; k < 6; ++k) {
-    const uint4 q = __ldg(v + k);
-    const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+    if (8 * k < 3 * nb) {  // grid-uniform
+      float c[8];
+      if (wide) {
+        uint32_t w[8];
+        ld_row32(row + 8 * k, w);
 #pragma unroll
-    for (int h = 0; h < 4; ++h) bf16_pair(w[h], c + 8 * k + 2 * h);
+        for (int h = 0; h < 8; ++h) c[h] = __uint_as_float(w[h]);
+      } else {
+        const float4 a = __ldg((const float4*)row + 2 * k), b = __ldg((const float4*)row + 2 * k + 1);
+        c[0] = a.x; c[1] = a.y; c[2] = a.z; c[3] = a.w;
+        c[4] = b.x; c[5] = b.y; c[6] = b.z; c[7] = b.w;
+      }
+      sh_add<8>(k, c, nb, Y, raw);
+    }
   }
+#pragma unroll
+  for (int k = 0; k < 3; ++k) raw[k] += 0.5f;
+}
+__device__ __forceinline__ void sh_raw_row(const __nv_bfloat16* __restrict__ row, int nb, const float* dir,
+                                           float* raw) {
+  float Y[16];
+  sh_basis(dir[0], dir[1], dir[2], Y);
+  raw[0] = raw[1] = raw[2] = 0.f;
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    if (8 * k < 3 * nb) {  // grid-uniform
+      const uint4 q = __ldg((const uint4*)row + k);
+      float c[8];
+      bf16_pair(q.x, c);
+      bf16_pair(q.y, c + 2);
+      bf16_pair(q.z, c + 4);
+      bf16_pair(q.w, c + 6);
+      sh_add<8>(k, c, nb, Y, raw);
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < 3; ++k) raw[k] += 0.5f;
 }
 
 // one voxel's 8 corner densities (any alignment)
@@ -591,22 +620,6 @@ __device__ __forceinline__ void load_corners(const __half* __restrict__ row, flo
   }
 }
 
-// c = max(0, raw) with raw = sum_j coef[j] Y_j + 0.5 per channel; coef laid out [j][rgb] with stride cs
-__device__ __forceinline__ void sh_raw(const float* coef, int cs, int nb, const float* Y, float* raw) {
-  float r = 0.f, g = 0.f, b = 0.f;
-#pragma unroll
-  for (int j = 0; j < 16; ++j) {
-    if (j < nb) {
-      r = fmaf(coef[(3 * j + 0) * cs], Y[j], r);
-      g = fmaf(coef[(3 * j + 1) * cs], Y[j], g);
-      b = fmaf(coef[(3 * j + 2) * cs], Y[j], b);
-    }
-  }
-  raw[0] = r + 0.5f;
-  raw[1] = g + 0.5f;
-  raw[2] = b + 0.5f;
-}
-
 __device__ __forceinline__ void unit_dir(float rx, float ry, float rz, float* d) {
   float nn = rx * rx + ry * ry + rz * rz;
   if (nn > 0.f) {
@@ -629,7 +642,7 @@ __device__ __forceinline__ void unit_dir(float rx, float ry, float rz, float* d)
 // and h | 8 corner densities | clamped SH colour and 1/(2h)), the slot's order
 // key, and the colour-gradient scratch (cleared; w = clamp mask).
 template <typename DT, typename ST>
-__global__ void __launch_bounds__(256) k_emit(const float4* __restrict__ geom, const DT* __restrict__ dens,
+__global__ void __launch_bounds__(BIN_THREADS, sizeof(ST) == 4 ? 6 : 8) k_emit(const float4* __restrict__ geom, const DT* __restrict__ dens,
                                               const ST* __restrict__ sh, int sh_nb, int64_t n,
                                               const __grid_constant__ ViewSet vs, const uint32_t* __restrict__ cnt,
                                               const uint2* __restrict__ rect,
@@ -687,20 +700,30 @@ __global__ void __launch_bounds__(256) k_emit(const float4* __restrict__ geom, c
   }
   uint32_t sl = blk_slots[blk];
   unsigned long long p_block = blk_pairs[blk];
+  // the groups before this block's: summed by the first warp (none up to 1M items)
+  __shared__ unsigned long long s_gp;
+  __shared__ uint32_t s_gs;
   const int64_t grp = blk / BO_GROUP;
-  if (grp) {  // grid-uniform within a group: every warp sums the groups before
+  if (warp == 0) {
     unsigned long long a = 0;
     uint32_t b = 0;
     for (int64_t g = lane; g < grp; g += 32) {
       a += grp_pairs[g];
       b += grp_slots[g];
     }
+    if (grp) {  // block-uniform
 #pragma unroll
-    for (int o = 16; o; o >>= 1) a += __shfl_xor_sync(FULL, a, o);
-    p_block += a;
-    sl += __reduce_add_sync(FULL, b);
+      for (int o = 16; o; o >>= 1) a += __shfl_xor_sync(FULL, a, o);
+      b = __reduce_add_sync(FULL, b);
+    }
+    if (lane == 0) {
+      s_gp = a;
+      s_gs = b;
+    }
   }
   __syncthreads();
+  p_block += s_gp;
+  sl += s_gs;
   uint32_t wp = 0;
 #pragma unroll
   for (int w = 0; w < 8; ++w) {
@@ -756,12 +779,8 @@ __global__ void __launch_bounds__(256) k_emit(const float4* __restrict__ geom, c
   const float rx = g.x - c.o[0], ry = g.y - c.o[1], rz = g.z - c.o[2];
   float dir[3];
   unit_dir(rx, ry, rz, dir);
-  float Y[16];
-  sh_basis(dir[0], dir[1], dir[2], Y);
-  float coef[48];
-  load_sh_row(sh + 48 * vox, coef);
   float raw[3];
-  sh_raw(coef, 1, sh_nb, Y, raw);
+  sh_raw_row(sh + 48 * vox, sh_nb, dir, raw);
   float d[8];
   if (vidx) {  // shared grid-vertex densities
     const uint4 i0 = *(const uint4*)(vidx + 8 * vox), i1 = *(const uint4*)(vidx + 8 * vox + 4);
@@ -771,10 +790,10 @@ __global__ void __launch_bounds__(256) k_emit(const float4* __restrict__ geom, c
     load_corners(dens + 8 * vox, d);
   }
   float4* r = rec + 4 * (int64_t)s;
-  r[0] = make_float4(rx, ry, rz, g.w);
-  r[1] = make_float4(d[0], d[1], d[2], d[3]);
-  r[2] = make_float4(d[4], d[5], d[6], d[7]);
-  r[3] = make_float4(fmaxf(raw[0], 0.f), fmaxf(raw[1], 0.f), fmaxf(raw[2], 0.f), __fdiv_rn(0.5f, g.w));
+  // whole sectors: a lane's rows are 64 bytes apart, and 16-byte stores would write each sector twice
+  st_row32(r, make_float4(rx, ry, rz, g.w), make_float4(d[0], d[1], d[2], d[3]));
+  st_row32(r + 2, make_float4(d[4], d[5], d[6], d[7]),
+           make_float4(fmaxf(raw[0], 0.f), fmaxf(raw[1], 0.f), fmaxf(raw[2], 0.f), __fdiv_rn(0.5f, g.w)));
   slot_vox[s] = (uint32_t)vox;
   // colour-gradient scratch: xyz cleared, w = which channels passed the clamp
   // (bit c set when raw_c > 0) as a small exact float, read by the SH backward
@@ -807,20 +826,20 @@ __device__ __forceinline__ int64_t usable_pairs(const unsigned long long* d_coun
 //   k_tile_sort       persistent blocks of 512 threads: lists of up to TS_CHUNK
 //                     pairs in one go, longer ones range of keys by range of
 //                     keys, and of those above TS_LAZY only the front, the
-//                     TS_FRONT to TS_CHUNK nearest pairs;
+//                     nearest pairs up to TS_CHUNK;
 //   k_tile_rest       the rest of those whose pixels are still open after the
 //                     composite of the sorted parts.
 // Opaque scenes seldom read a long list past its front: of eight 980 x 545
-// views of 6M voxels with tile 32 (lists of up to 68,000 pairs, 38M in all) 2-5 %
-// of the tiles do.  Sorting every list whole, in chunks merged afterwards, took
-// 4.7 ms of those views' 8.2 ms.  Lists of a few chunks are sorted whole: where
+// views of 6M voxels with tile 32 (lists of up to 68,000 pairs, 38M in all) hardly
+// a tile does (with fronts of 2048 pairs 2 to 5 % of them, and 480 us for the rest
+// and the resumed composite).  Sorting every list whole, in chunks merged
+// afterwards, took 4.7 ms of those views' 8.2 ms; their fronts take 0.41 ms.  Lists of a few chunks are sorted whole: where
 // their pixels stay open, the composite in two launches costs more than the sort
 // saves (one 1237 x 822 view of 2M voxels, lists of up to 7,800 pairs: 217 + 151 us
 // against 297 us).  Scenes of up to TS_LAZY_VOXELS seldom have longer lists, and go
 // without the two launches that the rest takes (6 us when there is none).
 constexpr int TS_BITS = 9, TS_BINS = 1 << TS_BITS;
 constexpr int TS_THREADS = 512, TS_WARPS = TS_THREADS / 32, TS_ITEMS = 8, TS_CHUNK = TS_THREADS * TS_ITEMS;
-constexpr int TS_FRONT = 2048;                      // pairs of a long list sorted at first (at least, if its keys allow)
 constexpr uint32_t TS_LAZY = 4 * TS_CHUNK;          // lists up to here are sorted whole at once
 constexpr int64_t TS_LAZY_VOXELS = 1 << 19;         // and all lists of scenes up to here
 constexpr int TL_BITS = 11, TL_BINS = 1 << TL_BITS;  // key histogram of a long list
@@ -1272,8 +1291,8 @@ __device__ __forceinline__ void tl_collect(TileSortSmem& S, const uint32_t* __re
 // collected in item order and sorted in shared memory.  A bin of more than
 // TS_CHUNK entries is cut by a finer histogram of its own keys; once a bin is one
 // key, item order is the order.  START: the keys are gathered first (to xk), and above
-// `lazy` entries the work stops after one range, of TS_FRONT entries or more where the
-// bins allow it; else it goes on from the progress of such a start.
+// `lazy` entries the work stops after one range; else it goes on from the progress of
+// such a start.
 template <bool START>
 __device__ __noinline__ void tl_order(uint32_t lo, uint32_t L, uint32_t lazy, const uint32_t* __restrict__ sv_all,
                          uint32_t* xk_all, const uint32_t* __restrict__ s_dkey, TileProg* prog,
@@ -1348,18 +1367,15 @@ __device__ __noinline__ void tl_order(uint32_t lo, uint32_t L, uint32_t lazy, co
     bool finer = false;
     while (cum < total) {  // block-uniform
       if (t == 0) {
-        // bins [b0, b1): as many as fit (b1 == b0: bin b0 alone does not), and for the front no more
-        // than reach TS_FRONT
+        // bins [b0, b1): as many as fit (b1 == b0: bin b0 alone does not)
         auto count_upto = [&](uint32_t limit) {  // bins with inc <= limit
           uint32_t n = 0;
           for (uint32_t step = TL_BINS; step; step >>= 1)
             if (n + step <= (uint32_t)TL_BINS && M.inc[n + step - 1] <= limit) n += step;
           return n;
         };
-        uint32_t b1 = count_upto(cum + TS_CHUNK);
-        if (front) b1 = min(b1, count_upto(cum + TS_FRONT - 1) + 1u);
         M.b0 = count_upto(cum);  // past empty bins, so that an oversized bin is met as b0
-        M.b1 = b1;
+        M.b1 = count_upto(cum + TS_CHUNK);
       }
       __syncthreads();
       b0 = M.b0;
