@@ -95,6 +95,35 @@ static void make_views(const lv_camera* cams, int nv, int ts, ViewSet* vs, int64
 }
 
 // ------------------------------------------------------------------ workspace
+// Tiles by list length, longest first: class 0 above 4096 pairs (long), 1 to 4 above 2048, 1024, 512 and
+// 256 (medium), 5 to 7 above 128, 64 and the rest (short).  The depth sort and the composites take them
+// in this order: a long list begun last would keep its warps marching after all others have ended.
+constexpr int TILE_CLASSES = 8, TILE_CLASS_SHORT = 5;
+struct TileOrder {
+  uint32_t* tiles;      // [TILE_CLASSES][stride]
+  unsigned int* count;  // [TILE_CLASSES], 16-byte aligned
+  uint32_t stride;
+  static __device__ __forceinline__ int cls(uint32_t length) {
+    // 12 bits and more: 0 and 1, each bit less a class on, at most 64: 7
+    return length > 4096u ? 0 : (length <= 64u ? 7 : __clz(length - 1u) - 19);
+  }
+  // the i-th tile, and (nullable) its class
+  __device__ __forceinline__ uint32_t tile(uint32_t i, int* c_out = nullptr) const {
+    const uint4 a = *(const uint4*)count, b = *(const uint4*)(count + 4);
+    const uint32_t n[TILE_CLASSES] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+    int c = 0;
+    uint32_t at = i;
+#pragma unroll
+    for (int k = 0; k + 1 < TILE_CLASSES; ++k) {
+      if (c == k && at >= n[k]) {
+        at -= n[k];
+        c = k + 1;
+      }
+    }
+    if (c_out) *c_out = c;
+    return tiles[(size_t)c * stride + at];
+  }
+};
 // progress of a long tile's depth order
 struct TileProg {
   uint32_t done;  // entries sorted
@@ -118,14 +147,11 @@ struct FwdWs {
   uint2* rec_bb;                 // [slots] pixel box of the render record
   uint32_t* slot_vox;            // [slots] voxel id of the render record
   uint32_t* s_dkey;              // [slots] order key
-  unsigned int* work;            // [16] work-item counters: [0..1] the persistent composites, [2] the
-                                 // resumed composite, [3] k_tile_rest, [4..5] count of the medium tiles
-                                 // and k_tile_sort's work counter, [6] count of the long tiles, [7] count
-                                 // of the open tiles, [11] count of the short tiles; [8..10] block arrivals of the persistent forward,
-                                 // backward and resumed composites (sm_leave)
-  uint32_t* mid_tiles;           // [tiles] tiles of medium-length lists
-  uint32_t* long_tiles;          // [tiles] tiles of long lists
-  uint32_t* short_tiles;         // [tiles] the other tiles
+  unsigned int* work;            // [32] work-item counters: [0..1] the persistent composites, [2] the
+                                 // resumed composite, [3] k_tile_rest, [5] k_tile_sort, [7] count of the
+                                 // open tiles; [8..10] block arrivals of the persistent forward, backward
+                                 // and resumed composites (sm_leave); [16..23] tiles per length class
+  uint32_t* class_tiles;         // [TILE_CLASSES][tiles] the tiles of each length class
   uint32_t* open_tiles;          // [tiles] long tiles with pixels open at the end of the sorted part
   uint32_t* ready;               // [tiles] end of the list's depth-sorted part
   TileProg* prog;                // [tiles] progress of the long tiles' depth order
@@ -161,7 +187,7 @@ static FwdWs carve_fwd(void* base, int64_t n, int nv, int64_t tiles, int64_t pix
   int64_t items = n * nv;
   w.counters = c.take<unsigned long long>(8);
   w.status = c.take<int32_t>(4);
-  w.work = c.take<unsigned int>(16);
+  w.work = c.take<unsigned int>(32);
   w.cnt = c.take<uint32_t>(items);
   w.rect = c.take<uint2>(items);
   w.pbox = c.take<uint2>(items);
@@ -177,9 +203,7 @@ static FwdWs carve_fwd(void* base, int64_t n, int nv, int64_t tiles, int64_t pix
   w.rec = c.take<float4>(items * 4);
   w.d_rgb = c.take<float4>(items);
   w.ranges = c.take<uint32_t>(tiles * 2);
-  w.mid_tiles = c.take<uint32_t>(tiles);
-  w.long_tiles = c.take<uint32_t>(tiles);
-  w.short_tiles = c.take<uint32_t>(tiles);
+  w.class_tiles = c.take<uint32_t>(TILE_CLASSES * tiles);
   w.open_tiles = c.take<uint32_t>(tiles);
   w.ready = c.take<uint32_t>(tiles);
   w.prog = c.take<TileProg>(tiles);
@@ -987,12 +1011,7 @@ __global__ void __launch_bounds__(TW_WARPS * 32, 2) k_tile_sort_warp(const uint3
                                                                     const unsigned long long* __restrict__ d_count,
                                                                     int64_t cap, bool ranges_ready, int64_t tiles,
                                                                     uint32_t* __restrict__ ranges,
-                                                                    uint32_t* __restrict__ mid_tiles,
-                                                                    unsigned int* __restrict__ n_mid,
-                                                                    uint32_t* __restrict__ long_tiles,
-                                                                    unsigned int* __restrict__ n_long,
-                                                                    uint32_t* __restrict__ short_tiles,
-                                                                    unsigned int* __restrict__ n_short,
+                                                                    const TileOrder order,
                                                                     uint32_t* __restrict__ ready,
                                                                     TileProg* __restrict__ prog,
                                                                     const __grid_constant__ ViewSet vs,
@@ -1002,31 +1021,28 @@ __global__ void __launch_bounds__(TW_WARPS * 32, 2) k_tile_sort_warp(const uint3
   extern __shared__ __align__(16) unsigned char tw_raw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   WarpSortSmem& W = reinterpret_cast<TileSortWarpSmem*>(tw_raw)->w[warp];
-  __shared__ uint32_t s_cnt[3], s_at[3];
+  __shared__ uint32_t s_cnt[TILE_CLASSES], s_at[TILE_CLASSES];
   const int64_t tile64 = (int64_t)blockIdx.x * TW_WARPS + warp;
   const uint32_t tile = (uint32_t)tile64;
   uint32_t lo = 0, hi = 0, at = 0;
-  int cls = 0;  // 0 short, 1 medium, 2 long
-  if (threadIdx.x < 3) s_cnt[threadIdx.x] = 0u;
+  int cls = 0;
+  if (threadIdx.x < TILE_CLASSES) s_cnt[threadIdx.x] = 0u;
   __syncthreads();
   if (lane == 0 && tile64 < tiles) {
     ts_range(ranges, tile, usable_pairs(d_count, cap), ranges_ready, &lo, &hi);
     reinterpret_cast<uint2*>(ranges)[tile] = make_uint2(lo, hi);
     const uint32_t L = hi - lo;
     ready[tile] = hi;
-    cls = L > (uint32_t)TS_CHUNK ? 2 : (L > (uint32_t)TW_MAX ? 1 : 0);
-    if (cls == 2) prog[tile].open = 0u;
+    cls = TileOrder::cls(L);
+    if (cls == 0) prog[tile].open = 0u;
     at = atomicAdd(&s_cnt[cls], 1u);
   }
   __syncthreads();
-  // the tiles by length class, for the longer lists' sorts and the composites' order of work
-  if (threadIdx.x < 3) {
-    unsigned int* n_cls = threadIdx.x == 0 ? n_short : (threadIdx.x == 1 ? n_mid : n_long);
-    s_at[threadIdx.x] = s_cnt[threadIdx.x] ? atomicAdd(n_cls, s_cnt[threadIdx.x]) : 0u;
-  }
+  if (threadIdx.x < TILE_CLASSES)
+    s_at[threadIdx.x] = s_cnt[threadIdx.x] ? atomicAdd(&order.count[threadIdx.x], s_cnt[threadIdx.x]) : 0u;
   __syncthreads();
   if (tile64 >= tiles) return;  // warp-uniform; no block-wide barrier below
-  if (lane == 0) (cls == 0 ? short_tiles : (cls == 1 ? mid_tiles : long_tiles))[s_at[cls] + at] = tile;
+  if (lane == 0) order.tiles[(size_t)cls * order.stride + s_at[cls] + at] = tile;
   lo = __shfl_sync(FULL, lo, 0);
   const int L = (int)(__shfl_sync(FULL, hi, 0) - lo);
   if (L < 1 || L > TW_MAX) return;  // warp-uniform
@@ -1435,16 +1451,12 @@ __device__ __noinline__ void tl_order(uint32_t lo, uint32_t L, uint32_t lazy, co
   }
 }
 
-// Persistent blocks over the long tiles (their fronts; first, as they take
-// longest), then over the medium tiles.
+// Persistent blocks over the long tiles, then over the medium ones.
 __global__ void __launch_bounds__(TS_THREADS, 2) k_tile_sort(const uint32_t* __restrict__ tvals,
                                                             uint32_t* xk,
                                                             const uint32_t* __restrict__ s_dkey,
                                                             const uint32_t* __restrict__ ranges,
-                                                            const uint32_t* __restrict__ mid_tiles,
-                                                            const unsigned int* __restrict__ n_mid,
-                                                            const uint32_t* __restrict__ long_tiles,
-                                                            const unsigned int* __restrict__ n_long,
+                                                            const TileOrder order,
                                                             unsigned int* __restrict__ work,
                                                             uint32_t* ready, TileProg* prog, uint32_t lazy,
                                                             const __grid_constant__ ViewSet vs,
@@ -1452,17 +1464,21 @@ __global__ void __launch_bounds__(TS_THREADS, 2) k_tile_sort(const uint32_t* __r
                                                             uint2* __restrict__ plist) {
   grid_begin();
   TileLongSmem& M = ts_smem();
-  const unsigned int nl = *n_long, total = nl + *n_mid;
+  static_assert(TILE_CLASS_SHORT == 5 && TS_CHUNK == 4096 && TW_MAX == 256, "the length classes");
+  unsigned int total = 0;
+#pragma unroll
+  for (int c = 0; c < TILE_CLASS_SHORT; ++c) total += order.count[c];
   while (true) {
     if (threadIdx.x == 0) M.s.item = atomicAdd(work, 1u);
     __syncthreads();
     const unsigned int item = M.s.item;
     __syncthreads();  // everyone has read the item before it is overwritten
     if (item >= total) return;  // block-uniform
-    const uint32_t tile = item < nl ? long_tiles[item] : mid_tiles[item - nl];
+    int cls;
+    const uint32_t tile = order.tile(item, &cls);
     const uint2 r = reinterpret_cast<const uint2*>(ranges)[tile];
     const TileBox tb(vs, tile);
-    if (item < nl)
+    if (cls == 0)
       tl_order<true>(r.x, r.y - r.x, lazy, tvals, xk, s_dkey, prog + tile, ready + tile, tb, rec_bb, plist);
     else
       ts_sort_list(tvals + r.x, s_dkey, (int)(r.y - r.x), tb, rec_bb, plist + r.x);
@@ -1589,18 +1605,6 @@ __device__ __forceinline__ float one_minus_exp(float x, float e) {
   p *= x;
   return x < 0.125f ? p : 1.f - e;
 }
-
-// The composites take the tiles by length class, long lists first: a long list
-// begun last would keep its warps marching after all others have ended.
-struct TileOrder {
-  const uint32_t *long_tiles, *mid_tiles, *short_tiles;
-  const unsigned int *n_long, *n_mid;
-  __device__ __forceinline__ int tile(uint32_t i) const {
-    const uint32_t nl = *n_long, nm = *n_mid;
-    if (nl + nm == 0u) return (int)i;  // short lists only: any order does, without one more load
-    return (int)(i < nl ? long_tiles[i] : (i < nl + nm ? mid_tiles[i - nl] : short_tiles[i - nl - nm]));
-  }
-};
 
 __device__ __forceinline__ int find_view(const ViewSet& vs, int gtile) {
   int v = 0;
@@ -1824,11 +1828,21 @@ struct Front {
   bool resume;
 };
 
-template <int TS>
-constexpr int min_blocks() { return TS == 16 ? 4 : (TS == 8 ? 16 : 1); }
+// A strip's march needs no other warp, so a block is a few warps whatever the
+// tile size, few where each warp has one item (a block's place is free once its
+// last warp ends), and as many blocks share an SM as leave a thread the 72
+// (forward) to 80 registers below which the march spills: the composites are
+// bound by instruction issue, for which 24 to 28 warps are enough.  1237 x 822
+// view of 2M voxels with long open lists, tile 16, forward + backward: 493 + 480 us
+// at 48 registers, 286 + 330 at 64 (8 warps a block), 261 + 310 at 80, 320 + 335 at
+// 128; fog view of 979 x 545 79 + 130 at 8 warps a block, 75 + 125 at 4.
+template <int TS, bool PERSIST>
+__host__ __device__ constexpr int comp_warps() { return PERSIST ? 8 : (TS == 8 ? 1 : 4); }
+template <int TS, bool PERSIST>
+__host__ __device__ constexpr int comp_blocks(int warps_sm) { return warps_sm / comp_warps<TS, PERSIST>(); }
 
 template <int TS, bool SEG, bool PERSIST>
-__global__ void __launch_bounds__(TS* TS, min_blocks<TS>()) k_fwd(const __grid_constant__ ViewSet vs, const uint32_t* __restrict__ ranges,
+__global__ void __launch_bounds__(comp_warps<TS, PERSIST>() * 32, comp_blocks<TS, PERSIST>(28)) k_fwd(const __grid_constant__ ViewSet vs, const uint32_t* __restrict__ ranges,
                                                 const uint2* __restrict__ plist, const float4* __restrict__ rec,
                                                 const uint32_t* __restrict__ slot_vox, float t_stop,
                                                 float* __restrict__ rgb, float* __restrict__ depth,
@@ -1838,7 +1852,7 @@ __global__ void __launch_bounds__(TS* TS, min_blocks<TS>()) k_fwd(const __grid_c
                                                 uint32_t n_items, int sm_cut, int n_sms, unsigned int* arrivals,
                                                 const TileOrder order, const Front fr) {
   grid_wait();
-  constexpr int NW = TS * TS / 32;
+  constexpr int NW = TS * TS / 32, CW = comp_warps<TS, PERSIST>();
   extern __shared__ float4 smem_f4[];
   if (PERSIST && sm_leave(sm_cut, n_sms, arrivals)) return;  // block-uniform
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -1854,9 +1868,9 @@ __global__ void __launch_bounds__(TS* TS, min_blocks<TS>()) k_fwd(const __grid_c
   walk.s_rec = (float4*)((char*)smem_f4 + WARP_SLICE * warp);
   walk.s_vox = (uint32_t*)(walk.s_rec + 2 * 32 * 4);
   walk.s_q = (uint2*)(walk.s_vox + 2 * 32);
-  for (uint32_t item = PERSIST ? next_item(work, lane) : blockIdx.x * NW + warp; item < n_items;
+  for (uint32_t item = PERSIST ? next_item(work, lane) : blockIdx.x * CW + warp; item < n_items;
        item = PERSIST ? next_item(work, lane) : n_items) {  // warp-uniform
-    const int gtile = PERSIST && fr.resume ? (int)fr.open_tiles[item / NW] : order.tile(item / NW);
+    const int gtile = PERSIST && fr.resume ? (int)fr.open_tiles[item / NW] : (int)order.tile(item / NW);
     const int view = find_view(vs, gtile);
     const DevView& c = vs.v[view];
     const uint32_t start = ranges[2 * gtile], end = fr.ready[gtile];
@@ -2011,7 +2025,7 @@ __device__ __forceinline__ float warp_reduce16(float* v, int lane) {
 // per-record gradients (8 corners + colour) are
 // reduced over the warp and sent with three 16-byte global reductions.
 template <int TS, bool SEG, bool PERSIST>
-__global__ void __launch_bounds__(TS* TS, min_blocks<TS>()) k_bwd(const __grid_constant__ ViewSet vs, const uint32_t* __restrict__ ranges,
+__global__ void __launch_bounds__(comp_warps<TS, PERSIST>() * 32, comp_blocks<TS, PERSIST>(24)) k_bwd(const __grid_constant__ ViewSet vs, const uint32_t* __restrict__ ranges,
                                                 const uint2* __restrict__ plist, const float4* __restrict__ rec,
                                                 const uint32_t* __restrict__ slot_vox, const float* __restrict__ T_fwd,
                                                 const float* __restrict__ tau_in,
@@ -2022,9 +2036,9 @@ __global__ void __launch_bounds__(TS* TS, min_blocks<TS>()) k_bwd(const __grid_c
                                                 int sm_cut, int n_sms, unsigned int* arrivals, const TileOrder order,
                                                 const LfFuse lf) {
   grid_wait();
-  constexpr int NW = TS * TS / 32;
+  constexpr int NW = TS * TS / 32, CW = comp_warps<TS, PERSIST>();
   extern __shared__ float4 smem_f4[];
-  __shared__ double s_lf[NW][LV_MAX_VIEWS];  // each warp's loss sums (fused LF loss; no atomics)
+  __shared__ double s_lf[CW][LV_MAX_VIEWS];  // each warp's loss sums (fused LF loss; no atomics)
   __shared__ float s_mean[LV_MAX_VIEWS], s_gscale[LV_MAX_VIEWS];  // the fused LF loss's per-view constants
   if (PERSIST && sm_leave(sm_cut, n_sms, arrivals)) return;  // block-uniform
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -2032,7 +2046,7 @@ __global__ void __launch_bounds__(TS* TS, min_blocks<TS>()) k_bwd(const __grid_c
     for (int v = lane; v < vs.n; v += 32) s_lf[warp][v] = 0.0;
     // each view's mean weight and gradient scale, rounded from FP64 as the loss kernel rounds them,
     // once per block (FP64 division is slow on this part)
-    for (int v = tid; v < vs.n; v += TS * TS) {
+    for (int v = tid; v < vs.n; v += CW * 32) {
       const double np = (double)vs.v[v].W * (double)vs.v[v].H;
       s_mean[v] = (float)(lf.wsum[v] / np);
       s_gscale[v] = (float)(2.0 / (3.0 * np));
@@ -2047,9 +2061,9 @@ __global__ void __launch_bounds__(TS* TS, min_blocks<TS>()) k_bwd(const __grid_c
   walk.s_rec = (float4*)((char*)smem_f4 + WARP_SLICE * warp);
   walk.s_vox = (uint32_t*)(walk.s_rec + 2 * 32 * 4);
   walk.s_q = (uint2*)(walk.s_vox + 2 * 32);
-  for (uint32_t item = PERSIST ? next_item(work, lane) : blockIdx.x * NW + warp; item < n_items;
+  for (uint32_t item = PERSIST ? next_item(work, lane) : blockIdx.x * CW + warp; item < n_items;
        item = PERSIST ? next_item(work, lane) : n_items) {  // warp-uniform
-    const int gtile = order.tile(item / NW);
+    const int gtile = (int)order.tile(item / NW);
     const int view = find_view(vs, gtile);
     const DevView& c = vs.v[view];
     const int lt = gtile - c.tile_off;
@@ -2189,9 +2203,9 @@ __global__ void __launch_bounds__(TS* TS, min_blocks<TS>()) k_bwd(const __grid_c
   }
   if (lf.w) {
     __syncthreads();
-    for (int v = tid; v < vs.n; v += TS * TS) {
+    for (int v = tid; v < vs.n; v += CW * 32) {
       double t = 0.0;
-      for (int w = 0; w < NW; ++w) t += s_lf[w][v];
+      for (int w = 0; w < CW; ++w) t += s_lf[w][v];
       if (t != 0.0) atomicAdd(&lf.lsum[v], t);
     }
   }
@@ -2484,8 +2498,9 @@ static void sm_limits(int sm_limit, int dev, int* sms, int* sm_cut) {
   *sm_cut = (sm_limit > 0 && *sms > 0 && sm_limit < *sms) ? sm_limit : 0;
 }
 
-static TileOrder tile_order(const FwdWs& w) {
-  return {w.long_tiles, w.mid_tiles, w.short_tiles, w.work + 6, w.work + 4};
+
+static TileOrder tile_order(const FwdWs& w, int64_t tiles) {
+  return {w.class_tiles, w.work + 16, (uint32_t)tiles};
 }
 
 // resume: the second launch, over the open tiles (its grid is persistent whatever the schedule: only the
@@ -2493,54 +2508,56 @@ static TileOrder tile_order(const FwdWs& w) {
 template <int TS, bool SEG, bool PERSIST>
 static void launch_fwd_t(int64_t tiles, cudaStream_t s, const ViewSet& vs, const FwdWs& w, float t_stop,
                          const lv_fwd_out* out, int sm_limit, bool resume) {
-  const size_t smem = WARP_SLICE * (TS * TS / 32);
+  constexpr int CW = comp_warps<TS, PERSIST>();
+  const size_t smem = WARP_SLICE * CW;
   static int pblocks[64];  // per device
   static std::atomic<unsigned long long> done{0};
   const int dev = current_device();
   once_per_device(done, [&] {
     cudaFuncSetAttribute(k_fwd<TS, SEG, PERSIST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (PERSIST && dev < 64) pblocks[dev] = persistent_blocks(k_fwd<TS, SEG, PERSIST>, TS * TS, smem);
+    if (PERSIST && dev < 64) pblocks[dev] = persistent_blocks(k_fwd<TS, SEG, PERSIST>, CW * 32, smem);
   });
-  const int pb = dev < 64 ? pblocks[dev] : persistent_blocks(k_fwd<TS, SEG, PERSIST>, TS * TS, smem);
+  const int pb = dev < 64 ? pblocks[dev] : persistent_blocks(k_fwd<TS, SEG, PERSIST>, CW * 32, smem);
   int sms = 0, sm_cut = 0;
   sm_limits(sm_limit, dev, &sms, &sm_cut);
   const uint32_t n_items = (uint32_t)tiles * (TS * TS / 32);
-  unsigned grid = (unsigned)tiles;
-  if (PERSIST) grid = (unsigned)(tiles < pb ? tiles : pb);  // the work counters were cleared at the start of the forward
+  unsigned grid = (n_items + CW - 1) / CW;
+  if (PERSIST) grid = std::min(grid, (unsigned)pb);  // the work counters were cleared at the start of the forward
   const Front fr = {w.ready, w.prog, w.open_tiles, w.work + 7, w.dep, w.nsamp, resume};
-  auto k = out->composite_event && !resume ? launch(k_fwd<TS, SEG, PERSIST>, grid, TS * TS, smem, s)
-                                           : chain(k_fwd<TS, SEG, PERSIST>, grid, TS * TS, smem, s);
+  auto k = out->composite_event && !resume ? launch(k_fwd<TS, SEG, PERSIST>, grid, CW * 32, smem, s)
+                                           : chain(k_fwd<TS, SEG, PERSIST>, grid, CW * 32, smem, s);
   k(vs, w.ranges, w.plist, w.rec, w.slot_vox, t_stop,
                                                        out->rgb, out->depth, out->T, out->n_contrib,
                                                        out->n_samples, w.tau, out->wmax_packed,
                                                        w.work + (resume ? 2 : 0), n_items, sm_cut, sms,
-                                                       w.work + (resume ? 10 : 8), tile_order(w), fr);
+                                                       w.work + (resume ? 10 : 8), tile_order(w, tiles), fr);
 }
 
 template <int TS, bool SEG, bool PERSIST>
 static void launch_bwd_t(int64_t tiles, cudaStream_t s, const ViewSet& vs, const FwdWs& w, const lv_fwd_out* fwd,
                          const float* gC, const float* gD, const float* gT, float* dd,
                          int sm_limit, const LfFuse& lf) {
-  const size_t smem = WARP_SLICE * (TS * TS / 32);
+  constexpr int CW = comp_warps<TS, PERSIST>();
+  const size_t smem = WARP_SLICE * CW;
   static int pblocks[64];  // per device
   static std::atomic<unsigned long long> done{0};
   const int dev = current_device();
   once_per_device(done, [&] {
     cudaFuncSetAttribute(k_bwd<TS, SEG, PERSIST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (PERSIST && dev < 64) pblocks[dev] = persistent_blocks(k_bwd<TS, SEG, PERSIST>, TS * TS, smem);
+    if (PERSIST && dev < 64) pblocks[dev] = persistent_blocks(k_bwd<TS, SEG, PERSIST>, CW * 32, smem);
   });
-  const int pb = dev < 64 ? pblocks[dev] : persistent_blocks(k_bwd<TS, SEG, PERSIST>, TS * TS, smem);
+  const int pb = dev < 64 ? pblocks[dev] : persistent_blocks(k_bwd<TS, SEG, PERSIST>, CW * 32, smem);
   int sms = 0, sm_cut = 0;
   sm_limits(sm_limit, dev, &sms, &sm_cut);
   const uint32_t n_items = (uint32_t)tiles * (TS * TS / 32);
-  unsigned grid = (unsigned)tiles;
+  unsigned grid = (n_items + CW - 1) / CW;
   if (PERSIST) {
     zero_async(s, w.work + 1, sizeof(unsigned int), w.work + 9, sizeof(unsigned int));
-    grid = (unsigned)(tiles < pb ? tiles : pb);
+    grid = std::min(grid, (unsigned)pb);
   }
-  launch(k_bwd<TS, SEG, PERSIST>, grid, TS * TS, smem, s)(vs, w.ranges, w.plist, w.rec, w.slot_vox, fwd->T,
+  launch(k_bwd<TS, SEG, PERSIST>, grid, CW * 32, smem, s)(vs, w.ranges, w.plist, w.rec, w.slot_vox, fwd->T,
                                                        w.tau, fwd->n_contrib, gC, gD, gT, dd, w.d_rgb, w.work + 1,
-                                                       n_items, sm_cut, sms, w.work + 9, tile_order(w), lf);
+                                                       n_items, sm_cut, sms, w.work + 9, tile_order(w, tiles), lf);
 }
 
 // tile size, density model (midpoint, or the exact-segment variant) and scheduling (one block per
@@ -2566,12 +2583,11 @@ static void launch_tile_sort(const FwdWs& w, const ViewSet& vs, int64_t n, int64
   const uint32_t* sv = w.tile_slots;
   const unsigned wblocks = (unsigned)((tiles + TW_WARPS - 1) / TW_WARPS);
   chain(k_tile_sort_warp, wblocks, TW_WARPS * 32, sizeof(TileSortWarpSmem), s)(
-      sv, w.s_dkey, w.counters, pair_cap, ready, tiles, w.ranges, w.mid_tiles, w.work + 4, w.long_tiles, w.work + 6,
-      w.short_tiles, w.work + 11, w.ready, w.prog, vs, w.rec_bb, w.plist);
+      sv, w.s_dkey, w.counters, pair_cap, ready, tiles, w.ranges, tile_order(w, tiles), w.ready, w.prog, vs, w.rec_bb, w.plist);
   count_launch(1);
   if (n <= TW_MAX) return;  // a tile lists a voxel once: every list is short
   chain(k_tile_sort, (unsigned)nb, TS_THREADS, sizeof(TileLongSmem), s)(
-      sv, w.long_keys, w.s_dkey, w.ranges, w.mid_tiles, w.work + 4, w.long_tiles, w.work + 6, w.work + 5,
+      sv, w.long_keys, w.s_dkey, w.ranges, tile_order(w, tiles), w.work + 5,
       w.ready, w.prog, n > TS_LAZY_VOXELS ? TS_LAZY : ~0u, vs, w.rec_bb, w.plist);
   count_launch(1);
 }
@@ -2580,8 +2596,8 @@ static void launch_tile_rest(const FwdWs& w, const ViewSet& vs, int64_t tiles, b
   const int64_t nb = std::min<int64_t>(tile_sort_blocks(), tiles);
   if (all) zero_async(s, w.work + 3, sizeof(unsigned int));
   chain(k_tile_rest, (unsigned)nb, TS_THREADS, sizeof(TileLongSmem), s)(
-      w.tile_slots, w.long_keys, w.ranges, all ? w.long_tiles : w.open_tiles,
-      w.work + (all ? 6 : 7), w.work + 3, w.ready, w.prog, vs, w.rec_bb, w.plist);
+      w.tile_slots, w.long_keys, w.ranges, all ? w.class_tiles : w.open_tiles,
+      w.work + (all ? 16 : 7), w.work + 3, w.ready, w.prog, vs, w.rec_bb, w.plist);
   count_launch(1);
 }
 
@@ -2656,7 +2672,7 @@ extern "C" lv_status lv_rasterize_forward(const lv_voxels* vox, const lv_camera*
   const int passes = std::min(sort_passes(tile_bits(tiles)), 4);
   const bool own_status = d_status == w.status;
   const ZeroRanges zr = {{w.counters, w.status, w.work, sc.counts},
-                         {8 * sizeof(unsigned long long), own_status ? sizeof(int32_t) : 0, 16 * sizeof(unsigned int),
+                         {8 * sizeof(unsigned long long), own_status ? sizeof(int32_t) : 0, 32 * sizeof(unsigned int),
                           sc.zero_bytes}};
   if (items == 0)
     zero_async(s, zr.p[0], zr.bytes[0], zr.p[1], zr.bytes[1], zr.p[2], zr.bytes[2], zr.p[3], zr.bytes[3]);
