@@ -1922,8 +1922,9 @@ __global__ void __launch_bounds__(comp_warps<TS, PERSIST>() * 32, comp_blocks<TS
         const bool hit = h && !done;
         const float4 gj = g;
         const float ti = t_in, to = t_out;
-        // the next record's chord does not wait for this sample (past the last one: the last again)
-        g = wr[4 * min(j + 1, m - 1)];
+        // the next record's chord does not wait for this sample (past the last one: whatever follows in
+        // the slice, and the result is not used)
+        g = wr[4 * (j + 1)];
         h = chord(r, g, t_in, t_out);
         if (!__any_sync(FULL, hit)) continue;
         float w = 0.f;
@@ -2135,10 +2136,10 @@ __global__ void __launch_bounds__(comp_warps<TS, PERSIST>() * 32, comp_blocks<TS
         const float4 g = gn;
         const float t_in = tn_in, t_out = tn_out;
         const uint32_t slot = qe.x;
-        // the next record's chord does not wait for this sample (past the last one: the last again)
-        const int jn = min(j + 1, m - 1);
-        qe = walk.s_q[(q0 + jn) & walk.QM];
-        gn = wr[4 * jn];
+        // the next record's chord does not wait for this sample (past the last one: whatever follows in
+        // the slice, and the result is not used)
+        qe = walk.s_q[(q0 + j + 1) & walk.QM];
+        gn = wr[4 * (j + 1)];
         h = chord(r, gn, tn_in, tn_out) && qe.y < my_hi;
         const unsigned hb = __ballot_sync(FULL, hit);
         if (!hb) continue;
