@@ -154,14 +154,19 @@ class Workload:
             self.tile, self.persistent, self.batch = schedule
         elif tuned:
             self.tile, self.persistent, self.batch, self.tune_ms = tuned_schedule(self.scene, self.cams)
-        # the persistent backward composite leaves 80 SMs to the pruning and selection kernels
-        # that the four-stream step runs beside it; with more SMs for the backward the chain ends
-        # last, with fewer the backward (graph-replayed step, batch 32: 0.828-0.832 ms with the
-        # backward on 72 SMs, 0.832 on 68, 0.833 on 76, 0.839 on 64, 0.843 on 80, 0.847 on 88);
-        # the forward composite runs alone and keeps every SM
+            # forward + backward alone, as the tuner times them, tell the schedules apart by a few per
+            # cent; the step needs the persistent one, which can leave SMs to its other streams
+            # (0.88 ms a step against 0.94)
+            t0 = 6 * TUNE_TILES.index(self.tile) + TUNE_BATCHES.index(self.batch)
+            if not self.persistent and 0 < self.tune_ms[t0 + 3] <= 1.05 * self.tune_ms[t0]:
+                self.persistent = True
+        # the persistent backward composite leaves 64 SMs to the pruning and selection kernels
+        # that the four-stream step runs beside it (graph-replayed step: 0.876 ms with the backward
+        # on 88 SMs, 0.881 on 72, 0.879 on 104, 0.883 on 112, 0.912 on 128); the forward composite
+        # runs alone and keeps every SM
         self.persistent_sms = 0
         if self.persistent:
-            self.persistent_sms = max(1, torch.cuda.get_device_properties(0).multi_processor_count - 80)
+            self.persistent_sms = max(1, torch.cuda.get_device_properties(0).multi_processor_count - 64)
         self.rctx = RasterContext(self.cams, n, tile=self.tile, batch=self.batch, persistent=self.persistent)
         self.bwd_opts = L.make_opts(self.tile, self.batch, persistent=self.persistent,
                                     persistent_sms=self.persistent_sms)
