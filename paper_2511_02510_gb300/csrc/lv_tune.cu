@@ -1,7 +1,6 @@
 // lv_tune.cu -- autotuner of the composite schedule (host code).  Every
-// candidate (tile edge 8 / 16 / 32, one block per tile or persistent warps
-// on a work counter, batch of 32 / 64 / 128 list entries staged per warp
-// round) runs the caller's forward + backward on the caller's
+// candidate (tile edge 8 / 16 / 32, a warp per item or persistent warps on a
+// work counter, batch 32 / 64 / 128, which no longer changes what runs) runs the caller's forward + backward on the caller's
 // scene and views; the fastest one, timed with CUDA events on the caller's
 // stream, is returned and optionally remembered in a text cache file.
 #include <stdio.h>
