@@ -42,7 +42,7 @@ template <> struct Vec4T<float> { using V = float4; };
 static_assert(IPT == 4, "the vector accesses move four elements");
 
 template <typename T>
-__device__ __forceinline__ void load4(const T* __restrict__ p, int64_t i0, int64_t n, T* v, T fill) {
+__device__ __forceinline__ void load4(const T* p, int64_t i0, int64_t n, T* v, T fill) {
   using V = typename Vec4T<T>::V;
   if (i0 + 3 < n && ((uintptr_t)p & (sizeof(V) - 1)) == 0) {
     const V q = *(const V*)(p + i0);
@@ -54,7 +54,7 @@ __device__ __forceinline__ void load4(const T* __restrict__ p, int64_t i0, int64
 }
 
 template <typename T>
-__device__ __forceinline__ void store4(T* __restrict__ p, int64_t i0, int64_t n, const T* v) {
+__device__ __forceinline__ void store4(T* p, int64_t i0, int64_t n, const T* v) {
   using V = typename Vec4T<T>::V;
   if (i0 + 3 < n && ((uintptr_t)p & (sizeof(V) - 1)) == 0) {
     V q;
@@ -82,7 +82,7 @@ __device__ __forceinline__ uint32_t block_total(uint32_t c) {
 
 // sum of the per-block counts of all earlier blocks (every thread calls): the
 // block's offset among the flagged items, read straight from the counts
-__device__ __forceinline__ uint32_t block_offset(const uint32_t* __restrict__ blk) {
+__device__ __forceinline__ uint32_t block_offset(const uint32_t* blk) {
   uint32_t c = 0;
   for (unsigned k = threadIdx.x; k < blockIdx.x; k += TPB) c += blk[k];
   return block_total(c);
@@ -229,8 +229,8 @@ __global__ void k_pr_seen(int64_t n, const uint8_t* __restrict__ seen, const flo
 
 // order keys of w_max for the per-bin quantiles and the cap
 // order keys of w_max; the per-bin selection's first digit is counted here (row = depth bin)
-__global__ void k_pr_wkey(int64_t n, const float* __restrict__ w_max, const uint16_t* __restrict__ grp,
-                          uint32_t* __restrict__ wkey, const FirstHist fh) {
+__global__ void k_pr_wkey(int64_t n, const float* __restrict__ w_max, const uint16_t* grp,
+                          uint32_t* wkey, const FirstHist fh) {
   grid_begin();
   __shared__ uint32_t sh[FH_WORDS];
   fh_clear(fh, sh);
@@ -344,7 +344,7 @@ struct Halo {
   const float* w_max;
 };
 
-__global__ void k_pr_update(int64_t n, const uint16_t* __restrict__ grp, const uint32_t* __restrict__ wkey,
+__global__ void k_pr_update(int64_t n, const uint16_t* grp, const uint32_t* wkey,
                             const SelectQuery* tau, float alpha, float oma, float m_low, float m_high, float* ema_m,
                             uint8_t* state, const Halo halo, uint8_t* mask, uint16_t* cand_grp, PruneState* st,
                             const FirstHist fh) {
@@ -410,8 +410,8 @@ __global__ void k_pr_cap_query(SelectQuery* q, PruneState* st, uint32_t cap, voi
 
 // candidates strictly below the threshold, and per block the candidates at it
 // (the ties compete by id: the need = cap - c_lt smallest ids among them go)
-__global__ void k_pr_ties(int64_t n, const uint32_t* __restrict__ wkey, const SelectQuery* thr,
-                          const uint8_t* __restrict__ cand, uint32_t* blk, PruneState* st) {
+__global__ void k_pr_ties(int64_t n, const uint32_t* wkey, const SelectQuery* thr,
+                          const uint8_t* cand, uint32_t* blk, PruneState* st) {
   grid_begin();
   const int64_t i0 = first_item();
   uint32_t clt = 0, ceq = 0;
@@ -441,8 +441,8 @@ __global__ void k_pr_ties(int64_t n, const uint32_t* __restrict__ wkey, const Se
 // mask holds the candidate flags on entry and the pruning decision on exit;
 // a tie's rank among the ties (in id order) is its block's offset plus its
 // rank inside the block
-__global__ void k_pr_mask(int64_t n, const uint32_t* __restrict__ wkey, const SelectQuery* thr,
-                          const uint32_t* __restrict__ blk, const PruneState* st, uint8_t* mask,
+__global__ void k_pr_mask(int64_t n, const uint32_t* wkey, const SelectQuery* thr,
+                          const uint32_t* blk, const PruneState* st, uint8_t* mask,
                           int64_t* n_pruned, uint32_t cap) {
   grid_begin();
   const int64_t i0 = first_item();
@@ -654,8 +654,8 @@ __global__ void k_sd_k(SelectQuery* q, SubState* st, uint32_t top_ppm, long long
 
 // eligible voxels above the k-th priority, and per block those tied with it
 // (the ties compete by id: the need = k - c_gt smallest ids among them split)
-__global__ void k_sd_ties(int64_t n, const uint32_t* __restrict__ pkey, const SelectQuery* thr,
-                          const uint16_t* __restrict__ grp, uint32_t* blk, SubState* st) {
+__global__ void k_sd_ties(int64_t n, const uint32_t* pkey, const SelectQuery* thr,
+                          const uint16_t* grp, uint32_t* blk, SubState* st) {
   grid_begin();
   const int64_t i0 = first_item();
   uint32_t cgt = 0, ceq = 0;
@@ -684,9 +684,9 @@ __global__ void k_sd_ties(int64_t n, const uint32_t* __restrict__ pkey, const Se
 
 // grp == 0 marks the eligible voxels (set by the priority kernel); a tie's
 // rank among the ties is its block's offset plus its rank inside the block
-__global__ void k_sd_select(int64_t n, const uint8_t* __restrict__ pm, const uint16_t* __restrict__ grp,
-                            const uint32_t* __restrict__ pkey, const SelectQuery* q,
-                            const uint32_t* __restrict__ blk, const SubState* st, uint8_t* selected,
+__global__ void k_sd_select(int64_t n, const uint8_t* __restrict__ pm, const uint16_t* grp,
+                            const uint32_t* pkey, const SelectQuery* q,
+                            const uint32_t* blk, const SubState* st, uint8_t* selected,
                             uint32_t* surv, uint32_t* sel, uint32_t* blk_surv, uint32_t* blk_sel) {
   grid_begin();
   const int64_t i0 = first_item();
@@ -798,8 +798,8 @@ __device__ __forceinline__ void warp_copy_rows(const char* __restrict__ in, char
 }
 
 template <typename DT, typename ST>
-__device__ __forceinline__ void write_survivors(int64_t i0, int64_t n, const uint32_t* __restrict__ surv,
-                                                const unsigned long long* __restrict__ pos,
+__device__ __forceinline__ void write_survivors(int64_t i0, int64_t n, const uint32_t* surv,
+                                                const unsigned long long* pos,
                                                 const float4* __restrict__ geom, const uint8_t* __restrict__ level,
                                                 const DT* __restrict__ dens, const ST* __restrict__ sh, float4* ogeom,
                                                 uint8_t* olevel, DT* odens, ST* osh, const AuxSet& aux) {
@@ -845,10 +845,10 @@ __global__ void k_cp_flags(int64_t n, const uint8_t* __restrict__ keep, uint32_t
 // parents and checks the grown count against the output capacity.  It runs
 // with the selection (on the caller's side stream in a training step) so that
 // the in-place write does not read these arrays again.
-__global__ void k_sd_list(int64_t n, const uint32_t* __restrict__ sel, const uint32_t* __restrict__ surv,
-                          const uint32_t* __restrict__ blk_surv, const uint32_t* __restrict__ blk_sel,
-                          unsigned long long* __restrict__ surv_pos, uint32_t* __restrict__ list,
-                          uint32_t* __restrict__ holes, unsigned long long* totals, SubState* st, int64_t capacity,
+__global__ void k_sd_list(int64_t n, const uint32_t* sel, const uint32_t* surv,
+                          const uint32_t* blk_surv, const uint32_t* blk_sel,
+                          unsigned long long* surv_pos, uint32_t* list,
+                          uint32_t* holes, unsigned long long* totals, SubState* st, int64_t capacity,
                           int64_t* n_new, int32_t* status) {
   grid_begin();
   const int64_t i0 = first_item();
@@ -890,7 +890,7 @@ __global__ void k_sd_list(int64_t n, const uint32_t* __restrict__ sel, const uin
 // the auxiliary rows are written cooperatively in 16-byte words so that the
 // stores coalesce (the 8 children of a parent read the same parent row).
 template <typename DT, typename ST>
-__device__ __forceinline__ void write_children(int64_t t0, const uint32_t* __restrict__ list,
+__device__ __forceinline__ void write_children(int64_t t0, const uint32_t* list,
                                                const unsigned long long* totals, const float4* __restrict__ geom,
                                                const uint8_t* __restrict__ level, const DT* __restrict__ dens,
                                                const ST* __restrict__ sh, float4* ogeom, uint8_t* olevel, DT* odens,
@@ -950,8 +950,8 @@ __device__ __forceinline__ void write_children(int64_t t0, const uint32_t* __res
 // All the writes of a topology change in one launch: warps [0, sw) copy the
 // survivors of 32 consecutive voxels each, warps [sw, ...) write 32 children each.
 template <typename DT, typename ST>
-__global__ void k_sd_write(int64_t n, int64_t max_children, const uint32_t* __restrict__ surv,
-                           const unsigned long long* __restrict__ pos, const uint32_t* __restrict__ list,
+__global__ void k_sd_write(int64_t n, int64_t max_children, const uint32_t* surv,
+                           const unsigned long long* pos, const uint32_t* list,
                            const unsigned long long* totals, const SubState* st, const float4* __restrict__ geom,
                            const uint8_t* __restrict__ level, const DT* __restrict__ dens, const ST* __restrict__ sh,
                            float4* ogeom, uint8_t* olevel, DT* odens, ST* osh, const __grid_constant__ AuxSet aux) {

@@ -56,6 +56,14 @@ void once_per_device(std::atomic<unsigned long long>& done, F&& f) {
 // pruning) spent 1 to 2 us of each on that latency.  launch(...) does not
 // overlap: for the first kernel of a call and after an event record, where what
 // comes before in the stream is the caller's.
+//
+// A chained kernel begins while the grids before it still write, so what they
+// write is not constant over its lifetime.  `const __restrict__`, __ldg and
+// ld.global.nc say that it is: the compiler may then load it ahead of the wait, or
+// through a path that is not coherent with those writes.  Chained kernels have
+// them only for what was complete before the call's last plain launch and no grid
+// since has written (the caller's inputs, an earlier call's results), and a
+// __restrict__ output only where no other grid of the call touches it.
 template <typename T>
 struct SameType {
   using type = T;

@@ -92,7 +92,7 @@ __device__ __forceinline__ int view_of_block(const int* first, int n, int b) {
 // caches before), and the next tile's pixels are loaded while this one is worked on.
 constexpr int ST = 32, SP = ST + 2;
 __global__ void __launch_bounds__(TPB) k_lf_sobel(const float* __restrict__ gt, const __grid_constant__ ViewPix vp,
-                                                 int per, uint32_t* __restrict__ mkey, uint32_t* __restrict__ hist) {
+                                                 int per, uint32_t* mkey, uint32_t* hist) {
   grid_begin();
   __shared__ uint32_t s_h[D1_BINS];
   __shared__ float s_y[SP * SP];
@@ -160,7 +160,7 @@ __global__ void __launch_bounds__(TPB) k_lf_sobel(const float* __restrict__ gt, 
 // the counters 32 at a time (coalesced), one thread per 32 scans the sums, and
 // the warp of the group that holds the key finds it there.
 template <int NB>
-__device__ __forceinline__ LfPick block_pick(const uint32_t* __restrict__ h, uint32_t k) {
+__device__ __forceinline__ LfPick block_pick(const uint32_t* h, uint32_t k) {
   constexpr int PER = NB / TPB;  // groups of 32 counters per warp
   static_assert(PER >= 1 && PER <= 32, "a lane for each of a warp's groups");
   __shared__ uint32_t s_part[TPB / 32];
@@ -210,7 +210,7 @@ __device__ __forceinline__ LfPick block_pick(const uint32_t* __restrict__ h, uin
 // LAST, of the third.  Every block picks for its view; the view's first block
 // leaves the pick for the next step.
 template <bool LAST>
-__global__ void __launch_bounds__(TPB) k_lf_digit(const uint32_t* __restrict__ mkey, const __grid_constant__ ViewPix vp,
+__global__ void __launch_bounds__(TPB) k_lf_digit(const uint32_t* mkey, const __grid_constant__ ViewPix vp,
                                                  uint32_t* hist, LfPick* pick) {
   grid_begin();
   constexpr int NB = LAST ? D3_BINS : D2_BINS;
@@ -265,10 +265,10 @@ __device__ __forceinline__ void block_add_f64(double v, double* dst) {
 // Eq. 7: w = (eps + 1 - s)^gamma, s = clip(|grad| / P, 0, 1); blocks never span views.
 // Grid-stride over the view's pixels with a bounded block count: one FP64
 // atomic per block (a per-256-pixel atomic would serialise at the L2).
-__global__ void __launch_bounds__(TPB) k_lf_weight(const uint32_t* __restrict__ mkey, const uint32_t* __restrict__ hist,
-                                                  const LfPick* __restrict__ pick,
+__global__ void __launch_bounds__(TPB) k_lf_weight(const uint32_t* mkey, const uint32_t* hist,
+                                                  const LfPick* pick,
                                                   const __grid_constant__ ViewPix vp, float eps, float gamma,
-                                                  float* __restrict__ w, double* wsum, float* __restrict__ edge_out) {
+                                                  float* w, double* wsum, float* edge_out) {
   grid_begin();
   const int v = view_of_block(vp.blk, vp.n, blockIdx.x);
   const int b0 = vp.blk[v], nb = vp.blk[v + 1] - b0;

@@ -238,9 +238,9 @@ SortTmp carve_sort(void* base, int64_t cap) {
 // Digit counts of all passes (block-private shared histograms, one global
 // atomic per nonzero bin), and clears the look-back words of the first pass.
 template <typename K>
-__global__ void __launch_bounds__(OS_HIST_THREADS) k_os_hist(const K* __restrict__ keys, const unsigned long long* d_count,
-                                                       int64_t cap, int passes, uint32_t* __restrict__ ghist,
-                                                       unsigned long long* __restrict__ look0) {
+__global__ void __launch_bounds__(OS_HIST_THREADS) k_os_hist(const K* keys, const unsigned long long* d_count,
+                                                       int64_t cap, int passes, uint32_t* ghist,
+                                                       unsigned long long* look0) {
   grid_begin();
   __shared__ uint32_t sh[OS_MAX_PASSES * RADIX];
   for (int i = threadIdx.x; i < passes * RADIX; i += OS_HIST_THREADS) sh[i] = 0;
@@ -286,13 +286,13 @@ __device__ __forceinline__ uint32_t os_block_excl(uint32_t c, uint32_t* s_w) {
 }
 
 template <typename K>
-__global__ void __launch_bounds__(Os<K>::THREADS, Os<K>::MIN_BLOCKS) k_os_pass(const K* __restrict__ kin, const uint32_t* __restrict__ vin,
-                                                         K* __restrict__ kout, uint32_t* __restrict__ vout,
+__global__ void __launch_bounds__(Os<K>::THREADS, Os<K>::MIN_BLOCKS) k_os_pass(const K* kin, const uint32_t* vin,
+                                                         K* kout, uint32_t* vout,
                                                          const unsigned long long* d_count, int64_t cap, int pass,
-                                                         const uint32_t* __restrict__ ghist, uint32_t* ticket,
+                                                         const uint32_t* ghist, uint32_t* ticket,
                                                          unsigned long long* look, unsigned long long* look_next,
                                                          int32_t* status, unsigned spin_limit,
-                                                         uint32_t* __restrict__ key_ranges) {
+                                                         uint32_t* key_ranges) {
   grid_begin();
   constexpr int OS_THREADS = Os<K>::THREADS, OS_WARPS = Os<K>::WARPS, OS_TILE = Os<K>::TILE;
   __shared__ uint32_t s_wh[OS_WARPS][RADIX + 1];  // warp digit counts -> warp prefixes (bin RADIX: padding items)
@@ -319,9 +319,22 @@ __global__ void __launch_bounds__(Os<K>::THREADS, Os<K>::MIN_BLOCKS) k_os_pass(c
     // every key has the same digit (the high bytes of keys packed from the bottom): the pass is a copy.
     // (32-bit keys are tile ids, whose digits differ whenever there is a second tile.)
     if (__syncthreads_or(gcount == (uint32_t)n)) {
-      for (int64_t i = tile * OS_TILE + t; i < min(n, (tile + 1) * OS_TILE); i += OS_THREADS) {
-        kout[i] = kin[i];
-        vout[i] = vin ? vin[i] : (uint32_t)i;
+      const int64_t i0 = tile * OS_TILE + t;
+      K kc[OS_ITEMS];
+      uint32_t vc[OS_ITEMS];
+#pragma unroll
+      for (int j = 0; j < OS_ITEMS; ++j) {
+        const int64_t i = i0 + j * OS_THREADS;
+        kc[j] = i < n ? kin[i] : (K)0;
+        vc[j] = i < n && vin ? vin[i] : (uint32_t)i;
+      }
+#pragma unroll
+      for (int j = 0; j < OS_ITEMS; ++j) {
+        const int64_t i = i0 + j * OS_THREADS;
+        if (i < n) {
+          kout[i] = kc[j];
+          vout[i] = vc[j];
+        }
       }
       return;
     }
@@ -617,7 +630,7 @@ constexpr int SEL_ITEMS = 16;       // items per thread per iteration, loads iss
 // One warp per query: find the digit holding the k-th item (warp scan over
 // RADIX / 32 digits per lane) and extend the prefix; returns the updated query.
 template <int RADIX>
-__device__ __forceinline__ SelectQuery warp_pick(const uint32_t* __restrict__ row, SelectQuery s, int shift,
+__device__ __forceinline__ SelectQuery warp_pick(const uint32_t* row, SelectQuery s, int shift,
                                                  int lane) {
   constexpr int PER = RADIX / 32;  // 8 or 64 digits per lane, contiguous
   const uint4* hrow = (const uint4*)(row + lane * PER);

@@ -435,11 +435,11 @@ __global__ void __launch_bounds__(BIN_THREADS, 6) k_bin(const float4* __restrict
 // to 1M items there is one group, at 48M items 46.  (One block over all entries
 // took 196 us for 48M items, 4 us a round of 4096.)
 constexpr int BO_THREADS = 1024, BO_ITEMS = 4, BO_GROUP = BO_THREADS * BO_ITEMS;
-__global__ void __launch_bounds__(BO_THREADS) k_block_offsets(unsigned long long* __restrict__ pairs,
-                                                              uint32_t* __restrict__ slots, int64_t m,
-                                                              unsigned long long* __restrict__ grp_pairs,
-                                                              uint32_t* __restrict__ grp_slots,
-                                                              unsigned long long* __restrict__ counters) {
+__global__ void __launch_bounds__(BO_THREADS) k_block_offsets(unsigned long long* pairs,
+                                                              uint32_t* slots, int64_t m,
+                                                              unsigned long long* grp_pairs,
+                                                              uint32_t* grp_slots,
+                                                              unsigned long long* counters) {
   grid_begin();
   __shared__ unsigned long long s_a[BO_THREADS / 32];
   __shared__ uint32_t s_b[BO_THREADS / 32];
@@ -668,22 +668,22 @@ __device__ __forceinline__ void unit_dir(float rx, float ry, float rz, float* d)
 template <typename DT, typename ST>
 __global__ void __launch_bounds__(BIN_THREADS, sizeof(ST) == 4 ? 6 : 8) k_emit(const float4* __restrict__ geom, const DT* __restrict__ dens,
                                               const ST* __restrict__ sh, int sh_nb, int64_t n,
-                                              const __grid_constant__ ViewSet vs, const uint32_t* __restrict__ cnt,
-                                              const uint2* __restrict__ rect,
-                                              const uint2* __restrict__ pbox, uint2* __restrict__ rec_bb,
-                                              uint32_t* __restrict__ slot_vox,
-                                              const uint32_t* __restrict__ dkey,
-                                              uint32_t* __restrict__ slot, int64_t blocks,
-                                              const unsigned long long* __restrict__ blk_pairs,
-                                              const uint32_t* __restrict__ blk_slots,
-                                              const unsigned long long* __restrict__ grp_pairs,
-                                              const uint32_t* __restrict__ grp_slots,
-                                              const unsigned long long* __restrict__ counters, int64_t pair_cap,
-                                              uint32_t* __restrict__ pair_tile, uint32_t* __restrict__ pair_slot,
-                                              int32_t* status, uint2* __restrict__ ranges, int64_t tiles,
+                                              const __grid_constant__ ViewSet vs, const uint32_t* cnt,
+                                              const uint2* rect,
+                                              const uint2* pbox, uint2* rec_bb,
+                                              uint32_t* slot_vox,
+                                              const uint32_t* dkey,
+                                              uint32_t* slot, int64_t blocks,
+                                              const unsigned long long* blk_pairs,
+                                              const uint32_t* blk_slots,
+                                              const unsigned long long* grp_pairs,
+                                              const uint32_t* grp_slots,
+                                              const unsigned long long* counters, int64_t pair_cap,
+                                              uint32_t* pair_tile, uint32_t* pair_slot,
+                                              int32_t* status, uint2* ranges, int64_t tiles,
                                               const SortCountTargets sc, int passes,
-                                              float4* __restrict__ rec,
-                                              float4* __restrict__ d_rgb, uint32_t* __restrict__ s_dkey,
+                                              float4* rec,
+                                              float4* d_rgb, uint32_t* s_dkey,
                                               const uint32_t* __restrict__ vidx) {
   grid_begin();
   // Block b covers 256 consecutive voxels of view b % views, so the blocks of
@@ -818,13 +818,15 @@ __global__ void __launch_bounds__(BIN_THREADS, sizeof(ST) == 4 ? 6 : 8) k_emit(c
   st_row32(r, make_float4(rx, ry, rz, g.w), make_float4(d[0], d[1], d[2], d[3]));
   st_row32(r + 2, make_float4(d[4], d[5], d[6], d[7]),
            make_float4(fmaxf(raw[0], 0.f), fmaxf(raw[1], 0.f), fmaxf(raw[2], 0.f), __fdiv_rn(0.5f, g.w)));
+  const uint2 box = pbox[i];
+  const uint32_t key = dkey[i];
   slot_vox[s] = (uint32_t)vox;
   // colour-gradient scratch: xyz cleared, w = which channels passed the clamp
   // (bit c set when raw_c > 0) as a small exact float, read by the SH backward
   d_rgb[s] = make_float4(0.f, 0.f, 0.f,
                          (float)((raw[0] > 0.f ? 1 : 0) | (raw[1] > 0.f ? 2 : 0) | (raw[2] > 0.f ? 4 : 0)));
-  rec_bb[s] = pbox[i];
-  s_dkey[s] = dkey[i];
+  rec_bb[s] = box;
+  s_dkey[s] = key;
 }
 
 // pairs usable by the later stages: all of them, or none after an overflow
@@ -1006,17 +1008,17 @@ struct TileBox {
 };
 
 // ---- short lists: one warp each, TW_WARPS tiles per block
-__global__ void __launch_bounds__(TW_WARPS * 32, 2) k_tile_sort_warp(const uint32_t* __restrict__ tvals,
-                                                                    const uint32_t* __restrict__ s_dkey,
-                                                                    const unsigned long long* __restrict__ d_count,
+__global__ void __launch_bounds__(TW_WARPS * 32, 2) k_tile_sort_warp(const uint32_t* tvals,
+                                                                    const uint32_t* s_dkey,
+                                                                    const unsigned long long* d_count,
                                                                     int64_t cap, bool ranges_ready, int64_t tiles,
-                                                                    uint32_t* __restrict__ ranges,
+                                                                    uint32_t* ranges,
                                                                     const TileOrder order,
-                                                                    uint32_t* __restrict__ ready,
-                                                                    TileProg* __restrict__ prog,
+                                                                    uint32_t* ready,
+                                                                    TileProg* prog,
                                                                     const __grid_constant__ ViewSet vs,
-                                                                    const uint2* __restrict__ rec_bb,
-                                                                    uint2* __restrict__ plist) {
+                                                                    const uint2* rec_bb,
+                                                                    uint2* plist) {
   grid_begin();
   extern __shared__ __align__(16) unsigned char tw_raw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1151,8 +1153,8 @@ __device__ __forceinline__ TileLongSmem& ts_smem() {
 // Sorts the m <= TS_CHUNK (key, slot) pairs of S by key, stably, with the whole
 // block (all of it past a barrier since they were written, and S.kmin and S.kmax
 // their extremes), and writes (slot, strip mask) to plist[0, m).
-__device__ __noinline__ void ts_sort_smem(int m, const TileBox& tb, const uint2* __restrict__ rec_bb,
-                                          uint2* __restrict__ plist) {
+__device__ __noinline__ void ts_sort_smem(int m, const TileBox& tb, const uint2* rec_bb,
+                                          uint2* plist) {
   TileSortSmem& S = ts_smem().s;
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   const int R = (m + TS_THREADS - 1) / TS_THREADS;  // items per thread, and rounds per warp
@@ -1205,9 +1207,9 @@ __device__ __noinline__ void ts_sort_smem(int m, const TileBox& tb, const uint2*
 }
 
 // a whole list of m <= TS_CHUNK slots
-__device__ __noinline__ void ts_sort_list(const uint32_t* __restrict__ src, const uint32_t* __restrict__ s_dkey,
-                                          int m, const TileBox& tb, const uint2* __restrict__ rec_bb,
-                                          uint2* __restrict__ plist) {
+__device__ __noinline__ void ts_sort_list(const uint32_t* src, const uint32_t* s_dkey,
+                                          int m, const TileBox& tb, const uint2* rec_bb,
+                                          uint2* plist) {
   TileSortSmem& S = ts_smem().s;
   const int t = threadIdx.x;
   if (t == 0) {
@@ -1251,10 +1253,10 @@ __device__ __noinline__ void ts_sort_list(const uint32_t* __restrict__ src, cons
 // (key, slot) with their extremes (there are at most TS_CHUNK of them), or, with
 // ALL_EQUAL, straight to plist (any number: one key, so item order is the order).
 template <bool ALL_EQUAL>
-__device__ __forceinline__ void tl_collect(TileSortSmem& S, const uint32_t* __restrict__ sv,
+__device__ __forceinline__ void tl_collect(TileSortSmem& S, const uint32_t* sv,
                                            const uint32_t* xk, uint32_t L, uint32_t k0, uint32_t k1,
-                                           const TileBox& tb, const uint2* __restrict__ rec_bb,
-                                           uint2* __restrict__ plist) {
+                                           const TileBox& tb, const uint2* rec_bb,
+                                           uint2* plist) {
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   if (t == 0) {
     S.kmin = ~0u;
@@ -1310,10 +1312,10 @@ __device__ __forceinline__ void tl_collect(TileSortSmem& S, const uint32_t* __re
 // `lazy` entries the work stops after one range; else it goes on from the progress of
 // such a start.
 template <bool START>
-__device__ __noinline__ void tl_order(uint32_t lo, uint32_t L, uint32_t lazy, const uint32_t* __restrict__ sv_all,
-                         uint32_t* xk_all, const uint32_t* __restrict__ s_dkey, TileProg* prog,
-                         uint32_t* ready, const TileBox& tb, const uint2* __restrict__ rec_bb,
-                         uint2* __restrict__ plist_all) {
+__device__ __noinline__ void tl_order(uint32_t lo, uint32_t L, uint32_t lazy, const uint32_t* sv_all,
+                         uint32_t* xk_all, const uint32_t* s_dkey, TileProg* prog,
+                         uint32_t* ready, const TileBox& tb, const uint2* rec_bb,
+                         uint2* plist_all) {
   TileLongSmem& M = ts_smem();
   TileSortSmem& S = M.s;
   const int t = threadIdx.x;
@@ -1452,16 +1454,16 @@ __device__ __noinline__ void tl_order(uint32_t lo, uint32_t L, uint32_t lazy, co
 }
 
 // Persistent blocks over the long tiles, then over the medium ones.
-__global__ void __launch_bounds__(TS_THREADS, 2) k_tile_sort(const uint32_t* __restrict__ tvals,
+__global__ void __launch_bounds__(TS_THREADS, 2) k_tile_sort(const uint32_t* tvals,
                                                             uint32_t* xk,
-                                                            const uint32_t* __restrict__ s_dkey,
-                                                            const uint32_t* __restrict__ ranges,
+                                                            const uint32_t* s_dkey,
+                                                            const uint32_t* ranges,
                                                             const TileOrder order,
-                                                            unsigned int* __restrict__ work,
+                                                            unsigned int* work,
                                                             uint32_t* ready, TileProg* prog, uint32_t lazy,
                                                             const __grid_constant__ ViewSet vs,
-                                                            const uint2* __restrict__ rec_bb,
-                                                            uint2* __restrict__ plist) {
+                                                            const uint2* rec_bb,
+                                                            uint2* plist) {
   grid_begin();
   TileLongSmem& M = ts_smem();
   static_assert(TILE_CLASS_SHORT == 5 && TS_CHUNK == 4096 && TW_MAX == 256, "the length classes");
@@ -1487,16 +1489,16 @@ __global__ void __launch_bounds__(TS_THREADS, 2) k_tile_sort(const uint32_t* __r
 }
 
 // Persistent blocks over the listed long tiles: what k_tile_sort left unsorted.
-__global__ void __launch_bounds__(TS_THREADS, 2) k_tile_rest(const uint32_t* __restrict__ tvals,
+__global__ void __launch_bounds__(TS_THREADS, 2) k_tile_rest(const uint32_t* tvals,
                                                             uint32_t* xk,
-                                                            const uint32_t* __restrict__ ranges,
-                                                            const uint32_t* __restrict__ list,
-                                                            const unsigned int* __restrict__ n_list,
-                                                            unsigned int* __restrict__ work,
+                                                            const uint32_t* ranges,
+                                                            const uint32_t* list,
+                                                            const unsigned int* n_list,
+                                                            unsigned int* work,
                                                             uint32_t* ready, TileProg* prog,
                                                             const __grid_constant__ ViewSet vs,
-                                                            const uint2* __restrict__ rec_bb,
-                                                            uint2* __restrict__ plist) {
+                                                            const uint2* rec_bb,
+                                                            uint2* plist) {
   grid_begin();
   TileLongSmem& M = ts_smem();
   const unsigned int total = *n_list;
@@ -1715,9 +1717,9 @@ template <bool REV>
 struct StripWalk {
   static constexpr int K = WALK_ENTRIES / 32;
   static constexpr uint32_t QM = QUEUE_LEN - 1;
-  const uint2* __restrict__ plist;
-  const float4* __restrict__ rec;
-  const uint32_t* __restrict__ slot_vox;
+  const uint2* plist;
+  const float4* rec;
+  const uint32_t* slot_vox;
   float4* s_rec;     // [2][32][4]
   uint32_t* s_vox;   // [2][32]
   uint2* s_q;        // (slot, entry)
@@ -1842,13 +1844,13 @@ template <int TS, bool PERSIST>
 __host__ __device__ constexpr int comp_blocks(int warps_sm) { return warps_sm / comp_warps<TS, PERSIST>(); }
 
 template <int TS, bool SEG, bool PERSIST>
-__global__ void __launch_bounds__(comp_warps<TS, PERSIST>() * 32, comp_blocks<TS, PERSIST>(28)) k_fwd(const __grid_constant__ ViewSet vs, const uint32_t* __restrict__ ranges,
-                                                const uint2* __restrict__ plist, const float4* __restrict__ rec,
-                                                const uint32_t* __restrict__ slot_vox, float t_stop,
-                                                float* __restrict__ rgb, float* __restrict__ depth,
-                                                float* __restrict__ T_out, uint32_t* __restrict__ n_contrib,
-                                                uint32_t* __restrict__ n_samples, float* __restrict__ tau_out,
-                                                unsigned long long* __restrict__ wmax, unsigned int* work,
+__global__ void __launch_bounds__(comp_warps<TS, PERSIST>() * 32, comp_blocks<TS, PERSIST>(28)) k_fwd(const __grid_constant__ ViewSet vs, const uint32_t* ranges,
+                                                const uint2* plist, const float4* rec,
+                                                const uint32_t* slot_vox, float t_stop,
+                                                float* rgb, float* depth,
+                                                float* T_out, uint32_t* n_contrib,
+                                                uint32_t* n_samples, float* tau_out,
+                                                unsigned long long* wmax, unsigned int* work,
                                                 uint32_t n_items, int sm_cut, int n_sms, unsigned int* arrivals,
                                                 const TileOrder order, const Front fr) {
   grid_wait();
@@ -2223,7 +2225,7 @@ __global__ void __launch_bounds__(comp_warps<TS, PERSIST>() * 32, comp_blocks<TS
 __global__ void __launch_bounds__(128) k_sh_bwd(const float4* __restrict__ rec, int sh_nb, int64_t n,
                                                 const __grid_constant__ ViewSet vs,
                                                 const uint32_t* __restrict__ cnt, const uint32_t* __restrict__ slot,
-                                                float4* __restrict__ d_rgb, float* __restrict__ d_sh,
+                                                float4* d_rgb, float* d_sh,
                                                 int accumulate) {
   grid_wait();
   constexpr int RS = 49;
@@ -2310,7 +2312,7 @@ __global__ void k_gather_edge(const int64_t* __restrict__ argmax, int64_t n, con
 }
 
 // a block per tile, in turn
-__global__ void k_debug_pairs(const uint2* __restrict__ ranges, int64_t tiles, const uint2* __restrict__ plist,
+__global__ void k_debug_pairs(const uint2* ranges, int64_t tiles, const uint2* plist,
                               const uint32_t* __restrict__ slot_vox, const uint32_t* __restrict__ s_dkey,
                               uint64_t* ko, uint32_t* vo) {
   grid_begin();
@@ -2345,12 +2347,12 @@ __device__ __forceinline__ void sh_basis64(double x, double y, double z, double*
 }
 
 template <typename DT, typename ST>
-__global__ void k_render_f64(const __grid_constant__ ViewSet vs, const uint32_t* __restrict__ ranges,
-                             const uint2* __restrict__ plist, const uint32_t* __restrict__ slot_vox,
+__global__ void k_render_f64(const __grid_constant__ ViewSet vs, const uint32_t* ranges,
+                             const uint2* plist, const uint32_t* __restrict__ slot_vox,
                              const float4* __restrict__ geom, const DT* __restrict__ dens, const ST* __restrict__ sh,
                              int sh_nb, const int64_t* __restrict__ pixels, int64_t n_px, double t_stop,
-                             int segment, const uint32_t* __restrict__ vidx, double* __restrict__ rgb_out,
-                             double* __restrict__ T_out) {
+                             int segment, const uint32_t* __restrict__ vidx, double* rgb_out,
+                             double* T_out) {
   grid_begin();
   const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (q >= n_px) return;

@@ -91,8 +91,8 @@ __device__ __forceinline__ bool grid_coord(float x, float h, double inv_unit, fl
 // passes over all corners (the whole index of 300,000 voxels: 404 -> 176 us, of
 // which this kernel is 40 and the sort 95, bound by its passes' latencies).
 __global__ void __launch_bounds__(TPB) k_vx_hash(const float4* __restrict__ geom, int64_t n, double inv_unit,
-                                                unsigned long long* table, int bits, uint32_t* __restrict__ vidx,
-                                                uint64_t* __restrict__ keys, uint32_t* __restrict__ slots,
+                                                unsigned long long* table, int bits, uint32_t* vidx,
+                                                uint64_t* keys, uint32_t* slots,
                                                 unsigned long long* count, uint32_t* bounds, int32_t* status) {
   grid_begin();
   __shared__ uint32_t s_b[6], s_n;
@@ -157,8 +157,8 @@ __global__ void __launch_bounds__(TPB) k_vx_hash(const float4* __restrict__ geom
 // The distinct keys packed: each coordinate less its smallest value, in just the
 // bits its range needs.  The order stays, and the sort's passes over the high
 // bytes, all zero, are plain copies.
-__global__ void __launch_bounds__(TPB) k_vx_pack(uint64_t* __restrict__ keys, const unsigned long long* count,
-                                                const uint32_t* __restrict__ bounds) {
+__global__ void __launch_bounds__(TPB) k_vx_pack(uint64_t* keys, const unsigned long long* count,
+                                                const uint32_t* bounds) {
   grid_begin();
   const int64_t m = (int64_t)*count;
   uint32_t lo[3];
@@ -179,8 +179,8 @@ __global__ void __launch_bounds__(TPB) k_vx_pack(uint64_t* __restrict__ keys, co
 }
 
 // a vertex's id is its key's rank
-__global__ void __launch_bounds__(TPB) k_vx_rank(const uint32_t* __restrict__ slots, const unsigned long long* count,
-                                                uint64_t* __restrict__ table, int64_t* __restrict__ n_vert) {
+__global__ void __launch_bounds__(TPB) k_vx_rank(const uint32_t* slots, const unsigned long long* count,
+                                                uint64_t* table, int64_t* n_vert) {
   grid_begin();
   const int64_t m = (int64_t)*count;
   for (int64_t i = blockIdx.x * (int64_t)TPB + threadIdx.x; i < m; i += (int64_t)gridDim.x * TPB)
@@ -189,8 +189,8 @@ __global__ void __launch_bounds__(TPB) k_vx_rank(const uint32_t* __restrict__ sl
 }
 
 // four corners per thread
-__global__ void __launch_bounds__(TPB) k_vx_assign(const uint64_t* __restrict__ table, int64_t n4,
-                                                  uint32_t* __restrict__ vidx) {
+__global__ void __launch_bounds__(TPB) k_vx_assign(const uint64_t* table, int64_t n4,
+                                                  uint32_t* vidx) {
   grid_begin();
   const int64_t i = blockIdx.x * (int64_t)TPB + threadIdx.x;
   if (i >= n4) return;
