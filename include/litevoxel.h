@@ -279,7 +279,8 @@ lv_status lv_gather_edge(const int64_t* argmax, int64_t n, const float* edge_map
  * voxel[i] = voxel id; ranges [tiles][2] = [start, end) per global tile.
  * keys / voxel hold at least min(pairs, pair_capacity) entries.  Any of the
  * outputs may be NULL.  n, cams, n_views, opts and pair_capacity are those
- * of the forward call.  For tests and debugging. */
+ * of the forward call.  Only reads the workspace, so calls on several streams
+ * may share one.  For tests and debugging. */
 lv_status lv_debug_pairs(int64_t n, const lv_camera* cams, int n_views, const lv_raster_opts* opts,
                          const void* workspace, size_t ws_bytes, int64_t pair_capacity, uint64_t* keys,
                          uint32_t* voxel, uint32_t* ranges, void* stream);
@@ -305,7 +306,8 @@ lv_status lv_debug_sort_timeout(int32_t spin_limit, void* workspace, size_t ws_b
  * near-plane, ordering, colour and stop rules as the forward.  The lists
  * depend on geometry only, so corner densities and SH may be changed between
  * the forward and this call.  rgb [n_px][3] and T [n_px] (nullable) are FP64
- * device outputs. */
+ * device outputs.  Only reads the workspace, so calls on several streams may
+ * share one. */
 lv_status lv_render_pixels_f64(const lv_voxels* vox, const lv_camera* cams, int n_views, const lv_raster_opts* opts,
                                const void* workspace, size_t ws_bytes, int64_t pair_capacity, const int64_t* pixels,
                                int64_t n_px, double* rgb, double* T, void* stream);

@@ -1152,9 +1152,8 @@ __device__ __forceinline__ TileLongSmem& ts_smem() {
 
 // Sorts the m <= TS_CHUNK (key, slot) pairs of S by key, stably, with the whole
 // block (all of it past a barrier since they were written, and S.kmin and S.kmax
-// their extremes), and writes (slot, strip mask) to plist[0, m).
-__device__ __noinline__ void ts_sort_smem(int m, const TileBox& tb, const uint2* rec_bb,
-                                          uint2* plist) {
+// their extremes); ends with a barrier where it moved anything.
+__device__ __noinline__ void ts_sort_smem(int m) {
   TileSortSmem& S = ts_smem().s;
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   const int R = (m + TS_THREADS - 1) / TS_THREADS;  // items per thread, and rounds per warp
@@ -1200,7 +1199,13 @@ __device__ __noinline__ void ts_sort_smem(int m, const TileBox& tb, const uint2*
     }
     __syncthreads();
   }
-  for (int q = t; q < m; q += TS_THREADS) {
+}
+
+// the sorted pairs of S as (slot, strip mask) to plist[0, m)
+__device__ __forceinline__ void ts_write(int m, const TileBox& tb, const uint2* rec_bb,
+                                         uint2* plist) {
+  const TileSortSmem& S = ts_smem().s;
+  for (int q = threadIdx.x; q < m; q += TS_THREADS) {
     const uint32_t v = S.v[q];
     plist[q] = make_uint2(v, tb.mask(rec_bb[v]));
   }
@@ -1246,17 +1251,17 @@ __device__ __noinline__ void ts_sort_list(const uint32_t* src, const uint32_t* s
   }
   ts_min_max(mn, mx, &S.kmin, &S.kmax);
   __syncthreads();
-  ts_sort_smem(m, tb, rec_bb, plist);
+  ts_sort_smem(m);
+  ts_write(m, tb, rec_bb, plist);
 }
 
-// The entries of a long list with keys in [k0, k1], in item order: to S as
-// (key, slot) with their extremes (there are at most TS_CHUNK of them), or, with
-// ALL_EQUAL, straight to plist (any number: one key, so item order is the order).
-template <bool ALL_EQUAL>
-__device__ __forceinline__ void tl_collect(TileSortSmem& S, const uint32_t* sv,
-                                           const uint32_t* xk, uint32_t L, uint32_t k0, uint32_t k1,
-                                           const TileBox& tb, const uint2* rec_bb,
-                                           uint2* plist) {
+// The entries of a long list with keys in [k0, k1], in item order, to S as (key,
+// slot).  Without ONE_KEY there are at most TS_CHUNK of them, and their extremes go
+// to S too.  With ONE_KEY (k0 == k1: item order is the order) there may be any
+// number: flush(m) gets each round's, at most TS_CHUNK, at S's start.
+template <bool ONE_KEY, typename Flush>
+__device__ __forceinline__ void tl_collect(TileSortSmem& S, const uint32_t* sv, const uint32_t* xk, uint32_t L,
+                                           uint32_t k0, uint32_t k1, Flush&& flush) {
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   if (t == 0) {
     S.kmin = ~0u;
@@ -1274,9 +1279,10 @@ __device__ __forceinline__ void tl_collect(TileSortSmem& S, const uint32_t* sv,
       in[j] = __ballot_sync(FULL, e0 + 32 * j < L && k[j] >= k0 && k[j] <= k1);
       c += __popc(in[j]);
     }
-    __syncthreads();  // the last round's counts are read
+    __syncthreads();  // the last round's counts are read, and its entries flushed
     if (lane == 0) S.w[warp] = c;
     __syncthreads();
+    if (ONE_KEY) at = 0;
     uint32_t pos = at;
 #pragma unroll
     for (int w = 0; w < TS_WARPS; ++w) {
@@ -1287,74 +1293,41 @@ __device__ __forceinline__ void tl_collect(TileSortSmem& S, const uint32_t* sv,
 #pragma unroll
     for (int j = 0; j < TS_ITEMS; ++j) {
       if ((in[j] >> lane) & 1u) {
-        const uint32_t q = pos + __popc(in[j] & ((1u << lane) - 1u)), v = sv[e0 + 32 * j];
-        if (ALL_EQUAL) {
-          plist[q] = make_uint2(v, tb.mask(rec_bb[v]));
-        } else {
-          S.k[q] = k[j];
-          S.v[q] = v;
-          mn = min(mn, k[j]);
-          mx = max(mx, k[j]);
-        }
+        const uint32_t q = pos + __popc(in[j] & ((1u << lane) - 1u));
+        S.k[q] = k[j];
+        S.v[q] = sv[e0 + 32 * j];
+        mn = min(mn, k[j]);
+        mx = max(mx, k[j]);
       }
       pos += __popc(in[j]);
     }
+    if (ONE_KEY && at) {  // block-uniform
+      __syncthreads();
+      flush(at);
+    }
   }
-  if (!ALL_EQUAL) ts_min_max(mn, mx, &S.kmin, &S.kmax);
+  if (!ONE_KEY) ts_min_max(mn, mx, &S.kmin, &S.kmax);
   __syncthreads();
 }
 
-// Depth order of a long list, nearest entries first: a histogram of the keys not
-// sorted yet cuts them into ranges of at most TS_CHUNK entries, and each range is
-// collected in item order and sorted in shared memory.  A bin of more than
-// TS_CHUNK entries is cut by a finer histogram of its own keys; once a bin is one
-// key, item order is the order.  START: the keys are gathered first (to xk), and above
-// `lazy` entries the work stops after one range; else it goes on from the progress of
-// such a start.
-template <bool START>
-__device__ __noinline__ void tl_order(uint32_t lo, uint32_t L, uint32_t lazy, const uint32_t* sv_all,
-                         uint32_t* xk_all, const uint32_t* s_dkey, TileProg* prog,
-                         uint32_t* ready, const TileBox& tb, const uint2* rec_bb,
-                         uint2* plist_all) {
+// Depth order of a long list's entries with keys from cur up (`done` of its L
+// entries have smaller ones), nearest first: a histogram of the keys not sorted yet
+// cuts them into ranges of at most TS_CHUNK entries, and each range is collected in
+// item order and sorted in shared memory.  A bin of more than TS_CHUNK entries is
+// cut by a finer histogram of its own keys; once a bin is one key, item order is the
+// order.  sink(at, m) gets the pieces in order: the m (key, slot) pairs at S's start
+// are the list's entries from `at` on; once it returns true (to the whole block) the
+// work stops after that key.
+struct TlAt {
+  uint32_t done;  // entries handed out
+  uint32_t next;  // smallest key not handed out yet
+};
+template <typename Sink>
+__device__ __forceinline__ TlAt tl_ranges(uint32_t L, const uint32_t* sv, const uint32_t* xk, uint32_t done,
+                                          uint32_t cur, uint32_t kmax, Sink&& sink) {
   TileLongSmem& M = ts_smem();
   TileSortSmem& S = M.s;
   const int t = threadIdx.x;
-  const uint32_t* sv = sv_all + lo;
-  uint32_t* xk = xk_all + lo;
-  uint2* plist = plist_all + lo;
-  uint32_t done, cur, kmax;
-  const bool front = START && L > lazy;
-  if (START) {
-    if (t == 0) {
-      S.kmin = ~0u;
-      S.kmax = 0u;
-    }
-    __syncthreads();
-    uint32_t mn = ~0u, mx = 0u;
-    for (uint32_t base = t; base < L; base += TS_CHUNK) {
-      uint32_t v[TS_ITEMS], k[TS_ITEMS];
-#pragma unroll
-      for (int j = 0; j < TS_ITEMS; ++j) v[j] = base + j * TS_THREADS < L ? sv[base + j * TS_THREADS] : 0u;
-#pragma unroll
-      for (int j = 0; j < TS_ITEMS; ++j) k[j] = base + j * TS_THREADS < L ? s_dkey[v[j]] : 0u;
-#pragma unroll
-      for (int j = 0; j < TS_ITEMS; ++j)
-        if (base + j * TS_THREADS < L) {
-          xk[base + j * TS_THREADS] = k[j];
-          mn = min(mn, k[j]);
-          mx = max(mx, k[j]);
-        }
-    }
-    ts_min_max(mn, mx, &S.kmin, &S.kmax);
-    __syncthreads();  // also orders the block's writes of xk before its reads below
-    done = 0u;
-    cur = S.kmin;
-    kmax = S.kmax;
-  } else {
-    done = prog->done;
-    cur = prog->next;
-    kmax = prog->kmax;
-  }
   uint32_t top = kmax;  // keys [cur, top] are cut by one histogram
   while (done < L) {    // block-uniform
     const uint32_t span = top - cur;
@@ -1399,57 +1372,98 @@ __device__ __noinline__ void tl_order(uint32_t lo, uint32_t L, uint32_t lazy, co
       b0 = M.b0;
       const uint32_t b1 = M.b1;
       __syncthreads();
+      bool stop = false;
+      uint32_t k1;
       if (b1 > b0) {
         const uint32_t k0 = cur + (b0 << shift);
-        const uint32_t k1 = b1 < (uint32_t)TL_BINS && top - cur >= b1 << shift ? cur + ((b1 << shift) - 1u) : top;
+        k1 = b1 < (uint32_t)TL_BINS && top - cur >= b1 << shift ? cur + ((b1 << shift) - 1u) : top;
         const uint32_t m = M.inc[b1 - 1] - cum;
-        tl_collect<false>(S, sv, xk, L, k0, k1, tb, rec_bb, plist);
-        ts_sort_smem((int)m, tb, rec_bb, plist + done);
+        tl_collect<false>(S, sv, xk, L, k0, k1, [](uint32_t) {});
+        ts_sort_smem((int)m);
+        stop = sink(done, m);
         __syncthreads();  // S is reused
         done += m;
         cum += m;
         b0 = b1;
-        if (front) {
-          if (t == 0) {
-            prog->done = done;
-            prog->next = k1 + 1u;
-            prog->kmax = kmax;
-            *ready = lo + done;
-          }
-          return;
-        }
       } else if (shift == 0) {  // one key with more entries than TS_CHUNK
-        const uint32_t m = M.inc[b0] - cum;
-        tl_collect<true>(S, sv, xk, L, cur + b0, cur + b0, tb, rec_bb, plist + done);
-        done += m;
-        cum += m;
-        const uint32_t k1 = cur + b0;
+        k1 = cur + b0;
+        cum = M.inc[b0];
+        tl_collect<true>(S, sv, xk, L, k1, k1, [&](uint32_t m) {
+          stop |= sink(done, m);
+          done += m;
+        });
         ++b0;
-        if (front) {
-          if (t == 0) {
-            prog->done = done;
-            prog->next = k1 + 1u;
-            prog->kmax = kmax;
-            *ready = lo + done;
-          }
-          return;
-        }
       } else {  // the bin's own keys, finer
         cur += b0 << shift;
         if (top - cur >= 1u << shift) top = cur + ((1u << shift) - 1u);
         finer = true;
         break;
       }
+      if (stop) return {done, k1 + 1u};
     }
     if (!finer) {  // everything up to top is sorted
       cur = top + 1u;
       top = kmax;
     }
   }
+  return {done, kmax};
+}
+
+// A long list's depth order to plist.  START: the keys are gathered first (to xk), and
+// above `lazy` entries the work stops after one range; else it goes on from the progress
+// of such a start.
+template <bool START>
+__device__ __noinline__ void tl_order(uint32_t lo, uint32_t L, uint32_t lazy, const uint32_t* sv_all,
+                         uint32_t* xk_all, const uint32_t* s_dkey, TileProg* prog,
+                         uint32_t* ready, const TileBox& tb, const uint2* rec_bb,
+                         uint2* plist_all) {
+  TileSortSmem& S = ts_smem().s;
+  const int t = threadIdx.x;
+  const uint32_t* sv = sv_all + lo;
+  uint32_t* xk = xk_all + lo;
+  uint2* plist = plist_all + lo;
+  uint32_t done, cur, kmax;
+  const bool front = START && L > lazy;
+  if (START) {
+    if (t == 0) {
+      S.kmin = ~0u;
+      S.kmax = 0u;
+    }
+    __syncthreads();
+    uint32_t mn = ~0u, mx = 0u;
+    for (uint32_t base = t; base < L; base += TS_CHUNK) {
+      uint32_t v[TS_ITEMS], k[TS_ITEMS];
+#pragma unroll
+      for (int j = 0; j < TS_ITEMS; ++j) v[j] = base + j * TS_THREADS < L ? sv[base + j * TS_THREADS] : 0u;
+#pragma unroll
+      for (int j = 0; j < TS_ITEMS; ++j) k[j] = base + j * TS_THREADS < L ? s_dkey[v[j]] : 0u;
+#pragma unroll
+      for (int j = 0; j < TS_ITEMS; ++j)
+        if (base + j * TS_THREADS < L) {
+          xk[base + j * TS_THREADS] = k[j];
+          mn = min(mn, k[j]);
+          mx = max(mx, k[j]);
+        }
+    }
+    ts_min_max(mn, mx, &S.kmin, &S.kmax);
+    __syncthreads();  // also orders the block's writes of xk before its reads below
+    done = 0u;
+    cur = S.kmin;
+    kmax = S.kmax;
+  } else {
+    done = prog->done;
+    cur = prog->next;
+    kmax = prog->kmax;
+  }
+  const TlAt end = tl_ranges(L, sv, xk, done, cur, kmax, [&](uint32_t at, uint32_t m) {
+    ts_write((int)m, tb, rec_bb, plist + at);
+    return front;
+  });
   if (t == 0) {
-    prog->done = done;
-    prog->next = prog->kmax = kmax;
-    *ready = lo + done;
+    prog->done = end.done;
+    prog->next = end.next;
+    prog->kmax = kmax;
+    *ready = lo + end.done;
   }
 }
 
@@ -2311,26 +2325,52 @@ __global__ void k_gather_edge(const int64_t* __restrict__ argmax, int64_t n, con
   edge[i] = (a >= 0 && a < n_pix) ? edge_map[a] : 0.f;
 }
 
+// The lists of a forward workspace, for the calls that read them whole.  A list the
+// forward left partly sorted is put in order in shared memory, by the cuts k_tile_rest
+// makes, so these calls only read the workspace and any number may share one.
+struct ListView {
+  const uint2* ranges;
+  const uint32_t* ready;
+  const uint2* plist;
+  const uint32_t* tile_slots;
+  const uint32_t* long_keys;
+  const TileProg* prog;
+  const uint32_t* slot_vox;
+};
+// sink as in tl_ranges (`at` counts from the list's start); the whole block calls
+template <typename Sink>
+__device__ __forceinline__ void list_rest(const ListView& lv, uint32_t tile, uint2 r, Sink&& sink) {
+  const TileProg p = lv.prog[tile];
+  tl_ranges(r.y - r.x, lv.tile_slots + r.x, lv.long_keys + r.x, p.done, p.next, p.kmax, sink);
+}
+
 // a block per tile, in turn
-__global__ void k_debug_pairs(const uint2* ranges, int64_t tiles, const uint2* plist,
-                              const uint32_t* __restrict__ slot_vox, const uint32_t* __restrict__ s_dkey,
-                              uint64_t* ko, uint32_t* vo) {
+__global__ void __launch_bounds__(TS_THREADS) k_debug_pairs(const ListView lv, int64_t tiles,
+                                                           const uint32_t* __restrict__ s_dkey, uint64_t* ko,
+                                                           uint32_t* vo) {
   grid_begin();
   for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
-    const uint2 r = ranges[tile];
-    for (uint32_t i = r.x + threadIdx.x; i < r.y; i += blockDim.x) {
-      const uint32_t s = plist[i].x;
+    const uint2 r = lv.ranges[tile];
+    auto put = [&](uint32_t i, uint32_t s) {
       if (ko) ko[i] = ((uint64_t)tile << 32) | s_dkey[s];
-      if (vo) vo[i] = slot_vox[s];
-    }
+      if (vo) vo[i] = lv.slot_vox[s];
+    };
+    const uint32_t sorted = lv.ready[tile];
+    for (uint32_t i = r.x + threadIdx.x; i < sorted; i += TS_THREADS) put(i, lv.plist[i].x);
+    if (sorted < r.y)  // block-uniform
+      list_rest(lv, (uint32_t)tile, r, [&](uint32_t at, uint32_t m) {
+        const TileSortSmem& S = ts_smem().s;
+        for (uint32_t q = threadIdx.x; q < m; q += TS_THREADS) put(r.x + at + q, S.v[q]);
+        return false;
+      });
   }
 }
 
 // ------------------------------------------------------------------ FP64 re-render (gradient checks)
-// One thread per listed pixel: the pixel's tile list (from a forward
-// workspace) is walked front to back in FP64 from the original voxel arrays
-// (geometry, corner densities and SH converted exactly to double): the FP64
-// counterpart of k_fwd, used only to take finite differences of the loss.
+// Each listed pixel's tile list (from a forward workspace) is walked front to
+// back in FP64 from the original voxel arrays (geometry, corner densities and SH
+// converted exactly to double): the FP64 counterpart of k_fwd, used only to take
+// finite differences of the loss.
 __device__ __forceinline__ void sh_basis64(double x, double y, double z, double* Y) {
   const double pi = 3.14159265358979323846;
   Y[0] = 0.5 / sqrt(pi);
@@ -2346,42 +2386,47 @@ __device__ __forceinline__ void sh_basis64(double x, double y, double z, double*
   Y[15] = c3a * x * (x * x - 3.0 * y * y);
 }
 
+// the voxel arrays and options of an FP64 march
 template <typename DT, typename ST>
-__global__ void k_render_f64(const __grid_constant__ ViewSet vs, const uint32_t* ranges,
-                             const uint2* plist, const uint32_t* __restrict__ slot_vox,
-                             const float4* __restrict__ geom, const DT* __restrict__ dens, const ST* __restrict__ sh,
-                             int sh_nb, const int64_t* __restrict__ pixels, int64_t n_px, double t_stop,
-                             int segment, const uint32_t* __restrict__ vidx, double* rgb_out,
-                             double* T_out) {
-  grid_begin();
-  const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (q >= n_px) return;
-  const long long gp = pixels[q];
-  int view = 0;
-  while (view + 1 < vs.n && gp >= vs.v[view + 1].pix_off) ++view;
-  const DevView& c = vs.v[view];
-  const long long loc = gp - c.pix_off;
-  const int px = (int)(loc % c.W), py = (int)(loc / c.W);
-  const int ts = vs.ts;
-  const int gtile = c.tile_off + (py / ts) * c.tiles_x + px / ts;
-  double o[3], d[3];
-  for (int k = 0; k < 3; ++k)
-    o[k] = -((double)c.R[k] * c.t[0] + (double)c.R[3 + k] * c.t[1] + (double)c.R[6 + k] * c.t[2]);
-  const double dcx = ((double)px + 0.5 - (double)c.cx) / (double)c.fx;
-  const double dcy = ((double)py + 0.5 - (double)c.cy) / (double)c.fy;
-  double nn = 0.0;
-  for (int k = 0; k < 3; ++k) {
-    d[k] = (double)c.R[k] * dcx + (double)c.R[3 + k] * dcy + (double)c.R[6 + k];
-    nn += d[k] * d[k];
+struct Scene64 {
+  const float4* geom;
+  const DT* dens;
+  const ST* sh;
+  const uint32_t* vidx;
+  int sh_nb, segment;
+  double t_stop;
+};
+
+// one pixel's FP64 march
+struct March64 {
+  int gtile;
+  double o[3], d[3], t_near;
+  double T, cr, cg, cb;
+
+  __device__ March64(const ViewSet& vs, long long gp) {
+    int view = 0;
+    while (view + 1 < vs.n && gp >= vs.v[view + 1].pix_off) ++view;
+    const DevView& c = vs.v[view];
+    const long long loc = gp - c.pix_off;
+    const int px = (int)(loc % c.W), py = (int)(loc / c.W);
+    const int ts = vs.ts;
+    gtile = c.tile_off + (py / ts) * c.tiles_x + px / ts;
+    for (int k = 0; k < 3; ++k)
+      o[k] = -((double)c.R[k] * c.t[0] + (double)c.R[3 + k] * c.t[1] + (double)c.R[6 + k] * c.t[2]);
+    const double dcx = ((double)px + 0.5 - (double)c.cx) / (double)c.fx;
+    const double dcy = ((double)py + 0.5 - (double)c.cy) / (double)c.fy;
+    double nn = 0.0;
+    for (int k = 0; k < 3; ++k) {
+      d[k] = (double)c.R[k] * dcx + (double)c.R[3 + k] * dcy + (double)c.R[6 + k];
+      nn += d[k] * d[k];
+    }
+    nn = sqrt(nn);
+    for (int k = 0; k < 3; ++k) d[k] /= nn;
+    t_near = (double)c.z_near * nn;  // camera depth z_near along this ray
+    T = 1.0;
+    cr = cg = cb = 0.0;
   }
-  nn = sqrt(nn);
-  for (int k = 0; k < 3; ++k) d[k] /= nn;
-  const double t_near = (double)c.z_near * nn;  // camera depth z_near along this ray
-  double T = 1.0, cr = 0.0, cg = 0.0, cb = 0.0;
-  const uint32_t start = ranges[2 * gtile], end = ranges[2 * gtile + 1];
-  for (uint32_t e = start; e < end; ++e) {
-    const uint32_t vox = slot_vox[plist[e].x];
-    const float4 g = geom[vox];
+  __device__ bool chord(float4 g, double* lo_out, double* hi_out) const {
     const double h = (double)g.w, cc[3] = {(double)g.x, (double)g.y, (double)g.z};
     double lo_t = t_near, hi_t = 1e300;
     bool miss = false;
@@ -2395,20 +2440,30 @@ __global__ void k_render_f64(const __grid_constant__ ViewSet vs, const uint32_t*
       lo_t = fmax(lo_t, fmin(t1, t2));
       hi_t = fmin(hi_t, fmax(t1, t2));
     }
-    if (miss || !(hi_t - lo_t > 0.0)) continue;
+    *lo_out = lo_t;
+    *hi_out = hi_t;
+    return !(miss || !(hi_t - lo_t > 0.0));
+  }
+  // the list's next voxel; true once the ray stops
+  template <typename DT, typename ST>
+  __device__ bool add(const Scene64<DT, ST>& sc, uint32_t vox) {
+    const float4 g = sc.geom[vox];
+    const double h = (double)g.w, cc[3] = {(double)g.x, (double)g.y, (double)g.z};
+    double lo_t, hi_t;
+    if (!chord(g, &lo_t, &hi_t)) return false;
     const double l = hi_t - lo_t, tm = 0.5 * (lo_t + hi_t);
     // the trilinear field at the midpoint, or its mean over the chord (Simpson, exact for the cubic)
-    const double ts3[3] = {tm, lo_t, hi_t}, ws3[3] = {segment ? 4.0 / 6.0 : 1.0, 1.0 / 6.0, 1.0 / 6.0};
+    const double ts3[3] = {tm, lo_t, hi_t}, ws3[3] = {sc.segment ? 4.0 / 6.0 : 1.0, 1.0 / 6.0, 1.0 / 6.0};
     double sr = 0.0;
-    for (int q3 = 0; q3 < (segment ? 3 : 1); ++q3) {
+    for (int q3 = 0; q3 < (sc.segment ? 3 : 1); ++q3) {
       double u[3];
       for (int a = 0; a < 3; ++a)
         u[a] = fmin(fmax((o[a] + ts3[q3] * d[a] - (cc[a] - h)) / (2.0 * h), 0.0), 1.0);
       for (int i = 0; i < 8; ++i) {
         const double w =
             ((i & 1) ? u[0] : 1.0 - u[0]) * ((i & 2) ? u[1] : 1.0 - u[1]) * ((i & 4) ? u[2] : 1.0 - u[2]);
-        const size_t di = vidx ? (size_t)vidx[8 * (size_t)vox + i] : 8 * (size_t)vox + i;
-        sr += ws3[q3] * w * (double)to_f32(dens[di]);
+        const size_t di = sc.vidx ? (size_t)sc.vidx[8 * (size_t)vox + i] : 8 * (size_t)vox + i;
+        sr += ws3[q3] * w * (double)to_f32(sc.dens[di]);
       }
     }
     const double sigma = fmax(sr, 0.0);
@@ -2419,19 +2474,85 @@ __global__ void k_render_f64(const __grid_constant__ ViewSet vs, const uint32_t*
     double Y[16];
     sh_basis64(dir[0], dir[1], dir[2], Y);
     double col[3] = {0.5, 0.5, 0.5};
-    for (int j = 0; j < sh_nb; ++j)
-      for (int ch = 0; ch < 3; ++ch) col[ch] += (double)to_f32(sh[48 * (size_t)vox + 3 * j + ch]) * Y[j];
+    for (int j = 0; j < sc.sh_nb; ++j)
+      for (int ch = 0; ch < 3; ++ch) col[ch] += (double)to_f32(sc.sh[48 * (size_t)vox + 3 * j + ch]) * Y[j];
     const double w = T * alpha;
     cr += w * fmax(col[0], 0.0);
     cg += w * fmax(col[1], 0.0);
     cb += w * fmax(col[2], 0.0);
     T *= exp(-sigma * l);
-    if (T < t_stop) break;
+    return T < sc.t_stop;
   }
-  rgb_out[3 * q + 0] = cr;
-  rgb_out[3 * q + 1] = cg;
-  rgb_out[3 * q + 2] = cb;
-  if (T_out) T_out[q] = T;
+  __device__ void store(double* rgb_out, double* T_out, int64_t q) const {
+    rgb_out[3 * q + 0] = cr;
+    rgb_out[3 * q + 1] = cg;
+    rgb_out[3 * q + 2] = cb;
+    if (T_out) T_out[q] = T;
+  }
+};
+
+// a thread per pixel; those whose list is not sorted to its end are k_render_f64_rest's
+template <typename DT, typename ST>
+__global__ void k_render_f64(const __grid_constant__ ViewSet vs, const ListView lv, const Scene64<DT, ST> sc,
+                             const int64_t* __restrict__ pixels, int64_t n_px, double* __restrict__ rgb_out,
+                             double* __restrict__ T_out) {
+  grid_begin();
+  const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (q >= n_px) return;
+  March64 m(vs, pixels[q]);
+  const uint2 r = lv.ranges[m.gtile];
+  if (lv.ready[m.gtile] < r.y) return;
+  for (uint32_t e = r.x; e < r.y; ++e)
+    if (m.add(sc, lv.slot_vox[lv.plist[e].x])) break;
+  m.store(rgb_out, T_out, q);
+}
+
+// a block per pixel, in turn: it tests 512 of the list's entries at a time, and its first thread
+// marches through those the ray meets
+template <typename DT, typename ST>
+__global__ void __launch_bounds__(TS_THREADS) k_render_f64_rest(const __grid_constant__ ViewSet vs, const ListView lv,
+                                                               const Scene64<DT, ST> sc,
+                                                               const int64_t* __restrict__ pixels, int64_t n_px,
+                                                               double* __restrict__ rgb_out,
+                                                               double* __restrict__ T_out) {
+  grid_begin();
+  __shared__ uint32_t s_hit[TS_WARPS];
+  __shared__ int s_done;
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  for (int64_t q = blockIdx.x; q < n_px; q += gridDim.x) {  // block-uniform
+    March64 m(vs, pixels[q]);
+    const uint2 r = lv.ranges[m.gtile];
+    const uint32_t sorted = lv.ready[m.gtile];
+    if (sorted >= r.y) continue;
+    __syncthreads();  // the last pixel's s_done is read
+    if (t == 0) s_done = 0;
+    __syncthreads();
+    // entries [0, n) with the voxel of entry e given by vox_at(e); true once the ray stops
+    auto march = [&](uint32_t n, auto&& vox_at) {
+      for (uint32_t e0 = 0; e0 < n && !s_done; e0 += TS_THREADS) {  // block-uniform
+        double lo_t, hi_t;
+        const bool hit = e0 + t < n && m.chord(sc.geom[vox_at(e0 + t)], &lo_t, &hi_t);
+        const uint32_t who = __ballot_sync(FULL, hit);
+        if (lane == 0) s_hit[warp] = who;
+        __syncthreads();
+        if (t == 0) {
+          bool done = false;
+          for (int w = 0; w < TS_WARPS && !done; ++w)
+            for (uint32_t h = s_hit[w]; h && !done; h &= h - 1)
+              done = m.add(sc, vox_at(e0 + 32 * w + __ffs(h) - 1));
+          if (done) s_done = 1;
+        }
+        __syncthreads();
+      }
+      return s_done != 0;
+    };
+    if (!march(sorted - r.x, [&](uint32_t e) { return lv.slot_vox[lv.plist[r.x + e].x]; }))
+      list_rest(lv, (uint32_t)m.gtile, r, [&](uint32_t, uint32_t n) {
+        const TileSortSmem& S = ts_smem().s;
+        return march(n, [&](uint32_t e) { return lv.slot_vox[S.v[e]]; });
+      });
+    if (t == 0) m.store(rgb_out, T_out, q);
+  }
 }
 
 // ------------------------------------------------------------------ host side
@@ -2594,14 +2715,43 @@ static void launch_tile_sort(const FwdWs& w, const ViewSet& vs, int64_t n, int64
       w.ready, w.prog, n > TS_LAZY_VOXELS ? TS_LAZY : ~0u, vs, w.rec_bb, w.plist);
   count_launch(1);
 }
-// the rest of the open tiles' lists, or (all) of every long list, for the calls that read whole lists
-static void launch_tile_rest(const FwdWs& w, const ViewSet& vs, int64_t tiles, bool all, cudaStream_t s) {
+// the rest of the open tiles' lists
+static void launch_tile_rest(const FwdWs& w, const ViewSet& vs, int64_t tiles, cudaStream_t s) {
   const int64_t nb = std::min<int64_t>(tile_sort_blocks(), tiles);
-  if (all) zero_async(s, w.work + 3, sizeof(unsigned int));
   chain(k_tile_rest, (unsigned)nb, TS_THREADS, sizeof(TileLongSmem), s)(
-      w.tile_slots, w.long_keys, w.ranges, all ? w.class_tiles : w.open_tiles,
-      w.work + (all ? 16 : 7), w.work + 3, w.ready, w.prog, vs, w.rec_bb, w.plist);
+      w.tile_slots, w.long_keys, w.ranges, w.open_tiles, w.work + 7, w.work + 3, w.ready, w.prog, vs, w.rec_bb,
+      w.plist);
   count_launch(1);
+}
+
+static ListView list_view(const FwdWs& w) {
+  return {(const uint2*)w.ranges, w.ready, w.plist, w.tile_slots, w.long_keys, w.prog, w.slot_vox};
+}
+
+// dynamic shared memory for the kernels that put a list's rest in order (once per kernel and device)
+template <typename K>
+static void allow_long_smem(K kernel, std::atomic<unsigned long long>& done) {
+  once_per_device(done, [&] {
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TileLongSmem));
+  });
+}
+
+template <typename DT, typename ST>
+static void launch_render_f64(const lv_voxels* vox, const lv_raster_opts* o, const ViewSet& vs, const FwdWs& w,
+                              const int64_t* pixels, int64_t n_px, double* rgb, double* T, cudaStream_t s) {
+  const Scene64<DT, ST> sc = {(const float4*)vox->geom, (const DT*)vox->density, (const ST*)vox->sh, vox->vidx,
+                              (vox->sh_degree + 1) * (vox->sh_degree + 1),
+                              (o->flags & LV_FLAG_EXACT_SEGMENT) ? 1 : 0, (double)o->t_stop};
+  const ListView lv = list_view(w);
+  launch(k_render_f64<DT, ST>, (unsigned)((n_px + 127) / 128), 128, 0, s)(vs, lv, sc, pixels, n_px, rgb, T);
+  count_launch(1);
+  if (vox->n > TS_LAZY_VOXELS) {  // else every list is sorted whole
+    static std::atomic<unsigned long long> done{0};
+    allow_long_smem(k_render_f64_rest<DT, ST>, done);
+    const unsigned grid = (unsigned)std::min<int64_t>(n_px, 1216);
+    chain(k_render_f64_rest<DT, ST>, grid, TS_THREADS, sizeof(TileLongSmem), s)(vs, lv, sc, pixels, n_px, rgb, T);
+    count_launch(1);
+  }
 }
 
 static void launch_fwd(const lv_raster_opts* o, int64_t tiles, cudaStream_t s, const ViewSet& vs, const FwdWs& w,
@@ -2723,7 +2873,7 @@ extern "C" lv_status lv_rasterize_forward(const lv_voxels* vox, const lv_camera*
   launch_fwd(opts, tiles, s, vs, w, out, false);
   count_launch(2);
   if (n > TS_LAZY_VOXELS) {
-    launch_tile_rest(w, vs, tiles, false, s);
+    launch_tile_rest(w, vs, tiles, s);
     launch_fwd(opts, tiles, s, vs, w, out, true);
     count_launch(1);
   }
@@ -2889,8 +3039,9 @@ extern "C" lv_status lv_debug_pairs(int64_t n, const lv_camera* cams, int n_view
   FwdWs w = carve_fwd((void*)workspace, n, n_views, tiles, pixels, pair_capacity);
   if (ws_bytes < w.bytes) { set_error("workspace too small"); return LV_ERR_WORKSPACE; }
   if (keys || voxel) {
-    launch_tile_rest(w, vs, tiles, true, s);
-    chain(k_debug_pairs, 608, 256, 0, s)((const uint2*)w.ranges, tiles, w.plist, w.slot_vox, w.s_dkey, keys, voxel);
+    static std::atomic<unsigned long long> done{0};
+    allow_long_smem(k_debug_pairs, done);
+    launch(k_debug_pairs, 608, TS_THREADS, sizeof(TileLongSmem), s)(list_view(w), tiles, w.s_dkey, keys, voxel);
     count_launch(1);
   }
   if (ranges) cudaMemcpyAsync(ranges, w.ranges, sizeof(uint32_t) * 2 * tiles, cudaMemcpyDeviceToDevice, s);
@@ -2911,19 +3062,13 @@ extern "C" lv_status lv_render_pixels_f64(const lv_voxels* vox, const lv_camera*
   make_views(cams, n_views, opts->tile, &vs, &tiles, &npix);
   FwdWs w = carve_fwd((void*)workspace, vox->n, n_views, tiles, npix, pair_capacity);
   if (ws_bytes < w.bytes) { set_error("workspace too small"); return LV_ERR_WORKSPACE; }
-  launch_tile_rest(w, vs, tiles, true, s);
-  const int nb = (vox->sh_degree + 1) * (vox->sh_degree + 1);
-  const unsigned grid = (unsigned)((n_px + 127) / 128);
-#define LV_F64(DT, ST)                                                                                            \
-  chain(k_render_f64<DT, ST>, grid, 128, 0, s)(vs, w.ranges, w.plist, w.slot_vox, (const float4*)vox->geom,              \
-                                            (const DT*)vox->density, (const ST*)vox->sh, nb, pixels, n_px,       \
-                                            (double)opts->t_stop, (opts->flags & LV_FLAG_EXACT_SEGMENT) ? 1 : 0,  \
-                                            vox->vidx, rgb, T)
-  if (vox->density_dtype == LV_F32 && vox->sh_dtype == LV_F32) LV_F64(float, float);
-  else if (vox->density_dtype == LV_F16 && vox->sh_dtype == LV_F32) LV_F64(__half, float);
-  else if (vox->density_dtype == LV_F32 && vox->sh_dtype == LV_BF16) LV_F64(float, __nv_bfloat16);
-  else LV_F64(__half, __nv_bfloat16);
-#undef LV_F64
-  count_launch(1);
+  if (vox->density_dtype == LV_F32 && vox->sh_dtype == LV_F32)
+    launch_render_f64<float, float>(vox, opts, vs, w, pixels, n_px, rgb, T, s);
+  else if (vox->density_dtype == LV_F16 && vox->sh_dtype == LV_F32)
+    launch_render_f64<__half, float>(vox, opts, vs, w, pixels, n_px, rgb, T, s);
+  else if (vox->density_dtype == LV_F32 && vox->sh_dtype == LV_BF16)
+    launch_render_f64<float, __nv_bfloat16>(vox, opts, vs, w, pixels, n_px, rgb, T, s);
+  else
+    launch_render_f64<__half, __nv_bfloat16>(vox, opts, vs, w, pixels, n_px, rgb, T, s);
   return cuda_check(cudaGetLastError(), "lv_render_pixels_f64");
 }
