@@ -1658,6 +1658,15 @@ __device__ __forceinline__ uint32_t next_item(unsigned int* work, int lane) {
   if (lane == 0) it = atomicAdd(work, 1u);
   return __shfl_sync(FULL, it, 0);
 }
+// the same for a block of CW warps, which take CW items together (every thread calls)
+template <int CW>
+__device__ __forceinline__ uint32_t next_items(unsigned int* work) {
+  __shared__ uint32_t s_at;
+  __syncthreads();  // the last items' number is read
+  if (threadIdx.x == 0) s_at = atomicAdd(work, 1u);
+  __syncthreads();
+  return s_at * CW + (threadIdx.x >> 5);
+}
 
 // A persistent grid limited to sm_cut of the n_sms SMs (0: all) is launched at
 // full size; a block that lands on an SM outside the first sm_cut (by SM id,
@@ -1695,23 +1704,37 @@ __device__ __forceinline__ bool sm_leave(int sm_cut, int n_sms, unsigned int* ar
 // ------------------------------------------------------------------ forward composite
 // Each warp walks its strip's list on its own, with no block-wide barrier, and
 // stops as soon as all its pixels have.  The list entries carry the strips they
-// meet, so a warp reads WALK_ENTRIES of them at a time (coalesced 8-byte words,
-// four per lane) and queues the few that meet its strip; the records of 32
-// queued entries are then copied to shared memory and every lane marches its
-// pixel through them.  A pixel that stays open walks thousands of entries, and
+// meet, so a warp reads a round of them at a time (coalesced 8-byte words,
+// three or four per lane) and queues the few that meet its strip; the records of a
+// batch of queued entries are then copied to shared memory and every lane marches
+// its pixel through them.  A pixel that stays open walks thousands of entries, and
 // the walk is then one serial chain per warp, so its memory latency is taken out
 // of the chain: the entries of the next round are loaded before they are needed,
-// and the records of the next 32 are copied (cp.async) while the current 32 are
-// marched.  The rounds and batches are the same for every lv_raster_opts.batch,
-// which chose the entries per round when a round gathered pixel boxes and records.
+// and the records of the next batch are copied (cp.async) while the current ones are
+// marched.  The rounds and batches are the same for every lv_raster_opts.batch.
 //
-// per-warp slice of shared memory: two buffers of 32 records (64 B) and voxel
-// ids, and the queue of (slot, list entry): at most 32 marched, 32 in flight, 31
-// left over and one round of new ones
-constexpr int WALK_ENTRIES = 128;
-constexpr int QUEUE_LEN = 256;
-static_assert(32 + 32 + 31 + WALK_ENTRIES <= QUEUE_LEN, "the queue holds every entry in use");
-constexpr size_t WARP_SLICE = 2 * 32 * (64 + 4) + (size_t)QUEUE_LEN * 8;
+// Where strips fill the SMs the composites are bound by instruction issue, and in an
+// opaque scene most strips stop within some 20 records, so what is read, copied and
+// computed ahead is wasted: the first batch takes 16 records and more only if the round
+// holds them, the forward copies nothing ahead before that is marched, a march ends
+// where its last pixel does, and a record's chord is computed when its turn comes.  One
+// 1237 x 822 view of 2M opaque voxels, tile 16, forward (with statistics) + backward:
+// 62M + 99M warp instructions, 75 + 109 us, against 84M + 111M and 91 + 123 us with
+// batches of 32 copied ahead from the start and every chord a record ahead.
+// With LOOK they look ahead like that: where few strips are in flight the latency of one
+// march counts, and the next record's chord does not wait for a sample (256 x 256 view of
+// an open scene, 2048 strips: 1.57 ms against 1.76).
+//
+// per-warp slice of shared memory: two buffers of 32 records (64 B), voxel ids and
+// (slot, list entry), and the queue: at most 31 entries left over and one round of new ones
+template <bool LOOK>
+struct WalkShape {
+  static constexpr int ENTRIES = LOOK ? 128 : 96;
+  static constexpr uint32_t FIRST = LOOK ? 32 : 16;
+  static constexpr int QUEUE = LOOK ? 256 : 128;
+  static constexpr size_t SLICE = 2 * 32 * (64 + 4 + 8) + (size_t)QUEUE * 8;
+  static_assert(31 + ENTRIES <= QUEUE, "the queue holds every waiting entry");
+};
 
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
@@ -1726,61 +1749,63 @@ template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
 // The records of one strip in list order (REV: from the last entry to the
-// first), 32 at a time.  All members are called by the whole warp.
-template <bool REV>
+// first), a batch of up to 32 at a time.  All members are called by the whole warp.
+template <bool REV, bool LOOK>
 struct StripWalk {
-  static constexpr int K = WALK_ENTRIES / 32;
-  static constexpr uint32_t QM = QUEUE_LEN - 1;
+  using Shape = WalkShape<LOOK>;
+  static constexpr int K = Shape::ENTRIES / 32;
+  static constexpr uint32_t QM = Shape::QUEUE - 1;
   const uint2* plist;
   const float4* rec;
   const uint32_t* slot_vox;
   float4* s_rec;     // [2][32][4]
   uint32_t* s_vox;   // [2][32]
+  uint2* s_ent;      // [2][32] (slot, entry)
   uint2* s_q;        // (slot, entry)
   uint32_t lo, hi;   // entries [lo, hi) not scanned yet, those in `ahead` not counted
   uint32_t base;     // first entry of `ahead`
   uint2 ahead[K];
   uint32_t head, tail;  // queue positions: next to copy, next to fill
+  uint32_t want;        // records that a batch waits for
   uint32_t bit;
   bool live;            // `ahead` holds entries not queued yet
   int lane;
 
+  __device__ __forceinline__ StripWalk(const uint2* plist_, const float4* rec_, const uint32_t* slot_vox_,
+                                       char* smem, int warp, int lane_)
+      : plist(plist_), rec(rec_), slot_vox(slot_vox_), lane(lane_) {
+    s_rec = (float4*)(smem + Shape::SLICE * warp);
+    s_vox = (uint32_t*)(s_rec + 2 * 32 * 4);
+    s_ent = (uint2*)(s_vox + 2 * 32);
+    s_q = s_ent + 2 * 32;
+  }
   __device__ __forceinline__ void load_ahead() {
-    if (REV) {
-      base = hi - lo > (uint32_t)WALK_ENTRIES ? hi - WALK_ENTRIES : lo;
+    const uint32_t r = min((uint32_t)Shape::ENTRIES, hi - lo);
+    base = REV ? hi - r : lo;
+    const uint2* p = plist + (base + lane);
 #pragma unroll
-      for (int k = 0; k < K; ++k) {
-        const uint32_t e = base + 32 * k + lane;
-        ahead[k] = e < hi ? plist[e] : make_uint2(0u, 0u);
-      }
-      hi = base;
-    } else {
-      base = lo;
-#pragma unroll
-      for (int k = 0; k < K; ++k) {
-        const uint32_t e = base + 32 * k + lane;
-        ahead[k] = e < hi ? plist[e] : make_uint2(0u, 0u);
-      }
-      lo = hi - lo > (uint32_t)WALK_ENTRIES ? lo + WALK_ENTRIES : hi;
-    }
+    for (int k = 0; k < K; ++k) ahead[k] = 32 * k + lane < r ? p[32 * k] : make_uint2(0u, 0u);
+    if (REV) hi = base;
+    else lo += r;
   }
   __device__ __forceinline__ void begin(uint32_t start, uint32_t end, int strip) {
     lo = start;
     hi = end;
     head = tail = 0u;
+    want = Shape::FIRST;
     bit = 1u << strip;
     live = start < end;
     load_ahead();
   }
-  // queue entries until 32 wait or the list ends
+  // queue entries until a batch of them waits or the list ends
   __device__ __forceinline__ void fill() {
-    while (tail - head < 32u && live) {
+    while (tail - head < want && live) {
       const uint32_t b = base;
       uint2 cur[K];
 #pragma unroll
       for (int k = 0; k < K; ++k) cur[k] = ahead[k];
       live = lo < hi;
-      load_ahead();
+      if (live) load_ahead();
 #pragma unroll
       for (int kk = 0; kk < K; ++kk) {
         const int k = REV ? K - 1 - kk : kk;
@@ -1795,19 +1820,27 @@ struct StripWalk {
     }
     __syncwarp();
   }
-  // start copying the next (up to) 32 records into buffer b; returns their number
+  // start copying the next batch's records into buffer b; returns their number
   __device__ __forceinline__ int copy(int b) {
     const int m = (int)min(32u, tail - head);
-    // four lanes per record: a record's 64 bytes in one request
+    want = 32u;
+    if (m) {
+      // four lanes per record: a record's 64 bytes in one request
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const int r = 8 * k + (lane >> 2);
-      if (r < m) {
-        const uint32_t sl = s_q[(head + r) & QM].x;
-        cp_async16(s_rec + 128 * b + 4 * r + (lane & 3), rec + 4 * (size_t)sl + (lane & 3));
+      for (int k = 0; k < 4; ++k) {
+        const int r = 8 * k + (lane >> 2);
+        if (r < m) {
+          const uint32_t sl = s_q[(head + r) & QM].x;
+          cp_async16(s_rec + 128 * b + 4 * r + (lane & 3), rec + 4 * (size_t)sl + (lane & 3));
+        }
       }
+      if (lane < m) {
+        const uint2 e = s_q[(head + lane) & QM];
+        cp_async4(s_vox + 32 * b + lane, slot_vox + e.x);
+        s_ent[32 * b + lane] = e;
+      }
+      __syncwarp();  // the queue's words are read before they are filled again
     }
-    if (lane < m) cp_async4(s_vox + 32 * b + lane, slot_vox + s_q[(head + lane) & QM].x);
     cp_async_commit();
     head += m;
     return m;
@@ -1841,24 +1874,30 @@ struct Front {
   unsigned int* n_open;
   float* dep;
   uint32_t* nsamp;
-  bool resume;
 };
 
 // A strip's march needs no other warp, so a block is a few warps whatever the
 // tile size, few where each warp has one item (a block's place is free once its
-// last warp ends), and as many blocks share an SM as leave a thread the 72
-// (forward) to 80 registers below which the march spills: the composites are
-// bound by instruction issue, for which 24 to 28 warps are enough.  1237 x 822
-// view of 2M voxels with long open lists, tile 16, forward + backward: 493 + 480 us
-// at 48 registers, 286 + 330 at 64 (8 warps a block), 261 + 310 at 80, 320 + 335 at
-// 128; fog view of 979 x 545 79 + 130 at 8 warps a block, 75 + 125 at 4.
+// last warp ends).  Blocks of 4 share their tile's list entries and records in L1, so the
+// persistent forward takes 4 items at a time as well, with a barrier (an item per warp
+// and atomic, 8 warps a block: 97 us against 88 on an opaque view, 578 against 559 on an
+// open one, tile 32); the persistent backward, whose strips differ more, takes single items.
+// As many blocks share an SM as leave a thread 64 (forward) and 72 (backward)
+// registers: with fewer the march spills, with more too few warps hide the
+// memory's latency.  1237 x 822 views of 2M voxels, opaque and open, tile 16, forward:
+// 78 and 494 us at 72 registers, 74 and 490 at 64, 77 and 499 at 56; backward 115 and 714 us
+// at 80, 109 and 684 at 72, 115 and 715 at 64.  Looking ahead takes 8 more of them.
+template <int TS, bool PERSIST, bool LOOK>
+__host__ __device__ constexpr int fwd_warps() { return PERSIST ? (LOOK ? 8 : 4) : (TS == 8 ? 1 : 4); }
+template <int TS, bool PERSIST, bool LOOK>
+__host__ __device__ constexpr int fwd_blocks() { return (LOOK ? 28 : 32) / fwd_warps<TS, PERSIST, LOOK>(); }
 template <int TS, bool PERSIST>
-__host__ __device__ constexpr int comp_warps() { return PERSIST ? 8 : (TS == 8 ? 1 : 4); }
-template <int TS, bool PERSIST>
-__host__ __device__ constexpr int comp_blocks(int warps_sm) { return warps_sm / comp_warps<TS, PERSIST>(); }
+__host__ __device__ constexpr int bwd_warps() { return PERSIST ? 8 : (TS == 8 ? 1 : 4); }
+template <int TS, bool PERSIST, bool LOOK>
+__host__ __device__ constexpr int bwd_blocks() { return (PERSIST || LOOK ? 24 : 28) / bwd_warps<TS, PERSIST>(); }
 
-template <int TS, bool SEG, bool PERSIST>
-__global__ void __launch_bounds__(comp_warps<TS, PERSIST>() * 32, comp_blocks<TS, PERSIST>(28)) k_fwd(const __grid_constant__ ViewSet vs, const uint32_t* ranges,
+template <int TS, bool SEG, bool PERSIST, bool LOOK>
+__global__ void __launch_bounds__(fwd_warps<TS, PERSIST, LOOK>() * 32, fwd_blocks<TS, PERSIST, LOOK>()) k_fwd(const __grid_constant__ ViewSet vs, const uint32_t* ranges,
                                                 const uint2* plist, const float4* rec,
                                                 const uint32_t* slot_vox, float t_stop,
                                                 float* rgb, float* depth,
@@ -1868,29 +1907,28 @@ __global__ void __launch_bounds__(comp_warps<TS, PERSIST>() * 32, comp_blocks<TS
                                                 uint32_t n_items, int sm_cut, int n_sms, unsigned int* arrivals,
                                                 const TileOrder order, const Front fr) {
   grid_wait();
-  constexpr int NW = TS * TS / 32, CW = comp_warps<TS, PERSIST>();
+  constexpr int NW = TS * TS / 32, CW = fwd_warps<TS, PERSIST, LOOK>();
+  constexpr bool RESUME = PERSIST && LOOK;  // the second launch, over the open tiles
   extern __shared__ float4 smem_f4[];
   if (PERSIST && sm_leave(sm_cut, n_sms, arrivals)) return;  // block-uniform
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (PERSIST && fr.resume) {  // grid-uniform
+  if (RESUME) {
     n_items = *fr.n_open * NW;
     if (n_items == 0u) return;
   }
-  StripWalk<false> walk;
-  walk.plist = plist;
-  walk.rec = rec;
-  walk.slot_vox = slot_vox;
-  walk.lane = lane;
-  walk.s_rec = (float4*)((char*)smem_f4 + WARP_SLICE * warp);
-  walk.s_vox = (uint32_t*)(walk.s_rec + 2 * 32 * 4);
-  walk.s_q = (uint2*)(walk.s_vox + 2 * 32);
-  for (uint32_t item = PERSIST ? next_item(work, lane) : blockIdx.x * CW + warp; item < n_items;
-       item = PERSIST ? next_item(work, lane) : n_items) {  // warp-uniform
-    const int gtile = PERSIST && fr.resume ? (int)fr.open_tiles[item / NW] : (int)order.tile(item / NW);
+  StripWalk<false, LOOK> walk(plist, rec, slot_vox, (char*)smem_f4, warp, lane);
+  constexpr bool BY_BLOCK = PERSIST && !RESUME;  // items taken CW at a time
+  auto next = [&]() {
+    return BY_BLOCK ? next_items<CW>(work) : (PERSIST ? next_item(work, lane) : n_items);
+  };
+  for (uint32_t item = PERSIST ? next() : blockIdx.x * CW + warp; item - (BY_BLOCK ? warp : 0) < n_items;
+       item = next()) {  // warp-uniform
+    if (BY_BLOCK && item >= n_items) continue;
+    const int gtile = RESUME ? (int)fr.open_tiles[item / NW] : (int)order.tile(item / NW);
     const int view = find_view(vs, gtile);
     const DevView& c = vs.v[view];
     const uint32_t start = ranges[2 * gtile], end = fr.ready[gtile];
-    walk.begin(PERSIST && fr.resume ? fr.prog[gtile].front : start, end, (int)(item % NW));
+    walk.begin(RESUME ? fr.prog[gtile].front : start, end, (int)(item % NW));
     const int lt = gtile - c.tile_off;
     const int tile_x = lt % c.tiles_x, tile_y = lt / c.tiles_x;
     const Strip<TS> strip(tile_x, tile_y, (int)(item % NW));
@@ -1902,7 +1940,7 @@ __global__ void __launch_bounds__(comp_warps<TS, PERSIST>() * 32, comp_blocks<TS
     float T = 1.f, tau = 0.f, cr = 0.f, cg = 0.f, cb = 0.f, dep = 0.f;
     uint32_t last = 0, nsamp = 0;
     bool done = !inside;
-    if (PERSIST && fr.resume) {
+    if (RESUME) {
       if (inside) {
         const size_t p = (size_t)gid;
         T = T_out[p];
@@ -1922,33 +1960,53 @@ __global__ void __launch_bounds__(comp_warps<TS, PERSIST>() * 32, comp_blocks<TS
     }
     walk.fill();
     int m = walk.copy(0);
+    bool ahead = LOOK;  // batches are copied ahead from the second one on
     for (int b = 0; m; b ^= 1) {  // warp-uniform
-      const uint32_t q0 = walk.head - (uint32_t)m;  // this batch's queue entries
-      walk.fill();
-      const int m_next = walk.copy(b ^ 1);
-      cp_async_wait<1>();
+      int m_next = 0;
+      if (ahead) {
+        walk.fill();
+        m_next = walk.copy(b ^ 1);
+        cp_async_wait<1>();
+      } else {
+        cp_async_wait<0>();
+      }
       __syncwarp();
       const float4* wr = walk.s_rec + 128 * b;
       const uint32_t* w_vox = walk.s_vox + 32 * b;
       int last_j = -1;  // the lane's last sample of this batch (its list entry is read once, below)
-      float4 g = wr[0];
-      float t_in, t_out;
-      bool h = chord(r, g, t_in, t_out);
+      float4 g_n;
+      float in_n, out_n;
+      bool h_n = false;
+      if (LOOK) {
+        g_n = wr[0];
+        h_n = chord(r, g_n, in_n, out_n);
+      }
       for (int j = 0; j < m; ++j) {
-        const bool hit = h && !done;
-        const float4 gj = g;
-        const float ti = t_in, to = t_out;
-        // the next record's chord does not wait for this sample (past the last one: whatever follows in
-        // the slice, and the result is not used)
-        g = wr[4 * (j + 1)];
-        h = chord(r, g, t_in, t_out);
-        if (!__any_sync(FULL, hit)) continue;
+        float4 g;
+        float t_in, t_out;
+        bool hit;
+        if (LOOK) {
+          hit = h_n && !done;
+          g = g_n;
+          t_in = in_n;
+          t_out = out_n;
+          // (past the last record: whatever follows in the slice, and the result is not used)
+          g_n = wr[4 * (j + 1)];
+          h_n = chord(r, g_n, in_n, out_n);
+        } else {
+          g = wr[4 * j];
+          hit = chord(r, g, t_in, t_out) && !done;
+        }
+        if (!__any_sync(FULL, hit)) {
+          if (!LOOK && __all_sync(FULL, done)) break;
+          continue;
+        }
         float w = 0.f;
         if (hit) {
           const float4 d0 = wr[4 * j + 1], d1 = wr[4 * j + 2], col = wr[4 * j + 3];
-          const float l = to - ti, tm = 0.5f * (ti + to);
+          const float l = t_out - t_in, tm = 0.5f * (t_in + t_out);
           float u[SEG ? 9 : 3];
-          const float sigma = fmaxf(sample_density<SEG>(r, gj, d0, d1, col.w, ti, tm, to, u), 0.f);
+          const float sigma = fmaxf(sample_density<SEG>(r, g, d0, d1, col.w, t_in, tm, t_out, u), 0.f);
           const float x = sigma * l;
           const float ex = __expf(-x);
           const float alpha = one_minus_exp(x, ex);
@@ -1972,10 +2030,15 @@ __global__ void __launch_bounds__(comp_warps<TS, PERSIST>() * 32, comp_blocks<TS
             atomicMax(&wmax[w_vox[j]], ((unsigned long long)(mx - 1u) << 32) | gid_key);
         }
       }
-      if (last_j >= 0) last = walk.s_q[(q0 + last_j) & walk.QM].y - start + 1;
-      m = m_next;
+      if (last_j >= 0) last = walk.s_ent[32 * b + last_j].y - start + 1;
       if (__all_sync(FULL, done)) break;
       __syncwarp();  // the buffer is copied into next
+      if (!ahead) {
+        ahead = true;
+        walk.fill();
+        m_next = walk.copy(b ^ 1);
+      }
+      m = m_next;
     }
     cp_async_wait<0>();  // a batch copied ahead of the stop
     // a long list sorted only so far, and pixels that go on: listed for k_tile_rest and the second launch
@@ -2041,8 +2104,8 @@ __device__ __forceinline__ float warp_reduce16(float* v, int lane) {
 // any of its pixels used, through the same queue and copies as the forward; the
 // per-record gradients (8 corners + colour) are
 // reduced over the warp and sent with three 16-byte global reductions.
-template <int TS, bool SEG, bool PERSIST>
-__global__ void __launch_bounds__(comp_warps<TS, PERSIST>() * 32, comp_blocks<TS, PERSIST>(24)) k_bwd(const __grid_constant__ ViewSet vs, const uint32_t* __restrict__ ranges,
+template <int TS, bool SEG, bool PERSIST, bool LOOK>
+__global__ void __launch_bounds__(bwd_warps<TS, PERSIST>() * 32, bwd_blocks<TS, PERSIST, LOOK>()) k_bwd(const __grid_constant__ ViewSet vs, const uint32_t* __restrict__ ranges,
                                                 const uint2* __restrict__ plist, const float4* __restrict__ rec,
                                                 const uint32_t* __restrict__ slot_vox, const float* __restrict__ T_fwd,
                                                 const float* __restrict__ tau_in,
@@ -2053,7 +2116,7 @@ __global__ void __launch_bounds__(comp_warps<TS, PERSIST>() * 32, comp_blocks<TS
                                                 int sm_cut, int n_sms, unsigned int* arrivals, const TileOrder order,
                                                 const LfFuse lf) {
   grid_wait();
-  constexpr int NW = TS * TS / 32, CW = comp_warps<TS, PERSIST>();
+  constexpr int NW = TS * TS / 32, CW = bwd_warps<TS, PERSIST>();
   extern __shared__ float4 smem_f4[];
   __shared__ double s_lf[CW][LV_MAX_VIEWS];  // each warp's loss sums (fused LF loss; no atomics)
   __shared__ float s_mean[LV_MAX_VIEWS], s_gscale[LV_MAX_VIEWS];  // the fused LF loss's per-view constants
@@ -2070,14 +2133,7 @@ __global__ void __launch_bounds__(comp_warps<TS, PERSIST>() * 32, comp_blocks<TS
     }
     __syncthreads();
   }
-  StripWalk<true> walk;
-  walk.plist = plist;
-  walk.rec = rec;
-  walk.slot_vox = slot_vox;
-  walk.lane = lane;
-  walk.s_rec = (float4*)((char*)smem_f4 + WARP_SLICE * warp);
-  walk.s_vox = (uint32_t*)(walk.s_rec + 2 * 32 * 4);
-  walk.s_q = (uint2*)(walk.s_vox + 2 * 32);
+  StripWalk<true, LOOK> walk(plist, rec, slot_vox, (char*)smem_f4, warp, lane);
   for (uint32_t item = PERSIST ? next_item(work, lane) : blockIdx.x * CW + warp; item < n_items;
        item = PERSIST ? next_item(work, lane) : n_items) {  // warp-uniform
     const int gtile = (int)order.tile(item / NW);
@@ -2136,27 +2192,43 @@ __global__ void __launch_bounds__(comp_warps<TS, PERSIST>() * 32, comp_blocks<TS
     walk.fill();
     int m = walk.copy(0);
     for (int b = 0; m; b ^= 1) {  // warp-uniform
-      const uint32_t q0 = walk.head - (uint32_t)m;  // this batch's queue entries
       walk.fill();
       const int m_next = walk.copy(b ^ 1);
       cp_async_wait<1>();
       __syncwarp();
       const float4* wr = walk.s_rec + 128 * b;
       const uint32_t* w_vox = walk.s_vox + 32 * b;
-      uint2 qe = walk.s_q[q0 & walk.QM];
-      float4 gn = wr[0];
-      float tn_in, tn_out;
-      bool h = chord(r, gn, tn_in, tn_out) && qe.y < my_hi;
+      const uint2* w_ent = walk.s_ent + 32 * b;
+      float4 g_n;
+      uint2 ent_n;
+      float in_n, out_n;
+      bool h_n = false;
+      if (LOOK) {
+        g_n = wr[0];
+        ent_n = w_ent[0];
+        h_n = chord(r, g_n, in_n, out_n) && ent_n.y < my_hi;
+      }
       for (int j = 0; j < m; ++j) {
-        const bool hit = h;
-        const float4 g = gn;
-        const float t_in = tn_in, t_out = tn_out;
-        const uint32_t slot = qe.x;
-        // the next record's chord does not wait for this sample (past the last one: whatever follows in
-        // the slice, and the result is not used)
-        qe = walk.s_q[(q0 + j + 1) & walk.QM];
-        gn = wr[4 * (j + 1)];
-        h = chord(r, gn, tn_in, tn_out) && qe.y < my_hi;
+        float4 g;
+        uint2 ent;
+        float t_in, t_out;
+        bool hit;
+        if (LOOK) {
+          hit = h_n;
+          g = g_n;
+          ent = ent_n;
+          t_in = in_n;
+          t_out = out_n;
+          // (past the last record: whatever follows in the slice, and the result is not used)
+          g_n = wr[4 * (j + 1)];
+          ent_n = w_ent[j + 1];
+          h_n = chord(r, g_n, in_n, out_n) && ent_n.y < my_hi;
+        } else {
+          g = wr[4 * j];
+          ent = w_ent[j];
+          hit = chord(r, g, t_in, t_out) && ent.y < my_hi;
+        }
+        const uint32_t slot = ent.x;
         const unsigned hb = __ballot_sync(FULL, hit);
         if (!hb) continue;
         float v[16];
@@ -2623,65 +2695,66 @@ static void sm_limits(int sm_limit, int dev, int* sms, int* sm_cut) {
 }
 
 
+static uint32_t strip_items(int ts, int64_t tiles) { return (uint32_t)tiles * (uint32_t)(ts * ts / 32); }
+
 static TileOrder tile_order(const FwdWs& w, int64_t tiles) {
   return {w.class_tiles, w.work + 16, (uint32_t)tiles};
 }
 
-// resume: the second launch, over the open tiles (its grid is persistent whatever the schedule: only the
-// device knows their number)
-template <int TS, bool SEG, bool PERSIST>
+template <int TS, bool SEG, bool PERSIST, bool LOOK>
 static void launch_fwd_t(int64_t tiles, cudaStream_t s, const ViewSet& vs, const FwdWs& w, float t_stop,
-                         const lv_fwd_out* out, int sm_limit, bool resume) {
-  constexpr int CW = comp_warps<TS, PERSIST>();
-  const size_t smem = WARP_SLICE * CW;
+                         const lv_fwd_out* out, int sm_limit) {
+  constexpr int CW = fwd_warps<TS, PERSIST, LOOK>();
+  constexpr bool RESUME = PERSIST && LOOK;
+  const auto kernel = k_fwd<TS, SEG, PERSIST, LOOK>;
+  const size_t smem = WalkShape<LOOK>::SLICE * CW;
   static int pblocks[64];  // per device
   static std::atomic<unsigned long long> done{0};
   const int dev = current_device();
   once_per_device(done, [&] {
-    cudaFuncSetAttribute(k_fwd<TS, SEG, PERSIST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (PERSIST && dev < 64) pblocks[dev] = persistent_blocks(k_fwd<TS, SEG, PERSIST>, CW * 32, smem);
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (PERSIST && dev < 64) pblocks[dev] = persistent_blocks(kernel, CW * 32, smem);
   });
-  const int pb = dev < 64 ? pblocks[dev] : persistent_blocks(k_fwd<TS, SEG, PERSIST>, CW * 32, smem);
+  const int pb = dev < 64 ? pblocks[dev] : persistent_blocks(kernel, CW * 32, smem);
   int sms = 0, sm_cut = 0;
   sm_limits(sm_limit, dev, &sms, &sm_cut);
-  const uint32_t n_items = (uint32_t)tiles * (TS * TS / 32);
+  const uint32_t n_items = strip_items(TS, tiles);
   unsigned grid = (n_items + CW - 1) / CW;
   if (PERSIST) grid = std::min(grid, (unsigned)pb);  // the work counters were cleared at the start of the forward
-  const Front fr = {w.ready, w.prog, w.open_tiles, w.work + 7, w.dep, w.nsamp, resume};
-  auto k = out->composite_event && !resume ? launch(k_fwd<TS, SEG, PERSIST>, grid, CW * 32, smem, s)
-                                           : chain(k_fwd<TS, SEG, PERSIST>, grid, CW * 32, smem, s);
-  k(vs, w.ranges, w.plist, w.rec, w.slot_vox, t_stop,
-                                                       out->rgb, out->depth, out->T, out->n_contrib,
-                                                       out->n_samples, w.tau, out->wmax_packed,
-                                                       w.work + (resume ? 2 : 0), n_items, sm_cut, sms,
-                                                       w.work + (resume ? 10 : 8), tile_order(w, tiles), fr);
+  const Front fr = {w.ready, w.prog, w.open_tiles, w.work + 7, w.dep, w.nsamp};
+  auto k = out->composite_event && !RESUME ? launch(kernel, grid, CW * 32, smem, s)
+                                           : chain(kernel, grid, CW * 32, smem, s);
+  k(vs, w.ranges, w.plist, w.rec, w.slot_vox, t_stop, out->rgb, out->depth, out->T, out->n_contrib, out->n_samples,
+    w.tau, out->wmax_packed, w.work + (RESUME ? 2 : 0), n_items, sm_cut, sms, w.work + (RESUME ? 10 : 8),
+    tile_order(w, tiles), fr);
 }
 
-template <int TS, bool SEG, bool PERSIST>
+template <int TS, bool SEG, bool PERSIST, bool LOOK>
 static void launch_bwd_t(int64_t tiles, cudaStream_t s, const ViewSet& vs, const FwdWs& w, const lv_fwd_out* fwd,
                          const float* gC, const float* gD, const float* gT, float* dd,
                          int sm_limit, const LfFuse& lf) {
-  constexpr int CW = comp_warps<TS, PERSIST>();
-  const size_t smem = WARP_SLICE * CW;
+  constexpr int CW = bwd_warps<TS, PERSIST>();
+  const auto kernel = k_bwd<TS, SEG, PERSIST, LOOK>;
+  const size_t smem = WalkShape<LOOK>::SLICE * CW;
   static int pblocks[64];  // per device
   static std::atomic<unsigned long long> done{0};
   const int dev = current_device();
   once_per_device(done, [&] {
-    cudaFuncSetAttribute(k_bwd<TS, SEG, PERSIST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (PERSIST && dev < 64) pblocks[dev] = persistent_blocks(k_bwd<TS, SEG, PERSIST>, CW * 32, smem);
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (PERSIST && dev < 64) pblocks[dev] = persistent_blocks(kernel, CW * 32, smem);
   });
-  const int pb = dev < 64 ? pblocks[dev] : persistent_blocks(k_bwd<TS, SEG, PERSIST>, CW * 32, smem);
+  const int pb = dev < 64 ? pblocks[dev] : persistent_blocks(kernel, CW * 32, smem);
   int sms = 0, sm_cut = 0;
   sm_limits(sm_limit, dev, &sms, &sm_cut);
-  const uint32_t n_items = (uint32_t)tiles * (TS * TS / 32);
+  const uint32_t n_items = strip_items(TS, tiles);
   unsigned grid = (n_items + CW - 1) / CW;
   if (PERSIST) {
     zero_async(s, w.work + 1, sizeof(unsigned int), w.work + 9, sizeof(unsigned int));
     grid = std::min(grid, (unsigned)pb);
   }
-  launch(k_bwd<TS, SEG, PERSIST>, grid, CW * 32, smem, s)(vs, w.ranges, w.plist, w.rec, w.slot_vox, fwd->T,
-                                                       w.tau, fwd->n_contrib, gC, gD, gT, dd, w.d_rgb, w.work + 1,
-                                                       n_items, sm_cut, sms, w.work + 9, tile_order(w, tiles), lf);
+  launch(kernel, grid, CW * 32, smem, s)(vs, w.ranges, w.plist, w.rec, w.slot_vox, fwd->T, w.tau, fwd->n_contrib, gC,
+                                         gD, gT, dd, w.d_rgb, w.work + 1, n_items, sm_cut, sms, w.work + 9,
+                                         tile_order(w, tiles), lf);
 }
 
 // tile size, density model (midpoint, or the exact-segment variant) and scheduling (one block per
@@ -2754,20 +2827,38 @@ static void launch_render_f64(const lv_voxels* vox, const lv_raster_opts* o, con
   }
 }
 
+// The looking-ahead composites, with either schedule, where few strips are in flight on an SM (see WalkShape):
+// up to `waves` times 28 an SM, in the forward 5 with tile 8 and 3 with the others, in the backward 1.  Forward
+// and backward in us, open 2M-voxel scene, looking ahead against not: tile 8, 2,048 strips 1611 + 714 against
+// 1759 + 755; 9,600 strips 511 + 487 against 559 + 489; 17,000 strips 348 + 459 against 379 + 426 (opaque 57 + 74
+// against 51 + 68), 32,400 strips 480 + 735 against 479 + 681; tile 16, 9,600 strips 503 + 524 against 536 + 504,
+// 17,000 strips 363 + 485 against 363 + 440 (opaque 57 + 74 against 49 + 68).
+static bool look_ahead(const lv_raster_opts* o, int64_t tiles, uint32_t waves) {
+  int sms = 0, cut = 0;
+  sm_limits((o->flags & LV_FLAG_PERSISTENT) ? o->persistent_sms : 0, current_device(), &sms, &cut);
+  return cut == 0 && strip_items(o->tile, tiles) <= waves * 28u * (uint32_t)sms;
+}
+
+// resume: the second launch, over the open tiles (its grid is persistent whatever the schedule: only the
+// device knows their number)
 static void launch_fwd(const lv_raster_opts* o, int64_t tiles, cudaStream_t s, const ViewSet& vs, const FwdWs& w,
                        const lv_fwd_out* out, bool resume) {
-  const bool seg = (o->flags & LV_FLAG_EXACT_SEGMENT) != 0, flag = (o->flags & LV_FLAG_PERSISTENT) != 0;
-  const bool per = flag || resume;
-  const int sml = flag ? o->persistent_sms : 0;
-#define LV_FWD(TS)                                                                          \
-  if (seg && per) launch_fwd_t<TS, true, true>(tiles, s, vs, w, o->t_stop, out, sml, resume);   \
-  else if (seg) launch_fwd_t<TS, true, false>(tiles, s, vs, w, o->t_stop, out, 0, false);      \
-  else if (per) launch_fwd_t<TS, false, true>(tiles, s, vs, w, o->t_stop, out, sml, resume);    \
-  else launch_fwd_t<TS, false, false>(tiles, s, vs, w, o->t_stop, out, 0, false)
+  const bool seg = (o->flags & LV_FLAG_EXACT_SEGMENT) != 0, per = (o->flags & LV_FLAG_PERSISTENT) != 0;
+  const int sml = per ? o->persistent_sms : 0;
+  const bool look = look_ahead(o, tiles, o->tile == 8 ? 5 : 3);
+#define LV_FWD_S(TS, SEG)                                                                        \
+  if (resume) launch_fwd_t<TS, SEG, true, true>(tiles, s, vs, w, o->t_stop, out, sml);           \
+  else if (look) launch_fwd_t<TS, SEG, false, true>(tiles, s, vs, w, o->t_stop, out, 0);         \
+  else if (per) launch_fwd_t<TS, SEG, true, false>(tiles, s, vs, w, o->t_stop, out, sml);        \
+  else launch_fwd_t<TS, SEG, false, false>(tiles, s, vs, w, o->t_stop, out, 0)
+#define LV_FWD(TS)                 \
+  if (seg) { LV_FWD_S(TS, true); } \
+  else { LV_FWD_S(TS, false); }
   if (o->tile == 8) { LV_FWD(8); }
   else if (o->tile == 16) { LV_FWD(16); }
   else { LV_FWD(32); }
 #undef LV_FWD
+#undef LV_FWD_S
 }
 
 static void launch_bwd(const lv_raster_opts* o, int64_t tiles, cudaStream_t s, const ViewSet& vs, const FwdWs& w,
@@ -2775,14 +2866,18 @@ static void launch_bwd(const lv_raster_opts* o, int64_t tiles, cudaStream_t s, c
                        float* dd, const LfFuse& lf) {
   const bool seg = (o->flags & LV_FLAG_EXACT_SEGMENT) != 0, per = (o->flags & LV_FLAG_PERSISTENT) != 0;
   const int sml = per ? o->persistent_sms : 0;
-#define LV_BWD(TS)                                                                                \
-  if (seg && per) launch_bwd_t<TS, true, true>(tiles, s, vs, w, fwd, gC, gD, gT, dd, sml, lf);    \
-  else if (seg) launch_bwd_t<TS, true, false>(tiles, s, vs, w, fwd, gC, gD, gT, dd, 0, lf);       \
-  else if (per) launch_bwd_t<TS, false, true>(tiles, s, vs, w, fwd, gC, gD, gT, dd, sml, lf);     \
-  else launch_bwd_t<TS, false, false>(tiles, s, vs, w, fwd, gC, gD, gT, dd, 0, lf)
+  const bool look = look_ahead(o, tiles, 1);
+#define LV_BWD_S(TS, SEG)                                                                              \
+  if (look) launch_bwd_t<TS, SEG, false, true>(tiles, s, vs, w, fwd, gC, gD, gT, dd, 0, lf);           \
+  else if (per) launch_bwd_t<TS, SEG, true, false>(tiles, s, vs, w, fwd, gC, gD, gT, dd, sml, lf);     \
+  else launch_bwd_t<TS, SEG, false, false>(tiles, s, vs, w, fwd, gC, gD, gT, dd, 0, lf)
+#define LV_BWD(TS)                 \
+  if (seg) { LV_BWD_S(TS, true); } \
+  else { LV_BWD_S(TS, false); }
   if (o->tile == 8) { LV_BWD(8); }
   else if (o->tile == 16) { LV_BWD(16); }
   else { LV_BWD(32); }
+#undef LV_BWD_S
 #undef LV_BWD
 }
 
