@@ -93,7 +93,7 @@ __device__ __forceinline__ int view_of_block(const int* first, int n, int b) {
 constexpr int ST = 32, SP = ST + 2;
 __global__ void __launch_bounds__(TPB) k_lf_sobel(const float* __restrict__ gt, const __grid_constant__ ViewPix vp,
                                                  int per, uint32_t* mkey, uint32_t* hist) {
-  grid_begin();
+  grid_wait();
   __shared__ uint32_t s_h[D1_BINS];
   __shared__ float s_y[SP * SP];
   const int t = threadIdx.x;
@@ -212,7 +212,7 @@ __device__ __forceinline__ LfPick block_pick(const uint32_t* h, uint32_t k) {
 template <bool LAST>
 __global__ void __launch_bounds__(TPB) k_lf_digit(const uint32_t* mkey, const __grid_constant__ ViewPix vp,
                                                  uint32_t* hist, LfPick* pick) {
-  grid_begin();
+  grid_wait();
   constexpr int NB = LAST ? D3_BINS : D2_BINS;
   __shared__ uint32_t s_h[NB];
   const int t = threadIdx.x, v = view_of_block(vp.blk, vp.n, blockIdx.x);
@@ -269,7 +269,7 @@ __global__ void __launch_bounds__(TPB) k_lf_weight(const uint32_t* mkey, const u
                                                   const LfPick* pick,
                                                   const __grid_constant__ ViewPix vp, float eps, float gamma,
                                                   float* w, double* wsum, float* edge_out) {
-  grid_begin();
+  grid_wait();
   const int v = view_of_block(vp.blk, vp.n, blockIdx.x);
   const int b0 = vp.blk[v], nb = vp.blk[v + 1] - b0;
   const long long lo = vp.off[v], hi = vp.off[v + 1];
@@ -316,7 +316,7 @@ __device__ __forceinline__ void lf_view_constants(const double* wsum, int v, lon
 __global__ void k_lf_loss(const float* __restrict__ rgb, const float* __restrict__ gt, const float* __restrict__ w,
                           const __grid_constant__ ViewPix vp, const double* wsum, double* lsum,
                           float* __restrict__ grad) {
-  grid_begin();
+  grid_wait();
   const int v = view_of_block(vp.blk, vp.n, blockIdx.x);
   const int b0 = vp.blk[v], nb = vp.blk[v + 1] - b0;
   const long long lo = vp.off[v], hi = vp.off[v + 1];
@@ -348,7 +348,7 @@ __global__ void k_lf_loss(const float* __restrict__ rgb, const float* __restrict
 __global__ void k_lf_loss4(const float* __restrict__ rgb, const float* __restrict__ gt, const float* __restrict__ w,
                            const __grid_constant__ ViewPix vp, const double* wsum, double* lsum,
                            float* __restrict__ grad) {
-  grid_begin();
+  grid_wait();
   const int v = view_of_block(vp.blk, vp.n, blockIdx.x);
   const int b0 = vp.blk[v], nb = vp.blk[v + 1] - b0;
   const long long lo = vp.off[v], hi = vp.off[v + 1];

@@ -96,3 +96,18 @@ def test_nothing_in_a_walk_or_list_is_restrict():
         body = s[m.end():closing(s, m.end(), "{}")]
         fields = [f for f in re.findall(r"__restrict__\s+(\w+)\s*;", body)]
         assert not fields, fields
+
+
+def test_no_two_grids_of_a_stream_wait():
+    """grid_begin lets the next grid in only after its own wait: else every grid behind a slow one becomes
+    resident, and their waiting blocks keep other streams' kernels out."""
+    s = text()
+    m = re.search(r"void grid_begin\(\)\s*\{([^}]*)\}", s)
+    assert 0 <= m.group(1).find("grid_wait()") < m.group(1).find("launch_dependents")
+
+
+def test_kernels_that_fill_the_gpu_let_no_grid_wait():
+    """The LF steps run beside a forward: a grid waiting behind one of them would hold what that needs."""
+    for name, _, body in kernels():
+        if name in ("k_lf_sobel", "k_lf_digit", "k_lf_weight", "k_lf_loss", "k_lf_loss4", "k_fwd", "k_bwd"):
+            assert re.match(r"\s*grid_wait\(\);", body), name
