@@ -239,17 +239,17 @@ lv_status lv_sh_backward(const lv_voxels* vox, const lv_camera* cams, int n_view
 
 /* Autotuner of the composite schedule (batched views in one launch: tile
  * size, batch and scheduling chosen per scene and view set).  Each candidate
- * -- tile edge 8, 16, 32 x one block per tile or persistent warps
- * (LV_FLAG_PERSISTENT) x batch 32, 64, 128 (not 128 with tile 32) -- runs one
- * warm-up forward + backward and then `reps` (1 .. 1000) timed ones on the
+ * -- tile edge 8, 16, 32 x a warp per strip or persistent warps
+ * (LV_FLAG_PERSISTENT) -- runs one warm-up forward + backward and then `reps` (1 .. 1000) timed ones on the
  * caller's scene and views, timed with CUDA events on `stream`; the call
  * synchronises the stream.  *best receives *base with the fastest tile,
- * batch and LV_FLAG_PERSISTENT choice.  ms_out (host float[18], nullable)
- * receives each candidate's mean forward + backward time in ms at index
- * (6 t + 3 p + b) for tile t (0: 8, 1: 16, 2: 32), schedule p (0: block per
- * tile, 1: persistent) and batch b (0: 32, 1: 64, 2: 128); -1 for a candidate
- * that is refused or needs more than pair_capacity pairs (skipped), and -1
- * everywhere on a cache hit.  cache_path (nullable) is a text file of
+ * LV_FLAG_PERSISTENT choice, and batch 32: the batch changes no launch, so a
+ * candidate is timed once.  ms_out (host float[18], nullable) receives each
+ * candidate's mean forward + backward time in ms at index (6 t + 3 p + b) for
+ * tile t (0: 8, 1: 16, 2: 32), schedule p (0: a warp per strip, 1: persistent),
+ * the same for every batch b (0: 32, 1: 64, 2: 128); -1 for tile 32 with batch
+ * 128, which is refused, for a candidate that needs more than pair_capacity
+ * pairs (skipped), and everywhere on a cache hit.  cache_path (nullable) is a text file of
  * "key tile persistent batch" lines keyed by device name, voxel count, view
  * sizes and the other flags (a line without the batch means 32): a hit
  * returns at once, a tuned result is appended.  workspace:

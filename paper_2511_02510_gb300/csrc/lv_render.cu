@@ -2640,7 +2640,7 @@ static lv_status check_common(const lv_voxels* vox, const lv_camera* cams, int n
   if (o->tile != 8 && o->tile != 16 && o->tile != 32) { set_error("tile must be 8, 16 or 32"); return LV_ERR_INVALID_ARG; }
   if (o->batch != 32 && o->batch != 64 && o->batch != 128) { set_error("batch must be 32, 64 or 128"); return LV_ERR_INVALID_ARG; }
   if (o->tile == 32 && o->batch == 128) {
-    set_error("batch 128 with 32x32 tiles needs more than 227 KB of shared memory per block");
+    set_error("tile 32 takes batch 32 or 64 (as it always has; the batch changes no launch)");
     return LV_ERR_UNSUPPORTED;
   }
   if (!(o->t_stop >= 0.f && o->t_stop < 1.f)) { set_error("t_stop must be in [0, 1)"); return LV_ERR_INVALID_ARG; }
@@ -2757,8 +2757,6 @@ static void launch_bwd_t(int64_t tiles, cudaStream_t s, const ViewSet& vs, const
                                          tile_order(w, tiles), lf);
 }
 
-// tile size, density model (midpoint, or the exact-segment variant) and scheduling (one block per
-// tile, or persistent warps on a work counter) from the options
 // One warp per tile first (short lists, ranges, the lists of longer tiles), then persistent blocks over
 // the long tiles' fronts and the medium tiles.
 static int tile_sort_blocks() {

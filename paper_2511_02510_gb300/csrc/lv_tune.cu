@@ -1,8 +1,10 @@
 // lv_tune.cu -- autotuner of the composite schedule (host code).  Every
 // candidate (tile edge 8 / 16 / 32, a warp per item or persistent warps on a
-// work counter, batch 32 / 64 / 128, which no longer changes what runs) runs the caller's forward + backward on the caller's
+// work counter) runs the caller's forward + backward on the caller's
 // scene and views; the fastest one, timed with CUDA events on the caller's
-// stream, is returned and optionally remembered in a text cache file.
+// stream, is returned and optionally remembered in a text cache file.  The batch
+// (lv_raster_opts.batch) changes no launch: a candidate is timed once, its time
+// stands for every batch that is accepted, and batch 32 is returned.
 #include <stdio.h>
 #include <string.h>
 
@@ -160,13 +162,12 @@ extern "C" lv_status lv_autotune(const lv_voxels* vox, const lv_camera* cams, in
   if (cuda_check(cudaEventCreate(&e1), "lv_autotune") != LV_OK) { cudaEventDestroy(e0); return LV_ERR_CUDA; }
   float best_ms = -1.f;
   lv_status result = LV_OK;
-  for (int c = 0; c < 2 * N_TILES * N_BATCH && result == LV_OK; ++c) {
-    const int t = c / (2 * N_BATCH), p = (c / N_BATCH) % 2, b = c % N_BATCH;
-    if (TILES[t] == 32 && BATCHES[b] == 128) continue;  // more shared memory than a block has
+  for (int c = 0; c < 2 * N_TILES && result == LV_OK; ++c) {
+    const int t = c / 2, p = c % 2;
     {
       lv_raster_opts o = *base;
       o.tile = TILES[t];
-      o.batch = BATCHES[b];
+      o.batch = BATCHES[0];
       o.flags = (base->flags & ~(uint32_t)(LV_FLAG_PERSISTENT | LV_FLAG_SYNC_CHECK)) | (p ? LV_FLAG_PERSISTENT : 0u);
       auto step = [&]() -> lv_status {
         lv_status e = lv_rasterize_forward(vox, cams, n_views, &o, &out, w.fwd, w.fwd_bytes, pair_capacity,
@@ -188,12 +189,14 @@ extern "C" lv_status lv_autotune(const lv_voxels* vox, const lv_camera* cams, in
       float ms = 0.f;
       cudaEventElapsedTime(&ms, e0, e1);
       ms /= (float)reps;
-      if (ms_out) ms_out[c] = ms;
+      if (ms_out)
+        for (int b = 0; b < N_BATCH; ++b)
+          if (TILES[t] != 32 || BATCHES[b] != 128) ms_out[c * N_BATCH + b] = ms;  // (refused: stays -1)
       if (best_ms < 0.f || ms < best_ms) {
         best_ms = ms;
         tile = TILES[t];
         persistent = p;
-        batch = BATCHES[b];
+        batch = BATCHES[0];
       }
     }
   }

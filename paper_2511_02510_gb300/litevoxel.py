@@ -464,7 +464,7 @@ def lv_autotune_workspace_size(n, cams_arr, n_views, base, pair_capacity) -> int
 
 
 def lv_autotune(vox, cams_arr, n_views, base, pair_capacity, reps, workspace, cache_path=None):
-    """Time every (tile, schedule, batch) candidate; returns (best lv_raster_opts, [18] ms per candidate at
+    """Time every (tile, schedule) candidate (the batch changes no launch); returns (best lv_raster_opts, [18] ms per candidate at
     6 tile + 3 schedule + batch, -1 = skipped)."""
     best = lv_raster_opts()
     ms = (C.c_float * 18)()

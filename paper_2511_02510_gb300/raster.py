@@ -216,7 +216,7 @@ class CapturedStep:
 
 def autotune_tile(scene: Scene, cams, tiles=(8, 16, 32), steps=5, cache_path=None, t_stop=1e-4,
                   schedules=(False, True)):
-    """Pick the tile size and composite scheduling (one block per tile, or persistent warps on a
+    """Pick the tile size and composite scheduling (a warp per strip, or persistent warps on a
     work counter) with the fastest forward + backward for this scene and camera set.
 
     Each candidate is timed with CUDA events over ``steps`` forward + backward passes after one
