@@ -75,8 +75,8 @@ def max_over_ranks(x: float, world: int, device=None) -> float:
 
 
 def tuned_schedule(scene, cams):
-    """Tile size, batch and composite schedule from the library's autotuner (lv_autotune: every
-    tile size and batch with and without persistent warps, forward + backward timed with CUDA
+    """Tile size and composite schedule from the library's autotuner (lv_autotune: every
+    tile size with and without persistent warps, forward + backward timed with CUDA
     events on this scene and these views), as a user of the library would pick them."""
     import torch
 
@@ -101,10 +101,7 @@ TUNE_TILES, TUNE_BATCHES = (8, 16, 32), (32, 64, 128)
 def step_batch_candidates(tile, persistent, batch, tune_ms, within=0.03):
     """Batches of the tuner's tile and schedule whose forward + backward time (lv_autotune's
     ms_out, index 6 t + 3 p + b) lies within `within` of the fastest: the tuner's pick first.
-    The tuner times forward + backward alone; in the step the backward composite shares the
-    GPU with the pruning and selection chain, whose blocks fit on the backward's SMs only when
-    its staging slices leave shared memory free, so close batches are told apart by timing
-    the step itself."""
+    (All of them while the batch changes no launch, so the step does not choose among them.)"""
     if not tune_ms or tile not in TUNE_TILES:
         return [batch]
     t, p = TUNE_TILES.index(tile), 1 if persistent else 0
@@ -154,22 +151,13 @@ class Workload:
             self.tile, self.persistent, self.batch = schedule
         elif tuned:
             self.tile, self.persistent, self.batch, self.tune_ms = tuned_schedule(self.scene, self.cams)
-            # forward + backward alone, as the tuner times them, tell the schedules apart by a few per
-            # cent; the step needs the persistent one, which can leave SMs to its other streams
-            # (0.88 ms a step against 0.94)
-            t0 = 6 * TUNE_TILES.index(self.tile) + TUNE_BATCHES.index(self.batch)
-            if not self.persistent and 0 < self.tune_ms[t0 + 3] <= 1.05 * self.tune_ms[t0]:
-                self.persistent = True
-        # the persistent backward composite leaves 64 SMs to the pruning and selection kernels
-        # that the four-stream step runs beside it (graph-replayed step: 0.876 ms with the backward
-        # on 88 SMs, 0.881 on 72, 0.879 on 104, 0.883 on 112, 0.912 on 128); the forward composite
-        # runs alone and keeps every SM
-        self.persistent_sms = 0
-        if self.persistent:
-            self.persistent_sms = max(1, torch.cuda.get_device_properties(0).multi_processor_count - 64)
         self.rctx = RasterContext(self.cams, n, tile=self.tile, batch=self.batch, persistent=self.persistent)
-        self.bwd_opts = L.make_opts(self.tile, self.batch, persistent=self.persistent,
-                                    persistent_sms=self.persistent_sms)
+        # the step's backward composite is the persistent one, on all but 64 SMs, which it leaves to the
+        # pruning and selection kernels that the four-stream step runs beside it (graph-replayed step:
+        # 0.811 ms with the backward on 88 SMs, 0.814 on 80, 0.819 on 72, 0.823 on 96, 0.830 on 120);
+        # the forward composite runs alone, by the schedule the tuner picks
+        self.persistent_sms = max(1, torch.cuda.get_device_properties(0).multi_processor_count - 64)
+        self.bwd_opts = L.make_opts(self.tile, self.batch, persistent=True, persistent_sms=self.persistent_sms)
         self.vox = self.scene.voxels()
         self.rctx.fit_capacity(self.vox)
         self.npix = self.rctx.n_pix
@@ -228,13 +216,6 @@ class Workload:
     # stage boundaries, for the per-kernel breakdown
     STAGES = ["reset", "forward", "loss", "backward", "sh_backward", "unpack", "prune", "subdivide_select",
               "subdivide_inplace", "restore"]
-
-    def set_batch(self, batch):
-        """Stage `batch` list entries per warp round in both composites (changes no result; a
-        captured step must be captured again)."""
-        self.batch = int(batch)
-        self.rctx.opts.batch = self.batch
-        self.bwd_opts.batch = self.batch
 
     def _state_arrays(self):
         """The per-voxel arrays the next step reads that an in-place topology change overwrites below
@@ -865,34 +846,6 @@ def run_next_rows(torch, L, wl, reps, hbm_peak):
     return out
 
 
-def choose_step_batch(torch, wl, CapturedStep, reps=10):
-    """Among step_batch_candidates, the batch whose captured step (step_concurrent, the timed
-    step) replays fastest, timed with CUDA events over `reps` replays after 3 warm-up replays;
-    wl is left on that batch.  Returns what was timed (None when the tuner left one candidate)."""
-    cands = step_batch_candidates(wl.tile, wl.persistent, wl.batch, wl.tune_ms)
-    if len(cands) < 2:
-        return None
-    tuner_batch, ms = wl.batch, {}
-    for b in cands:
-        wl.set_batch(b)
-        g = CapturedStep(wl.step_concurrent)
-        for _ in range(3):
-            g()
-        e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-        e0.record()
-        for _ in range(reps):
-            g()
-        e1.record()
-        torch.cuda.synchronize()
-        ms[b] = e0.elapsed_time(e1) / reps
-        del g
-    best = min(ms, key=ms.get)
-    wl.set_batch(best)
-    return {"tuner_batch": tuner_batch, "step_ms_by_batch": {str(b): v for b, v in ms.items()}, "batch": best,
-            "how": "batches whose forward + backward time lies within 3 % of the tuner's pick, each timed "
-                   "as the captured step (10 replays after 3); the fastest is the bench's batch"}
-
-
 def run_ours(args, rank, world, local):
     import torch
     import torch.distributed as dist
@@ -935,9 +888,6 @@ def run_ours(args, rank, world, local):
     if any(cnt[k] != first[k] for k in ("n_pruned", "n_new", "split", "pairs")):
         raise RuntimeError(f"the restored state does not repeat the first step: {first} vs {cnt}")
     from paper_2511_02510_gb300.raster import CapturedStep
-    batch_choice = None
-    if fixed is None:
-        batch_choice = choose_step_batch(torch, wl, CapturedStep)
 
     # ---- per-stage breakdown: K eager steps with an event at every stage boundary
     K = args.steps
@@ -1128,9 +1078,9 @@ def run_ours(args, rank, world, local):
                           "global_batch": world, "seq_len": None, "parallelism": f"replicas x{world}",
                           "voxels": wl.n, "pixels_per_rank": wl.npix, "pairs": cnt["pairs"],
                           "visible_slots": cnt["visible_slots"], "tile": wl.tile, "batch": wl.batch,
-                          "schedule": (f"persistent warps (backward on {wl.persistent_sms} SMs)" if wl.persistent
-                                       else "one block per tile"),
-                          "autotune_ms": wl.tune_ms, "batch_choice": batch_choice,
+                          "schedule": ("forward: " + ("persistent warps" if wl.persistent else "a warp per strip") +
+                                       f" (autotuned); backward: persistent warps on {wl.persistent_sms} SMs"),
+                          "autotune_ms": wl.tune_ms,
                           "l2": "inputs larger than L2 (scene arrays 480 MB, per-step outputs > 600 MB)"},
                "roofline": roofline,
                "stages_ms": stage_ms, "eager_ms_per_step": eager_ms,
