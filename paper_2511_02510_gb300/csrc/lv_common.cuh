@@ -21,10 +21,15 @@ constexpr unsigned FULL = 0xffffffffu;
 void set_error(const char* fmt, ...);
 lv_status cuda_check(cudaError_t e, const char* what);
 void count_launch(int k = 1);
-// The weights, their per-view sums and the loss sums in a workspace of
-// lv_lf_weights for the given views (the backward's fused LF loss).
+// The weights, their per-view sums, every view's (mean weight, gradient scale) and
+// the loss sums, each in LF_SLOTS parts [slot][LV_MAX_VIEWS], in a workspace of
+// lv_lf_weights for the given views (the backward's fused LF loss).  The backward's
+// many blocks spread their sums over the slots: FP64 atomics on one word serialise
+// at the L2.
+constexpr unsigned LF_SLOTS = 4;
 lv_status lf_fused_buffers(const int32_t* widths, const int32_t* heights, int n_views, void* workspace,
-                           size_t ws_bytes, const float** w, const double** wsum, double** lsum);
+                           size_t ws_bytes, const float** w, const double** wsum, const float2** view_k,
+                           double** lsum);
 
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 

@@ -47,7 +47,9 @@ struct LfPick {
 struct LfWs {
   LfPick* pick;   // [2][views] after the first and the second digit
   double* wsum;   // [views]
-  double* lsum;   // [views]
+  double* lsum;   // [LF_SLOTS][views]
+  float2* view_k; // [views] mean weight, gradient scale
+  uint32_t* done; // [views] blocks that have added to wsum
   uint32_t* hist; // [views][HIST_WORDS]
   uint32_t* mkey; // [pixels] bits of three times the Sobel magnitude
   float* w;       // [pixels] unnormalised weight
@@ -59,7 +61,9 @@ LfWs carve_lf(void* base, int nv, int64_t pixels) {
   Carve c(base);
   w.pick = c.take<LfPick>(2 * LV_MAX_VIEWS);
   w.wsum = c.take<double>(LV_MAX_VIEWS);
-  w.lsum = c.take<double>(LV_MAX_VIEWS);
+  w.lsum = c.take<double>(LF_SLOTS * LV_MAX_VIEWS);
+  w.view_k = c.take<float2>(LV_MAX_VIEWS);
+  w.done = c.take<uint32_t>(LV_MAX_VIEWS);
   w.hist = c.take<uint32_t>((size_t)nv * HIST_WORDS);
   w.mkey = c.take<uint32_t>(pixels);
   w.w = c.take<float>(pixels);
@@ -268,11 +272,14 @@ __device__ __forceinline__ void block_add_f64(double v, double* dst) {
 __global__ void __launch_bounds__(TPB) k_lf_weight(const uint32_t* mkey, const uint32_t* hist,
                                                   const LfPick* pick,
                                                   const __grid_constant__ ViewPix vp, float eps, float gamma,
-                                                  float* w, double* wsum, float* edge_out) {
+                                                  float* w, double* wsum, float2* view_k, uint32_t* done,
+                                                  float* edge_out) {
   grid_wait();
   const int v = view_of_block(vp.blk, vp.n, blockIdx.x);
   const int b0 = vp.blk[v], nb = vp.blk[v + 1] - b0;
   const long long lo = vp.off[v], hi = vp.off[v + 1];
+  // the view's gradient scale 2 / (3 |P|), rounded to FP32 from FP64
+  if ((int)blockIdx.x == b0 && threadIdx.x == 0) view_k[v].y = (float)(2.0 / (3.0 * (double)(hi - lo)));
   const LfPick p2 = pick[LV_MAX_VIEWS + v];
   const LfPick p3 = block_pick<D3_BINS>(hist + (size_t)v * HIST_WORDS + D1_BINS + D2_BINS, p2.k);
   const float P = __uint_as_float(p2.prefix << D2_SHIFT | p3.prefix);
@@ -300,30 +307,27 @@ __global__ void __launch_bounds__(TPB) k_lf_weight(const uint32_t* mkey, const u
     acc += (double)part;
   }
   block_add_f64(acc, &wsum[v]);
-}
-
-// the view's mean weight <w> and gradient scale 2 / (3 |P|), rounded to FP32 from FP64, once per
-// block (thread 0; FP64 division is slow on this part) into *mean and *gscale (shared memory)
-__device__ __forceinline__ void lf_view_constants(const double* wsum, int v, long long np, float* mean, float* gscale) {
-  if (threadIdx.x == 0) {
-    *mean = (float)(wsum[v] / (double)np);
-    *gscale = (float)(2.0 / (3.0 * (double)np));
+  // the view's mean weight <w>, rounded to FP32 from FP64, once, by its last block (FP64 division is slow on
+  // this part: not in every block that uses it)
+  if (threadIdx.x == 0) {  // the thread that added
+    __threadfence();
+    if (atomicAdd(&done[v], 1u) == (uint32_t)nb - 1u) {
+      __threadfence();
+      view_k[v].x = (float)(__ldcg(&wsum[v]) / (double)(hi - lo));
+    }
   }
-  __syncthreads();
 }
 
 // Eq. 8 + Eq. 18: w~ = w / <w>, L = 1/|P| sum w~ mean_c r^2, dL/drgb = 2/(3|P|) w~ r
 __global__ void k_lf_loss(const float* __restrict__ rgb, const float* __restrict__ gt, const float* __restrict__ w,
-                          const __grid_constant__ ViewPix vp, const double* wsum, double* lsum,
+                          const __grid_constant__ ViewPix vp, const float2* view_k, double* lsum,
                           float* __restrict__ grad) {
   grid_wait();
   const int v = view_of_block(vp.blk, vp.n, blockIdx.x);
   const int b0 = vp.blk[v], nb = vp.blk[v + 1] - b0;
   const long long lo = vp.off[v], hi = vp.off[v + 1];
-  const long long np = hi - lo;
-  __shared__ float s_mean, s_gscale;
-  lf_view_constants(wsum, v, np, &s_mean, &s_gscale);
-  const float mean = s_mean, gscale = s_gscale;
+  const float2 vk = view_k[v];
+  const float mean = vk.x, gscale = vk.y;
   double acc = 0.0;  // sum of w~ (r0^2 + r1^2 + r2^2) over this thread's pixels; the 1/3 is applied at the end
   for (long long p = lo + (blockIdx.x - b0) * (long long)TPB + threadIdx.x; p < hi; p += (long long)nb * TPB) {
     const float wt = w[p] / mean;
@@ -336,7 +340,7 @@ __global__ void k_lf_loss(const float* __restrict__ rgb, const float* __restrict
       grad[3 * p + 2] = c * r2;
     }
   }
-  block_add_f64(acc, &lsum[v]);
+  block_add_f64(acc, &lsum[v]);  // few blocks: the first slot
 }
 
 // k_lf_loss over groups of four pixels: three 16-byte loads of rgb and of gt,
@@ -346,16 +350,14 @@ __global__ void k_lf_loss(const float* __restrict__ rgb, const float* __restrict
 // per-pixel arithmetic is that of k_lf_loss; only the summation order of the
 // partial sums differs.
 __global__ void k_lf_loss4(const float* __restrict__ rgb, const float* __restrict__ gt, const float* __restrict__ w,
-                           const __grid_constant__ ViewPix vp, const double* wsum, double* lsum,
+                           const __grid_constant__ ViewPix vp, const float2* view_k, double* lsum,
                            float* __restrict__ grad) {
   grid_wait();
   const int v = view_of_block(vp.blk, vp.n, blockIdx.x);
   const int b0 = vp.blk[v], nb = vp.blk[v + 1] - b0;
   const long long lo = vp.off[v], hi = vp.off[v + 1];
-  const long long np = hi - lo;
-  __shared__ float s_mean, s_gscale;
-  lf_view_constants(wsum, v, np, &s_mean, &s_gscale);
-  const float mean = s_mean, gscale = s_gscale;
+  const float2 vk = view_k[v];
+  const float mean = vk.x, gscale = vk.y;
   const long long g0 = (lo + 3) >> 2, g1 = hi >> 2;  // whole groups [4 g0, 4 g1)
   double acc = 0.0;  // four pixels' terms are summed in FP32
   auto one = [&](long long p) {
@@ -406,7 +408,7 @@ __global__ void k_lf_loss4(const float* __restrict__ rgb, const float* __restric
       d4[3 * g + 2] = make_float4(o[8], o[9], o[10], o[11]);
     }
   }
-  block_add_f64(acc, &lsum[v]);
+  block_add_f64(acc, &lsum[v]);  // few blocks: the first slot
 }
 
 // clear: the sums are zeroed once read (the fused backward's sums start from zero next time)
@@ -415,8 +417,13 @@ __global__ void k_lf_finish(const __grid_constant__ ViewPix vp, double* lsum, fl
   int v = threadIdx.x;
   if (v < vp.n) {
     const long long np = vp.off[v + 1] - vp.off[v];
-    loss[v] = np > 0 ? (float)(lsum[v] / (3.0 * (double)np)) : 0.f;
-    if (clear) lsum[v] = 0.0;
+    double sum = 0.0;
+#pragma unroll
+    for (unsigned k = 0; k < LF_SLOTS; ++k) sum += lsum[k * LV_MAX_VIEWS + v];
+    loss[v] = np > 0 ? (float)(sum / (3.0 * (double)np)) : 0.f;
+    if (clear)
+#pragma unroll
+      for (unsigned k = 0; k < LF_SLOTS; ++k) lsum[k * LV_MAX_VIEWS + v] = 0.0;
   }
 }
 
@@ -496,15 +503,16 @@ extern "C" lv_status lv_lf_weights(const float* gt, const int32_t* widths, const
   cudaStream_t s = (cudaStream_t)stream;
   const float gamma = lv_lf_gamma(t, p);
   // the weight sums, the loss sums a backward with the fused loss accumulates, and the counters
-  zero_async(s, w.wsum, sizeof(double) * LV_MAX_VIEWS, w.lsum, sizeof(double) * LV_MAX_VIEWS, w.hist,
-             sizeof(uint32_t) * HIST_WORDS * (size_t)n_views);
+  zero_async(s, w.wsum, sizeof(double) * LV_MAX_VIEWS, w.lsum, sizeof(double) * LF_SLOTS * LV_MAX_VIEWS, w.hist,
+             sizeof(uint32_t) * HIST_WORDS * (size_t)n_views, w.done, sizeof(uint32_t) * LV_MAX_VIEWS);
   // a block clears and adds up all the counters, so it takes several tiles once there are enough
   const int tiles = vp.tile[n_views], per = (tiles + SOBEL_BLOCKS - 1) / SOBEL_BLOCKS;
   chain(k_lf_sobel, (unsigned)((tiles + per - 1) / per), TPB, 0, s)(gt, vp, per, w.mkey, w.hist);
   const unsigned blocks = (unsigned)vp.blk[n_views];
   chain(k_lf_digit<false>, blocks, TPB, 0, s)(w.mkey, vp, w.hist, w.pick);
   chain(k_lf_digit<true>, blocks, TPB, 0, s)(w.mkey, vp, w.hist, w.pick);
-  chain(k_lf_weight, blocks, TPB, 0, s)(w.mkey, w.hist, w.pick, vp, p->eps, gamma, w.w, w.wsum, p->edge_out);
+  chain(k_lf_weight, blocks, TPB, 0, s)(w.mkey, w.hist, w.pick, vp, p->eps, gamma, w.w, w.wsum, w.view_k, w.done,
+                                       p->edge_out);
   count_launch(4);
   return cuda_check(cudaGetLastError(), "lv_lf_weights");
 }
@@ -518,12 +526,12 @@ extern "C" lv_status lv_lf_loss_from_weights(const float* rgb, const float* gt, 
   lv_status e = lf_setup(widths, heights, n_views, 990000, workspace, ws_bytes, &vp, &w);
   if (e != LV_OK) return e;
   cudaStream_t s = (cudaStream_t)stream;
-  zero_async(s, w.lsum, sizeof(double) * LV_MAX_VIEWS);
+  zero_async(s, w.lsum, sizeof(double) * LF_SLOTS * LV_MAX_VIEWS);
   // four pixels (three 16-byte words of rgb, gt and dL_drgb) per step where the buffers allow it
   const bool vec = aligned16(rgb) && aligned16(gt) && aligned16(w.w) && (!dL_drgb || aligned16(dL_drgb));
   const unsigned blocks = (unsigned)vp.blk[n_views];
-  if (vec) chain(k_lf_loss4, blocks, TPB, 0, s)(rgb, gt, w.w, vp, w.wsum, w.lsum, dL_drgb);
-  else chain(k_lf_loss, blocks, TPB, 0, s)(rgb, gt, w.w, vp, w.wsum, w.lsum, dL_drgb);
+  if (vec) chain(k_lf_loss4, blocks, TPB, 0, s)(rgb, gt, w.w, vp, w.view_k, w.lsum, dL_drgb);
+  else chain(k_lf_loss, blocks, TPB, 0, s)(rgb, gt, w.w, vp, w.view_k, w.lsum, dL_drgb);
   chain(k_lf_finish, 1, LV_MAX_VIEWS, 0, s)(vp, w.lsum, loss, false);
   count_launch(2);
   return cuda_check(cudaGetLastError(), "lv_lf_loss_from_weights");
@@ -543,13 +551,15 @@ extern "C" lv_status lv_lf_loss_finish(const int32_t* widths, const int32_t* hei
 
 namespace lv {
 lv_status lf_fused_buffers(const int32_t* widths, const int32_t* heights, int n_views, void* workspace,
-                           size_t ws_bytes, const float** w_out, const double** wsum, double** lsum) {
+                           size_t ws_bytes, const float** w_out, const double** wsum, const float2** view_k,
+                           double** lsum) {
   ViewPix vp;
   LfWs w;
   lv_status e = lf_setup(widths, heights, n_views, 990000, workspace, ws_bytes, &vp, &w);
   if (e != LV_OK) return e;
   *w_out = w.w;
   *wsum = w.wsum;
+  *view_k = w.view_k;
   *lsum = w.lsum;
   return LV_OK;
 }

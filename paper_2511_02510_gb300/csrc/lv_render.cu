@@ -1851,14 +1851,17 @@ struct StripWalk {
 // 18): per pixel dL/drgb = 2 / (3 |P_v|) * (w / <w>) * (rgb - gt), in the
 // operation order lv_lf_loss_from_weights uses, and the view's summed
 // weighted squared error (FP32 per warp item, FP64 per warp in shared memory,
-// summed per block, one global FP64 atomic per block and view).  w == nullptr:
-// not fused.
+// summed per block, one global FP64 atomic per block and view into one of
+// LF_SLOTS sums; a block is 1 to 8 warps, and with one sum a view and each view's
+// constants computed in every block 16 views took 1708 us instead of 1608).
+// w == nullptr: not fused.
 struct LfFuse {
   const float* rgb;    // [P][3] the forward's image
   const float* gt;     // [P][3]
   const float* w;      // [P] unnormalised weights (lv_lf_weights)
   const double* wsum;  // [views] their sums
-  double* lsum;        // [views] loss sums
+  const float2* view_k;  // [views] mean weight, gradient scale
+  double* lsum;        // [LF_SLOTS][LV_MAX_VIEWS] loss sums
   float* dL;           // [P][3] dL/drgb, also written out (nullable)
 };
 
@@ -2119,19 +2122,20 @@ __global__ void __launch_bounds__(bwd_warps<TS, PERSIST>() * 32, bwd_blocks<TS, 
   constexpr int NW = TS * TS / 32, CW = bwd_warps<TS, PERSIST>();
   extern __shared__ float4 smem_f4[];
   __shared__ double s_lf[CW][LV_MAX_VIEWS];  // each warp's loss sums (fused LF loss; no atomics)
-  __shared__ float s_mean[LV_MAX_VIEWS], s_gscale[LV_MAX_VIEWS];  // the fused LF loss's per-view constants
+  __shared__ float2 s_vk[PERSIST ? LV_MAX_VIEWS : 1];  // view_k, computed by a block of many items (reading it: +1.5 % with 16 views)
   if (PERSIST && sm_leave(sm_cut, n_sms, arrivals)) return;  // block-uniform
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if (lf.w) {  // grid-uniform; a warp clears and then adds to its own row only
     for (int v = lane; v < vs.n; v += 32) s_lf[warp][v] = 0.0;
-    // each view's mean weight and gradient scale, rounded from FP64 as the loss kernel rounds them,
-    // once per block (FP64 division is slow on this part)
-    for (int v = tid; v < vs.n; v += CW * 32) {
-      const double np = (double)vs.v[v].W * (double)vs.v[v].H;
-      s_mean[v] = (float)(lf.wsum[v] / np);
-      s_gscale[v] = (float)(2.0 / (3.0 * np));
+    if (PERSIST) {
+      for (int v = tid; v < vs.n; v += CW * 32) {
+        const double np = (double)vs.v[v].W * (double)vs.v[v].H;
+        s_vk[v] = make_float2((float)(lf.wsum[v] / np), (float)(2.0 / (3.0 * np)));
+      }
+      __syncthreads();
+    } else {
+      __syncwarp();
     }
-    __syncthreads();
   }
   StripWalk<true, LOOK> walk(plist, rec, slot_vox, (char*)smem_f4, warp, lane);
   for (uint32_t item = PERSIST ? next_item(work, lane) : blockIdx.x * CW + warp; item < n_items;
@@ -2162,7 +2166,8 @@ __global__ void __launch_bounds__(bwd_warps<TS, PERSIST>() * 32, bwd_blocks<TS, 
       if (dL_dT) gT = dL_dT[p];
     }
     if (lf.w) {  // grid-uniform: dL/drgb of the LF-weighted loss from the forward's image
-      const float mean = s_mean[view], gscale = s_gscale[view];
+      const float2 vk = PERSIST ? s_vk[view] : lf.view_k[view];
+      const float mean = vk.x, gscale = vk.y;
       float part = 0.f;
       if (inside) {
         const float wt = lf.w[p] / mean;
@@ -2295,7 +2300,7 @@ __global__ void __launch_bounds__(bwd_warps<TS, PERSIST>() * 32, bwd_blocks<TS, 
     for (int v = tid; v < vs.n; v += CW * 32) {
       double t = 0.0;
       for (int w = 0; w < CW; ++w) t += s_lf[w][v];
-      if (t != 0.0) atomicAdd(&lf.lsum[v], t);
+      if (t != 0.0) atomicAdd(&lf.lsum[(blockIdx.x % LF_SLOTS) * LV_MAX_VIEWS + v], t);
     }
   }
 }
@@ -3060,7 +3065,7 @@ extern "C" lv_status lv_rasterize_backward(const lv_voxels* vox, const lv_camera
   if (ws_bytes < w.bytes) { set_error("workspace %zu bytes < required %zu", ws_bytes, w.bytes); return LV_ERR_WORKSPACE; }
   if (!d_status) d_status = w.status;
   // the LF-weighted loss fused in: dL/drgb from the forward's image, the ground truth and the weights
-  LfFuse lf = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
+  LfFuse lf = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
   if (!dL_drgb) {
     if (!fwd->lf_gt || !fwd->rgb) { set_error("the fused LF loss needs lf_gt and the forward's rgb"); return LV_ERR_INVALID_ARG; }
     int32_t wd[LV_MAX_VIEWS], ht[LV_MAX_VIEWS];
@@ -3068,7 +3073,7 @@ extern "C" lv_status lv_rasterize_backward(const lv_voxels* vox, const lv_camera
       wd[v] = cams[v].width;
       ht[v] = cams[v].height;
     }
-    lv_status e = lf_fused_buffers(wd, ht, n_views, fwd->lf_workspace, fwd->lf_ws_bytes, &lf.w, &lf.wsum, &lf.lsum);
+    lv_status e = lf_fused_buffers(wd, ht, n_views, fwd->lf_workspace, fwd->lf_ws_bytes, &lf.w, &lf.wsum, &lf.view_k, &lf.lsum);
     if (e != LV_OK) return e;
     lf.rgb = fwd->rgb;
     lf.gt = fwd->lf_gt;
