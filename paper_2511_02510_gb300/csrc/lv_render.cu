@@ -851,8 +851,10 @@ __device__ __forceinline__ int64_t usable_pairs(const unsigned long long* d_coun
 //                     and lists the longer tiles;
 //   k_tile_sort       persistent blocks of 512 threads: lists of up to TS_CHUNK
 //                     pairs in one go, longer ones range of keys by range of
-//                     keys, and of those above TS_LAZY only the front, the
-//                     nearest pairs up to TS_CHUNK;
+//                     keys (as many whole bins of a histogram of the keys as
+//                     hold TS_CHUNK pairs), and of those above TS_LAZY only
+//                     the front, the nearest ranges up to TS_FRONT pairs: one
+//                     range, unless a crowded bin cut it short;
 //   k_tile_rest       the rest of those whose pixels are still open after the
 //                     composite of the sorted parts.
 // Opaque scenes seldom read a long list past its front: of eight 980 x 545
@@ -867,6 +869,7 @@ __device__ __forceinline__ int64_t usable_pairs(const unsigned long long* d_coun
 constexpr int TS_BITS = 9, TS_BINS = 1 << TS_BITS;
 constexpr int TS_THREADS = 512, TS_WARPS = TS_THREADS / 32, TS_ITEMS = 8, TS_CHUNK = TS_THREADS * TS_ITEMS;
 constexpr uint32_t TS_LAZY = 4 * TS_CHUNK;          // lists up to here are sorted whole at once
+constexpr uint32_t TS_FRONT = TS_CHUNK / 2;         // at least this many entries of the others are
 constexpr int64_t TS_LAZY_VOXELS = 1 << 19;         // and all lists of scenes up to here
 constexpr int TL_BITS = 11, TL_BINS = 1 << TL_BITS;  // key histogram of a long list
 constexpr int TW_MAX = 256, TW_ITEMS = TW_MAX / 32, TW_WARPS = 16;
@@ -1410,8 +1413,8 @@ __device__ __forceinline__ TlAt tl_ranges(uint32_t L, const uint32_t* sv, const 
 }
 
 // A long list's depth order to plist.  START: the keys are gathered first (to xk), and
-// above `lazy` entries the work stops after one range; else it goes on from the progress
-// of such a start.
+// above `lazy` entries the work stops at the first range's end past TS_FRONT entries; else
+// it goes on from the progress of such a start.
 template <bool START>
 __device__ __noinline__ void tl_order(uint32_t lo, uint32_t L, uint32_t lazy, const uint32_t* sv_all,
                          uint32_t* xk_all, const uint32_t* s_dkey, TileProg* prog,
@@ -1457,7 +1460,7 @@ __device__ __noinline__ void tl_order(uint32_t lo, uint32_t L, uint32_t lazy, co
   }
   const TlAt end = tl_ranges(L, sv, xk, done, cur, kmax, [&](uint32_t at, uint32_t m) {
     ts_write((int)m, tb, rec_bb, plist + at);
-    return front;
+    return front && at + m >= TS_FRONT;
   });
   if (t == 0) {
     prog->done = end.done;
