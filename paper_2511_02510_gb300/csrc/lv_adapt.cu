@@ -1380,10 +1380,10 @@ extern "C" lv_status lv_subdivide_apply(const lv_voxels* in, const lv_subdiv_par
   const int64_t warps = (n + 31) / 32 + (max_children + 31) / 32;
   const unsigned grid = (unsigned)((warps * 32 + TPB - 1) / TPB);
 #define LV_SUB(DT, ST)                                                                                                 \
-  launch(k_sd_write<DT, ST>, grid, TPB, 0, s)(n, max_children, w.surv, w.surv_pos, w.sel_list, w.totals, w.st,           \
-                                          (const float4*)in->geom, in->level, (const DT*)in->density,                \
-                                          (const ST*)in->sh, (float4*)out->geom, (uint8_t*)out->level,               \
-                                          (DT*)out->density, (ST*)out->sh, as)
+  launch(k_sd_write<DT, ST>, grid, TPB, 0, s)(n, max_children, w.surv, w.surv_pos, w.sel_list, w.totals, w.st,         \
+                                              (const float4*)in->geom, in->level, (const DT*)in->density,            \
+                                              (const ST*)in->sh, (float4*)out->geom, (uint8_t*)out->level,           \
+                                              (DT*)out->density, (ST*)out->sh, as)
   if (in->density_dtype == LV_F32 && in->sh_dtype == LV_F32) LV_SUB(float, float);
   else if (in->density_dtype == LV_F16 && in->sh_dtype == LV_F32) LV_SUB(__half, float);
   else if (in->density_dtype == LV_F32 && in->sh_dtype == LV_BF16) LV_SUB(float, __nv_bfloat16);
@@ -1431,10 +1431,11 @@ extern "C" lv_status lv_subdivide_apply_inplace(const lv_voxels* vox, int64_t ca
 #define LV_IP(DT, ST)                                                                                                  \
   do {                                                                                                                \
     if (grid > 0)                                                                                                     \
-      launch(k_ip_children<DT, ST>, grid, TPB, 0, s)(n, w.sel_list, holes, w.totals, w.st, (float4*)vox->geom,            \
-                                                 (uint8_t*)vox->level, (DT*)vox->density, (ST*)vox->sh, as);          \
-    chain(k_ip_tail<DT, ST>, tail_grid, TPB, 0, s)(n, holes, w.totals, w.st, (float4*)vox->geom, (uint8_t*)vox->level,   \
-                                                (DT*)vox->density, (ST*)vox->sh, as);                                 \
+      launch(k_ip_children<DT, ST>, grid, TPB, 0, s)(n, w.sel_list, holes, w.totals, w.st, (float4*)vox->geom,        \
+                                                     (uint8_t*)vox->level, (DT*)vox->density, (ST*)vox->sh, as);      \
+    auto tail = grid > 0 ? chain(k_ip_tail<DT, ST>, tail_grid, TPB, 0, s)                                             \
+                         : launch(k_ip_tail<DT, ST>, tail_grid, TPB, 0, s);                                           \
+    tail(n, holes, w.totals, w.st, (float4*)vox->geom, (uint8_t*)vox->level, (DT*)vox->density, (ST*)vox->sh, as);    \
   } while (0)
   if (vox->density_dtype == LV_F32 && vox->sh_dtype == LV_F32) LV_IP(float, float);
   else if (vox->density_dtype == LV_F16 && vox->sh_dtype == LV_F32) LV_IP(__half, float);

@@ -30,9 +30,9 @@ struct ViewPix {
 };
 
 // The percentile is selected by the magnitudes' bits, digit by digit from the
-// top: 14 bits (the highest, the sign, is always 0), then 9 and 9.  The first digit is wide so that the few octaves an image's
-// gradients span fall into hundreds of counters: with 11 bits about 24 counters
-// took all the shared-memory atomics.  It is counted where the magnitudes are
+// top: 14 bits (the highest, the sign, is always 0), then 9 and 9.  The first digit is
+// wide so that the few octaves an image's gradients span fall into hundreds of
+// counters: with 11 bits about 24 counters took all the shared-memory atomics.  It is counted where the magnitudes are
 // computed, and no group array is read, as a block's pixels are one view's.
 constexpr int D1_SHIFT = 18, D1_BINS = 1 << (31 - D1_SHIFT);
 constexpr int D2_SHIFT = 9, D2_BINS = 1 << (D1_SHIFT - D2_SHIFT);

@@ -185,8 +185,8 @@ constexpr int OS_MATCH_MAX_GROUPS = 16;          // distinct digits in a warp's 
 constexpr int OS_HIST_THREADS = 256;
 
 // Tile shape of the pass kernel: 512 threads (4096 items, about 52 KB of
-// static shared memory) for 32-bit keys, three blocks an SM at 42 registers (two at
-// 64: 325 us a pass over 38M pairs, against 278), 256 threads (2048 items, about
+// static shared memory) for 32-bit keys, three blocks an SM at 40 registers and 144
+// bytes spilled (two at 64: 325 us a pass over 38M pairs, against 278), 256 threads (2048 items, about
 // 36 KB) for 64-bit keys, whose staged keys are twice as large, four blocks.
 // Threads d < RADIX look after digit d.
 template <typename K>

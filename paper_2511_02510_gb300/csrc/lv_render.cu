@@ -137,10 +137,12 @@ struct FwdWs {
   unsigned long long* counters;  // [0] pairs, [1] slots
   uint32_t* cnt;                 // [items] tiles covered (visible: not 0)
   uint2* rect;                   // [items] of visible items: (tx0 | tx1 << 16, ty0 | ty1 << 16)
-  uint2* pbox;                   // [items] of visible items: conservative pixel box (x0 | x1 << 16, y0 | y1 << 16), [x0, x1)
+  uint2* pbox;                   // [items] of visible items: conservative pixel box (x0 | x1 << 16,
+                                 // y0 | y1 << 16), [x0, x1)
   uint32_t* dkey;                // [items] of visible items: order key of z_centre
   uint32_t* slot;                // [items] of visible items: render slot
-  unsigned long long* blk_pairs; // [blocks of 256 voxels x views, view-major] pairs, then the block's first within its group
+  unsigned long long* blk_pairs; // [blocks of 256 voxels x views, view-major] pairs, then the block's first
+                                 // within its group
   uint32_t* blk_slots;           // the same for slots
   unsigned long long* grp_pairs; // totals of groups of BO_GROUP blocks
   uint32_t* grp_slots;
@@ -173,6 +175,7 @@ struct FwdWs {
 };
 
 constexpr int BIN_THREADS = 256;  // voxels per block of k_bin and k_emit
+constexpr int BO_THREADS = 1024, BO_ITEMS = 4, BO_GROUP = BO_THREADS * BO_ITEMS;  // blocks per group of their offsets
 static int64_t bin_blocks(int64_t n) { return (n + BIN_THREADS - 1) / BIN_THREADS; }
 
 static int tile_bits(int64_t tiles) {
@@ -195,8 +198,8 @@ static FwdWs carve_fwd(void* base, int64_t n, int nv, int64_t tiles, int64_t pix
   w.slot = c.take<uint32_t>(items);
   w.blk_pairs = c.take<unsigned long long>(bin_blocks(n) * nv);
   w.blk_slots = c.take<uint32_t>(bin_blocks(n) * nv);
-  w.grp_pairs = c.take<unsigned long long>(bin_blocks(n) * nv / 4096 + 1);
-  w.grp_slots = c.take<uint32_t>(bin_blocks(n) * nv / 4096 + 1);
+  w.grp_pairs = c.take<unsigned long long>(bin_blocks(n) * nv / BO_GROUP + 1);
+  w.grp_slots = c.take<uint32_t>(bin_blocks(n) * nv / BO_GROUP + 1);
   w.rec_bb = c.take<uint2>(items);
   w.slot_vox = c.take<uint32_t>(items);
   w.s_dkey = c.take<uint32_t>(items);
@@ -380,14 +383,13 @@ __device__ __forceinline__ uint32_t bin_item(const DevView& c, int ts, const flo
 // offsets, scanned by three more launches, cost 28 bytes of traffic an item
 // (48M items: 290 us), and only visible items write anything but their count
 // (48M items: 854 -> 607 us with that, the geometry read once, the usual case's
-// projections without a test per corner and six blocks an SM; 2M items: 39 -> 31 us).
-__global__ void __launch_bounds__(BIN_THREADS, 6) k_bin(const float4* __restrict__ geom, int64_t n, int64_t blocks,
-                                                     const __grid_constant__ ViewSet vs, uint32_t* __restrict__ cnt,
-                                                     uint2* __restrict__ rect, uint2* __restrict__ pbox,
-                                                     uint32_t* __restrict__ dkey,
-                                                     unsigned long long* __restrict__ blk_pairs,
-                                                     uint32_t* __restrict__ blk_slots, float* z_min,
-                                                     float* delta_min, uint8_t* seen, const ZeroRanges zr) {
+// projections without a test per corner and six blocks an SM, for which 56 bytes a
+// thread are spilled; 2M items: 39 -> 31 us).
+__global__ void __launch_bounds__(BIN_THREADS, 6)
+    k_bin(const float4* __restrict__ geom, int64_t n, int64_t blocks, const __grid_constant__ ViewSet vs,
+          uint32_t* __restrict__ cnt, uint2* __restrict__ rect, uint2* __restrict__ pbox, uint32_t* __restrict__ dkey,
+          unsigned long long* __restrict__ blk_pairs, uint32_t* __restrict__ blk_slots, float* z_min,
+          float* delta_min, uint8_t* seen, const ZeroRanges zr) {
   grid_begin();
   __shared__ unsigned long long s_pairs[BIN_THREADS / 32];
   __shared__ uint32_t s_slots[BIN_THREADS / 32];
@@ -434,7 +436,6 @@ __global__ void __launch_bounds__(BIN_THREADS, 6) k_bin(const float4* __restrict
 // counters[0] and [1] (zero before).  k_emit sums the groups before its own: up
 // to 1M items there is one group, at 48M items 46.  (One block over all entries
 // took 196 us for 48M items, 4 us a round of 4096.)
-constexpr int BO_THREADS = 1024, BO_ITEMS = 4, BO_GROUP = BO_THREADS * BO_ITEMS;
 __global__ void __launch_bounds__(BO_THREADS) k_block_offsets(unsigned long long* pairs,
                                                               uint32_t* slots, int64_t m,
                                                               unsigned long long* grp_pairs,
@@ -561,7 +562,7 @@ __device__ __forceinline__ void bf16_pair(uint32_t w, float* c) {
 // asked for, and only as far as the degree needs, to keep k_emit's registers few: it is bound by the
 // latency of its scattered reads and writes, so warps in flight count for more than loads in flight per
 // warp.  Eight views of 6M voxels, FP16 and BF16: 1474 us at 5 blocks an SM, 1362 at 6, 1271 at 8 (32
-// registers), 1100 with the records stored in whole sectors; one view of 2M, FP32: 97, 91, 97 us, and 86.
+// registers and 16 bytes spilled), 1100 with the records stored in whole sectors; one view of 2M, FP32: 97, 91, 97 us, and 86.
 template <int PER, typename F>
 __device__ __forceinline__ void sh_add(int k, const F (&c)[PER], int nb, const float* Y, float* raw) {
 #pragma unroll
@@ -666,25 +667,14 @@ __device__ __forceinline__ void unit_dir(float rx, float ry, float rz, float* d)
 // and h | 8 corner densities | clamped SH colour and 1/(2h)), the slot's order
 // key, and the colour-gradient scratch (cleared; w = clamp mask).
 template <typename DT, typename ST>
-__global__ void __launch_bounds__(BIN_THREADS, sizeof(ST) == 4 ? 6 : 8) k_emit(const float4* __restrict__ geom, const DT* __restrict__ dens,
-                                              const ST* __restrict__ sh, int sh_nb, int64_t n,
-                                              const __grid_constant__ ViewSet vs, const uint32_t* cnt,
-                                              const uint2* rect,
-                                              const uint2* pbox, uint2* rec_bb,
-                                              uint32_t* slot_vox,
-                                              const uint32_t* dkey,
-                                              uint32_t* slot, int64_t blocks,
-                                              const unsigned long long* blk_pairs,
-                                              const uint32_t* blk_slots,
-                                              const unsigned long long* grp_pairs,
-                                              const uint32_t* grp_slots,
-                                              const unsigned long long* counters, int64_t pair_cap,
-                                              uint32_t* pair_tile, uint32_t* pair_slot,
-                                              int32_t* status, uint2* ranges, int64_t tiles,
-                                              const SortCountTargets sc, int passes,
-                                              float4* rec,
-                                              float4* d_rgb, uint32_t* s_dkey,
-                                              const uint32_t* __restrict__ vidx) {
+__global__ void __launch_bounds__(BIN_THREADS, sizeof(ST) == 4 ? 6 : 8)
+    k_emit(const float4* __restrict__ geom, const DT* __restrict__ dens, const ST* __restrict__ sh, int sh_nb,
+           int64_t n, const __grid_constant__ ViewSet vs, const uint32_t* cnt, const uint2* rect, const uint2* pbox,
+           uint2* rec_bb, uint32_t* slot_vox, const uint32_t* dkey, uint32_t* slot, int64_t blocks,
+           const unsigned long long* blk_pairs, const uint32_t* blk_slots, const unsigned long long* grp_pairs,
+           const uint32_t* grp_slots, const unsigned long long* counters, int64_t pair_cap, uint32_t* pair_tile,
+           uint32_t* pair_slot, int32_t* status, uint2* ranges, int64_t tiles, const SortCountTargets sc, int passes,
+           float4* rec, float4* d_rgb, uint32_t* s_dkey, const uint32_t* __restrict__ vidx) {
   grid_begin();
   // Block b covers 256 consecutive voxels of view b % views, so the blocks of
   // all views of one voxel range run side by side: a voxel's SH row comes
@@ -861,8 +851,8 @@ __device__ __forceinline__ int64_t usable_pairs(const unsigned long long* d_coun
 // views of 6M voxels with tile 32 (lists of up to 68,000 pairs, 38M in all) hardly
 // a tile does (with fronts of 2048 pairs 2 to 5 % of them, and 480 us for the rest
 // and the resumed composite).  Sorting every list whole, in chunks merged
-// afterwards, took 4.7 ms of those views' 8.2 ms; their fronts take 0.41 ms.  Lists of a few chunks are sorted whole: where
-// their pixels stay open, the composite in two launches costs more than the sort
+// afterwards, took 4.7 ms of those views' 8.2 ms; their fronts take 0.41 ms.  Lists
+// of a few chunks are sorted whole: where their pixels stay open, the composite in two launches costs more than the sort
 // saves (one 1237 x 822 view of 2M voxels, lists of up to 7,800 pairs: 217 + 151 us
 // against 297 us).  Scenes of up to TS_LAZY_VOXELS seldom have longer lists, and go
 // without the two launches that the rest takes (6 us when there is none).
@@ -1011,17 +1001,10 @@ struct TileBox {
 };
 
 // ---- short lists: one warp each, TW_WARPS tiles per block
-__global__ void __launch_bounds__(TW_WARPS * 32, 2) k_tile_sort_warp(const uint32_t* tvals,
-                                                                    const uint32_t* s_dkey,
-                                                                    const unsigned long long* d_count,
-                                                                    int64_t cap, bool ranges_ready, int64_t tiles,
-                                                                    uint32_t* ranges,
-                                                                    const TileOrder order,
-                                                                    uint32_t* ready,
-                                                                    TileProg* prog,
-                                                                    const __grid_constant__ ViewSet vs,
-                                                                    const uint2* rec_bb,
-                                                                    uint2* plist) {
+__global__ void __launch_bounds__(TW_WARPS * 32, 2)
+    k_tile_sort_warp(const uint32_t* tvals, const uint32_t* s_dkey, const unsigned long long* d_count, int64_t cap,
+                     bool ranges_ready, int64_t tiles, uint32_t* ranges, const TileOrder order, uint32_t* ready,
+                     TileProg* prog, const __grid_constant__ ViewSet vs, const uint2* rec_bb, uint2* plist) {
   grid_begin();
   extern __shared__ __align__(16) unsigned char tw_raw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1471,16 +1454,10 @@ __device__ __noinline__ void tl_order(uint32_t lo, uint32_t L, uint32_t lazy, co
 }
 
 // Persistent blocks over the long tiles, then over the medium ones.
-__global__ void __launch_bounds__(TS_THREADS, 2) k_tile_sort(const uint32_t* tvals,
-                                                            uint32_t* xk,
-                                                            const uint32_t* s_dkey,
-                                                            const uint32_t* ranges,
-                                                            const TileOrder order,
-                                                            unsigned int* work,
-                                                            uint32_t* ready, TileProg* prog, uint32_t lazy,
-                                                            const __grid_constant__ ViewSet vs,
-                                                            const uint2* rec_bb,
-                                                            uint2* plist) {
+__global__ void __launch_bounds__(TS_THREADS, 2)
+    k_tile_sort(const uint32_t* tvals, uint32_t* xk, const uint32_t* s_dkey, const uint32_t* ranges,
+                const TileOrder order, unsigned int* work, uint32_t* ready, TileProg* prog, uint32_t lazy,
+                const __grid_constant__ ViewSet vs, const uint2* rec_bb, uint2* plist) {
   grid_begin();
   TileLongSmem& M = ts_smem();
   static_assert(TILE_CLASS_SHORT == 5 && TS_CHUNK == 4096 && TW_MAX == 256, "the length classes");
@@ -1506,16 +1483,10 @@ __global__ void __launch_bounds__(TS_THREADS, 2) k_tile_sort(const uint32_t* tva
 }
 
 // Persistent blocks over the listed long tiles: what k_tile_sort left unsorted.
-__global__ void __launch_bounds__(TS_THREADS, 2) k_tile_rest(const uint32_t* tvals,
-                                                            uint32_t* xk,
-                                                            const uint32_t* ranges,
-                                                            const uint32_t* list,
-                                                            const unsigned int* n_list,
-                                                            unsigned int* work,
-                                                            uint32_t* ready, TileProg* prog,
-                                                            const __grid_constant__ ViewSet vs,
-                                                            const uint2* rec_bb,
-                                                            uint2* plist) {
+__global__ void __launch_bounds__(TS_THREADS, 2)
+    k_tile_rest(const uint32_t* tvals, uint32_t* xk, const uint32_t* ranges, const uint32_t* list,
+                const unsigned int* n_list, unsigned int* work, uint32_t* ready, TileProg* prog,
+                const __grid_constant__ ViewSet vs, const uint2* rec_bb, uint2* plist) {
   grid_begin();
   TileLongSmem& M = ts_smem();
   const unsigned int total = *n_list;
@@ -1889,8 +1860,8 @@ struct Front {
 // and atomic, 8 warps a block: 97 us against 88 on an opaque view, 578 against 559 on an
 // open one, tile 32); the persistent backward, whose strips differ more, takes single items.
 // As many blocks share an SM as leave a thread 64 (forward) and 72 (backward)
-// registers: with fewer the march spills, with more too few warps hide the
-// memory's latency.  1237 x 822 views of 2M voxels, opaque and open, tile 16, forward:
+// registers: with fewer the march spills (at these the exact-segment forward of
+// tile 8, 28 bytes), with more too few warps hide the memory's latency.  1237 x 822 views of 2M voxels, opaque and open, tile 16, forward:
 // 78 and 494 us at 72 registers, 74 and 490 at 64, 77 and 499 at 56; backward 115 and 714 us
 // at 80, 109 and 684 at 72, 115 and 715 at 64.  Looking ahead takes 8 more of them.
 template <int TS, bool PERSIST, bool LOOK>
@@ -1903,15 +1874,11 @@ template <int TS, bool PERSIST, bool LOOK>
 __host__ __device__ constexpr int bwd_blocks() { return (PERSIST || LOOK ? 24 : 28) / bwd_warps<TS, PERSIST>(); }
 
 template <int TS, bool SEG, bool PERSIST, bool LOOK>
-__global__ void __launch_bounds__(fwd_warps<TS, PERSIST, LOOK>() * 32, fwd_blocks<TS, PERSIST, LOOK>()) k_fwd(const __grid_constant__ ViewSet vs, const uint32_t* ranges,
-                                                const uint2* plist, const float4* rec,
-                                                const uint32_t* slot_vox, float t_stop,
-                                                float* rgb, float* depth,
-                                                float* T_out, uint32_t* n_contrib,
-                                                uint32_t* n_samples, float* tau_out,
-                                                unsigned long long* wmax, unsigned int* work,
-                                                uint32_t n_items, int sm_cut, int n_sms, unsigned int* arrivals,
-                                                const TileOrder order, const Front fr) {
+__global__ void __launch_bounds__(fwd_warps<TS, PERSIST, LOOK>() * 32, fwd_blocks<TS, PERSIST, LOOK>())
+    k_fwd(const __grid_constant__ ViewSet vs, const uint32_t* ranges, const uint2* plist, const float4* rec,
+          const uint32_t* slot_vox, float t_stop, float* rgb, float* depth, float* T_out, uint32_t* n_contrib,
+          uint32_t* n_samples, float* tau_out, unsigned long long* wmax, unsigned int* work, uint32_t n_items,
+          int sm_cut, int n_sms, unsigned int* arrivals, const TileOrder order, const Front fr) {
   grid_wait();
   constexpr int NW = TS * TS / 32, CW = fwd_warps<TS, PERSIST, LOOK>();
   constexpr bool RESUME = PERSIST && LOOK;  // the second launch, over the open tiles
@@ -2111,21 +2078,19 @@ __device__ __forceinline__ float warp_reduce16(float* v, int lane) {
 // per-record gradients (8 corners + colour) are
 // reduced over the warp and sent with three 16-byte global reductions.
 template <int TS, bool SEG, bool PERSIST, bool LOOK>
-__global__ void __launch_bounds__(bwd_warps<TS, PERSIST>() * 32, bwd_blocks<TS, PERSIST, LOOK>()) k_bwd(const __grid_constant__ ViewSet vs, const uint32_t* __restrict__ ranges,
-                                                const uint2* __restrict__ plist, const float4* __restrict__ rec,
-                                                const uint32_t* __restrict__ slot_vox, const float* __restrict__ T_fwd,
-                                                const float* __restrict__ tau_in,
-                                                const uint32_t* __restrict__ n_contrib,
-                                                const float* __restrict__ dL_drgb, const float* __restrict__ dL_ddepth,
-                                                const float* __restrict__ dL_dT, float* __restrict__ d_density,
-                                                float4* __restrict__ d_rgb, unsigned int* work, uint32_t n_items,
-                                                int sm_cut, int n_sms, unsigned int* arrivals, const TileOrder order,
-                                                const LfFuse lf) {
+__global__ void __launch_bounds__(bwd_warps<TS, PERSIST>() * 32, bwd_blocks<TS, PERSIST, LOOK>())
+    k_bwd(const __grid_constant__ ViewSet vs, const uint32_t* __restrict__ ranges, const uint2* __restrict__ plist,
+          const float4* __restrict__ rec, const uint32_t* __restrict__ slot_vox, const float* __restrict__ T_fwd,
+          const float* __restrict__ tau_in, const uint32_t* __restrict__ n_contrib, const float* __restrict__ dL_drgb,
+          const float* __restrict__ dL_ddepth, const float* __restrict__ dL_dT, float* __restrict__ d_density,
+          float4* __restrict__ d_rgb, unsigned int* work, uint32_t n_items, int sm_cut, int n_sms,
+          unsigned int* arrivals, const TileOrder order, const LfFuse lf) {
   grid_wait();
   constexpr int NW = TS * TS / 32, CW = bwd_warps<TS, PERSIST>();
   extern __shared__ float4 smem_f4[];
   __shared__ double s_lf[CW][LV_MAX_VIEWS];  // each warp's loss sums (fused LF loss; no atomics)
-  __shared__ float2 s_vk[PERSIST ? LV_MAX_VIEWS : 1];  // view_k, computed by a block of many items (reading it: +1.5 % with 16 views)
+  // view_k, computed by a block of many items (reading it there: +1.5 % with 16 views)
+  __shared__ float2 s_vk[PERSIST ? LV_MAX_VIEWS : 1];
   if (PERSIST && sm_leave(sm_cut, n_sms, arrivals)) return;  // block-uniform
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if (lf.w) {  // grid-uniform; a warp clears and then adds to its own row only
@@ -2316,11 +2281,10 @@ __global__ void __launch_bounds__(bwd_warps<TS, PERSIST>() * 32, bwd_blocks<TS, 
 // views; the 32 rows leave through shared memory as coalesced 16-byte stores
 // (row stride 49 floats: conflict-free per lane).  With `accumulate`, warps
 // without any visible voxel touch nothing.
-__global__ void __launch_bounds__(128) k_sh_bwd(const float4* __restrict__ rec, int sh_nb, int64_t n,
-                                                const __grid_constant__ ViewSet vs,
-                                                const uint32_t* __restrict__ cnt, const uint32_t* __restrict__ slot,
-                                                float4* d_rgb, float* d_sh,
-                                                int accumulate) {
+__global__ void __launch_bounds__(128)
+    k_sh_bwd(const float4* __restrict__ rec, int sh_nb, int64_t n, const __grid_constant__ ViewSet vs,
+             const uint32_t* __restrict__ cnt, const uint32_t* __restrict__ slot, float4* d_rgb, float* d_sh,
+             int accumulate) {
   grid_wait();
   constexpr int RS = 49;
   __shared__ float s_rows[4][32 * RS];
@@ -2786,7 +2750,8 @@ static void launch_tile_sort(const FwdWs& w, const ViewSet& vs, int64_t n, int64
   const uint32_t* sv = w.tile_slots;
   const unsigned wblocks = (unsigned)((tiles + TW_WARPS - 1) / TW_WARPS);
   chain(k_tile_sort_warp, wblocks, TW_WARPS * 32, sizeof(TileSortWarpSmem), s)(
-      sv, w.s_dkey, w.counters, pair_cap, ready, tiles, w.ranges, tile_order(w, tiles), w.ready, w.prog, vs, w.rec_bb, w.plist);
+      sv, w.s_dkey, w.counters, pair_cap, ready, tiles, w.ranges, tile_order(w, tiles), w.ready, w.prog, vs, w.rec_bb,
+      w.plist);
   count_launch(1);
   if (n <= TW_MAX) return;  // a tile lists a voxel once: every list is short
   chain(k_tile_sort, (unsigned)nb, TS_THREADS, sizeof(TileLongSmem), s)(
@@ -2934,20 +2899,19 @@ extern "C" lv_status lv_rasterize_forward(const lv_voxels* vox, const lv_camera*
     const int64_t blocks = bin_blocks(n);
     const unsigned item_blocks = (unsigned)(blocks * n_views);  // (voxel range, view) blocks
     const unsigned bo_blocks = (unsigned)((blocks * n_views + BO_GROUP - 1) / BO_GROUP);
-    launch(k_bin, item_blocks, BIN_THREADS, 0, s)((const float4*)vox->geom, n, blocks, vs, w.cnt, w.rect, w.pbox, w.dkey,
-                                              w.blk_pairs, w.blk_slots, out->z_min, out->delta_min, out->seen, zr);
+    launch(k_bin, item_blocks, BIN_THREADS, 0, s)(
+        (const float4*)vox->geom, n, blocks, vs, w.cnt, w.rect, w.pbox, w.dkey, w.blk_pairs, w.blk_slots, out->z_min,
+        out->delta_min, out->seen, zr);
     if (out->stats_event) cudaEventRecord((cudaEvent_t)out->stats_event, s);  // statistics final
     auto offsets = out->stats_event ? launch(k_block_offsets, bo_blocks, BO_THREADS, 0, s)
                                     : chain(k_block_offsets, bo_blocks, BO_THREADS, 0, s);
     offsets(w.blk_pairs, w.blk_slots, blocks * n_views, w.grp_pairs, w.grp_slots, w.counters);
     const int nb = (vox->sh_degree + 1) * (vox->sh_degree + 1);
-#define LV_EMIT(DT, ST)                                                                                             \
-  chain(k_emit<DT, ST>, item_blocks, BIN_THREADS, 0, s)((const float4*)vox->geom, (const DT*)vox->density, (const ST*)vox->sh, \
-                                             nb, n, vs, w.cnt, w.rect, w.pbox, w.rec_bb, w.slot_vox, w.dkey,          \
-                                             w.slot, blocks, w.blk_pairs, w.blk_slots, w.grp_pairs, w.grp_slots,     \
-                                             w.counters, pair_capacity, w.k0, w.v0, d_status,         \
-                                             (uint2*)w.ranges, tiles, sc, passes, w.rec, w.d_rgb, w.s_dkey,   \
-                                             vox->vidx)
+#define LV_EMIT(DT, ST)                                                                                              \
+  chain(k_emit<DT, ST>, item_blocks, BIN_THREADS, 0, s)(                                                             \
+      (const float4*)vox->geom, (const DT*)vox->density, (const ST*)vox->sh, nb, n, vs, w.cnt, w.rect, w.pbox,       \
+      w.rec_bb, w.slot_vox, w.dkey, w.slot, blocks, w.blk_pairs, w.blk_slots, w.grp_pairs, w.grp_slots, w.counters,  \
+      pair_capacity, w.k0, w.v0, d_status, (uint2*)w.ranges, tiles, sc, passes, w.rec, w.d_rgb, w.s_dkey, vox->vidx)
     if (vox->density_dtype == LV_F32 && vox->sh_dtype == LV_F32) LV_EMIT(float, float);
     else if (vox->density_dtype == LV_F16 && vox->sh_dtype == LV_F32) LV_EMIT(__half, float);
     else if (vox->density_dtype == LV_F32 && vox->sh_dtype == LV_BF16) LV_EMIT(float, __nv_bfloat16);

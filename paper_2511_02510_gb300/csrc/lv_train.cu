@@ -262,7 +262,8 @@ extern "C" lv_status lv_transmittance_loss(const float* T, int64_t n_pix, float 
   cudaMemsetAsync(w.acc, 0, sizeof(double), s);
   if (n_pix > 0)
     launch(k_tc, grid_for(n_pix), TPB, 0, s)(T, n_pix, weight, 1.0f / (float)n_pix, dL_dT, accumulate, w.acc);
-  chain(k_train_finish, 1, 32, 0, s)(w.acc, n_pix > 0 ? (double)weight / (double)n_pix : 0.0, loss);
+  auto last = n_pix > 0 ? chain(k_train_finish, 1, 32, 0, s) : launch(k_train_finish, 1, 32, 0, s);
+  last(w.acc, n_pix > 0 ? (double)weight / (double)n_pix : 0.0, loss);
   count_launch(n_pix > 0 ? 2 : 1);
   return cuda_check(cudaGetLastError(), "lv_transmittance_loss");
 }
@@ -311,11 +312,26 @@ extern "C" lv_status lv_adam_voxels(int64_t n, void* density, lv_dtype density_d
     }
   }
   if (tv_loss) {
-    chain(k_train_finish, 1, 32, 0, s)(tv_acc, n > 0 ? (double)p->tv_weight / (double)n : 0.0, tv_loss);
+    auto last = n > 0 ? chain(k_train_finish, 1, 32, 0, s) : launch(k_train_finish, 1, 32, 0, s);
+    last(tv_acc, n > 0 ? (double)p->tv_weight / (double)n : 0.0, tv_loss);
     count_launch(1);
   }
   return cuda_check(cudaGetLastError(), "lv_adam_voxels");
 }
+
+namespace {
+// whole words, then the ragged end (the call's first kernel when there is no whole word)
+template <typename P>
+void adam_array(int64_t count, void* param, const float* grad, float* m, float* v, const AdamK& k, cudaStream_t s) {
+  const int64_t n4 = count / 4, first = 4 * n4;
+  if (n4)
+    launch(k_adam_flat<P>, grid_for(n4), TPB, 0, s)(n4, (P*)param, (const float4*)grad, (float4*)m, (float4*)v, k);
+  if (first < count) {
+    auto tail = n4 ? chain(k_adam_tail<P>, 1, 32, 0, s) : launch(k_adam_tail<P>, 1, 32, 0, s);
+    tail(first, count, (P*)param, grad, m, v, k);
+  }
+}
+}  // namespace
 
 extern "C" lv_status lv_adam_array(int64_t count, void* param, lv_dtype dtype, const float* grad, float* m, float* v,
                                    float lr, const lv_adam_params* p, void* stream) {
@@ -329,20 +345,9 @@ extern "C" lv_status lv_adam_array(int64_t count, void* param, lv_dtype dtype, c
   if (count == 0) return LV_OK;
   cudaStream_t s = (cudaStream_t)stream;
   const AdamK k = make_adam(lr, p);
-  const int64_t n4 = count / 4, first = 4 * n4;
-  if (dtype == LV_F32) {
-    if (n4) launch(k_adam_flat<float>, grid_for(n4), TPB, 0, s)(n4, (float*)param, (const float4*)grad, (float4*)m,
-                                                           (float4*)v, k);
-    if (first < count) chain(k_adam_tail<float>, 1, 32, 0, s)(first, count, (float*)param, grad, m, v, k);
-  } else if (dtype == LV_F16) {
-    if (n4) launch(k_adam_flat<__half>, grid_for(n4), TPB, 0, s)(n4, (__half*)param, (const float4*)grad, (float4*)m,
-                                                            (float4*)v, k);
-    if (first < count) chain(k_adam_tail<__half>, 1, 32, 0, s)(first, count, (__half*)param, grad, m, v, k);
-  } else {
-    if (n4) launch(k_adam_flat<__nv_bfloat16>, grid_for(n4), TPB, 0, s)(n4, (__nv_bfloat16*)param, (const float4*)grad,
-                                                                    (float4*)m, (float4*)v, k);
-    if (first < count) chain(k_adam_tail<__nv_bfloat16>, 1, 32, 0, s)(first, count, (__nv_bfloat16*)param, grad, m, v, k);
-  }
+  if (dtype == LV_F32) adam_array<float>(count, param, grad, m, v, k, s);
+  else if (dtype == LV_F16) adam_array<__half>(count, param, grad, m, v, k, s);
+  else adam_array<__nv_bfloat16>(count, param, grad, m, v, k, s);
   count_launch(2);
   return cuda_check(cudaGetLastError(), "lv_adam_array");
 }
